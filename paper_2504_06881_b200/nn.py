@@ -17,6 +17,13 @@ import torch.nn as nn
 from . import tconv
 
 
+def _emit_winners(recording, *tensors):
+    """Whether a forward has to leave the winners a backward will need.  `recording` is
+    ``torch.is_grad_enabled()`` where the layer was called: inside a Function's forward the grad mode is
+    always off, and parameters keep ``requires_grad`` under ``torch.no_grad``."""
+    return recording and any(t is not None and t.requires_grad for t in tensors)
+
+
 class TropicalConvFn(torch.autograd.Function):
     """y = tconv_forward(x, w, w2, alpha, beta, bias); backward = tconv_backward with the stored winners.
 
@@ -32,7 +39,7 @@ class TropicalConvFn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, w2, alpha, beta, bias, geom):
-        mode, chan, dtype, stride, pad, dil = geom
+        mode, chan, dtype, stride, pad, dil, recording = geom
         dt = tconv.TORCH_DTYPE[dtype]
         N, C, H, W = x.shape
         K, _, R, S = w.shape
@@ -49,7 +56,7 @@ class TropicalConvFn(torch.autograd.Function):
         al = alpha.detach().float().contiguous() if alpha is not None else None
         be = beta.detach().float().contiguous() if beta is not None else None
         bi = bias.detach().float().contiguous() if bias is not None else None
-        need_grad = any(t is not None and t.requires_grad for t in (x, w, w2, alpha, beta, bias))
+        need_grad = _emit_winners(recording, x, w, w2, alpha, beta, bias)
         ev = TropicalConvFn.events
         if ev is not None:
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -273,7 +280,7 @@ class TropicalConv2d(nn.Module):
                 beta = -alpha
             elif self.params == "fixed":
                 alpha, beta = self.alpha_fixed, self.beta_fixed
-        geom = (self.mode, self.chan, self.dtype, self.stride, self.padding, self.dilation)
+        geom = (self.mode, self.chan, self.dtype, self.stride, self.padding, self.dilation, torch.is_grad_enabled())
         return self.FN.apply(x, self.weight, self.weight2, alpha, beta, self.bias, geom)
 
 
@@ -343,7 +350,7 @@ class TropicalDepthwiseFn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, w2, alpha, beta, bias, geom):
-        mode, dtype, stride, pad, dil = geom
+        mode, dtype, stride, pad, dil, recording = geom
         dt = tconv.TORCH_DTYPE[dtype]
         N, C, H, W = x.shape
         _, R, S = w.shape
@@ -355,7 +362,7 @@ class TropicalDepthwiseFn(torch.autograd.Function):
         al = alpha.detach().float().contiguous() if alpha is not None else None
         be = beta.detach().float().contiguous() if beta is not None else None
         bi = bias.detach().float().contiguous() if bias is not None else None
-        need_grad = any(t is not None and t.requires_grad for t in (x, w, w2, alpha, beta, bias))
+        need_grad = _emit_winners(recording, x, w, w2, alpha, beta, bias)
         y, winners = tconv.dw_forward(d, xc, wc, w2c, al, be, bi, want_winners=need_grad)
         ctx.d, ctx.in_dtype = d, x.dtype
         ctx.save_for_backward(xc, wc, w2c, al, be, winners)
@@ -421,7 +428,7 @@ class TropicalDepthwiseConv2d(nn.Module):
                 beta = -alpha
             elif self.params == "fixed":
                 alpha, beta = self.alpha_fixed, self.beta_fixed
-        geom = (self.mode, self.dtype, self.stride, self.padding, self.dilation)
+        geom = (self.mode, self.dtype, self.stride, self.padding, self.dilation, torch.is_grad_enabled())
         return TropicalDepthwiseFn.apply(x, self.weight, self.weight2, alpha, beta, self.bias, geom)
 
 
@@ -431,7 +438,7 @@ class TropicalConv3dFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, w, w2, alpha, beta, bias, geom):
         from . import tconv3d
-        mode, chan, dtype, stride, pad, dil = geom
+        mode, chan, dtype, stride, pad, dil, recording = geom
         dt = tconv.TORCH_DTYPE[dtype]
         N, C, D, H, W = x.shape
         K, _, T, R, S = w.shape
@@ -440,7 +447,7 @@ class TropicalConv3dFn(torch.autograd.Function):
         cast = lambda t, ty: t.detach().to(ty).contiguous() if t is not None else None
         xc, wc, w2c = cast(x, dt), cast(w, dt), cast(w2, dt)
         al, be, bi = cast(alpha, torch.float32), cast(beta, torch.float32), cast(bias, torch.float32)
-        need_grad = any(t is not None and t.requires_grad for t in (x, w, w2, alpha, beta, bias))
+        need_grad = _emit_winners(recording, x, w, w2, alpha, beta, bias)
         y, winners = tconv3d.forward(d, xc, wc, w2c, al, be, bi, want_winners=need_grad)
         ctx.d, ctx.in_dtype = d, x.dtype
         ctx.save_for_backward(xc, wc, w2c, al, be, winners)
