@@ -52,6 +52,7 @@ def build(force: bool = False, verbose: bool = False) -> Path:
         return LIB
     OBJ.mkdir(exist_ok=True)
     jobs = [(CSRC / "tconv_api.cu", OBJ / "tconv_api.o", [], verbose),
+            (CSRC / "tconv_bwd_sum.cu", OBJ / "tconv_bwd_sum.o", [], verbose),
             (CSRC / "tconv3d_api.cu", OBJ / "tconv3d_api.o", [], verbose)]
     for name, mode, chan in FWD_INSTANCES:
         defs = [f"-DTCONV_INST_NAME={name}", f"-DTCONV_INST_MODE={mode}", f"-DTCONV_INST_CHAN={chan}"]

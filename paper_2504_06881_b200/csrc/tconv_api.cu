@@ -7,6 +7,7 @@
 #include "alu_probe.cuh"
 #include "tconv_common.cuh"
 #include "tconv_bwd.cuh"
+#include "tconv_bwd_sum.cuh"
 #include "tconv_depthwise.cuh"
 #include "tconv_generic.cuh"
 #include "tconv_tiled.cuh"
@@ -225,8 +226,8 @@ void bias_gradient(const Geo& g, const void* gy, float* gbias, void* ws, size_t 
 }
 
 template <typename T>
-int backward_sum_t(const Geo& g0, const void* x, const void* w, const void* w2, const float* alpha,
-                   const float* beta, const void* gy0, const void* winners, void* gx, float* gw,
+int backward_sum_t(const Geo& g, const void* x, const void* w, const void* w2, const float* alpha,
+                   const float* beta, const void* gy, const void* winners, void* gx, float* gw,
                    float* gw2, float* galpha, float* gbeta, float* gbias, void* ws, size_t ws_bytes,
                    cudaStream_t st);
 
@@ -235,7 +236,6 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
                const float* beta, const void* gy, const void* winners, void* gx, float* gw,
                float* gw2, float* galpha, float* gbeta, float* gbias, void* ws, size_t ws_bytes,
                cudaStream_t st) {
-    const bool twob = two_branch(g.mode);
     const bool tiled = !force_generic();
     const char* name = "bwd_generic";
     bool bias_done = false;
@@ -341,150 +341,57 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
 
 // Backward of the Sum channel combine (layers (i), (ii), compound, parallel): per-channel winner codes.
 template <typename T>
-int backward_sum_t(const Geo& g0, const void* x, const void* w, const void* w2, const float* alpha,
-                   const float* beta, const void* gy0, const void* winners, void* gx, float* gw,
+int backward_sum_t(const Geo& g, const void* x, const void* w, const void* w2, const float* alpha,
+                   const float* beta, const void* gy, const void* winners, void* gx, float* gw,
                    float* gw2, float* galpha, float* gbeta, float* gbias, void* ws, size_t ws_bytes,
                    cudaStream_t st) {
-    const bool twob = two_branch(g0.mode);
     const bool tiled = !force_generic();
-    const char* name = "bwd_generic";
-    // output widths that are not a multiple of 4: the code-driven kernels see a layer of width OWP
-    // and a zero-padded copy of grad_y (last block of the workspace)
-    Geo g = g0;
-    const void* gy = gy0;
-    const size_t bias_part = ((size_t)16 * g0.K * sizeof(float) + 255) / 256 * 256;
-    if (tiled && (g0.OW & 3) != 0 && ws) {
-        const Geo gq = widened_geo(g0);
-        const size_t off = bias_part + padded_x_bytes(gq, (int)sizeof(T));
-        const size_t need = padded_gy_bytes(g0, (int)sizeof(T));
-        if (ws_bytes >= off + need) {
-            T* gpad = (T*)((char*)ws + off);
-            const size_t total = (size_t)g0.N * g0.K * g0.OH * g0.OWP;
-            pad_grad_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(g0, (const T*)gy0, gpad);
-            g_launches += 1;
-            g = gq;
-            gy = gpad;
-        }
-    }
-    const bool quads = tiled && (g.OW & 3) == 0;   // the code-driven kernels read whole, aligned quads
-    {
-        const uint8_t* codes = (const uint8_t*)winners;
-        const int br = twob ? 0 : (g.mode == TCONV_MIN_PLUS ? 1 : 2);
-        CodeGxPlan pl;
-        if (gx) {
-            if (quads && plan_code_gx(g, &pl)) {
-                const dim3 grid(pl.grid);
-#define TCONV_GXM(BR, CBV, MULTI, NTH)                                                               \
-    {                                                                                                \
-        auto kern = bwd_code_gx_kernel<T, BR, CBV, MULTI, NTH, false>;                               \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) \
-            return cuda_fail(cudaGetLastError());                                                    \
-        kern<<<grid, pl.threads, pl.smem, st>>>(g, alpha, beta, (const T*)gy, codes, (T*)gx, pl);   \
-    }
-#define TCONV_GXW(BR, CBV)                                                                           \
-    {                                                                                                \
-        auto kern = bwd_code_gx_kernel<T, BR, CBV, false, 256, true>;                                \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) \
-            return cuda_fail(cudaGetLastError());                                                    \
-        kern<<<grid, pl.threads, pl.smem, st>>>(g, alpha, beta, (const T*)gy, codes, (T*)gx, pl);   \
-    }
-#define TCONV_GXC(BR, CBV, NTH)                                                                      \
-    {                                                                                                \
-        auto kern = bwd_code_gx_kernel<T, BR, CBV, false, NTH, false, true>;                         \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) \
-            return cuda_fail(cudaGetLastError());                                                    \
-        kern<<<grid, pl.threads, pl.smem, st>>>(g, alpha, beta, (const T*)gy, codes, (T*)gx, pl);   \
-    }
-#define TCONV_GX(BR, CBV)                                                                            \
-    {                                                                                                \
-        if (pl.ncol > 1 && !g.wide) { if (pl.threads > 256) TCONV_GXC(BR, CBV, 1024) else TCONV_GXC(BR, CBV, 256) } \
-        else if (g.wide) TCONV_GXW(BR, CBV)                                                          \
-        else if (pl.imgs > 1) TCONV_GXM(BR, CBV, true, 256)                                          \
-        else if (pl.threads > 256) TCONV_GXM(BR, CBV, false, 1024)                                   \
-        else TCONV_GXM(BR, CBV, false, 256)                                                          \
-    }
-#define TCONV_GX2(BR) TCONV_GX(BR, 1)
-                if (br == 0) TCONV_GX2(0) else if (br == 1) TCONV_GX2(1) else TCONV_GX2(2)
-#undef TCONV_GX2
-#undef TCONV_GX
-#undef TCONV_GXM
-#undef TCONV_GXW
-#undef TCONV_GXC
-                name = "bwd_code";
-            } else {
-                const size_t total = (size_t)g0.N * g0.C * g0.H * g0.W;
-                bwd_gx_generic_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(
-                    g0, alpha, beta, (const T*)gy0, winners, (T*)gx);
-            }
-            g_launches += 1;
-        }
-        if (gw || gw2 || galpha || gbeta) {
-            CodeGwPlan gp;
-            plan_code_gw(g, &gp);
-            if (quads && gp.smem <= kBwdSmemLimit) {
-                // zero-padded copy of x for the branch values of grad_alpha / grad_beta, placed after
-                // the grad_bias partials in the workspace
-                const size_t pad_bytes = padded_x_bytes(g, (int)sizeof(T));
-                if (br == 0 && (galpha || gbeta) && ws && ws_bytes >= bias_part + pad_bytes &&
-                    (double)g.N * g.C * gp.HP * gp.WP < 2.0e9) {
-                    T* xpad = (T*)((char*)ws + bias_part);
-                    const size_t total = (size_t)g.N * g.C * gp.HP * gp.WP;
-                    if (g.xf32) pad_input_kernel<float, T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(g, (const float*)x, xpad, gp.HP, gp.WP);
-                    else pad_input_kernel<T, T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(g, (const T*)x, xpad, gp.HP, gp.WP);
-                    g_launches += 1;
-                    gp.xs_elems = gp.HP * gp.WP;
-                    gp.xpad = xpad;
-                } else if (g.xf32 && br == 0 && (galpha || gbeta)) {
-                    return TCONV_ERR_UNSUPPORTED;   // float x is only read through the padded (converted) copy
-                }
-#define TCONV_GWK(BR, XSV, WARPV, GRID)                                                               \
-    {                                                                                                \
-        auto kern = bwd_code_gw_kernel<T, BR, XSV, WARPV, false>;                                    \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) \
-            return cuda_fail(cudaGetLastError());                                                    \
-        kern<<<(unsigned)(GRID), 256, gp.smem, st>>>(g, (const T*)x, (const T*)w, (const T*)w2, alpha, beta, \
-                                                      (const T*)gy, codes, gw, gw2, galpha, gbeta, gp); \
-    }
-#define TCONV_GWW(BR, XSV)                                                                           \
-    {                                                                                                \
-        auto kern = bwd_code_gw_kernel<T, BR, XSV, false, true>;                                     \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) \
-            return cuda_fail(cudaGetLastError());                                                    \
-        kern<<<(unsigned)((size_t)g.K * g.C), 256, gp.smem, st>>>(g, (const T*)x, (const T*)w, (const T*)w2, alpha, beta, \
-                                                      (const T*)gy, codes, gw, gw2, galpha, gbeta, gp); \
-    }
-#define TCONV_GW(BR, XSV)                                                                            \
-    {                                                                                                \
-        if (g.wide) TCONV_GWW(BR, XSV)                                                               \
-        else if (gp.warp) TCONV_GWK(BR, XSV, true, ((size_t)g.K * g.C + 7) / 8)                      \
-        else TCONV_GWK(BR, XSV, false, (size_t)g.K * g.C)                                            \
-    }
-#define TCONV_GWV(BR, XSV) TCONV_GW(BR, XSV)
-                if (br == 0) { if (gp.xs_elems) TCONV_GWV(0, true) else TCONV_GWV(0, false) }
-                else if (br == 1) TCONV_GWV(1, false) else TCONV_GWV(2, false)
-#undef TCONV_GWV
-#undef TCONV_GW
-#undef TCONV_GWK
-#undef TCONV_GWW
+    if (tiled && ws) {
+        // output widths that are not a multiple of 4: the kernels see a layer of width OWP and a
+        // zero-padded copy of grad_y (front of the workspace)
+        SumBwdArgs a;
+        a.g = widened_geo(g);
+        const size_t part_bytes = sum_ws_bytes(a.g, (int)sizeof(T));
+        const size_t pad_bytes = padded_gy_bytes(g, (int)sizeof(T));
+        if (part_bytes && ws_bytes >= pad_bytes + part_bytes) {
+            a.gy = gy;
+            if (pad_bytes) {
+                const size_t total = (size_t)g.N * g.K * g.OH * g.OWP;
+                pad_grad_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(g, (const T*)gy, (T*)ws);
                 g_launches += 1;
-                name = "bwd_code";
-            } else {
-                if (gw || gw2) {
-                    bwd_gw_generic_kernel<T><<<(unsigned)((size_t)g0.K * g0.C * g0.RS), 256, 0, st>>>(
-                        g0, alpha, beta, (const T*)gy0, winners, gw, gw2);
-                    g_launches += 1;
-                }
-                if (twob && (galpha || gbeta) && g0.xf32) return TCONV_ERR_UNSUPPORTED;
-                if (twob && (galpha || gbeta)) {
-                    bwd_gab_generic_kernel<T><<<(unsigned)((size_t)g0.K * g0.C), 256, 0, st>>>(
-                        g0, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy0, winners, galpha, gbeta);
-                    g_launches += 1;
-                }
+                a.gy = ws;
             }
+            a.dtype = sizeof(T) == 4 ? TCONV_F32 : TCONV_BF16;
+            a.x = x; a.w = w; a.w2 = w2; a.alpha = alpha; a.beta = beta; a.codes = (const uint8_t*)winners;
+            a.gx = gx; a.gw = gw; a.gw2 = gw2; a.galpha = galpha; a.gbeta = gbeta; a.gbias = gbias;
+            a.ws = (float*)((char*)ws + pad_bytes); a.st = st; a.launches = 0;
+            const int rc = bwd_sum_launch(a);
+            g_launches += a.launches;
+            if (rc == TCONV_OK) {
+                snprintf(g_last_kernel, sizeof(g_last_kernel), "bwd_sum");
+                return check_launch();
+            }
+            if (rc != TCONV_ERR_UNSUPPORTED) return rc == TCONV_ERR_CUDA ? cuda_fail(cudaGetLastError()) : rc;
         }
     }
-    snprintf(g_last_kernel, sizeof(g_last_kernel), "%s", name);
-    if (gbias) bias_gradient<T>(g0, gy0, gbias, ws, ws_bytes, tiled, st);
+    const bool twob = two_branch(g.mode);
+    if (gx) {
+        const size_t total = (size_t)g.N * g.C * g.H * g.W;
+        bwd_gx_generic_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(g, alpha, beta, (const T*)gy, winners, (T*)gx);
+        g_launches += 1;
+    }
+    if (gw || gw2) {
+        bwd_gw_generic_kernel<T><<<(unsigned)((size_t)g.K * g.C * g.RS), 256, 0, st>>>(g, alpha, beta, (const T*)gy, winners, gw, gw2);
+        g_launches += 1;
+    }
+    if (twob && (galpha || gbeta)) {
+        if (g.xf32) return TCONV_ERR_UNSUPPORTED;   // (the any-shape kernel reads x in the layer's type)
+        bwd_gab_generic_kernel<T><<<(unsigned)((size_t)g.K * g.C), 256, 0, st>>>(
+            g, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, winners, galpha, gbeta);
+        g_launches += 1;
+    }
+    snprintf(g_last_kernel, sizeof(g_last_kernel), "bwd_generic");
+    if (gbias) bias_gradient<T>(g, gy, gbias, ws, ws_bytes, tiled, st);
     return check_launch();
 }
 
@@ -697,7 +604,12 @@ size_t tconv_workspace_bytes(const tconv_desc_t* desc, int backward) {
     if (!backward) return fwd;
     // winners recomputed (by a forward pass) into the workspace when the caller passes none;
     // the forward scratch and the backward partial sums are not live at the same time
-    const size_t bwd = align_up(bwd_ws_bytes(g), 256);
+    size_t bwd = align_up(bwd_ws_bytes(g), 256);
+    if (g.chan == CH_SUM) {
+        const int es = desc->dtype == TCONV_F32 ? 4 : 2;
+        const size_t part = padded_gy_bytes(g, es) + sum_ws_bytes(widened_geo(g), es);
+        if (part > bwd) bwd = part;
+    }
     return align_up(winner_bytes(g), 256) + (fwd > bwd ? fwd : bwd);
 }
 

@@ -1,0 +1,79 @@
+// Launches of the Sum-form backward kernels (tconv_bwd_sum.cuh).
+#include "tconv_bwd_sum.cuh"
+
+namespace tconv {
+namespace {
+
+template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW>
+int launch_gx(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx) {
+    auto kern = bwd_sum_gx_kernel<T, BR, GX, AB, WIDE, KW>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
+    kern<<<pl.ctas * (unsigned)a.g.C, pl.threads, pl.smem, a.st>>>(
+        a.g, a.x, a.alpha, a.beta, (const T*)a.gy, a.codes, (T*)a.gx, part_ab, part_gx, pl);
+    ++a.launches;
+    return TCONV_OK;
+}
+// 3 x 3 and 5 x 5 windows have instances of their own (constant address offsets, unrolled windows).
+template <typename T, int BR, bool GX, bool AB>
+int launch_gx_window(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx) {
+    const Geo& g = a.g;
+    if (g.wide) return g.R == 5 && g.S == 5 ? launch_gx<T, BR, GX, AB, true, 5>(a, pl, part_ab, part_gx)
+                                            : launch_gx<T, BR, GX, AB, true, 0>(a, pl, part_ab, part_gx);
+    return g.R == 3 && g.S == 3 ? launch_gx<T, BR, GX, AB, false, 3>(a, pl, part_ab, part_gx)
+                                : launch_gx<T, BR, GX, AB, false, 0>(a, pl, part_ab, part_gx);
+}
+
+template <typename T, int BR, bool PAIRS, bool WIDE>
+int launch_gw(SumBwdArgs& a, const SumGwPlan& pl, float* part) {
+    auto kern = pl.flat ? bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, true> : bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
+    kern<<<pl.grid, 128, pl.smem, a.st>>>(a.g, (const T*)a.gy, a.codes, part, pl);
+    ++a.launches;
+    return TCONV_OK;
+}
+template <typename T, int BR>
+int launch_gw_window(SumBwdArgs& a, const SumGwPlan& pl, float* part) {
+    if (a.g.wide) return launch_gw<T, BR, false, true>(a, pl, part);
+    if (BR == 0 && pl.pairs) return launch_gw<T, BR, BR == 0, false>(a, pl, part);
+    return launch_gw<T, BR, false, false>(a, pl, part);
+}
+
+template <typename T>
+int launch_all(SumBwdArgs& a) {
+    const Geo& g = a.g;
+    const SumPlans& plans = sum_plans(g, (int)sizeof(T));
+    if (!plans.ok) return TCONV_ERR_UNSUPPORTED;
+    const SumGxPlan& xp = plans.gx;
+    const SumGwPlan& gp = plans.gw;
+    const bool two = two_branch(g.mode);
+    const int br = two ? 0 : (g.mode == TCONV_MIN_PLUS ? 1 : 2);
+    const bool ab = two && (a.galpha || a.gbeta), params = a.gw || a.gw2 || a.gbias || ab;
+    float* part = a.ws;
+    float* part_ab = a.ws + sum_part_gw_bytes(g, gp) / sizeof(float);
+    float* part_gx = part_ab + sum_part_ab_bytes(g, xp) / sizeof(float);
+    int rc = TCONV_OK;
+    if (ab) rc = a.gx ? launch_gx_window<T, 0, true, true>(a, xp, part_ab, part_gx) : launch_gx_window<T, 0, false, true>(a, xp, part_ab, part_gx);
+    else if (a.gx) rc = br == 0 ? launch_gx_window<T, 0, true, false>(a, xp, part_ab, part_gx)
+                        : br == 1 ? launch_gx_window<T, 1, true, false>(a, xp, part_ab, part_gx) : launch_gx_window<T, 2, true, false>(a, xp, part_ab, part_gx);
+    if (rc == TCONV_OK && a.gx && xp.nrow * xp.ncol > 1) {
+        bwd_sum_edges_kernel<T><<<dim3((unsigned)(g.N * g.C), (unsigned)((g.H * g.W + 255) / 256)), 256, 0, a.st>>>(g, part_gx, (T*)a.gx, xp);
+        ++a.launches;
+    }
+    if (rc != TCONV_OK || !params) return rc;
+    rc = br == 0 ? launch_gw_window<T, 0>(a, gp, part) : br == 1 ? launch_gw_window<T, 1>(a, gp, part) : launch_gw_window<T, 2>(a, gp, part);
+    if (rc != TCONV_OK) return rc;
+    const size_t pairs = (size_t)g.K * g.C;
+    const unsigned nb_w = a.gw || a.gw2 || a.gbias ? (unsigned)((pairs * g.RS + 255) / 256) : 0u, nb_ab = ab ? (unsigned)((pairs + 31) / 32) : 0u;
+    bwd_sum_finish_kernel<T><<<nb_w + nb_ab, 256, 0, a.st>>>(g, br, gp.splits, part, (int)xp.ctas, part_ab, (const T*)a.w,
+                                                            (const T*)a.w2, a.alpha, a.beta, a.gw, a.gw2, a.galpha, a.gbeta, a.gbias, nb_w);
+    ++a.launches;
+    return TCONV_OK;
+}
+
+}  // namespace
+
+int bwd_sum_launch(SumBwdArgs& a) {
+    return a.dtype == TCONV_F32 ? launch_all<float>(a) : launch_all<__nv_bfloat16>(a);
+}
+
+}  // namespace tconv

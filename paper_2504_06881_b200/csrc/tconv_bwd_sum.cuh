@@ -1,0 +1,727 @@
+// Backward of the Sum channel combine (layers (i), (ii), compound, parallel): two kernels over the winner
+// codes and one that finishes their partial sums.
+//
+//   bwd_sum_gx_kernel   a CTA owns one input channel of a tile of outputs of one image (or of several
+//                       small images); a thread owns 4 adjacent output pixels and walks the output
+//                       channels k.  It adds coef * g into its private per-tap accumulators, which a
+//                       gather over the taps turns into grad_x at the end.  For grad_alpha / grad_beta
+//                       the inputs of its windows sit beside the accumulators, so the input of a winner
+//                       is read through the address of its accumulator; g * x is summed over the warp
+//                       per k.
+//   bwd_sum_edges_kernel  where an image is cut into tiles: adds the (overlapping) input regions the
+//                       tiles' outputs reach.
+//   bwd_sum_gw_kernel   a warp owns one (k, c) pair and a share of its (image, pixel) items; every
+//                       lane keeps a private histogram of g over the *pair* of winning taps, so that
+//                       an item costs one shared-memory read-modify-write for both branches.
+//   bwd_sum_finish_kernel  sums the partials in a fixed order, applies alpha / beta, and completes
+//                       grad_alpha = sum g * (x + w) at the winners with sum_tap w * histogram.
+//
+// No atomics; every accumulator has one writer and a fixed order.
+#pragma once
+#include <cstring>
+
+#include "tconv_bwd.cuh"
+
+namespace tconv {
+
+// ---------------------------------------------------------------------------------- plans
+constexpr int kSgThreads = 256;         // most threads of a grad_x CTA: one quad each
+constexpr int kSgKB = 32;               // output channels staged per round
+constexpr size_t kSgSmem = 112 * 1024;  // two CTAs per SM (other windows than 3 x 3)
+
+struct SumGxPlan {
+    int threads;
+    int imgs;                      // images per CTA (> 1: whole images of a small map)
+    int TR, TQ;                    // output rows and quads per row of a tile
+    int nrow, ncol;                // tiles of an image
+    int ER, EC;                    // input rows and columns the outputs of a tile reach
+    unsigned ctas;                 // tiles of all images (without the channels)
+    size_t smem;
+};
+
+struct SumGwPlan {
+    int flat;                      // items run over the flattened (image, quad) space
+    int splits;                    // shares of a pair's items
+    int per;                       // quads (flat) or rounds of 32 quads per share
+    int pairs;                     // 1: one table over the pair of winners, 0: one table per branch
+    int nbins;                     // bins of a lane's tables
+    unsigned grid;
+    size_t smem;
+};
+
+// Picks the tile of outputs with the least work: lanes (idle ones included) times output channels, and
+// the input region a tile leaves for the final sum.
+inline bool plan_sum_gx(const Geo& g, SumGxPlan* best) {
+    const bool ab = two_branch(g.mode), k3 = g.R == 3 && g.S == 3;
+    const size_t group = (size_t)g.RS * 256 * (ab ? 8 : 4);     // accumulators (and window inputs) of 64 threads
+    const int halo_h = (g.R - 1) * g.dh, halo_w = (g.S - 1) * g.dw, QPR = (g.OW + 3) / 4;
+    int most = kSgThreads;
+    while (most > 64 && most / 64 * group > kSgSmem) most -= 64;
+    if (most / 64 * group > kBwdSmemAttr) return false;
+    double best_cost = -1.0;
+    for (int ncol = 1; ncol <= QPR; ++ncol) {
+        SumGxPlan p;
+        p.TQ = (QPR + ncol - 1) / ncol;
+        if (p.TQ > most) continue;
+        p.ncol = (QPR + p.TQ - 1) / p.TQ;
+        if (p.ncol != ncol) continue;
+        if (p.TQ < 4 && ncol > 1) break;
+        const int rows = most / p.TQ < g.OH ? most / p.TQ : g.OH;
+        p.nrow = (g.OH + rows - 1) / rows;
+        p.TR = (g.OH + p.nrow - 1) / p.nrow;                    // even bands
+        p.nrow = (g.OH + p.TR - 1) / p.TR;
+        p.imgs = 1;
+        if (p.nrow * ncol == 1) {
+            int im = most / (p.TR * p.TQ);
+            if (im > g.N) im = g.N;
+            // (a thread addresses the codes of its CTA's images with a 32-bit count of quads)
+            const double per_img = (double)g.K * g.C * g.OH * g.OW;
+            while (im > 1 && per_img * im > 1.6e10) --im;
+            // small batches: as many CTAs as the SMs can take before a CTA takes a second image
+            while (im > 1 && (double)((g.N + im - 1) / im) * g.C < 148.0) --im;
+            const int groups = (g.N + im - 1) / im;             // even groups
+            p.imgs = (g.N + groups - 1) / groups;
+        }
+        p.ER = (p.TR - 1) * g.sh + halo_h + 1;
+        p.EC = (p.TQ * 4 - 1) * g.sw + halo_w + 1;
+        p.threads = (p.TR * p.TQ * p.imgs + 31) / 32 * 32;
+        const double ctas = (double)((g.N + p.imgs - 1) / p.imgs) * p.nrow * ncol;
+        if (ctas * g.C > 2.0e9) continue;
+        p.ctas = (unsigned)ctas;
+        p.smem = (k3 ? kSgThreads / 64 : (p.threads + 63) / 64) * group;
+        const double per_sm = ctas * g.C / 148.0;
+        const double cost = ctas * (4.0 * p.threads * g.K + (p.nrow * ncol > 1 ? 2.0 * p.ER * p.EC : 0.0)) * (per_sm < 1.0 ? 1.0 / per_sm : 1.0);
+        if (best_cost < 0.0 || cost < best_cost) { best_cost = cost; *best = p; }
+    }
+    return best_cost >= 0.0;
+}
+
+inline bool plan_sum_gw(const Geo& g, SumGwPlan* p) {
+    const long pairs = (long)g.K * g.C;
+    const long nq = (long)g.OH * ((g.OW + 3) / 4), rpi = nq / 32;
+    p->flat = nq % 32 != 0;
+    const long items = p->flat ? g.N * nq : g.N * rpi;
+    const long least = p->flat ? 256 : 8;              // a share is at least eight rounds
+    // one table over the pair of winners while it is small and a pair's items outweigh clearing and
+    // summing it (RS * RS columns against one access per item saved)
+    const bool two = two_branch(g.mode);
+    p->pairs = two && g.RS <= 9 && (double)g.N * nq * 4 / 32 >= 2.0 * g.RS * g.RS;
+    p->nbins = p->pairs ? g.RS * g.RS : two ? 2 * g.RS : g.RS;
+    p->smem = (size_t)4 * p->nbins * 32 * sizeof(float);
+    if (p->smem > kBwdSmemAttr) return false;
+    long per_sm = (long)((227 * 1024) / (p->smem + 1024)) * 4;
+    if (per_sm > 32) per_sm = 32;
+    const long slots = 148 * per_sm;
+    // among the counts that fill the SMs the one whose last round of resident warps is fullest
+    long most = items / least;
+    if (most < 1) most = 1;
+    if (most > 64) most = 64;
+    long s = 1;
+    double best = -1.0;
+    for (long c = 1; c <= most; ++c) {
+        const long w = pairs * c, rounds = (w + slots - 1) / slots;
+        const double eff = (double)w / (double)(rounds * slots);
+        if (eff > best + 0.02) { best = eff; s = c; }
+        if (best > 0.92) break;
+    }
+    p->per = (int)((items + s - 1) / s);
+    p->splits = (int)((items + p->per - 1) / p->per);
+    p->grid = (unsigned)((pairs * p->splits + 3) / 4);
+    return true;
+}
+
+// Both plans of a layer; the search above is host work of some microseconds, so the last few are kept
+// per host thread (they depend on nothing but the geometry).
+struct SumPlans {
+    Geo g;
+    int esize;
+    SumGxPlan gx;
+    SumGwPlan gw;
+    int ok;      // the layer fits both kernels
+};
+inline const SumPlans& sum_plans(const Geo& g, int esize) {
+    constexpr int kKept = 32;
+    static thread_local SumPlans kept[kKept];
+    static thread_local int used = 0, next = 0;
+    for (int i = 0; i < used; ++i)
+        if (kept[i].esize == esize && memcmp(&kept[i].g, &g, sizeof(Geo)) == 0) return kept[i];
+    SumPlans& p = kept[next];
+    p.g = g;
+    p.esize = esize;
+    p.ok = (double)g.N * g.OH * g.OWP < 2.0e9 && (double)g.H * g.W < 1.6e7 && (double)g.N * g.C < 2.0e9 && (double)g.OH * g.OWP * g.K < 1.0e9 &&
+           (double)g.OH * g.OWP * g.K * g.C < 1.6e10 && plan_sum_gx(g, &p.gx) &&
+           plan_sum_gw(g, &p.gw);
+    next = (next + 1) % kKept;
+    if (used < kKept) ++used;
+    return p;
+}
+// Partial sums of a call: [grad_w histograms | grad_alpha, grad_beta rows | input regions of the tiles].
+inline size_t sum_part_gw_bytes(const Geo& g, const SumGwPlan& p) {
+    return ((size_t)p.splits * g.K * g.C * 2 * g.RS * sizeof(float) + 255) / 256 * 256;
+}
+inline size_t sum_part_ab_bytes(const Geo& g, const SumGxPlan& p) {
+    return two_branch(g.mode) ? ((size_t)p.ctas * g.K * g.C * 2 * sizeof(float) + 255) / 256 * 256 : 0;
+}
+inline size_t sum_part_gx_bytes(const Geo& g, const SumGxPlan& p) {
+    return p.nrow * p.ncol > 1 ? ((size_t)p.ctas * g.C * p.ER * p.EC * sizeof(float) + 255) / 256 * 256 : 0;
+}
+// Bytes of all partial sums; 0 when the layer does not fit the kernels.  g: widened to whole quads.
+inline size_t sum_ws_bytes(const Geo& g, int esize) {
+    const SumPlans& p = sum_plans(g, esize);
+    return p.ok ? sum_part_gw_bytes(g, p.gw) + sum_part_ab_bytes(g, p.gx) + sum_part_gx_bytes(g, p.gx) : 0;
+}
+
+// ---------------------------------------------------------------------------------- loads
+// Operands requested ahead of their use: volatile, so that they stay where they are written.  KEEP: the
+// lines are shared with other warps of the CTA (grad_w); the grad_x kernel streams its operands past an L1
+// that the accumulators leave little of.
+template <typename T, bool KEEP>
+__device__ __forceinline__ void ahead_g4(const T* p, float* gv) {
+    if constexpr (sizeof(T) == 4) {
+        if constexpr (KEEP) asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(gv[0]), "=f"(gv[1]), "=f"(gv[2]), "=f"(gv[3]) : "l"(p));
+        else asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(gv[0]), "=f"(gv[1]), "=f"(gv[2]), "=f"(gv[3]) : "l"(p));
+    } else {
+        unsigned a, b;
+        if constexpr (KEEP) asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "l"(p));
+        else asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "l"(p));
+        gv[0] = __uint_as_float(a); gv[1] = __uint_as_float(b);      // (unpacked when used: unpack_g4)
+    }
+}
+template <typename T> __device__ __forceinline__ void unpack_g4(const float* raw, float* gv) {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) gv[j] = raw[j];
+    } else {
+        const unsigned a = __float_as_uint(raw[0]), b = __float_as_uint(raw[1]);
+        gv[0] = __uint_as_float(a << 16); gv[1] = __uint_as_float(a & 0xffff0000u);
+        gv[2] = __uint_as_float(b << 16); gv[3] = __uint_as_float(b & 0xffff0000u);
+    }
+}
+template <bool WIDE, bool KEEP>
+__device__ __forceinline__ Codes4<WIDE> ahead_codes4(const uint8_t* p) {
+    Codes4<WIDE> r;
+    if constexpr (!WIDE) {
+        if constexpr (KEEP) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(r.lo) : "l"(p));
+        else asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(r.lo) : "l"(p));
+    } else {
+        asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(r.lo), "=r"(r.hi) : "l"(p));
+    }
+    return r;
+}
+
+// ---------------------------------------------------------------------------------- grad_x, grad_alpha, grad_beta
+__device__ __forceinline__ float load_xf(const void* x, size_t i, int xf32, float) { return __ldg(reinterpret_cast<const float*>(x) + i); }
+__device__ __forceinline__ float load_xf(const void* x, size_t i, int xf32, __nv_bfloat16) {
+    if (xf32) return __bfloat162float(__float2bfloat16_rn(__ldg(reinterpret_cast<const float*>(x) + i)));
+    return __bfloat162float(__ldg(reinterpret_cast<const __nv_bfloat16*>(x) + i));
+}
+
+// Sums 16 values over the warp: halving butterfly, lane 2v (and 2v + 1) ends with the total of value v.
+__device__ __forceinline__ float warp_sum16(float* s, int lane) {
+#pragma unroll
+    for (int step = 0; step < 4; ++step) {
+        const int d = 16 >> step, n = 8 >> step;
+        const bool up = (lane & d) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const float keep = up ? s[i + n] : s[i];
+            const float send = up ? s[i] : s[i + n];
+            s[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+        }
+    }
+    return s[0] + __shfl_xor_sync(0xffffffffu, s[0], 1);
+}
+
+// Byte offset tap << SH of pixel j for the min / max branch (SH 8 or 10).  Narrow codes: the nibbles of a
+// quad's four codes, one per byte; one PRMT moves a byte to bits 8..15.
+template <bool WIDE, int SH> struct QuadTaps;
+template <int SH> struct QuadTaps<false, SH> {
+    static constexpr unsigned mask = 0x0f0f0f0fu << (SH - 8);
+    unsigned lo, hi;
+    __device__ __forceinline__ explicit QuadTaps(const Codes4<false>& c) : lo((c.lo << (SH - 8)) & mask), hi((c.lo >> (12 - SH)) & mask) {}
+    __device__ __forceinline__ unsigned tmin(int j) const { return __byte_perm(lo, 0u, 0x4404u + (unsigned)(j << 4)); }
+    __device__ __forceinline__ unsigned tmax(int j) const { return __byte_perm(hi, 0u, 0x4404u + (unsigned)(j << 4)); }
+};
+template <> struct QuadTaps<true, 8> {
+    Codes4<true> c;
+    __device__ __forceinline__ explicit QuadTaps(const Codes4<true>& c_) : c(c_) {}
+    __device__ __forceinline__ unsigned tmin(int j) const { return __byte_perm(j < 2 ? c.lo : c.hi, 0u, 0x4404u + (unsigned)((2 * (j & 1)) << 4)); }
+    __device__ __forceinline__ unsigned tmax(int j) const { return __byte_perm(j < 2 ? c.lo : c.hi, 0u, 0x4404u + (unsigned)((2 * (j & 1) + 1) << 4)); }
+};
+
+// BR: 0 both branches, 1 min branch only, 2 max branch only.  GX: grad_x.  AB: grad_alpha / grad_beta (BR 0).
+// KW: 3 or 5 for 3 x 3 (narrow codes) and 5 x 5 windows (wide codes), else 0 (any window).
+// Shared memory: accumulators [4][tap][TP] floats per TP threads, then (AB) the window inputs in the same
+// layout; TP is 256 for 3 x 3 windows (and the taps of a column lie 1024 bytes apart), 64 otherwise (256
+// bytes apart): one PRMT and one add address an accumulator, and the winner's input lies at a constant
+// distance from it.
+template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW>
+__global__ void __launch_bounds__(kSgThreads, KW == 3 ? 3 : 2)
+bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const float* __restrict__ alpha, const float* __restrict__ beta,
+                  const T* __restrict__ gy, const uint8_t* __restrict__ codes, T* __restrict__ gx,
+                  float* __restrict__ part_ab, float* __restrict__ part_gx, SumGxPlan pl) {
+    constexpr bool K3 = KW == 3;
+    constexpr int TP = K3 ? kSgThreads : 64, TS = TP * 4;      // columns side by side, bytes between two taps
+    const int RS = KW ? KW * KW : g.RS;
+    const int WR = KW ? KW : g.R, WS = KW ? KW : g.S;
+    const int gbytes = RS * TS * (AB ? 8 : 4);                 // bytes of TP threads
+    extern __shared__ __align__(16) char smem[];
+    __shared__ float coef[kSgKB * 2];                          // [KB] {alpha, beta}
+    __shared__ float part[kSgThreads / 32 * kSgKB * 2];        // [warps][KB][2]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int c = blockIdx.x % g.C;
+    const unsigned tile = blockIdx.x / g.C;
+    const int ct = tile % pl.ncol, rt = (tile / pl.ncol) % pl.nrow;
+    const int n_first = (tile / pl.ncol / pl.nrow) * pl.imgs;
+    const int nimg = min(pl.imgs, g.N - n_first);
+    const int oh0 = rt * pl.TR, oq0 = ct * pl.TQ;
+    const int tr = min(pl.TR, g.OH - oh0), tq = min(pl.TQ, (g.OW >> 2) - oq0);   // output rows, quads per row
+    const int NQ1 = tr * tq, NQ = NQ1 * nimg;
+    const unsigned plane = (unsigned)g.OH * (unsigned)g.OW;    // (below 2^30 with all K channels)
+    constexpr int CW = WIDE ? 2 : 1;                           // bytes per code
+    // addresses: a base of the CTA plus a 32-bit count of the thread, elements of grad_y and quads of codes
+    const T* gbase = gy + (size_t)n_first * g.K * plane;
+    const uint8_t* cbase = codes + ((size_t)n_first * g.K * g.C + c) * plane * CW;
+    const unsigned cstep = (unsigned)g.C * (plane >> 2);       // quads of codes between two output channels
+    {
+        // a thread without a quad repeats the last one into columns nobody reads
+        const bool live = tid < NQ;
+        const int q = min(tid, NQ - 1);
+        const int il = q / NQ1, q1 = q - il * NQ1, orow = q1 / tq;
+        const int oh = oh0 + orow, ow0 = (oq0 + q1 - orow * tq) * 4;
+        const unsigned pix = (unsigned)(oh * g.OW + ow0);
+        unsigned goff = (unsigned)(il * g.K) * plane + pix;
+        unsigned coff = (unsigned)(il * g.K) * cstep + (pix >> 2);
+        char* Ab = smem + (size_t)(tid / TP) * gbytes + (tid % TP) * 4;
+
+        // gradients and codes of a pair of output channels are requested together, one pair ahead: the loads
+        // of a pair share a scoreboard, which a longer chain of single requests would exhaust (past the last
+        // channel it is read again: the staged coefficients of such a channel are zero)
+        constexpr int PF = 4;
+        float raw[PF][sizeof(T)];      // (4 floats, or 4 bf16 in two registers)
+        Codes4<WIDE> cq[PF];
+        int more = g.K - 1;
+        auto request = [&](int u) {
+            ahead_g4<T, false>(gbase + goff, raw[u]);
+            cq[u] = ahead_codes4<WIDE, false>(cbase + (size_t)coff * (4 * CW));
+            if (more > 0) { goff += plane; coff += cstep; }
+            --more;
+        };
+        request(0);
+        request(1);
+
+        if constexpr (GX)
+            for (int e = 0; e < 4 * RS; ++e) *reinterpret_cast<float*>(Ab + e * TS) = 0.0f;
+        if constexpr (AB) {
+            // the inputs of the four windows; zero outside the image and for a repeated quad
+            const size_t xc = ((size_t)(n_first + il) * g.C + c) * g.H * g.W;
+            const int iwq = ow0 * g.sw - g.pw;
+            char* Xb = Ab + 4 * RS * TS;
+#pragma unroll
+            for (int r = 0; r < WR; ++r) {
+                const int ih = oh * g.sh - g.ph + r * g.dh;
+                const bool rok = live && ih >= 0 && ih < g.H;
+                const size_t xrow = xc + (size_t)(rok ? ih : 0) * g.W;
+                auto fetch = [&](int iw) { return rok && iw >= 0 && iw < g.W ? load_xf(x, xrow + iw, g.xf32, T()) : 0.0f; };
+                if (KW && g.sw == 1 && g.dw == 1) {       // neighbouring windows share their columns
+                    float col[KW + 3];
+#pragma unroll
+                    for (int i = 0; i < KW + 3; ++i) col[i] = fetch(iwq + i);
+#pragma unroll
+                    for (int t = 0; t < KW; ++t)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) *reinterpret_cast<float*>(Xb + (j * RS + r * KW + t) * TS) = col[t + j];
+                } else {
+                    for (int t = 0; t < WS; ++t)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            *reinterpret_cast<float*>(Xb + (j * RS + r * WS + t) * TS) = fetch(iwq + j * g.sw + t * g.dw);
+                }
+            }
+        }
+
+        for (int kb0 = 0; kb0 < g.K; kb0 += kSgKB) {
+            const int kn = min(kSgKB, g.K - kb0);
+            __syncthreads();     // the previous round's staging is consumed
+            for (int e = tid; e < kSgKB; e += blockDim.x) {
+                const bool ok = e < kn;
+                const size_t i = (size_t)(kb0 + e) * g.C + c;
+                coef[2 * e] = ok ? (alpha ? alpha[i] : 1.0f) : 0.0f;      // (no alpha / beta in single-branch layers)
+                coef[2 * e + 1] = ok ? (beta ? beta[i] : 1.0f) : 0.0f;
+            }
+            __syncthreads();
+            for (int k8 = 0; k8 < kn; k8 += 8) {
+                float s[AB ? 16 : 1];
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) {
+                    const int u = kk % PF;
+                    if (kk % 2 == 0) {
+                        request((u + 2) % PF);
+                        request((u + 3) % PF);
+                    }
+                    float gv[4];
+                    unpack_g4<T>(raw[u], gv);
+                    const float2 cf = *reinterpret_cast<const float2*>(coef + 2 * (k8 + kk));
+                    const QuadTaps<WIDE, K3 ? 10 : 8> taps(cq[u]);
+                    // one branch: the four pixels' accumulators are distinct, so their loads go out together
+                    auto branch = [&](bool is_min, float a) {
+                        char* p[4];
+                        float v[4], xv[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) p[j] = Ab + (is_min ? taps.tmin(j) : taps.tmax(j));
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if constexpr (GX) v[j] = *reinterpret_cast<const float*>(p[j] + j * RS * TS);
+                            if constexpr (AB) xv[j] = *reinterpret_cast<const float*>(p[j] + (4 + j) * RS * TS);
+                        }
+                        float sum = 0.0f;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if constexpr (GX) *reinterpret_cast<float*>(p[j] + j * RS * TS) = __fmaf_rn(a, gv[j], v[j]);
+                            if constexpr (AB) sum = __fmaf_rn(gv[j], xv[j], sum);
+                        }
+                        return sum;
+                    };
+                    float sa = 0.0f, sb = 0.0f;
+                    if constexpr (BR != 2) sa = branch(true, cf.x);
+                    if constexpr (BR != 1) sb = branch(false, cf.y);
+                    if constexpr (AB) { s[2 * kk] = sa; s[2 * kk + 1] = sb; }
+                }
+                if constexpr (AB) {
+                    const float v = warp_sum16(s, lane);
+                    if (!(lane & 1)) part[(warp * kSgKB + k8) * 2 + (lane >> 1)] = v;
+                }
+            }
+            if constexpr (AB) {
+                __syncthreads();
+                for (int e = tid; e < 2 * kn; e += blockDim.x) {
+                    float t = 0.0f;
+                    for (int i = 0; i < nwarps; ++i) t += part[i * kSgKB * 2 + e];
+                    part_ab[((size_t)tile * g.C + c) * g.K * 2 + 2 * kb0 + e] = t;
+                }
+            }
+        }
+    }
+    if constexpr (GX) {
+        __syncthreads();
+        // gather: an input element sums, over the taps, the accumulator of the output pixel that reads it
+        // through that tap (lanes along the columns, one warp per input row).  An image in one tile: all
+        // its inputs, straight to grad_x; else the region the tile reaches, as floats
+        const float* A = reinterpret_cast<const float*>(smem);
+        const int gfl = gbytes / 4;
+        const bool whole = pl.nrow * pl.ncol == 1;
+        const int rows = whole ? g.H : pl.ER, cols = whole ? g.W : pl.EC;
+        const int up = whole ? g.ph : 0, left = whole ? g.pw : 0;      // row / column 0 of the walk in the tile's region
+        float* region = part_gx + ((size_t)tile * g.C + c) * pl.ER * pl.EC;
+        auto index = [&](int q, int j, int tap) { return (q / TP) * gfl + (j * RS + tap) * TP + q % TP; };
+        auto store = [&](int il, int row, int col, float v) {
+            if (whole) gx[(((size_t)(n_first + il) * g.C + c) * g.H + row) * g.W + col] = from_f32<T>(v);
+            else region[(size_t)row * pl.EC + col] = v;
+        };
+        // (strides 1 and 2 divide by a shift)
+        const int lh = g.sh <= 2 ? g.sh - 1 : -1, lw = g.sw <= 2 ? g.sw - 1 : -1;
+        auto quot = [](int n, int stride, int shift) { return shift >= 0 ? n >> shift : n / stride; };
+        for (int col = lane; col < cols; col += 32) {
+            // output column that reads this one through tap column sx, or -1
+            int at[KW ? KW : 1];
+            auto column = [&](int sx) {
+                const int nw = col + left - sx * g.dw, ow = quot(nw, g.sw, lw);
+                return nw >= 0 && ow * g.sw == nw && ow < tq * 4 ? ow : -1;
+            };
+            if constexpr (KW != 0) {
+#pragma unroll
+                for (int sx = 0; sx < KW; ++sx) {
+                    at[sx] = column(sx);
+                    if (K3 && at[sx] >= 0) at[sx] = (at[sx] >> 2) + (at[sx] & 3) * RS * TP;   // its accumulator's index but for row and tap
+                }
+            }
+            for (int rr = warp; rr < nimg * rows; rr += nwarps) {
+                const int il = nimg == 1 ? 0 : rr / rows, row = rr - il * rows;
+                float sum = 0.0f;
+#pragma unroll
+                for (int r = 0; r < WR; ++r) {
+                    const int nh = row + up - r * g.dh, oh = quot(nh, g.sh, lh);
+                    if (nh < 0 || oh * g.sh != nh || oh >= tr) continue;
+                    const int qrow = il * NQ1 + oh * tq;
+#pragma unroll
+                    for (int sx = 0; sx < WS; ++sx) {
+                        const int ow = KW ? at[KW ? sx : 0] : column(sx);
+                        if constexpr (K3) {
+                            if (ow >= 0) sum += A[qrow + ow + (r * WS + sx) * TP];
+                        } else if (ow >= 0) sum += A[index(qrow + (ow >> 2), ow & 3, r * WS + sx)];
+                    }
+                }
+                store(il, row, col, sum);
+            }
+        }
+    }
+}
+
+// grad_x of an image cut into tiles: every input element adds the regions that cover it, tile rows and
+// columns ascending.  grid (N * C, blocks of 256 elements of a plane).
+template <typename T>
+__global__ void __launch_bounds__(256)
+bwd_sum_edges_kernel(Geo g, const float* __restrict__ part_gx, T* __restrict__ gx, SumGxPlan pl) {
+    const unsigned i = blockIdx.y * 256 + threadIdx.x;
+    if (i >= (unsigned)(g.H * g.W)) return;
+    const unsigned n = blockIdx.x / (unsigned)g.C, c = blockIdx.x - n * (unsigned)g.C;
+    const unsigned y = i / (unsigned)g.W + g.ph, x = i - (y - g.ph) * g.W + g.pw;
+    const unsigned sr = pl.TR * g.sh, sc = pl.TQ * 4 * g.sw;     // input distance between two tiles
+    const unsigned ER = pl.ER, EC = pl.EC, area = ER * EC;
+    const unsigned r1 = min((unsigned)pl.nrow - 1, y / sr), c1 = min((unsigned)pl.ncol - 1, x / sc);
+    const unsigned r0 = y < ER ? 0 : (y - ER) / sr + 1, c0 = x < EC ? 0 : (x - EC) / sc + 1;
+    float sum = 0.0f;
+    for (unsigned r = r0; r <= r1; ++r)
+        for (unsigned q = c0; q <= c1; ++q)
+            sum += __ldg(part_gx + ((size_t)((n * pl.nrow + r) * pl.ncol + q) * g.C + c) * area + (y - r * sr) * EC + (x - q * sc));
+    gx[(size_t)blockIdx.x * g.H * g.W + i] = from_f32<T>(sum);
+}
+
+// ---------------------------------------------------------------------------------- grad_w (and grad_bias)
+// A warp owns one (k, c) pair and one share of its (image, quad) items.  Lane-private histograms,
+// [bin][64] floats for two warps (bins 256 bytes apart: one PRMT turns a bin number into an offset).
+// PAIRS: with both branches the bin is the pair (argmax tap, argmin tap), RS * RS bins, so one
+// read-modify-write serves both; the finishing sums over rows / columns of the table give the two
+// histograms.  Else one table per branch.
+// FLAT: the share is a range of the flattened (image, quad) space; else an image is whole rounds of 32 quads.
+template <typename T, int BR, bool PAIRS, bool WIDE, bool FLAT>
+__global__ void __launch_bounds__(128)
+bwd_sum_gw_kernel(Geo g, const T* __restrict__ gy, const uint8_t* __restrict__ codes, float* __restrict__ part, SumGwPlan pl) {
+    extern __shared__ float tabs[];
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // (uniform: addresses below)
+    const long wid = (long)blockIdx.x * 4 + warp;
+    const int pairs = g.K * g.C;
+    if (wid >= (long)pairs * pl.splits) return;
+    const int split = (int)(wid / pairs), pair = (int)(wid - (long)split * pairs);
+    const int k = pair / g.C, c = pair - k * g.C;
+    float* tab = tabs + (size_t)(warp >> 1) * pl.nbins * 64 + (warp & 1) * 32;
+    char* mine = reinterpret_cast<char*>(tab + lane);
+    char* mine_max = mine + (BR == 0 ? g.RS * 256 : 0);      // (one table per branch)
+    for (int b = 0; b < pl.nbins; ++b) tab[b * 64 + lane] = 0.0f;
+    constexpr int CW = WIDE ? 2 : 1;
+    const int NQ = g.OH * (g.OW >> 2);
+    const size_t plane = (size_t)g.OH * g.OW, gstep = (size_t)g.K * plane, cstep = gstep * g.C * CW;
+    const unsigned skip = 16u - (unsigned)g.RS;
+    auto add_two = [&](char* base, unsigned o0, unsigned o1, float g0, float g1) {
+        float* p0 = reinterpret_cast<float*>(base + o0);
+        float* p1 = reinterpret_cast<float*>(base + o1);
+        // both loads first; where the two bins are one, the second store holds both gradients
+        const float v0 = *p0, v1 = *p1;
+        const float t0 = v0 + g0;
+        const float t1 = (o0 == o1 ? t0 : v1) + g1;
+        *p0 = t0;
+        *p1 = t1;
+    };
+    auto add_quad = [&](const float* gv, const Codes4<WIDE>& code) {
+        if constexpr (PAIRS) {
+            // four bins, one per byte (no borrow crosses a byte: each is at least skip * high nibble)
+            const unsigned top = (code.lo >> 4) & 0x0f0f0f0fu, bins = code.lo - skip * top;
+            auto at = [&](int j) { return __byte_perm(bins, 0u, 0x4404u + (unsigned)(j << 4)); };
+            add_two(mine, at(0), at(1), gv[0], gv[1]);
+            add_two(mine, at(2), at(3), gv[2], gv[3]);
+        } else {
+            const QuadTaps<WIDE, 8> t(code);
+            if constexpr (BR != 2) {
+                add_two(mine, t.tmin(0), t.tmin(1), gv[0], gv[1]);
+                add_two(mine, t.tmin(2), t.tmin(3), gv[2], gv[3]);
+            }
+            if constexpr (BR != 1) {
+                add_two(mine_max, t.tmax(0), t.tmax(1), gv[0], gv[1]);
+                add_two(mine_max, t.tmax(2), t.tmax(3), gv[2], gv[3]);
+            }
+        }
+    };
+    // FLAT: the operands of HB rounds are requested together, while the HB rounds before them are added (the
+    // loads of such a batch share a scoreboard: 290 against 270 us on the 28 x 28 transition layer); whole
+    // rounds: one at a time, PF ahead
+    constexpr int HB = FLAT && !PAIRS ? 2 : 4, PF = 2 * HB;
+    float raw[PF][sizeof(T)];
+    Codes4<WIDE> cq[PF];
+    if constexpr (FLAT) {
+        const int lo = split * pl.per, hi = min(g.N * NQ, lo + pl.per);
+        int it = lo + lane;
+        // lanes past the end read the share's last quad again; its gradient is dropped
+        const int first = min(it, hi - 1);
+        int n = first / NQ, q = first - n * NQ;
+        const T* gp = gy + ((size_t)n * g.K + k) * plane + 4 * q;
+        const uint8_t* cp = codes + ((((size_t)n * g.K + k) * g.C + c) * plane + 4 * q) * CW;
+        const int dn = 32 / NQ, dq = 32 - dn * NQ;
+        const size_t gadv = dn * gstep + 4 * dq, cadv = dn * cstep + 4 * dq * CW;
+        const size_t gwrap = gstep - plane, cwrap = cstep - plane * CW;
+        auto request = [&](int u) {
+            ahead_g4<T, true>(gp, raw[u]);
+            cq[u] = ahead_codes4<WIDE, true>(cp);
+            it += 32;
+            if (it < hi) {
+                q += dq;
+                gp += gadv;
+                cp += cadv;
+                if (q >= NQ) { q -= NQ; gp += gwrap; cp += cwrap; }
+            }
+        };
+#pragma unroll
+        for (int u = 0; u < HB; ++u) request(u);
+        const int rounds = (hi - lo + 31) / 32;
+        for (int r0 = 0; r0 < rounds; r0 += PF) {
+#pragma unroll
+            for (int u = 0; u < PF; ++u) {
+                if (u % HB == 0) {
+#pragma unroll
+                    for (int v = 0; v < HB; ++v) request((u + HB + v) % PF);
+                }
+                float gv[4];
+                unpack_g4<T>(raw[u], gv);
+                if (lo + (r0 + u + 1) * 32 > hi) {      // the last round, or a round past it
+                    const bool in = lo + (r0 + u) * 32 + lane < hi;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) gv[j] = in ? gv[j] : 0.0f;
+                }
+                add_quad(gv, cq[u]);
+            }
+        }
+    } else {
+        const int rpi = NQ / 32;
+        const int lo = split * pl.per, hi = min(g.N * rpi, lo + pl.per);
+        const int n0 = lo / rpi;
+        int rr = lo - n0 * rpi, left = hi - lo - 1;      // round of its image to request next, rounds behind it
+        const T* gp = gy + ((size_t)n0 * g.K + k) * plane;
+        const uint8_t* cp = codes + (((size_t)n0 * g.K + k) * g.C + c) * plane * CW;
+        auto request = [&](int u) {                      // (past the share its last round is read again)
+            const unsigned off = (unsigned)(rr * 32 + lane) * 4u;
+            ahead_g4<T, true>(gp + off, raw[u]);
+            cq[u] = ahead_codes4<WIDE, true>(cp + off * CW);
+            if (left > 0 && ++rr == rpi) {
+                rr = 0;
+                gp += gstep;
+                cp += cstep;
+            }
+            --left;
+        };
+#pragma unroll
+        for (int u = 0; u < PF; ++u) request(u);
+        int i = lo;
+        for (; i + PF <= hi; i += PF) {
+#pragma unroll
+            for (int u = 0; u < PF; ++u) {
+                float gv[4];
+                unpack_g4<T>(raw[u], gv);
+                add_quad(gv, cq[u]);
+                request(u);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < PF; ++u) {
+            if (i + u >= hi) break;
+            float gv[4];
+            unpack_g4<T>(raw[u], gv);
+            add_quad(gv, cq[u]);
+        }
+    }
+    __syncwarp();
+    // bin totals: lane l sums the bins l, l + 32, ..., starting at its own column (no bank conflicts)
+    for (int b = lane; b < pl.nbins; b += 32) {
+        float s = 0.0f;
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i) s += tab[b * 64 + ((i + lane) & 31)];
+        tab[b * 64 + lane] = s;      // (column b % 32 of its own row: read by this lane only)
+    }
+    __syncwarp();
+    auto total = [&](int b) { return tab[b * 64 + (b & 31)]; };
+    float* o = part + ((size_t)split * pairs + pair) * 2 * g.RS;
+    for (int t = lane; t < g.RS; t += 32) {
+        float smin = 0.0f, smax = 0.0f;
+        if constexpr (PAIRS) {
+            for (int i = 0; i < g.RS; ++i) { smin += total(i * g.RS + t); smax += total(t * g.RS + i); }
+        } else {
+            smin = total(t);
+            smax = BR == 0 ? total(g.RS + t) : smin;
+        }
+        o[t] = smin;
+        o[g.RS + t] = smax;
+    }
+}
+
+// ---------------------------------------------------------------------------------- finish
+// Blocks [0, nb_w): one thread per (k, c, tap): grad_w / grad_w2 over the splits, and grad_bias (the sum
+// of a pair's histogram is the sum of grad_y).  Blocks from nb_w on: grad_alpha / grad_beta, 32 (c, k)
+// entries per block; eight slices share the partial rows and the taps, and are added in slice order.
+template <typename T>
+__global__ void __launch_bounds__(256)
+bwd_sum_finish_kernel(Geo g, int br, int splits, const float* __restrict__ part, int rows, const float* __restrict__ part_ab,
+                      const T* __restrict__ w, const T* __restrict__ w2, const float* __restrict__ alpha,
+                      const float* __restrict__ beta, float* __restrict__ gw, float* __restrict__ gw2,
+                      float* __restrict__ galpha, float* __restrict__ gbeta, float* __restrict__ gbias, unsigned nb_w) {
+    const size_t pairs = (size_t)g.K * g.C, len = pairs * 2 * g.RS;
+    if (blockIdx.x < nb_w) {
+        const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+        if (i >= pairs * g.RS) return;
+        const size_t pair = i / g.RS;
+        const int t = (int)(i - pair * g.RS);
+        const float* p = part + pair * 2 * g.RS + t;
+        float smin = 0.0f, smax = 0.0f;
+        for (int s = 0; s < splits; ++s) { smin += p[s * len]; smax += p[s * len + g.RS]; }
+        if (br == 0) {
+            const float a = alpha ? alpha[pair] : 1.0f, b = beta ? beta[pair] : 1.0f;
+            if (g.mode == TCONV_COMPOUND) {
+                if (gw) gw[i] = __fmaf_rn(a, smin, b * smax);
+            } else {
+                if (gw) gw[i] = a * smin;
+                if (gw2) gw2[i] = b * smax;
+            }
+        } else if (gw) {
+            gw[i] = smin;
+        }
+        if (gbias && t == 0 && pair % g.C == 0) {
+            float s = 0.0f;
+            for (int sp = 0; sp < splits; ++sp)
+                for (int u = 0; u < g.RS; ++u) s += p[sp * len + u];
+            gbias[pair / g.C] = s;
+        }
+        return;
+    }
+    __shared__ float2 red[8][32];
+    const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+    const size_t e = (size_t)(blockIdx.x - nb_w) * 32 + lane;     // c * K + k
+    const size_t c = e / g.K, k = e - c * g.K;
+    float2 s = make_float2(0.0f, 0.0f);
+    if (e < pairs) {
+        for (int r = slice; r < rows; r += 8) {
+            const float2 v = __ldg(reinterpret_cast<const float2*>(part_ab) + r * pairs + e);
+            s.x += v.x; s.y += v.y;
+        }
+        const size_t pair = k * g.C + c;
+        const T* wm = g.mode == TCONV_PARALLEL ? w2 : w;
+        for (int t = slice; t < g.RS; t += 8) {
+            const float* p = part + pair * 2 * g.RS + t;
+            float smin = 0.0f, smax = 0.0f;
+            for (int sp = 0; sp < splits; ++sp) { smin += p[sp * len]; smax += p[sp * len + g.RS]; }
+            s.x = __fmaf_rn(to_f32(w[pair * g.RS + t]), smin, s.x);
+            s.y = __fmaf_rn(to_f32(wm[pair * g.RS + t]), smax, s.y);
+        }
+    }
+    red[slice][lane] = s;
+    __syncthreads();
+    if (slice == 0 && e < pairs) {
+        for (int i = 1; i < 8; ++i) { s.x += red[i][lane].x; s.y += red[i][lane].y; }
+        if (galpha) galpha[k * g.C + c] = s.x;
+        if (gbeta) gbeta[k * g.C + c] = s.y;
+    }
+}
+
+// Arguments of one backward call (host side).
+struct SumBwdArgs {
+    Geo g;             // widened to whole quads (OW a multiple of 4)
+    int dtype;
+    const void *x, *w, *w2;
+    const float *alpha, *beta;
+    const void* gy;    // rows of g.OW elements
+    const uint8_t* codes;
+    void* gx;
+    float *gw, *gw2, *galpha, *gbeta, *gbias;
+    float* ws;         // sum_ws_bytes()
+    cudaStream_t st;
+    int launches;      // out
+};
+int bwd_sum_launch(SumBwdArgs& a);
+
+}  // namespace tconv
