@@ -277,7 +277,7 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
                         thi2 = best;
                     }
                     auto kern = g.RS == 9 ? bwd_idx_gx2_kernel<T, 9> : bwd_idx_gx2_kernel<T, 0>;
-                    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess)
+                    if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess)
                         return cuda_fail(cudaGetLastError());
                     if (thi2 > 0) {
                         const int tiles2 = (g.H + thi2 - 1) / thi2;
@@ -285,13 +285,13 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
                             g, (const T*)gy, idx, (T*)gx, thi2, tiles2, magic);
                     } else {
                         auto kern1 = bwd_idx_gx_kernel<T>;
-                        if (cudaFuncSetAttribute(kern1, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess)
+                        if (allow_smem(kern1, kBwdSmemAttr) != cudaSuccess)
                             return cuda_fail(cudaGetLastError());
                         kern1<<<(unsigned)(g.N * tiles), 256, smem, st>>>(g, (const T*)gy, idx, (T*)gx, thi, tiles, magic);
                     }
                 } else {
                     auto kern = bwd_idx_gx_kernel<T>;
-                    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess)
+                    if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess)
                         return cuda_fail(cudaGetLastError());
                     kern<<<(unsigned)(g.N * tiles), 256, smem, st>>>(g, (const T*)gy, idx, (T*)gx, thi, tiles, magic);
                 }
@@ -309,7 +309,7 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
             float* pw = (float*)ws;
             float* pb = pw + (size_t)chunks * g.K * CRS;
             auto kern = bwd_idx_gw_kernel<T>;
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess)
+            if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess)
                 return cuda_fail(cudaGetLastError());
             const int npc = (g.N + chunks - 1) / chunks;
             kern<<<dim3((unsigned)g.K, (unsigned)chunks), 256, smem, st>>>(g, (const T*)gy, idx, pw, pb, npc);
@@ -539,7 +539,7 @@ int dw_backward_t(const Geo& g, const void* x, const void* w, const void* w2, co
 #define TCONV_DW_PAR(BR, PARV)                                                                        \
     {                                                                                                \
         auto kern = dw_bwd_params_kernel<T, BR, PARV>;                                               \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) \
+        if (allow_smem(kern, (int)smem) != cudaSuccess) \
             return cuda_fail(cudaGetLastError());                                                    \
         kern<<<grid, 256, smem, st>>>(g, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, codes, partial, nch, need_ab); \
     }
@@ -552,7 +552,7 @@ int dw_backward_t(const Geo& g, const void* x, const void* w, const void* w2, co
 #define TCONV_DW_P3(BR, PARV, SWV, VECV)                                                              \
     {                                                                                                \
         auto kern = dw_bwd_params3_kernel<T, BR, PARV, SWV, VECV>;                                   \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) \
+        if (allow_smem(kern, (int)smem) != cudaSuccess) \
             return cuda_fail(cudaGetLastError());                                                    \
         kern<<<grid, 256, smem, st>>>(g, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, codes, partial, nch, \
                                       need_ab, QPR3, strips3);                                       \

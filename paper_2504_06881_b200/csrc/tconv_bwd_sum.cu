@@ -7,7 +7,7 @@ namespace {
 template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW>
 int launch_gx(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx) {
     auto kern = bwd_sum_gx_kernel<T, BR, GX, AB, WIDE, KW>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
+    if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
     kern<<<pl.ctas * (unsigned)a.g.C, pl.threads, pl.smem, a.st>>>(
         a.g, a.x, a.alpha, a.beta, (const T*)a.gy, a.codes, (T*)a.gx, part_ab, part_gx, pl);
     ++a.launches;
@@ -26,7 +26,7 @@ int launch_gx_window(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* 
 template <typename T, int BR, bool PAIRS, bool WIDE>
 int launch_gw(SumBwdArgs& a, const SumGwPlan& pl, float* part) {
     auto kern = pl.flat ? bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, true> : bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
+    if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
     kern<<<pl.grid, 128, pl.smem, a.st>>>(a.g, (const T*)a.gy, a.codes, part, pl);
     ++a.launches;
     return TCONV_OK;

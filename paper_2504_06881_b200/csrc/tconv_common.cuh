@@ -56,6 +56,32 @@ template <> __device__ __forceinline__ __nv_bfloat16 zero_of<__nv_bfloat16>() {
     return __float2bfloat16_rn(0.0f);
 }
 
+// cudaFuncSetAttribute for the dynamic shared memory of a kernel, remembered per host thread and device: the
+// call costs the host about as much as a launch, and its effect lasts.
+inline cudaError_t allow_smem_ptr(const void* kern, int bytes) {
+    struct Entry { const void* kern; int dev, bytes; };
+    constexpr unsigned kEntries = 256;          // (power of two; a full neighbourhood only repeats the call)
+    static thread_local Entry table[kEntries];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned h = (unsigned)(((uintptr_t)kern >> 4) * 2654435761u) + (unsigned)dev;
+    Entry* slot = nullptr;
+    for (unsigned i = 0; i < 8; ++i) {
+        Entry& t = table[(h + i) & (kEntries - 1)];
+        if (t.kern == kern && t.dev == dev) {
+            if (t.bytes >= bytes) return cudaSuccess;
+            slot = &t;
+            break;
+        }
+        if (!t.kern) { slot = &t; break; }
+    }
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && slot) *slot = Entry{kern, dev, bytes};
+    return e;
+}
+template <typename F> inline cudaError_t allow_smem(F* kern, int bytes) { return allow_smem_ptr((const void*)kern, bytes); }
+
 // Deterministic block-wide sum (fixed tree): every thread passes its partial,
 // thread 0 receives the total.  `red` holds blockDim.x floats.
 __device__ __forceinline__ float block_sum(float v, float* red) {

@@ -1032,7 +1032,7 @@ int launch_tiled_variant(FwdArgs& a) {
 #define TCONV_LAUNCH_F32_S(XTMAV, RAGV, STATSV)                                                       \
     {                                                                                                \
         auto kern = fwd_tiled_f32_kernel<MODE, CHAN, WIN, XTMAV, RAGV, R, S, SW, DW, Q, KG, PW, TK, STATSV>; \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) \
+        if (allow_smem(kern, 200 * 1024) != cudaSuccess) \
             return TCONV_ERR_CUDA;                                                                   \
         kern<<<pl.grid, pl.threads, pl.smem, a.st>>>(xmap, pl.p);                                    \
     }

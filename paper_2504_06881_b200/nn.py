@@ -14,7 +14,7 @@ import math
 import torch
 import torch.nn as nn
 
-from . import tconv
+from . import tconv, tconv3d
 
 
 def _emit_winners(recording, *tensors):
@@ -22,6 +22,39 @@ def _emit_winners(recording, *tensors):
     ``torch.is_grad_enabled()`` where the layer was called: inside a Function's forward the grad mode is
     always off, and parameters keep ``requires_grad`` under ``torch.no_grad``."""
     return recording and any(t is not None and t.requires_grad for t in tensors)
+
+
+def _as(t, dtype):
+    """t in the given type, dense; None stays None.  (Called with the grad mode off.)"""
+    if t is None:
+        return None
+    if t.dtype != dtype:
+        t = t.to(dtype)
+    return t if t.is_contiguous() else t.contiguous()
+
+
+def _make_desc2d(xs, ws, geom, x_f32):
+    (N, C, H, W), (K, _, R, S), (mode, chan, dtype, stride, pad, dil, _rec) = xs, ws, geom
+    d = tconv.PlannedDesc(N=N, C=C, H=H, W=W, K=K, R=R, S=S, stride_h=stride[0], stride_w=stride[1], pad_h=pad[0],
+                          pad_w=pad[1], dil_h=dil[0], dil_w=dil[1], mode=mode, chan=chan, dtype=dtype)
+    if x_f32:
+        d["x_dtype"] = "f32"
+    return d
+
+
+def _make_desc_dw(xs, ws, geom):
+    (N, C, H, W), (_, R, S), (mode, dtype, stride, pad, dil, _rec) = xs, ws, geom
+    return tconv.PlannedDesc(N=N, C=C, H=H, W=W, K=C, R=R, S=S, stride_h=stride[0], stride_w=stride[1], pad_h=pad[0],
+                             pad_w=pad[1], dil_h=dil[0], dil_w=dil[1], mode=mode, chan="sum", dtype=dtype)
+
+
+def _make_desc3d(xs, ws, geom):
+    (N, C, D, H, W), (K, _, T, R, S), (mode, chan, dtype, stride, pad, dil, _rec) = xs, ws, geom
+    return tconv.PlannedDesc(N=N, C=C, D=D, H=H, W=W, K=K, T=T, R=R, S=S, stride=tuple(stride), pad=tuple(pad),
+                             dil=tuple(dil), mode=mode, chan=chan, dtype=dtype)
+
+
+_descs2d, _descs_dw, _descs3d = map(tconv.KeptPlans, (_make_desc2d, _make_desc_dw, _make_desc3d))
 
 
 class TropicalConvFn(torch.autograd.Function):
@@ -39,23 +72,16 @@ class TropicalConvFn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, w2, alpha, beta, bias, geom):
-        mode, chan, dtype, stride, pad, dil, recording = geom
+        dtype, recording = geom[2], geom[6]
         dt = tconv.TORCH_DTYPE[dtype]
-        N, C, H, W = x.shape
-        K, _, R, S = w.shape
-        d = dict(N=N, C=C, H=H, W=W, K=K, R=R, S=S, stride_h=stride[0], stride_w=stride[1],
-                 pad_h=pad[0], pad_w=pad[1], dil_h=dil[0], dil_w=dil[1], mode=mode, chan=chan, dtype=dtype)
         # a float x for a bf16 layer is rounded by the kernel while it stages x (no cast kernel, no
         # bf16 copy); layers the tiled kernels do not serve fall back to the explicit cast
         fused_cast = TropicalConvFn.fuse_cast and dtype == "bf16" and x.dtype == torch.float32
-        xc = x.detach().contiguous() if fused_cast else x.detach().to(dt).contiguous()
-        if fused_cast:
-            d["x_dtype"] = "f32"
-        wc = w.detach().to(dt).contiguous()
-        w2c = w2.detach().to(dt).contiguous() if w2 is not None else None
-        al = alpha.detach().float().contiguous() if alpha is not None else None
-        be = beta.detach().float().contiguous() if beta is not None else None
-        bi = bias.detach().float().contiguous() if bias is not None else None
+        desc_of = lambda f32x: _descs2d.get((x.shape, w.shape, geom, f32x), x.shape, w.shape, geom, f32x)
+        d = desc_of(fused_cast)
+        xc = _as(x, x.dtype if fused_cast else dt)
+        wc, w2c = _as(w, dt), _as(w2, dt)
+        al, be, bi = _as(alpha, torch.float32), _as(beta, torch.float32), _as(bias, torch.float32)
         need_grad = _emit_winners(recording, x, w, w2, alpha, beta, bias)
         ev = TropicalConvFn.events
         if ev is not None:
@@ -66,8 +92,8 @@ class TropicalConvFn(torch.autograd.Function):
         except tconv.TconvError as err:
             if not fused_cast or err.status != -2:
                 raise
-            d.pop("x_dtype")
-            xc = x.detach().to(dt).contiguous()
+            d = desc_of(False)
+            xc = _as(x, dt)
             y, winners = tconv.forward(d, xc, wc, w2c, al, be, bi, want_winners=need_grad)
         if ev is not None:
             e1.record()
@@ -83,7 +109,7 @@ class TropicalConvFn(torch.autograd.Function):
         xc, wc, w2c, al, be, winners = ctx.saved_tensors
         d = ctx.d
         dt = tconv.TORCH_DTYPE[d["dtype"]]
-        g = gy.to(dt).contiguous()
+        g = _as(gy, dt)
         ev = TropicalConvFn.events
         if ev is not None:
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -350,18 +376,10 @@ class TropicalDepthwiseFn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, w2, alpha, beta, bias, geom):
-        mode, dtype, stride, pad, dil, recording = geom
-        dt = tconv.TORCH_DTYPE[dtype]
-        N, C, H, W = x.shape
-        _, R, S = w.shape
-        d = dict(N=N, C=C, H=H, W=W, K=C, R=R, S=S, stride_h=stride[0], stride_w=stride[1],
-                 pad_h=pad[0], pad_w=pad[1], dil_h=dil[0], dil_w=dil[1], mode=mode, chan="sum", dtype=dtype)
-        xc = x.detach().to(dt).contiguous()
-        wc = w.detach().to(dt).contiguous()
-        w2c = w2.detach().to(dt).contiguous() if w2 is not None else None
-        al = alpha.detach().float().contiguous() if alpha is not None else None
-        be = beta.detach().float().contiguous() if beta is not None else None
-        bi = bias.detach().float().contiguous() if bias is not None else None
+        dt, recording = tconv.TORCH_DTYPE[geom[1]], geom[5]
+        d = _descs_dw.get((x.shape, w.shape, geom), x.shape, w.shape, geom)
+        xc, wc, w2c = _as(x, dt), _as(w, dt), _as(w2, dt)
+        al, be, bi = _as(alpha, torch.float32), _as(beta, torch.float32), _as(bias, torch.float32)
         need_grad = _emit_winners(recording, x, w, w2, alpha, beta, bias)
         y, winners = tconv.dw_forward(d, xc, wc, w2c, al, be, bi, want_winners=need_grad)
         ctx.d, ctx.in_dtype = d, x.dtype
@@ -373,7 +391,7 @@ class TropicalDepthwiseFn(torch.autograd.Function):
     def backward(ctx, gy):
         xc, wc, w2c, al, be, winners = ctx.saved_tensors
         d = ctx.d
-        g = gy.to(tconv.TORCH_DTYPE[d["dtype"]]).contiguous()
+        g = _as(gy, tconv.TORCH_DTYPE[d["dtype"]])
         grads = tconv.dw_backward(d, xc, wc, g, w2c, al, be, winners)
         has_w2, has_a, has_b, has_bias = ctx.has
         return (grads["grad_x"].to(ctx.in_dtype), grads["grad_w"], grads.get("grad_w2") if has_w2 else None,
@@ -437,16 +455,10 @@ class TropicalConv3dFn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, w2, alpha, beta, bias, geom):
-        from . import tconv3d
-        mode, chan, dtype, stride, pad, dil, recording = geom
-        dt = tconv.TORCH_DTYPE[dtype]
-        N, C, D, H, W = x.shape
-        K, _, T, R, S = w.shape
-        d = dict(N=N, C=C, D=D, H=H, W=W, K=K, T=T, R=R, S=S, stride=tuple(stride), pad=tuple(pad),
-                 dil=tuple(dil), mode=mode, chan=chan, dtype=dtype)
-        cast = lambda t, ty: t.detach().to(ty).contiguous() if t is not None else None
-        xc, wc, w2c = cast(x, dt), cast(w, dt), cast(w2, dt)
-        al, be, bi = cast(alpha, torch.float32), cast(beta, torch.float32), cast(bias, torch.float32)
+        dt, recording = tconv.TORCH_DTYPE[geom[2]], geom[6]
+        d = _descs3d.get((x.shape, w.shape, geom), x.shape, w.shape, geom)
+        xc, wc, w2c = _as(x, dt), _as(w, dt), _as(w2, dt)
+        al, be, bi = _as(alpha, torch.float32), _as(beta, torch.float32), _as(bias, torch.float32)
         need_grad = _emit_winners(recording, x, w, w2, alpha, beta, bias)
         y, winners = tconv3d.forward(d, xc, wc, w2c, al, be, bi, want_winners=need_grad)
         ctx.d, ctx.in_dtype = d, x.dtype
@@ -456,10 +468,9 @@ class TropicalConv3dFn(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, gy):
-        from . import tconv3d
         xc, wc, w2c, al, be, winners = ctx.saved_tensors
         d = ctx.d
-        g = gy.detach().to(tconv.TORCH_DTYPE[d["dtype"]]).contiguous()
+        g = _as(gy, tconv.TORCH_DTYPE[d["dtype"]])
         grads = tconv3d.backward(d, xc, wc, g, w2c, al, be, winners, need_grad_x=ctx.needs_input_grad[0])
         has_w2, has_a, has_b, has_bias = ctx.has
         gx = grads["grad_x"].to(ctx.in_dtype) if "grad_x" in grads else None
@@ -501,4 +512,7 @@ class TropicalConv1d(nn.Module):
     def forward(self, x):                      # x: [N, C, L]
         if self.tiled:
             return self.conv(x.unsqueeze(2)).squeeze(2)
-        return self.conv(x[:, :, None, None, :])[:, :, 0, 0, :]
+        # (reshapes, not slices: the gradient of a slice would be written into a zeroed copy)
+        N, C, L = x.shape
+        y = self.conv(x.reshape(N, C, 1, 1, L))
+        return y.reshape(N, y.shape[1], y.shape[4])

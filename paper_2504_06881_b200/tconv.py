@@ -8,6 +8,7 @@ library has not been built (``python paper_2504_06881_b200/build.py``).
 from __future__ import annotations
 
 import ctypes
+import threading
 from pathlib import Path
 
 import torch
@@ -232,10 +233,111 @@ def tconv_launch_count() -> int:
 
 
 # ---- convenience: allocate outputs with torch, check the status ----------------------
+class Plan:
+    """What a layer's calls need beside its tensors, worked out once per descriptor: the C descriptor and
+    the shapes and sizes derived from it.  (Building the C structure and asking the library for them took
+    half of the host time of a small layer's call.)"""
+
+    __slots__ = ("desc", "ref", "x", "w", "kc", "k", "y", "dt", "xdt", "two", "par", "winner_bytes", "fwd_ws",
+                 "bwd_ws", "bwd_ws_stored")
+
+    def __init__(self, d: dict):
+        self.desc = make_desc(d)
+        self.ref = ctypes.byref(self.desc)
+        N, C, H, W, K, R, S = (d[k] for k in "NCHWKRS")
+        OH, OW = tconv_output_shape(d)
+        self.x, self.w, self.kc, self.k, self.y = (N, C, H, W), (K, C, R, S), (K, C), (K,), (N, K, OH, OW)
+        self.dt, self.xdt = TORCH_DTYPE[d["dtype"]], _x_dtype(d)
+        self.two, self.par = d["mode"] in ("compound", "parallel"), d["mode"] == "parallel"
+        self.winner_bytes = int(_lib.tconv_winner_bytes(self.ref))
+        self.fwd_ws = int(_lib.tconv_workspace_bytes(self.ref, 0))
+        self.bwd_ws = int(_lib.tconv_workspace_bytes(self.ref, 1))
+        # the figure includes room for recomputed winners, not needed when they are passed
+        self.bwd_ws_stored = max(0, self.bwd_ws - (self.winner_bytes + 255) // 256 * 256)
+
+
+class PlannedDesc(dict):
+    """A descriptor dict that carries its plan (made on first use; the dict must not change after that)."""
+
+    __slots__ = ("plan",)
+
+    def __init__(self, *args, **kw):
+        super().__init__(*args, **kw)
+        self.plan = None
+
+
+class KeptPlans:
+    """A bounded table of plans by key; when it is full the oldest half goes."""
+
+    def __init__(self, make, most=512):
+        self.make, self.most, self.table, self.lock = make, most, {}, threading.Lock()
+
+    def get(self, key, *args):
+        p = self.table.get(key)
+        if p is None:
+            p = self.make(*args)
+            with self.lock:
+                if len(self.table) >= self.most:
+                    for k in list(self.table)[:self.most // 2]:
+                        del self.table[k]
+                self.table[key] = p
+        return p
+
+
+_FIELDS = ("N", "C", "H", "W", "K", "R", "S", "stride_h", "stride_w", "pad_h", "pad_w", "dil_h", "dil_w", "mode",
+           "chan", "dtype", "pad_mode", "x_dtype")
+_plans = KeptPlans(Plan)
+
+
+class DwPlan:
+    """Plan of a depthwise layer."""
+
+    __slots__ = ("desc", "ref", "x", "w", "k", "y", "dt", "two", "par", "bwd_ws")
+
+    def __init__(self, d: dict):
+        self.desc = make_desc(d)
+        self.ref = ctypes.byref(self.desc)
+        N, C, H, W, R, S = (d[k] for k in "NCHWRS")
+        OH, OW = tconv_output_shape(d)
+        self.x, self.w, self.k, self.y = (N, C, H, W), (C, R, S), (C,), (N, C, OH, OW)
+        self.dt = TORCH_DTYPE[d["dtype"]]
+        self.two, self.par = d["mode"] in ("compound", "parallel"), d["mode"] == "parallel"
+        self.bwd_ws = int(_lib.tconv_dw_workspace_bytes(self.ref, 1))
+
+
+_dw_plans = KeptPlans(DwPlan)
+
+
+def dw_plan_of(d: dict) -> DwPlan:
+    if type(d) is PlannedDesc:
+        if d.plan is None:
+            d.plan = DwPlan(d)
+        return d.plan
+    return _dw_plans.get(tuple(map(d.get, _FIELDS)), d)
+
+
+def plan_of(d: dict) -> Plan:
+    if type(d) is PlannedDesc:
+        if d.plan is None:
+            d.plan = Plan(d)
+        return d.plan
+    return _plans.get(tuple(map(d.get, _FIELDS)), d)
+
+
+def _ptr(t):
+    return None if t is None else t.data_ptr()
+
+
+def _raw_stream(stream):
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
 def _check(t, shape, dtype, name):
     if t is None:
         return
-    if not t.is_cuda or not t.is_contiguous() or tuple(t.shape) != tuple(shape) or t.dtype != dtype:
+    if not t.is_cuda or not t.is_contiguous() or t.shape != shape or t.dtype != dtype:
         raise ValueError(f"{name}: need a contiguous CUDA tensor of shape {tuple(shape)} and dtype "
                          f"{dtype}, got {tuple(t.shape)} {t.dtype} on {t.device}")
 
@@ -259,21 +361,24 @@ def winner_buffer(d: dict, device) -> torch.Tensor:
     return torch.empty(tconv_winner_bytes(d), dtype=torch.uint8, device=device)
 
 
+def _check_layer(p, x, w, w2, alpha, beta, bias):
+    _check(x, p.x, p.xdt, "x"); _check(w, p.w, p.dt, "w"); _check(w2, p.w, p.dt, "w2")
+    _check(alpha, p.kc, torch.float32, "alpha"); _check(beta, p.kc, torch.float32, "beta")
+    _check(bias, p.k, torch.float32, "bias")
+
+
 def forward(d: dict, x, w, w2=None, alpha=None, beta=None, bias=None, want_winners=False,
             stream=None):
     """Allocate y (and the winner buffer) and run tconv_forward.  Returns (y, winners)."""
-    N, C, H, W, K, R, S = (d[k] for k in "NCHWKRS")
-    dt = TORCH_DTYPE[d["dtype"]]
-    _check(x, (N, C, H, W), _x_dtype(d), "x"); _check(w, (K, C, R, S), dt, "w"); _check(w2, (K, C, R, S), dt, "w2")
-    _check(alpha, (K, C), torch.float32, "alpha"); _check(beta, (K, C), torch.float32, "beta")
-    _check(bias, (K,), torch.float32, "bias")
-    OH, OW = tconv_output_shape(d)
-    y = torch.empty((N, K, OH, OW), dtype=dt, device=x.device)
-    winners = winner_buffer(d, x.device) if want_winners else None
-    nws = tconv_workspace_bytes(d, False)
-    ws = torch.empty(nws, dtype=torch.uint8, device=x.device) if nws else None
+    p = plan_of(d)
+    _check_layer(p, x, w, w2, alpha, beta, bias)
+    dev = x.device
+    y = torch.empty(p.y, dtype=p.dt, device=dev)
+    winners = torch.empty(p.winner_bytes, dtype=torch.uint8, device=dev) if want_winners else None
+    ws = torch.empty(p.fwd_ws, dtype=torch.uint8, device=dev) if p.fwd_ws else None
     _on_stream(stream, y, winners, ws)
-    rc = tconv_forward(d, x, w, w2, alpha, beta, bias, y, winners, ws, stream)
+    rc = _lib.tconv_forward(p.ref, x.data_ptr(), w.data_ptr(), _ptr(w2), _ptr(alpha), _ptr(beta), _ptr(bias),
+                            y.data_ptr(), _ptr(winners), _ptr(ws), p.fwd_ws, _raw_stream(stream))
     if rc != 0:
         raise TconvError(rc, "tconv_forward")
     return y, winners
@@ -303,36 +408,32 @@ def forward_stats(d: dict, x, w, w2=None, alpha=None, beta=None, bias=None, want
 def backward(d: dict, x, w, grad_y, w2=None, alpha=None, beta=None, winners=None, stream=None,
              need=("grad_x", "grad_w", "grad_w2", "grad_alpha", "grad_beta", "grad_bias")):
     """Allocate the gradients named in `need` and run tconv_backward.  Returns a dict."""
-    N, C, H, W, K, R, S = (d[k] for k in "NCHWKRS")
-    dt = TORCH_DTYPE[d["dtype"]]
-    OH, OW = tconv_output_shape(d)
-    _check(x, (N, C, H, W), _x_dtype(d), "x"); _check(w, (K, C, R, S), dt, "w"); _check(w2, (K, C, R, S), dt, "w2")
-    _check(grad_y, (N, K, OH, OW), dt, "grad_y")
-    two = d["mode"] in ("compound", "parallel")
+    p = plan_of(d)
+    _check(x, p.x, p.xdt, "x"); _check(w, p.w, p.dt, "w"); _check(w2, p.w, p.dt, "w2")
+    _check(grad_y, p.y, p.dt, "grad_y")
     dev = x.device
     f32 = torch.float32
     out = {}
     if "grad_x" in need:
-        out["grad_x"] = torch.empty((N, C, H, W), dtype=dt, device=dev)
+        out["grad_x"] = torch.empty(p.x, dtype=p.dt, device=dev)
     if "grad_w" in need:
-        out["grad_w"] = torch.empty((K, C, R, S), dtype=f32, device=dev)
-    if "grad_w2" in need and d["mode"] == "parallel":
-        out["grad_w2"] = torch.empty((K, C, R, S), dtype=f32, device=dev)
-    if "grad_alpha" in need and two:
-        out["grad_alpha"] = torch.empty((K, C), dtype=f32, device=dev)
-    if "grad_beta" in need and two:
-        out["grad_beta"] = torch.empty((K, C), dtype=f32, device=dev)
+        out["grad_w"] = torch.empty(p.w, dtype=f32, device=dev)
+    if p.par and "grad_w2" in need:
+        out["grad_w2"] = torch.empty(p.w, dtype=f32, device=dev)
+    if p.two and "grad_alpha" in need:
+        out["grad_alpha"] = torch.empty(p.kc, dtype=f32, device=dev)
+    if p.two and "grad_beta" in need:
+        out["grad_beta"] = torch.empty(p.kc, dtype=f32, device=dev)
     if "grad_bias" in need:
-        out["grad_bias"] = torch.empty((K,), dtype=f32, device=dev)
-    nws = tconv_workspace_bytes(d, True)
-    if winners is not None:
-        # the figure includes room for recomputed winners, not needed when they are passed
-        nws -= (tconv_winner_bytes(d) + 255) // 256 * 256
+        out["grad_bias"] = torch.empty(p.k, dtype=f32, device=dev)
+    nws = p.bwd_ws if winners is None else p.bwd_ws_stored
     ws = torch.empty(nws, dtype=torch.uint8, device=dev) if nws > 0 else None
     _on_stream(stream, ws, *out.values())
-    rc = tconv_backward(d, x, w, w2, alpha, beta, grad_y, winners, out.get("grad_x"),
-                        out.get("grad_w"), out.get("grad_w2"), out.get("grad_alpha"),
-                        out.get("grad_beta"), out.get("grad_bias"), ws, stream)
+    get = out.get
+    rc = _lib.tconv_backward(p.ref, x.data_ptr(), w.data_ptr(), _ptr(w2), _ptr(alpha), _ptr(beta),
+                             grad_y.data_ptr(), _ptr(winners), _ptr(get("grad_x")), _ptr(get("grad_w")),
+                             _ptr(get("grad_w2")), _ptr(get("grad_alpha")), _ptr(get("grad_beta")),
+                             _ptr(get("grad_bias")), _ptr(ws), nws, _raw_stream(stream))
     if rc != 0:
         raise TconvError(rc, "tconv_backward")
     return out
@@ -340,16 +441,15 @@ def backward(d: dict, x, w, grad_y, w2=None, alpha=None, beta=None, winners=None
 
 def dw_forward(d: dict, x, w, w2=None, alpha=None, beta=None, bias=None, want_winners=False, stream=None):
     """Depthwise form: allocate y (and the winner codes) and run tconv_dw_forward.  Returns (y, winners)."""
-    N, C, H, W, R, S = (d[k] for k in "NCHWRS")
-    dt = TORCH_DTYPE[d["dtype"]]
-    _check(x, (N, C, H, W), dt, "x"); _check(w, (C, R, S), dt, "w"); _check(w2, (C, R, S), dt, "w2")
-    _check(alpha, (C,), torch.float32, "alpha"); _check(beta, (C,), torch.float32, "beta")
-    _check(bias, (C,), torch.float32, "bias")
-    OH, OW = tconv_output_shape(d)
-    y = torch.empty((N, C, OH, OW), dtype=dt, device=x.device)
-    winners = torch.empty((N, C, OH, OW), dtype=torch.uint8, device=x.device) if want_winners else None
+    p = dw_plan_of(d)
+    _check(x, p.x, p.dt, "x"); _check(w, p.w, p.dt, "w"); _check(w2, p.w, p.dt, "w2")
+    _check(alpha, p.k, torch.float32, "alpha"); _check(beta, p.k, torch.float32, "beta")
+    _check(bias, p.k, torch.float32, "bias")
+    y = torch.empty(p.y, dtype=p.dt, device=x.device)
+    winners = torch.empty(p.y, dtype=torch.uint8, device=x.device) if want_winners else None
     _on_stream(stream, y, winners)
-    rc = tconv_dw_forward(d, x, w, w2, alpha, beta, bias, y, winners, stream)
+    rc = _lib.tconv_dw_forward(p.ref, x.data_ptr(), w.data_ptr(), _ptr(w2), _ptr(alpha), _ptr(beta), _ptr(bias),
+                               y.data_ptr(), _ptr(winners), _raw_stream(stream))
     if rc != 0:
         raise TconvError(rc, "tconv_dw_forward")
     return y, winners
@@ -357,26 +457,25 @@ def dw_forward(d: dict, x, w, w2=None, alpha=None, beta=None, bias=None, want_wi
 
 def dw_backward(d: dict, x, w, grad_y, w2=None, alpha=None, beta=None, winners=None, stream=None):
     """Depthwise form: allocate every gradient the mode has and run tconv_dw_backward.  Returns a dict."""
-    N, C, H, W, R, S = (d[k] for k in "NCHWRS")
-    dt = TORCH_DTYPE[d["dtype"]]
-    OH, OW = tconv_output_shape(d)
-    _check(x, (N, C, H, W), dt, "x"); _check(w, (C, R, S), dt, "w"); _check(w2, (C, R, S), dt, "w2")
-    _check(grad_y, (N, C, OH, OW), dt, "grad_y")
-    two, par = d["mode"] in ("compound", "parallel"), d["mode"] == "parallel"
+    p = dw_plan_of(d)
+    _check(x, p.x, p.dt, "x"); _check(w, p.w, p.dt, "w"); _check(w2, p.w, p.dt, "w2")
+    _check(grad_y, p.y, p.dt, "grad_y")
     dev, f32 = x.device, torch.float32
-    out = {"grad_x": torch.empty((N, C, H, W), dtype=dt, device=dev),
-           "grad_w": torch.empty((C, R, S), dtype=f32, device=dev),
-           "grad_bias": torch.empty((C,), dtype=f32, device=dev)}
-    if par:
-        out["grad_w2"] = torch.empty((C, R, S), dtype=f32, device=dev)
-    if two:
-        out["grad_alpha"] = torch.empty((C,), dtype=f32, device=dev)
-        out["grad_beta"] = torch.empty((C,), dtype=f32, device=dev)
-    ws = torch.empty(tconv_dw_workspace_bytes(d, True), dtype=torch.uint8, device=dev)
+    out = {"grad_x": torch.empty(p.x, dtype=p.dt, device=dev), "grad_w": torch.empty(p.w, dtype=f32, device=dev),
+           "grad_bias": torch.empty(p.k, dtype=f32, device=dev)}
+    if p.par:
+        out["grad_w2"] = torch.empty(p.w, dtype=f32, device=dev)
+    if p.two:
+        out["grad_alpha"] = torch.empty(p.k, dtype=f32, device=dev)
+        out["grad_beta"] = torch.empty(p.k, dtype=f32, device=dev)
+    ws = torch.empty(p.bwd_ws, dtype=torch.uint8, device=dev)
     _on_stream(stream, ws, *out.values())
-    rc = tconv_dw_backward(d, x, w, w2, alpha, beta, grad_y, winners, out["grad_x"], out["grad_w"],
-                           out.get("grad_w2"), out.get("grad_alpha"), out.get("grad_beta"),
-                           out["grad_bias"], ws, stream)
+    get = out.get
+    rc = _lib.tconv_dw_backward(p.ref, x.data_ptr(), w.data_ptr(), _ptr(w2), _ptr(alpha), _ptr(beta),
+                                grad_y.data_ptr(), _ptr(winners), out["grad_x"].data_ptr(),
+                                out["grad_w"].data_ptr(), _ptr(get("grad_w2")), _ptr(get("grad_alpha")),
+                                _ptr(get("grad_beta")), out["grad_bias"].data_ptr(), ws.data_ptr(), p.bwd_ws,
+                                _raw_stream(stream))
     if rc != 0:
         raise TconvError(rc, "tconv_dw_backward")
     return out

@@ -10,7 +10,8 @@ import ctypes
 
 import torch
 
-from .tconv import CHANS, DTYPES, MODES, TORCH_DTYPE, TconvError, _check, _lib, _on_stream, _p, _stream
+from .tconv import (CHANS, DTYPES, MODES, TORCH_DTYPE, KeptPlans, PlannedDesc, TconvError, _check, _lib, _on_stream,
+                    _p, _ptr, _raw_stream, _stream)
 
 # every symbol include/tconv3d.h declares
 SYMBOLS = ("tconv3d_output_shape", "tconv3d_winner_bytes", "tconv3d_workspace_bytes", "tconv3d_forward",
@@ -90,28 +91,58 @@ def _shapes(d):
     return (N, C, D, H, W), (K, C, T, R, S), (N, K) + tconv3d_output_shape(d)
 
 
+class Plan3:
+    """What a layer's calls need beside its tensors (see tconv.Plan)."""
+
+    __slots__ = ("desc", "ref", "x", "w", "y", "kc", "k", "dt", "two", "par", "winner_shape", "winner_dtype", "bwd_ws")
+
+    def __init__(self, d: dict):
+        self.desc = make_desc(d)
+        self.ref = ctypes.byref(self.desc)
+        self.x, self.w, self.y = _shapes(d)
+        self.kc, self.k = (d["K"], d["C"]), (d["K"],)
+        self.dt = TORCH_DTYPE[d.get("dtype", "f32")]
+        self.two, self.par = d["mode"] in ("compound", "parallel"), d["mode"] == "parallel"
+        chan = d.get("chan", "default")
+        if chan == "default":
+            chan = {"max_plus": "max", "min_plus": "min"}.get(d["mode"], "sum")
+        if chan == "sum":
+            self.winner_shape, self.winner_dtype = self.y[:2] + (d["C"],) + self.y[2:], torch.int16
+        else:
+            self.winner_shape, self.winner_dtype = self.y, torch.int32
+        self.bwd_ws = int(_lib.tconv3d_workspace_bytes(self.ref, 1))
+
+
+_plans = KeptPlans(Plan3)
+_FIELDS = ("N", "C", "D", "H", "W", "K", "T", "R", "S", "stride", "pad", "dil", "mode", "chan", "dtype")
+
+
+def plan_of(d: dict) -> Plan3:
+    if type(d) is PlannedDesc:
+        if d.plan is None:
+            d.plan = Plan3(d)
+        return d.plan
+    return _plans.get(tuple(tuple(v) if isinstance(v, list) else v for v in map(d.get, _FIELDS)), d)
+
+
 def winner_buffer(d: dict, device):
     """Buffer for the winning taps: uint16 [N,K,C,OD,OH,OW] (Sum channel combine) or int32 [N,K,OD,OH,OW]."""
-    _, _, sy = _shapes(d)
-    chan = d.get("chan", "default")
-    if chan == "default":
-        chan = {"max_plus": "max", "min_plus": "min"}.get(d["mode"], "sum")
-    if chan == "sum":
-        return torch.empty((sy[0], sy[1], d["C"]) + sy[2:], dtype=torch.int16, device=device)
-    return torch.empty(sy, dtype=torch.int32, device=device)
+    p = plan_of(d)
+    return torch.empty(p.winner_shape, dtype=p.winner_dtype, device=device)
 
 
 def forward(d: dict, x, w, w2=None, alpha=None, beta=None, bias=None, want_winners=False, stream=None):
     """Allocate y (and the winners) and run tconv3d_forward.  Returns (y, winners)."""
-    sx, sw, sy = _shapes(d)
-    dt = TORCH_DTYPE[d.get("dtype", "f32")]
-    _check(x, sx, dt, "x"); _check(w, sw, dt, "w"); _check(w2, sw, dt, "w2")
-    _check(alpha, (d["K"], d["C"]), torch.float32, "alpha"); _check(beta, (d["K"], d["C"]), torch.float32, "beta")
-    _check(bias, (d["K"],), torch.float32, "bias")
-    y = torch.empty(sy, dtype=dt, device=x.device)
-    winners = winner_buffer(d, x.device) if want_winners else None
+    p = plan_of(d)
+    _check(x, p.x, p.dt, "x"); _check(w, p.w, p.dt, "w"); _check(w2, p.w, p.dt, "w2")
+    _check(alpha, p.kc, torch.float32, "alpha"); _check(beta, p.kc, torch.float32, "beta")
+    _check(bias, p.k, torch.float32, "bias")
+    dev = x.device
+    y = torch.empty(p.y, dtype=p.dt, device=dev)
+    winners = torch.empty(p.winner_shape, dtype=p.winner_dtype, device=dev) if want_winners else None
     _on_stream(stream, y, winners)
-    rc = tconv3d_forward(d, x, w, w2, alpha, beta, bias, y, winners, stream)
+    rc = _lib.tconv3d_forward(p.ref, x.data_ptr(), w.data_ptr(), _ptr(w2), _ptr(alpha), _ptr(beta), _ptr(bias),
+                              y.data_ptr(), _ptr(winners), _raw_stream(stream))
     if rc != 0:
         raise TconvError(rc, "tconv3d_forward")
     return y, winners
@@ -120,24 +151,24 @@ def forward(d: dict, x, w, w2=None, alpha=None, beta=None, bias=None, want_winne
 def backward(d: dict, x, w, grad_y, w2=None, alpha=None, beta=None, winners=None, need_grad_x=True,
              stream=None):
     """Allocate every gradient the mode has and run tconv3d_backward.  Returns a dict."""
-    sx, sw, sy = _shapes(d)
-    dt = TORCH_DTYPE[d.get("dtype", "f32")]
-    _check(x, sx, dt, "x"); _check(w, sw, dt, "w"); _check(w2, sw, dt, "w2"); _check(grad_y, sy, dt, "grad_y")
-    two, par = d["mode"] in ("compound", "parallel"), d["mode"] == "parallel"
+    p = plan_of(d)
+    _check(x, p.x, p.dt, "x"); _check(w, p.w, p.dt, "w"); _check(w2, p.w, p.dt, "w2"); _check(grad_y, p.y, p.dt, "grad_y")
     dev, f32 = x.device, torch.float32
-    out = {"grad_w": torch.empty(sw, dtype=f32, device=dev), "grad_bias": torch.empty((d["K"],), dtype=f32, device=dev)}
+    out = {"grad_w": torch.empty(p.w, dtype=f32, device=dev), "grad_bias": torch.empty(p.k, dtype=f32, device=dev)}
     if need_grad_x:
-        out["grad_x"] = torch.empty(sx, dtype=dt, device=dev)
-    if par:
-        out["grad_w2"] = torch.empty(sw, dtype=f32, device=dev)
-    if two:
-        out["grad_alpha"] = torch.empty((d["K"], d["C"]), dtype=f32, device=dev)
-        out["grad_beta"] = torch.empty((d["K"], d["C"]), dtype=f32, device=dev)
-    ws = torch.empty(tconv3d_workspace_bytes(d, True), dtype=torch.uint8, device=dev)
+        out["grad_x"] = torch.empty(p.x, dtype=p.dt, device=dev)
+    if p.par:
+        out["grad_w2"] = torch.empty(p.w, dtype=f32, device=dev)
+    if p.two:
+        out["grad_alpha"] = torch.empty(p.kc, dtype=f32, device=dev)
+        out["grad_beta"] = torch.empty(p.kc, dtype=f32, device=dev)
+    ws = torch.empty(p.bwd_ws, dtype=torch.uint8, device=dev)
     _on_stream(stream, ws, *out.values())
-    rc = tconv3d_backward(d, x, w, w2, alpha, beta, grad_y, winners, out.get("grad_x"), out["grad_w"],
-                          out.get("grad_w2"), out.get("grad_alpha"), out.get("grad_beta"), out["grad_bias"],
-                          ws, stream)
+    get = out.get
+    rc = _lib.tconv3d_backward(p.ref, x.data_ptr(), w.data_ptr(), _ptr(w2), _ptr(alpha), _ptr(beta),
+                               grad_y.data_ptr(), _ptr(winners), _ptr(get("grad_x")), out["grad_w"].data_ptr(),
+                               _ptr(get("grad_w2")), _ptr(get("grad_alpha")), _ptr(get("grad_beta")),
+                               out["grad_bias"].data_ptr(), ws.data_ptr(), p.bwd_ws, _raw_stream(stream))
     if rc != 0:
         raise TconvError(rc, "tconv3d_backward")
     return out
