@@ -124,6 +124,30 @@ __device__ __forceinline__ unsigned short load_x(const unsigned short* x, size_t
     return __bfloat16_as_ushort(__float2bfloat16_rn(reinterpret_cast<const float*>(x)[i]));
 }
 
+// Extremum m of R rows of three tap sums (pixel pairs) and, per half, the lowest tap that attains it,
+// shifted left by SH.  NaN taps (neutral padding) never equal it.
+template <int R, int SH>
+__device__ __forceinline__ unsigned win_taps(const unsigned* t, bool is_min, unsigned& m) {
+    auto eq = [](unsigned a, unsigned b) { return __heq2_mask(as_bf162(a), as_bf162(b)); };
+    auto pick = [](unsigned mask, unsigned a, unsigned b) { return (mask & a) | (~mask & b); };
+    constexpr unsigned one = 0x00010001u << SH;
+    unsigned row[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) row[r] = hext2u(hext2u(t[3 * r], t[3 * r + 1], is_min), t[3 * r + 2], is_min);
+    m = row[0];
+#pragma unroll
+    for (int r = 1; r < R; ++r) m = hext2u(m, row[r], is_min);
+    unsigned u = t[3 * (R - 1)], v = t[3 * (R - 1) + 1], first = 3 * (R - 1) * one;
+#pragma unroll
+    for (int r = R - 2; r >= 0; --r) {
+        const unsigned e = eq(row[r], m);
+        u = pick(e, t[3 * r], u);
+        v = pick(e, t[3 * r + 1], v);
+        first = pick(e, 3 * r * one, first);
+    }
+    return first + pick(eq(u, m), 0u, pick(eq(v, m), one, 2 * one));
+}
+
 // KPT words of packed weights of one tap (one or two 16-byte loads)
 template <int KPT>
 __device__ __forceinline__ void loadw(const unsigned* p, unsigned* out) {
@@ -326,6 +350,22 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
         }
 
     const size_t plane = (size_t)g.OH * g.OW;
+    // Sum forms with winners: where this thread's codes of (its first output channel, the next input
+    // channel) go, the distance between two output channels, and how many of its channels exist
+    const size_t cplane = (size_t)g.OH * g.OWP, kstep = (size_t)g.C * cplane;
+    const int klim = g.K - (kt * TILE_K + kg * KPT);
+    uint8_t* code_ptr[Q];
+    bool code_ok[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        code_ptr[q] = nullptr;
+        code_ok[q] = false;
+        if constexpr (WIN && SUMF) {
+            code_ok[q] = out_row[q] >= 0 && qcol[q] < g.OW;
+            const int n = max(out_row[q], 0) / g.OH, oh = max(out_row[q], 0) - n * g.OH;
+            code_ptr[q] = reinterpret_cast<uint8_t*>(p.winners) + ((size_t)n * g.K + kt * TILE_K + kg * KPT) * kstep + (size_t)oh * g.OWP + qcol[q];
+        }
+    }
     const int row_step = g.dh * pitch_w;
     const int chan_step = p.NSLOTS * pitch_w;
     issue_chunk(0, 0);
@@ -362,56 +402,68 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
 
             unsigned mx[CARRIED ? 1 : KPT][Q][2];
             unsigned mn[TWO ? KPT : 1][Q][2];
-            unsigned amx[(WIN && SUMF) ? KPT : 1][Q][2], amn[(WIN && TWO) ? KPT : 1][Q][2];
 
             if constexpr (WIN && SUMF) {
+                // Sum forms that emit winners, one output channel and one pixel pair at a time: the tap sums
+                // stay in registers, feed the extrema (three-input min / max, row by row), and then give the
+                // winning taps: the first row whose extremum is the window's, that row's first two taps by
+                // selects, and the first of its taps that equals the extremum (win_taps).  13 instructions
+                // per branch and pair; comparing every tap took 16 and tracking the tap while folding 26.
+                constexpr bool DO_MIN = TWO || TAP_MIN, DO_MAX = TWO || !TAP_MIN;
+                float av[KPT], bv[KPT];
+                if constexpr (TWO) {
+                    loadn<KPT>(as + cc * TILE_K, av);
+                    loadn<KPT>(bs + cc * TILE_K, bv);
+                }
 #pragma unroll
-                for (int tap = 0; tap < RS; ++tap) {
-                    constexpr unsigned one2 = 0x00010001u;
-                    const unsigned tap2 = one2 * (unsigned)tap;
-                    const int r = tap / S, sx = tap % S;
-                    unsigned wv[KPT], wv2[KPT];
-                    loadw<KPT>(wc + tap * TILE_K, wv);
-                    if constexpr (PAR) loadw<KPT>(wc2 + tap * TILE_K, wv2);
+                for (int q = 0; q < Q; ++q) {
+                    unsigned xp[RS][2];
 #pragma unroll
-                    for (int q = 0; q < Q; ++q)
+                    for (int r = 0; r < R; ++r) {
+                        xp[r * 3][0] = pixel_pair<SW, EODD + 0 * SW + 0 * DW>(xw[q][r]); xp[r * 3][1] = pixel_pair<SW, EODD + 2 * SW + 0 * DW>(xw[q][r]);
+                        xp[r * 3 + 1][0] = pixel_pair<SW, EODD + 0 * SW + 1 * DW>(xw[q][r]); xp[r * 3 + 1][1] = pixel_pair<SW, EODD + 2 * SW + 1 * DW>(xw[q][r]);
+                        xp[r * 3 + 2][0] = pixel_pair<SW, EODD + 0 * SW + 2 * DW>(xw[q][r]); xp[r * 3 + 2][1] = pixel_pair<SW, EODD + 2 * SW + 2 * DW>(xw[q][r]);
+                    }
+                    uint8_t* dst = code_ptr[q];
 #pragma unroll
-                        for (int pp = 0; pp < 2; ++pp) {
-                            unsigned xp;
-                            // compile-time element offset of this pair: unrolled over (sx, pp)
-                            if (sx == 0) xp = pp == 0 ? pixel_pair<SW, EODD + 0 * SW + 0 * DW>(xw[q][r]) : pixel_pair<SW, EODD + 2 * SW + 0 * DW>(xw[q][r]);
-                            else if (sx == 1) xp = pp == 0 ? pixel_pair<SW, EODD + 0 * SW + 1 * DW>(xw[q][r]) : pixel_pair<SW, EODD + 2 * SW + 1 * DW>(xw[q][r]);
-                            else xp = pp == 0 ? pixel_pair<SW, EODD + 0 * SW + 2 * DW>(xw[q][r]) : pixel_pair<SW, EODD + 2 * SW + 2 * DW>(xw[q][r]);
+                    for (int kp = 0; kp < KPT / 2; ++kp) {
+                        uint2 wa[RS], wb[PAR ? RS : 1];
 #pragma unroll
-                            for (int k = 0; k < KPT; ++k) {
-                                const unsigned t = hadd2u(xp, wv[k]);
-                                const unsigned t2 = PAR ? hadd2u(xp, wv2[k]) : t;
-                                if constexpr (TWO) {
-                                    if (tap == 0 && !g.neutral) {
-                                        mn[k][q][pp] = t; amn[k][q][pp] = 0u; mx[k][q][pp] = t2; amx[k][q][pp] = 0u;
-                                    } else {
-                                        if (tap == 0) {   // neutral padding: tap 0 may be a NaN; start from the identities
-                                            mn[k][q][pp] = kPosInf2; mx[k][q][pp] = kNegInf2; amn[k][q][pp] = amx[k][q][pp] = 0u;
-                                        }
-                                        const unsigned ml = hbetter_mask(t, mn[k][q][pp], true);
-                                        mn[k][q][pp] = hext2u(mn[k][q][pp], t, true);
-                                        amn[k][q][pp] = (tap2 & ml) | (amn[k][q][pp] & ~ml);
-                                        const unsigned mg = hbetter_mask(t2, mx[k][q][pp], false);
-                                        mx[k][q][pp] = hext2u(mx[k][q][pp], t2, false);
-                                        amx[k][q][pp] = (tap2 & mg) | (amx[k][q][pp] & ~mg);
-                                    }
-                                } else {
-                                    if (tap == 0 && !g.neutral) {
-                                        mx[k][q][pp] = t; amx[k][q][pp] = 0u;
-                                    } else {
-                                        if (tap == 0) { mx[k][q][pp] = TAP_MIN ? kPosInf2 : kNegInf2; amx[k][q][pp] = 0u; }
-                                        const unsigned mg = hbetter_mask(t, mx[k][q][pp], TAP_MIN);
-                                        mx[k][q][pp] = hext2u(mx[k][q][pp], t, TAP_MIN);
-                                        amx[k][q][pp] = (tap2 & mg) | (amx[k][q][pp] & ~mg);
-                                    }
-                                }
-                            }
+                        for (int tap = 0; tap < RS; ++tap) {
+                            wa[tap] = *reinterpret_cast<const uint2*>(wc + tap * TILE_K + 2 * kp);
+                            if constexpr (PAR) wb[tap] = *reinterpret_cast<const uint2*>(wc2 + tap * TILE_K + 2 * kp);
                         }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int k = 2 * kp + h;
+                            unsigned c2[2];
+#pragma unroll
+                            for (int pp = 0; pp < 2; ++pp) {
+                                unsigned ta[RS], tb[PAR ? RS : 1];
+#pragma unroll
+                                for (int tap = 0; tap < RS; ++tap) {
+                                    ta[tap] = hadd2u(xp[tap][pp], h == 0 ? wa[tap].x : wa[tap].y);
+                                    if constexpr (PAR) tb[tap] = hadd2u(xp[tap][pp], h == 0 ? wb[tap].x : wb[tap].y);
+                                }
+                                unsigned lo = 0u, hi = 0u, code = 0u;
+                                if constexpr (DO_MIN) code = win_taps<R, 0>(ta, true, lo);
+                                if constexpr (DO_MAX) code |= win_taps<R, 4>(PAR ? tb : ta, false, hi);
+                                float* a2 = acc[k][q] + 2 * pp;
+                                if constexpr (TWO) {
+                                    fma2(av[k], bf_lo(lo), bf_hi(lo), a2[0], a2[1]);
+                                    fma2(bv[k], bf_lo(hi), bf_hi(hi), a2[0], a2[1]);
+                                } else {
+                                    const unsigned m = TAP_MIN ? lo : hi;
+                                    addpair(bf_lo(m), bf_hi(m), a2[0], a2[1]);
+                                }
+                                c2[pp] = code;
+                            }
+                            // the quad's 4 codes in one store (code rows are padded to whole quads)
+                            if (k < klim && code_ok[q]) *reinterpret_cast<unsigned*>(dst) = __byte_perm(c2[0], c2[1], 0x6420);
+                            dst += kstep;
+                        }
+                    }
+                    code_ptr[q] += cplane;
                 }
             } else {
                 constexpr int FIRST = CARRIED ? 2 : (RS >= 3 ? 3 : RS);
@@ -474,7 +526,7 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
             }
 
             // channel combine
-            if constexpr (!CARRIED) {
+            if constexpr (!CARRIED && !(WIN && SUMF)) {
                 float av[KPT], bv[KPT];
                 if constexpr (TWO) {
                     loadn<KPT>(as + cc * TILE_K, av);
@@ -500,32 +552,6 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
                                 best[k][q][pp] = hext2u(best[k][q][pp], mx[k][q][pp], CHAN == CH_MIN);
                             }
                         }
-                if constexpr (WIN && SUMF) {
-                    uint8_t* codes = reinterpret_cast<uint8_t*>(p.winners);
-#pragma unroll
-                    for (int q = 0; q < Q; ++q) {
-                        if (out_row[q] < 0) continue;
-                        const int n = out_row[q] / g.OH, oh = out_row[q] - n * g.OH;
-#pragma unroll
-                        for (int k = 0; k < KPT; ++k) {
-                            const int kk = kt * TILE_K + kg * KPT + k;
-                            if (kk >= g.K) continue;
-                            uint8_t* dst = codes + (((size_t)n * g.K + kk) * g.C + c) * ((size_t)g.OH * g.OWP) +
-                                           (size_t)oh * g.OWP + qcol[q];
-                            unsigned c01, c23;
-                            if constexpr (TWO) {
-                                c01 = amn[k][q][0] | (amx[k][q][0] << 4);
-                                c23 = amn[k][q][1] | (amx[k][q][1] << 4);
-                            } else {
-                                c01 = TAP_MIN ? amx[k][q][0] : (amx[k][q][0] << 4);
-                                c23 = TAP_MIN ? amx[k][q][1] : (amx[k][q][1] << 4);
-                            }
-                            const unsigned packed = __byte_perm(c01, c23, 0x6420);
-                            // the quad's 4 codes in one store (code rows are padded to whole quads)
-                            if (qcol[q] < g.OW) *reinterpret_cast<unsigned*>(dst) = packed;
-                        }
-                    }
-                }
             }
         }
         __syncthreads();
@@ -666,7 +692,7 @@ int launch_tiled_variant_bf16(FwdArgs& a) {
 #define TCONV_LAUNCH_BF16_S(XTMAV, RAGV, STATSV)                                                      \
     {                                                                                                \
         auto kern = fwd_tiled_bf16_kernel<MODE, CHAN, WIN, XTMAV, RAGV, R, S, SW, DW, Q, KG, PW, KPT, STATSV>; \
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) \
+        if (allow_smem(kern, 200 * 1024) != cudaSuccess) \
             return TCONV_ERR_CUDA;                                                                   \
         kern<<<pl.grid, pl.threads, pl.smem, a.st>>>(xmap, pl.p);                                    \
     }
