@@ -161,11 +161,38 @@ Plan1 plan_1d(const Geo3& g) {
     return p;
 }
 
+// Parameter gradients of the other layers: private columns per thread (a window's taps and branches decide how
+// many threads a block can have), the (n, position) range split so that the blocks fill the SMs once.
+struct PlanParams3 {
+    int tb, nsplit;
+    size_t smem, scratch_floats;
+};
+PlanParams3 plan_params3(const Geo3& g) {
+    PlanParams3 p;
+    const int branches = two_branch(g.mode) ? 2 : 1;
+    auto bytes = [&](int tb) { return ((size_t)branches * (g.taps + 1) * tb + 2 * (size_t)g.taps + 3 * (size_t)(tb / 32)) * 4; };
+    p.tb = 128;
+    while (p.tb > 32 && bytes(p.tb) > 48 * 1024) p.tb /= 2;
+    p.smem = bytes(p.tb);
+    const long long kc = (long long)g.K * g.C, total = (long long)g.N * g.vol;
+    long long per_sm = (long long)(200 * 1024 / (p.smem + 1024));
+    if (per_sm > 16) per_sm = 16;
+    long long want = 148 * per_sm / kc;
+    const long long most = (total + 8 * p.tb - 1) / (8 * p.tb);   // two batches of four items per thread
+    if (want > most) want = most;
+    if (want > 64) want = 64;
+    if (want < 1) want = 1;
+    p.nsplit = (int)want;
+    p.scratch_floats = (size_t)p.nsplit * (kc * 2 * g.taps + kc * 2 + g.K);
+    return p;
+}
+
 size_t backward_scratch_floats(const Geo3& g) {
-    const size_t ns = (size_t)gw_splits(g);
-    const size_t generic = 2 * ns * g.K * g.C * g.taps + 2 * ns * g.K * g.C + (size_t)bias_splits(g) * g.K;
     const Plan1 p = plan_1d(g);
-    return (p.ok && p.scratch_floats > generic) ? p.scratch_floats : generic;
+    if (p.ok) return p.scratch_floats;
+    if (!force_generic3()) return plan_params3(g).scratch_floats;
+    const size_t ns = (size_t)gw_splits(g);
+    return 2 * ns * g.K * g.C * g.taps + 2 * ns * g.K * g.C + (size_t)bias_splits(g) * g.K;
 }
 
 int check(cudaError_t e) { return e == cudaSuccess ? TCONV_OK : TCONV_ERR_CUDA; }
@@ -186,8 +213,7 @@ int forward1d_t(const Geo3& g, const void* x, const void* w, const void* w2, con
 #define TCONV1_LAUNCH(STV, BRV, WINV)                                                     \
     {                                                                                     \
         if (smem > 48 * 1024 &&                                                           \
-            cudaFuncSetAttribute(fwd1d_kernel<T, STV, BRV, WINV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                 (int)kSmem1d) != cudaSuccess)                            \
+            allow_smem(fwd1d_kernel<T, STV, BRV, WINV>, (int)kSmem1d) != cudaSuccess)     \
             return TCONV_ERR_CUDA;                                                        \
         fwd1d_kernel<T, STV, BRV, WINV><<<grid, kF1Threads, smem, st>>>(                   \
             g, q4, (const T*)x, (const T*)w, (const T*)w2, alpha, beta, bias, (T*)y, winners); \
@@ -222,11 +248,44 @@ int forward3_t(const Geo3& g, const void* x, const void* w, const void* w2, cons
     // two output channels per thread when K is small and not a multiple of four, else four
     const int kt = (g.K % 4 == 0 || g.K > 8) ? 4 : 2;
     const size_t per_c = (size_t)g.taps * kt * sizeof(T) * (par ? 2 : 1);
+    const long long flat = (long long)g.N * g.vol;
+    // Too few (position, output channel) threads for the GPU (1024 per SM): the channels and window planes of a
+    // position are split over 8, 16 or 32 threads (the 6 -> 16 channel layer on 6^3: 75 -> 4 us)
+    const long long base = flat * ((g.K + kt - 1) / kt), work = (long long)g.C * g.T;
+    if (base < 148 * 1024 && work > 1) {
+        int slots = 8;
+        while (slots < 32 && base * slots < 148 * 1024 && slots < work) slots *= 2;
+        // channels per group, planes per channel: the fewest rounds of the slots
+        const int wmax = (int)(34 * 1024 / per_c) < 1 ? 1 : (int)(34 * 1024 / per_c);
+        auto group = [&](int ts) { int c = slots / ts; if (c > g.C) c = g.C; return c < wmax ? c : wmax; };
+        int ts = 1, cg = group(1);
+        if (g.T > 1 && g.T <= slots && (g.C + group(g.T) - 1) / group(g.T) < (g.C + cg - 1) / cg * g.T) { ts = g.T; cg = group(g.T); }
+        const int px = 256 / slots;
+        const size_t smem = ((per_c * cg + 15) & ~(size_t)15) + (size_t)cg * ts * kt * px * 10;
+        const dim3 grid((unsigned)((flat + px - 1) / px), (unsigned)((g.K + kt - 1) / kt));
+#define TCONV3_SPLIT(KTV, WINV, SCV)                                                                      \
+    fwd3d_split_kernel<T, KTV, WINV, SCV><<<grid, 256, smem, st>>>(                                        \
+        g, px, ts, cg, (const T*)x, (const T*)w, (const T*)w2, alpha, beta, bias, (T*)y, winners)
+#define TCONV3_SPLIT_S(KTV, WINV)                                \
+    {                                                            \
+        if (g.S == 3) TCONV3_SPLIT(KTV, WINV, 3);                \
+        else if (g.S == 5) TCONV3_SPLIT(KTV, WINV, 5);           \
+        else TCONV3_SPLIT(KTV, WINV, 0);                         \
+    }
+        if (kt == 4) {
+            if (winners) TCONV3_SPLIT_S(4, true) else TCONV3_SPLIT_S(4, false)
+        } else {
+            if (winners) TCONV3_SPLIT_S(2, true) else TCONV3_SPLIT_S(2, false)
+        }
+#undef TCONV3_SPLIT_S
+#undef TCONV3_SPLIT
+        g3_launches += 1;
+        return check(cudaGetLastError());
+    }
     int cch = (int)(48 * 1024 / per_c);
     if (cch < 1) cch = 1;
     if (cch > g.C) cch = g.C;
     const size_t smem = per_c * cch;
-    const long long flat = (long long)g.N * g.vol;
     const dim3 grid((unsigned)((flat + kFwd3Threads - 1) / kFwd3Threads), (unsigned)((g.K + kt - 1) / kt));
 #define TCONV3_LAUNCH(KTV, WINV, SCV)                                                                     \
     fwd3d_kernel<T, KTV, WINV, SCV><<<grid, kFwd3Threads, smem, st>>>(                                     \
@@ -254,13 +313,8 @@ template <typename T>
 int backward1d_t(const Geo3& g, const Plan1& p, const void* x, const void* w, const void* w2,
                  const float* alpha, const float* beta, const void* gy, const void* winners, void* gx,
                  float* gw, float* gw2, float* galpha, float* gbeta, float* gbias, char* ws, cudaStream_t st) {
-    static const cudaError_t attr = [] {
-        cudaError_t e = cudaFuncSetAttribute(bwd1d_gx_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem1d);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(bwd1d_params_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem1d);
-        return e;
-    }();
-    if (attr != cudaSuccess) return TCONV_ERR_CUDA;
+    if (allow_smem(bwd1d_gx_kernel<T>, (int)kSmem1d) != cudaSuccess || allow_smem(bwd1d_params_kernel<T>, (int)kSmem1d) != cudaSuccess)
+        return TCONV_ERR_CUDA;
     const size_t kc = (size_t)g.K * g.C, count = kc * g.S;
     float* pmin = (float*)ws;
     float* pmax = pmin + (size_t)p.nsplit * count;
@@ -322,6 +376,21 @@ int backward3_t(const Geo3& g, const void* x, const void* w, const void* w2, con
         bwd3d_gx_kernel<T><<<(unsigned)((total + per_block - 1) / per_block), dim3(per_block, (unsigned)slices), 0, st>>>(
             g, alpha, beta, (const T*)gy, winners, (T*)gx);
         g3_launches += 1;
+    }
+    if (!force_generic3()) {
+        if (!(gw || gw2 || gbias || (two && (galpha || gbeta)))) return check(cudaGetLastError());
+        const PlanParams3 p = plan_params3(g);
+        const size_t kc = (size_t)g.K * g.C;
+        float* hist = (float*)ws;
+        float* ab = hist + (size_t)p.nsplit * kc * 2 * g.taps;
+        float* pb = ab + (size_t)p.nsplit * kc * 2;
+        if (allow_smem(bwd3d_params_kernel<T>, (int)kSmem1d) != cudaSuccess) return TCONV_ERR_CUDA;
+        bwd3d_params_kernel<T><<<dim3((unsigned)kc, (unsigned)p.nsplit), p.tb, p.smem, st>>>(
+            g, p.nsplit, (const T*)x, (const T*)gy, winners, hist, ab, pb);
+        bwd3d_params_finish_kernel<T><<<(unsigned)kc, 128, 0, st>>>(g, p.nsplit, (const T*)w, (const T*)w2, alpha, beta, hist, ab,
+                                                                  pb, gw, gw2, galpha, gbeta, gbias);
+        g3_launches += 2;
+        return check(cudaGetLastError());
     }
     const int nsplit = gw_splits(g);
     const size_t count = (size_t)g.K * g.C * g.taps;

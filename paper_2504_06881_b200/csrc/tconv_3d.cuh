@@ -160,6 +160,149 @@ fwd3d_kernel(Geo3 g, int cch, const T* __restrict__ x, const T* __restrict__ w, 
     }
 }
 
+// Forward for layers with too few (position, output channel) pairs to fill the GPU (a LeNet layer on 28^3
+// volumes has 1024 of them): a block owns PX positions x KT output channels and splits the taps of a group of
+// input channels over `parts` threads per position, one (channel, window plane) each; after every group the
+// block folds the planes of a channel and adds the channels in ascending order, one thread per (position,
+// output channel), so that the results are those of fwd3d_kernel.  256 threads = PX * parts.  Shared memory:
+// weights of the group [cc][tap][KT] (twice in parallel mode), then the partial extrema [part][KT][PX] (min,
+// max, and with winners both taps in 16 bits).  ts: planes per channel (1 or T), cg: channels per group.
+template <typename T, int KT, bool WIN, int SC>
+__global__ void __launch_bounds__(256)
+fwd3d_split_kernel(Geo3 g, int PX, int ts, int cg, const T* __restrict__ x, const T* __restrict__ w,
+                   const T* __restrict__ w2, const float* __restrict__ alpha, const float* __restrict__ beta,
+                   const float* __restrict__ bias, T* __restrict__ y, void* __restrict__ winners) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const bool par = g.mode == TCONV_PARALLEL, twob = two_branch(g.mode);
+    T* wmin_s = reinterpret_cast<T*>(smem_raw);
+    T* wmax_s = par ? wmin_s + (size_t)cg * g.taps * KT : wmin_s;
+    const int nparts = cg * ts;
+    float* pmn = reinterpret_cast<float*>(smem_raw + (((size_t)cg * g.taps * KT * (par ? 2 : 1) * sizeof(T) + 15) & ~(size_t)15));
+    float* pmx = pmn + nparts * KT * PX;
+    uint16_t* pcode = reinterpret_cast<uint16_t*>(pmx + nparts * KT * PX);
+    const int tid = threadIdx.x, px = tid % PX, part = tid / PX;
+    const int pc = part / ts, pt = part - pc * ts;             // this thread's channel of the group, window plane
+    const int k0 = blockIdx.y * KT;
+    const long long flat0 = (long long)blockIdx.x * PX, total = (long long)g.N * g.vol;
+    const long long flat = min(flat0 + px, total - 1);
+    const int n = (int)(flat / g.vol), pos = (int)(flat % g.vol);
+    const int ow = pos % g.OW, oh = (pos / g.OW) % g.OH, od = pos / (g.OW * g.OH);
+    const int d0 = od * g.sd - g.pd, h0 = oh * g.sh - g.ph, w0 = ow * g.sw - g.pw;
+    const int S = SC ? SC : g.S, RS = g.R * g.S;
+    // folding thread: (output channel, position) of the block
+    const int fj = tid / PX, fk = k0 + fj;
+    const bool folds = tid < KT * PX && flat0 + px < total && fk < g.K;
+    float acc = g.chan == CH_SUM ? 0.0f : (g.chan == CH_MAX ? -INFINITY : INFINITY);
+    int win = -1;
+    for (int c0 = 0; c0 < g.C; c0 += cg) {
+        const int ncc = min(cg, g.C - c0);
+        // (the folding threads are done with the previous group before its partials are overwritten: second barrier)
+        for (int i = tid; i < ncc * g.taps * KT; i += 256) {
+            // along the taps of one (channel, output channel): contiguous weights
+            const int tap = i % g.taps, j = (i / g.taps) % KT, cc = i / (KT * g.taps), k = k0 + j;
+            const size_t wi = ((size_t)k * g.C + c0 + cc) * g.taps + tap;
+            wmin_s[(cc * g.taps + tap) * KT + j] = k < g.K ? w[wi] : zero_of<T>();
+            if (par) wmax_s[(cc * g.taps + tap) * KT + j] = k < g.K ? w2[wi] : zero_of<T>();
+        }
+        __syncthreads();
+        if (pc < ncc) {
+            float mn[KT], mx[KT];
+            int amn[KT], amx[KT];
+#pragma unroll
+            for (int j = 0; j < KT; ++j) { mn[j] = INFINITY; mx[j] = -INFINITY; amn[j] = amx[j] = 0; }
+            const T* xc = x + ((size_t)n * g.C + c0 + pc) * g.D * g.H * g.W;
+            const T* wa = wmin_s + (size_t)pc * g.taps * KT;
+            const T* wb = wmax_s + (size_t)pc * g.taps * KT;
+            const int t_end = ts == 1 ? g.T : pt + 1;
+            for (int t = pt; t < t_end; ++t) {
+                const int id = d0 + t * g.dd;
+                const bool okd = id >= 0 && id < g.D;
+                for (int r = 0; r < g.R; ++r) {
+                    const int ih = h0 + r * g.dh;
+                    const bool okh = okd && ih >= 0 && ih < g.H;
+                    const T* xrow = xc + ((size_t)(okh ? id : 0) * g.H + (okh ? ih : 0)) * g.W;
+                    const int tap0 = t * RS + r * S;
+                    auto fold = [&](T xv, int tap) {
+#pragma unroll
+                        for (int j = 0; j < KT; ++j) {
+                            const float tmn = tap_add(xv, wa[tap * KT + j]);
+                            const float tmx = par ? tap_add(xv, wb[tap * KT + j]) : tmn;
+                            if constexpr (WIN) {
+                                if (tmn < mn[j]) { mn[j] = tmn; amn[j] = tap; }
+                                if (tmx > mx[j]) { mx[j] = tmx; amx[j] = tap; }
+                            } else {
+                                mn[j] = fminf(mn[j], tmn);
+                                mx[j] = fmaxf(mx[j], tmx);
+                            }
+                        }
+                    };
+                    if constexpr (SC != 0) {
+                        T xv[SC];
+#pragma unroll
+                        for (int s = 0; s < SC; ++s) {
+                            const int iw = w0 + s * g.dw;
+                            xv[s] = (okh && iw >= 0 && iw < g.W) ? xrow[iw] : zero_of<T>();
+                        }
+#pragma unroll
+                        for (int s = 0; s < SC; ++s) fold(xv[s], tap0 + s);
+                    } else {
+                        for (int s = 0; s < S; ++s) {
+                            const int iw = w0 + s * g.dw;
+                            fold((okh && iw >= 0 && iw < g.W) ? xrow[iw] : zero_of<T>(), tap0 + s);
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < KT; ++j) {
+                const int o = (part * KT + j) * PX + px;
+                pmn[o] = mn[j];
+                pmx[o] = mx[j];
+                if constexpr (WIN) pcode[o] = (uint16_t)(amn[j] | (amx[j] << 8));
+            }
+        }
+        __syncthreads();
+        if (folds) {
+            for (int cc = 0; cc < ncc; ++cc) {
+                const int c = c0 + cc;
+                float mn = INFINITY, mx = -INFINITY;
+                unsigned amn = 0, amx = 0;
+                for (int z = 0; z < ts; ++z) {          // planes ascending: the lowest winning tap stays
+                    const int o = ((cc * ts + z) * KT + fj) * PX + px;
+                    const float a = pmn[o], b = pmx[o];
+                    if constexpr (WIN) {
+                        const unsigned cd = pcode[o];
+                        if (a < mn) { mn = a; amn = cd & 0xFFu; }
+                        if (b > mx) { mx = b; amx = cd >> 8; }
+                    } else {
+                        mn = fminf(mn, a);
+                        mx = fmaxf(mx, b);
+                    }
+                }
+                if (twob) {
+                    acc = __fmaf_rn(alpha ? alpha[(size_t)fk * g.C + c] : 1.0f, mn, acc);
+                    acc = __fmaf_rn(beta ? beta[(size_t)fk * g.C + c] : 1.0f, mx, acc);
+                } else {
+                    const bool is_min = g.mode == TCONV_MIN_PLUS;
+                    const float m = is_min ? mn : mx;
+                    const int am = (int)(is_min ? amn : amx);
+                    if (g.chan == CH_SUM) acc = __fadd_rn(acc, m);
+                    else if (g.chan == CH_MAX ? m > acc : m < acc) { acc = m; win = c * g.taps + am; }
+                    if (is_min) amx = 0; else amn = 0;
+                }
+                if (WIN && g.chan == CH_SUM)
+                    ((uint16_t*)winners)[(((size_t)n * g.K + fk) * g.C + c) * g.vol + pos] = (uint16_t)(amn | (amx << 8));
+            }
+        }
+    }
+    if (!folds) return;
+    float out = acc;
+    if (bias) out = __fadd_rn(out, bias[fk]);
+    const size_t o = ((size_t)n * g.K + fk) * g.vol + pos;
+    if (y) y[o] = from_f32<T>(out);
+    if (WIN && g.chan != CH_SUM) ((int32_t*)winners)[o] = win;
+}
+
 // The winning taps of (n, k, c, position) as two ints; -1 where the layer has no such branch or
 // (Max / Min channel combine) another channel won.
 __device__ __forceinline__ void winners3(const Geo3& g, const void* winners, int n, int k, int c, int pos,
@@ -176,11 +319,27 @@ __device__ __forceinline__ void winners3(const Geo3& g, const void* winners, int
     }
 }
 
-// grad_x in gather form.  A block of 256 threads owns 256 / slices consecutive input elements
-// (threadIdx.x) and splits the output channels over blockDim.y = 1, 2, 4 or 8 slices (k = slice, slice + slices, ...): each thread visits,
-// taps ascending and its channels ascending inside a tap, the outputs whose window reads its
-// element; the slices' partial sums are then added in slice order.  (Small 3-D layers have few
-// input elements: the slices keep enough warps in flight to hide the dependent loads.)
+// Taps t of one axis through which an output reads input index i: i + pad - t * dil = stride * o with
+// 0 <= o < out.  The walk visits exactly those when dil is 1 (step = stride), else it tests every tap.
+struct TapRange {
+    int first, end, step;
+};
+__device__ __forceinline__ TapRange tap_range(int i, int pad, int dil, int stride, int taps, int out) {
+    TapRange r;
+    if (dil != 1) { r.first = 0; r.end = taps; r.step = 1; return r; }
+    const int u = i + pad, last = (out - 1) * stride;
+    r.first = u > last ? u - last : u % stride;      // (last is a multiple of the stride)
+    r.end = min(taps, u + 1);
+    r.step = stride;
+    return r;
+}
+
+// grad_x in gather form.  A block of 256 threads owns 256 / slices consecutive input elements (threadIdx.x)
+// and splits the output channels over blockDim.y = 1, 2, 4 or 8 slices (k = slice, slice + slices, ...): each
+// thread visits, taps ascending and its channels ascending inside a tap, the outputs whose window reads its
+// element; the slices' partial sums are then added in slice order.  (Small 3-D layers have few input elements:
+// the slices keep enough warps in flight to hide the dependent loads.)  Four channels' winners are requested
+// together; a gradient is only read where one of them is the tap.
 constexpr int kGx3Slices = 8;
 
 template <typename T>
@@ -192,35 +351,57 @@ bwd3d_gx_kernel(Geo3 g, const float* __restrict__ alpha, const float* __restrict
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int slice = threadIdx.y, slices = blockDim.y;
     const bool live = i < total;
-    const bool twob = two_branch(g.mode);
+    const bool twob = two_branch(g.mode), codes = g.chan == CH_SUM;
+    const bool use_min = g.mode != TCONV_MAX_PLUS, use_max = g.mode != TCONV_MIN_PLUS;
     float acc = 0.0f;
     if (live) {
-        const int iw = (int)(i % g.W), ih = (int)((i / g.W) % g.H), id = (int)((i / ((size_t)g.W * g.H)) % g.D);
-        const int c = (int)((i / ((size_t)g.W * g.H * g.D)) % g.C),
-                  n = (int)(i / ((size_t)g.W * g.H * g.D * g.C));
-        for (int t = 0; t < g.T; ++t) {
-            const int nd = id + g.pd - t * g.dd;
-            if (nd < 0 || nd % g.sd != 0 || nd / g.sd >= g.OD) continue;
-            for (int r = 0; r < g.R; ++r) {
-                const int nh = ih + g.ph - r * g.dh;
-                if (nh < 0 || nh % g.sh != 0 || nh / g.sh >= g.OH) continue;
-                for (int s = 0; s < g.S; ++s) {
-                    const int nw = iw + g.pw - s * g.dw;
-                    if (nw < 0 || nw % g.sw != 0 || nw / g.sw >= g.OW) continue;
-                    const int tap = (t * g.R + r) * g.S + s;
-                    const int pos = ((nd / g.sd) * g.OH + nh / g.sh) * g.OW + nw / g.sw;
-                    for (int k = slice; k < g.K; k += slices) {
-                        int amn, amx;
-                        winners3(g, winners, n, k, c, pos, amn, amx);
-                        if (amn != tap && amx != tap) continue;
-                        const float gv = to_f32(gy[((size_t)n * g.K + k) * g.vol + pos]);
-                        if (twob) {
-                            const float a = alpha ? alpha[(size_t)k * g.C + c] : 1.0f;
-                            const float b = beta ? beta[(size_t)k * g.C + c] : 1.0f;
-                            if (amn == tap) acc = __fmaf_rn(a, gv, acc);
-                            if (amx == tap) acc = __fmaf_rn(b, gv, acc);
-                        } else {
-                            acc += gv;
+        const unsigned ui = (unsigned)i;                    // (every tensor has fewer than 2^31 elements)
+        const int iw = (int)(ui % (unsigned)g.W);
+        const unsigned t1 = ui / (unsigned)g.W;
+        const int ih = (int)(t1 % (unsigned)g.H);
+        const unsigned t2 = t1 / (unsigned)g.H;
+        const int id = (int)(t2 % (unsigned)g.D);
+        const unsigned nc = t2 / (unsigned)g.D;
+        const int c = (int)(nc % (unsigned)g.C), n = (int)(nc / (unsigned)g.C);
+        const uint16_t* cbase = (const uint16_t*)winners + ((size_t)n * g.K * g.C + c) * g.vol;
+        const int32_t* ibase = (const int32_t*)winners + (size_t)n * g.K * g.vol;
+        const T* gbase = gy + (size_t)n * g.K * g.vol;
+        const int cstep = g.C * g.vol;
+        const TapRange rd = tap_range(id, g.pd, g.dd, g.sd, g.T, g.OD), rh = tap_range(ih, g.ph, g.dh, g.sh, g.R, g.OH),
+                       rw = tap_range(iw, g.pw, g.dw, g.sw, g.S, g.OW);
+        for (int t = rd.first; t < rd.end; t += rd.step) {
+            const int nd = id + g.pd - t * g.dd, od = nd / g.sd;
+            if (nd < 0 || od * g.sd != nd || od >= g.OD) continue;
+            for (int r = rh.first; r < rh.end; r += rh.step) {
+                const int nh = ih + g.ph - r * g.dh, oh = nh / g.sh;
+                if (nh < 0 || oh * g.sh != nh || oh >= g.OH) continue;
+                for (int s = rw.first; s < rw.end; s += rw.step) {
+                    const int nw = iw + g.pw - s * g.dw, ow = nw / g.sw;
+                    if (nw < 0 || ow * g.sw != nw || ow >= g.OW) continue;
+                    const unsigned tap = (unsigned)((t * g.R + r) * g.S + s);
+                    const int pos = (od * g.OH + oh) * g.OW + ow;
+                    for (int k0 = slice; k0 < g.K; k0 += 4 * slices) {
+                        bool hmin[4], hmax[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int k = min(k0 + u * slices, g.K - 1);
+                            if (codes) {
+                                const unsigned v = __ldg(cbase + (k * cstep + pos));
+                                hmin[u] = use_min && (v & 0xFFu) == tap;
+                                hmax[u] = use_max && (v >> 8) == tap;
+                            } else {
+                                const bool hit = (unsigned)__ldg(ibase + (k * g.vol + pos)) == (unsigned)(c * g.taps) + tap;
+                                hmin[u] = hit && use_min;
+                                hmax[u] = hit && !use_min;
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int k = k0 + u * slices;
+                            if (k >= g.K || !(hmin[u] || hmax[u])) continue;
+                            const float gv = to_f32(__ldg(gbase + (k * g.vol + pos)));
+                            if (hmin[u]) acc = __fmaf_rn(twob && alpha ? alpha[k * g.C + c] : 1.0f, gv, acc);
+                            if (hmax[u]) acc = __fmaf_rn(twob && beta ? beta[k * g.C + c] : 1.0f, gv, acc);
                         }
                     }
                 }
@@ -233,6 +414,180 @@ bwd3d_gx_kernel(Geo3 g, const float* __restrict__ alpha, const float* __restrict
         float total_acc = 0.0f;
         for (int j = 0; j < slices; ++j) total_acc += part[j * blockDim.x + threadIdx.x];
         gx[i] = from_f32<T>(total_acc);
+    }
+}
+
+// All parameter gradients but their last sum.  Block (k * C + c, split) walks its share of the (n, position)
+// range; every thread keeps private columns in shared memory, one per tap and branch (col[tap][tb], one more
+// for items that another channel won), so that an item costs one read-modify-write per branch; grad_alpha /
+// grad_beta: g * x at the winner (zero in the padding), the weights' share is added by the finishing kernel from
+// the same histograms.  part_hist [split][k*C+c][2][taps], part_ab [split][k*C+c][2], part_bias [split][k].
+template <typename T>
+__global__ void __launch_bounds__(128)
+bwd3d_params_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __restrict__ gy,
+                    const void* __restrict__ winners, float* __restrict__ part_hist, float* __restrict__ part_ab,
+                    float* __restrict__ part_bias) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int tid = threadIdx.x, tb = blockDim.x, taps = g.taps;
+    const int kc = blockIdx.x, k = kc / g.C, c = kc - k * g.C, split = blockIdx.y;
+    const bool twob = two_branch(g.mode), codes = g.chan == CH_SUM;
+    const bool use_min = g.mode != TCONV_MAX_PLUS, use_max = g.mode != TCONV_MIN_PLUS;
+    const int branches = (use_min ? 1 : 0) + (use_max ? 1 : 0);
+    float* cmin = reinterpret_cast<float*>(smem_raw);
+    float* cmax = cmin + (use_min ? (taps + 1) * tb : 0);
+    int* tofs = reinterpret_cast<int*>(cmin + branches * (taps + 1) * tb);   // input offset of a tap from its window's corner
+    int* tcrd = tofs + taps;                                                 // its (depth, row, column) distance, 10 bits each
+    float* red = reinterpret_cast<float*>(tcrd + taps);                      // [3][tb / 32]
+    for (int i = tid; i < branches * (taps + 1) * tb; i += tb) cmin[i] = 0.0f;
+    for (int i = tid; i < taps; i += tb) {
+        const int t = i / (g.R * g.S), r = (i / g.S) % g.R, s = i % g.S;
+        tofs[i] = (t * g.dd * g.H + r * g.dh) * g.W + s * g.dw;
+        tcrd[i] = (t << 20) | (r << 10) | s;
+    }
+    __syncthreads();
+    const int total = g.N * g.vol, per = (total + nsplit - 1) / nsplit;
+    const int j0 = min(total, split * per), j1 = min(total, j0 + per);
+    float sa = 0.0f, sb = 0.0f, sg = 0.0f;
+    constexpr int U = 4;          // items whose loads go out together
+    for (int jb = j0 + tid; jb < j1; jb += U * tb) {
+        unsigned raw[U];
+        float gv[U];
+        int n[U], pos[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = jb + u * tb, jj = j < j1 ? j : jb;
+            n[u] = (int)((unsigned)jj / (unsigned)g.vol);
+            pos[u] = jj - n[u] * g.vol;
+            const int row = n[u] * g.K + k;
+            raw[u] = codes ? (unsigned)__ldg((const uint16_t*)winners + ((row * g.C + c) * g.vol + pos[u]))
+                           : (unsigned)__ldg((const int32_t*)winners + (row * g.vol + pos[u]));
+            const float v = to_f32(__ldg(gy + (row * g.vol + pos[u])));
+            gv[u] = j < j1 ? v : 0.0f;
+        }
+        int amn[U], amx[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (codes) {
+                amn[u] = (int)(raw[u] & 0xFFu);
+                amx[u] = (int)(raw[u] >> 8);
+            } else {
+                const int v = (int)raw[u] - c * taps;
+                amn[u] = amx[u] = (v >= 0 && v < taps) ? v : taps;
+            }
+        }
+        if (twob) {
+            float xa[U], xb[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const unsigned q = (unsigned)pos[u] / (unsigned)g.OW;
+                const int ow = pos[u] - (int)q * g.OW, od = (int)(q / (unsigned)g.OH), oh = (int)q - od * g.OH;
+                const int d0 = od * g.sd - g.pd, h0 = oh * g.sh - g.ph, w0 = ow * g.sw - g.pw;
+                const T* xc = x + (size_t)(n[u] * g.C + c) * g.D * g.H * g.W;
+                const int corner = (d0 * g.H + h0) * g.W + w0;
+                auto at = [&](int tap) {
+                    const int p = tcrd[tap];
+                    const int id = d0 + (p >> 20) * g.dd, ih = h0 + ((p >> 10) & 1023) * g.dh, iw = w0 + (p & 1023) * g.dw;
+                    const bool ok = (unsigned)id < (unsigned)g.D && (unsigned)ih < (unsigned)g.H && (unsigned)iw < (unsigned)g.W;
+                    return ok ? to_f32(__ldg(xc + corner + tofs[tap])) : 0.0f;
+                };
+                xa[u] = at(amn[u]);
+                xb[u] = at(amx[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                sa = __fmaf_rn(gv[u], xa[u], sa);
+                sb = __fmaf_rn(gv[u], xb[u], sb);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            sg += gv[u];
+            if (use_min) cmin[amn[u] * tb + tid] += gv[u];
+            if (use_max) cmax[amx[u] * tb + tid] += gv[u];
+        }
+    }
+    __syncthreads();
+    float* hist = part_hist + ((size_t)split * g.K * g.C + kc) * 2 * taps;
+    for (int i = tid; i < 2 * taps; i += tb) {
+        const bool mx = i >= taps;
+        const float* col = (mx ? cmax : cmin) + (size_t)(mx ? i - taps : i) * tb;
+        float s = 0.0f;
+        if (mx ? use_max : use_min)
+            for (int q = 0; q < tb; ++q) s += col[(q + tid) & (tb - 1)];   // rotated start: different banks
+        hist[i] = s;
+    }
+    float v[3] = {sa, sb, sg};
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], d);
+        if ((tid & 31) == 0) red[q * (tb / 32) + (tid >> 5)] = v[q];
+    }
+    __syncthreads();
+    if (tid < 3) {
+        float s = 0.0f;
+        for (int q = 0; q < tb / 32; ++q) s += red[tid * (tb / 32) + q];
+        if (tid < 2) part_ab[((size_t)split * g.K * g.C + kc) * 2 + tid] = s;
+        else if (c == 0) part_bias[(size_t)split * g.K + k] = s;
+    }
+}
+
+// One block per (k, c): sums its partials over the splits in order, applies alpha / beta and completes
+// grad_alpha / grad_beta with sum_tap w * histogram.
+template <typename T>
+__global__ void __launch_bounds__(128)
+bwd3d_params_finish_kernel(Geo3 g, int nsplit, const T* __restrict__ w, const T* __restrict__ w2,
+                           const float* __restrict__ alpha, const float* __restrict__ beta,
+                           const float* __restrict__ part_hist, const float* __restrict__ part_ab,
+                           const float* __restrict__ part_bias, float* __restrict__ gw, float* __restrict__ gw2,
+                           float* __restrict__ galpha, float* __restrict__ gbeta, float* __restrict__ gbias) {
+    __shared__ float red[2][4];
+    const int kc = blockIdx.x, k = kc / g.C, c = kc - k * g.C, tid = threadIdx.x;
+    const size_t pairs = (size_t)g.K * g.C;
+    const bool twob = two_branch(g.mode), par = g.mode == TCONV_PARALLEL;
+    const float a = twob && alpha ? alpha[kc] : 1.0f, b = twob && beta ? beta[kc] : 1.0f;
+    float sa = 0.0f, sb = 0.0f;
+    for (int t = tid; t < g.taps; t += 128) {
+        float tmin = 0.0f, tmax = 0.0f;
+        for (int s = 0; s < nsplit; ++s) {
+            const float* h = part_hist + (s * pairs + kc) * 2 * g.taps;
+            tmin += h[t];
+            tmax += h[g.taps + t];
+        }
+        const size_t i = (size_t)kc * g.taps + t;
+        if (!twob) {
+            if (gw) gw[i] = g.mode == TCONV_MIN_PLUS ? tmin : tmax;
+        } else {
+            if (par) {
+                if (gw) gw[i] = a * tmin;
+                if (gw2) gw2[i] = b * tmax;
+            } else if (gw) {
+                gw[i] = __fmaf_rn(a, tmin, b * tmax);
+            }
+            sa = __fmaf_rn(to_f32(w[i]), tmin, sa);
+            sb = __fmaf_rn(to_f32(par ? w2[i] : w[i]), tmax, sb);
+        }
+    }
+    if (twob && (galpha || gbeta)) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            sa += __shfl_xor_sync(0xffffffffu, sa, d);
+            sb += __shfl_xor_sync(0xffffffffu, sb, d);
+        }
+        if ((tid & 31) == 0) { red[0][tid >> 5] = sa; red[1][tid >> 5] = sb; }
+        __syncthreads();
+        if (tid < 2) {
+            float s = 0.0f;
+            for (int sp = 0; sp < nsplit; ++sp) s += part_ab[(sp * pairs + kc) * 2 + tid];
+            for (int q = 0; q < 4; ++q) s += red[tid][q];
+            float* to = tid == 0 ? galpha : gbeta;
+            if (to) to[kc] = s;
+        }
+    }
+    if (gbias && c == 0 && tid == 2) {
+        float s = 0.0f;
+        for (int sp = 0; sp < nsplit; ++sp) s += part_bias[(size_t)sp * g.K + k];
+        gbias[k] = s;
     }
 }
 
