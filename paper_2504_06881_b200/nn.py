@@ -14,7 +14,14 @@ import math
 import torch
 import torch.nn as nn
 
-from . import tconv, tconv3d
+from . import tconv
+try:
+    from . import _tconv_torch as _native
+except ImportError as err:
+    raise ImportError(f"the layers' extension module is missing or does not load ({err}): build it with "
+                      f"`python -m paper_2504_06881_b200.build`") from err
+
+_native.set_error(tconv.TconvError)
 
 
 def _emit_winners(recording, *tensors):
@@ -42,23 +49,22 @@ def _make_desc2d(xs, ws, geom, x_f32):
     return d
 
 
-def _make_desc_dw(xs, ws, geom):
-    (N, C, H, W), (_, R, S), (mode, dtype, stride, pad, dil, _rec) = xs, ws, geom
-    return tconv.PlannedDesc(N=N, C=C, H=H, W=W, K=C, R=R, S=S, stride_h=stride[0], stride_w=stride[1], pad_h=pad[0],
-                             pad_w=pad[1], dil_h=dil[0], dil_w=dil[1], mode=mode, chan="sum", dtype=dtype)
+_descs2d = tconv.KeptPlans(_make_desc2d)
+
+_KINDS = {"dense": 0, "depthwise": 1, "volume": 2}
+_geoms = tconv.KeptPlans(lambda kind, mode, chan, dtype, stride, pad, dil: _native.Geom(
+    _KINDS[kind], tconv.MODES[mode], tconv.CHANS[chan], tconv.DTYPES[dtype], stride, pad, dil))
 
 
-def _make_desc3d(xs, ws, geom):
-    (N, C, D, H, W), (K, _, T, R, S), (mode, chan, dtype, stride, pad, dil, _rec) = xs, ws, geom
-    return tconv.PlannedDesc(N=N, C=C, D=D, H=H, W=W, K=K, T=T, R=R, S=S, stride=tuple(stride), pad=tuple(pad),
-                             dil=tuple(dil), mode=mode, chan=chan, dtype=dtype)
-
-
-_descs2d, _descs_dw, _descs3d = map(tconv.KeptPlans, (_make_desc2d, _make_desc_dw, _make_desc3d))
+def _layer(kind, mode, chan, dtype, stride, pad, dil, x, w, w2, alpha, beta, bias):
+    """One layer through the native autograd path (csrc/torch_layers.cpp)."""
+    geom = (kind, mode, chan, dtype, stride, pad, dil)
+    return _native.layer(_geoms.get(geom, *geom), x, w, w2, alpha, beta, bias)
 
 
 class TropicalConvFn(torch.autograd.Function):
     """y = tconv_forward(x, w, w2, alpha, beta, bias); backward = tconv_backward with the stored winners.
+    The layers take the native path (csrc/torch_layers.cpp) unless one of the two settings below is on.
 
     Master parameters may be fp32 while the layer computes in bf16: the cast happens here and the
     parameter gradients come back in fp32.  When ``TropicalConvFn.events`` is a list, every library
@@ -255,7 +261,7 @@ class TropicalConv2d(nn.Module):
 
     PARAMS = ("0p", "1p", "2p", "shared", "opposite", "fixed")
     ND = 2          # spatial dimensions
-    FN = None       # autograd Function of the layer (set below the class)
+    KIND = "dense"
 
     def __init__(self, in_channels, out_channels, kernel_size, stride=1, padding=0, dilation=1,
                  bias=True, mode="compound", chan="default", params="2p", dtype="f32", fixed=(0.5, 0.5)):
@@ -306,11 +312,11 @@ class TropicalConv2d(nn.Module):
                 beta = -alpha
             elif self.params == "fixed":
                 alpha, beta = self.alpha_fixed, self.beta_fixed
-        geom = (self.mode, self.chan, self.dtype, self.stride, self.padding, self.dilation, torch.is_grad_enabled())
-        return self.FN.apply(x, self.weight, self.weight2, alpha, beta, self.bias, geom)
-
-
-TropicalConv2d.FN = TropicalConvFn
+        if self.KIND == "dense" and (TropicalConvFn.events is not None or TropicalConvFn.fuse_cast):
+            geom = (self.mode, self.chan, self.dtype, self.stride, self.padding, self.dilation, torch.is_grad_enabled())
+            return TropicalConvFn.apply(x, self.weight, self.weight2, alpha, beta, self.bias, geom)
+        return _layer(self.KIND, self.mode, self.chan, self.dtype, self.stride, self.padding, self.dilation, x,
+                      self.weight, self.weight2, alpha, beta, self.bias)
 
 
 class TropicalBasicBlock(nn.Module):
@@ -371,34 +377,6 @@ class HybridResNet18(nn.Module):
         return [m for m in self.modules() if isinstance(m, TropicalConv2d)]
 
 
-class TropicalDepthwiseFn(torch.autograd.Function):
-    """Depthwise (groups = C) form over tconv_dw_forward / tconv_dw_backward; see TropicalConvFn."""
-
-    @staticmethod
-    def forward(ctx, x, w, w2, alpha, beta, bias, geom):
-        dt, recording = tconv.TORCH_DTYPE[geom[1]], geom[5]
-        d = _descs_dw.get((x.shape, w.shape, geom), x.shape, w.shape, geom)
-        xc, wc, w2c = _as(x, dt), _as(w, dt), _as(w2, dt)
-        al, be, bi = _as(alpha, torch.float32), _as(beta, torch.float32), _as(bias, torch.float32)
-        need_grad = _emit_winners(recording, x, w, w2, alpha, beta, bias)
-        y, winners = tconv.dw_forward(d, xc, wc, w2c, al, be, bi, want_winners=need_grad)
-        ctx.d, ctx.in_dtype = d, x.dtype
-        ctx.save_for_backward(xc, wc, w2c, al, be, winners)
-        ctx.has = (w2 is not None, alpha is not None, beta is not None, bias is not None)
-        return y.to(x.dtype) if x.dtype != dt else y
-
-    @staticmethod
-    def backward(ctx, gy):
-        xc, wc, w2c, al, be, winners = ctx.saved_tensors
-        d = ctx.d
-        g = _as(gy, tconv.TORCH_DTYPE[d["dtype"]])
-        grads = tconv.dw_backward(d, xc, wc, g, w2c, al, be, winners)
-        has_w2, has_a, has_b, has_bias = ctx.has
-        return (grads["grad_x"].to(ctx.in_dtype), grads["grad_w"], grads.get("grad_w2") if has_w2 else None,
-                grads.get("grad_alpha") if has_a else None, grads.get("grad_beta") if has_b else None,
-                grads["grad_bias"] if has_bias else None, None)
-
-
 class TropicalDepthwiseConv2d(nn.Module):
     """Depthwise tropical convolution (``nn.Conv2d(channels, channels, k, groups=channels)``'s place in
     a MobileNetV2 block): per channel one window of weights, one alpha and one beta.
@@ -446,37 +424,8 @@ class TropicalDepthwiseConv2d(nn.Module):
                 beta = -alpha
             elif self.params == "fixed":
                 alpha, beta = self.alpha_fixed, self.beta_fixed
-        geom = (self.mode, self.dtype, self.stride, self.padding, self.dilation, torch.is_grad_enabled())
-        return TropicalDepthwiseFn.apply(x, self.weight, self.weight2, alpha, beta, self.bias, geom)
-
-
-class TropicalConv3dFn(torch.autograd.Function):
-    """y = tconv3d_forward(...); backward = tconv3d_backward with the stored winners."""
-
-    @staticmethod
-    def forward(ctx, x, w, w2, alpha, beta, bias, geom):
-        dt, recording = tconv.TORCH_DTYPE[geom[2]], geom[6]
-        d = _descs3d.get((x.shape, w.shape, geom), x.shape, w.shape, geom)
-        xc, wc, w2c = _as(x, dt), _as(w, dt), _as(w2, dt)
-        al, be, bi = _as(alpha, torch.float32), _as(beta, torch.float32), _as(bias, torch.float32)
-        need_grad = _emit_winners(recording, x, w, w2, alpha, beta, bias)
-        y, winners = tconv3d.forward(d, xc, wc, w2c, al, be, bi, want_winners=need_grad)
-        ctx.d, ctx.in_dtype = d, x.dtype
-        ctx.save_for_backward(xc, wc, w2c, al, be, winners)
-        ctx.has = (w2 is not None, alpha is not None, beta is not None, bias is not None)
-        return y.to(x.dtype) if x.dtype != dt else y
-
-    @staticmethod
-    def backward(ctx, gy):
-        xc, wc, w2c, al, be, winners = ctx.saved_tensors
-        d = ctx.d
-        g = _as(gy, tconv.TORCH_DTYPE[d["dtype"]])
-        grads = tconv3d.backward(d, xc, wc, g, w2c, al, be, winners, need_grad_x=ctx.needs_input_grad[0])
-        has_w2, has_a, has_b, has_bias = ctx.has
-        gx = grads["grad_x"].to(ctx.in_dtype) if "grad_x" in grads else None
-        return (gx, grads["grad_w"], grads.get("grad_w2") if has_w2 else None,
-                grads.get("grad_alpha") if has_a else None, grads.get("grad_beta") if has_b else None,
-                grads["grad_bias"] if has_bias else None, None)
+        return _layer("depthwise", self.mode, "sum", self.dtype, self.stride, self.padding, self.dilation, x, self.weight,
+                      self.weight2, alpha, beta, self.bias)
 
 
 class TropicalConv3d(TropicalConv2d):
@@ -485,7 +434,7 @@ class TropicalConv3d(TropicalConv2d):
     as in TropicalConv2d.  Windows of up to 256 taps (the paper's 3-D LeNet uses 5 x 5 x 5)."""
 
     ND = 3
-    FN = TropicalConv3dFn
+    KIND = "volume"
 
 
 class TropicalConv1d(nn.Module):
