@@ -807,7 +807,7 @@ inline int round_up(int v, int a) { return (v + a - 1) / a * a; }
 
 // One candidate plan: ragged tiles allowed or not, cc input channels per staged chunk.
 template <int R, int S, int SW, int DW, int Q, int KG, int PW, int TK = 8>
-inline bool plan_tiles_opt(const Geo& g, bool par, bool two, int esize, bool allow_ragged, int cc, TiledPlan* pl) {
+inline bool plan_tiles_opt(const Geo& g, bool par, bool two, int esize, bool allow_ragged, int cc, TiledPlan* pl, bool plain = false) {
     TiledParams& p = pl->p;
     constexpr int TILE_K = KG * TK;
     constexpr int NQ = Q * 32 * PW;
@@ -840,7 +840,7 @@ inline bool plan_tiles_opt(const Geo& g, bool par, bool two, int esize, bool all
     const bool rows_fit = p.ragged ? (g.OH * p.QPR >= NQ)
                                    : ((double)g.OH / (tiles_img * th_img) >= 0.75 && th_img * p.QPR * 4 >= NQ * 3);
     // (a bf16 layer fed with float x converts while staging element by element: no tensor copy)
-    pl->xtma = !g.xf32 && ((g.W * esize) % 16 == 0) && (g.pw == (S - 1) * DW / 2) && rows_fit;
+    pl->xtma = !plain && !g.xf32 && ((g.W * esize) % 16 == 0) && (g.pw == (S - 1) * DW / 2) && rows_fit;
     p.XW = (p.TW - 1) * SW + (S - 1) * DW + 1;   // == (QPR-1)*4*SW + L
     if (pl->xtma && p.ragged) {
         p.TH = rows_max;
@@ -897,12 +897,18 @@ inline bool plan_tiles_opt(const Geo& g, bool par, bool two, int esize, bool all
 // blocks; the first candidate whose two stages leave room for four resident CTAs per SM wins, in
 // the order ragged / whole rows, 8 / 4 channels per chunk; else whole rows with 8 channels.
 template <int R, int S, int SW, int DW, int Q, int KG, int PW, int TK = 8>
-inline bool plan_tiles(const Geo& g, bool par, bool two, int esize, TiledPlan* pl) {
+inline bool plan_tiles(const Geo& g, bool par, bool two, int esize, TiledPlan* pl, bool plain = false) {
     // 8 channels per chunk when four CTAs stay resident, else 4 channels when three do (measured
     // on the stride-2 56 -> 28 layer: 8.06 against 7.86 Ttap/s for whole-row tiles at four CTAs)
     // (two-branch kernels with 8 channels per thread hold two CTAs per SM by their registers: their
     // stages may use half of the shared memory)
     const bool two_resident = two && TK == 8;
+    // (plain: whole rows, element staging; large windows stage fewer channels so that three CTAs stay resident)
+    if (plain) {
+        for (int cc = 8; cc > 2; cc -= 2)
+            if (plan_tiles_opt<R, S, SW, DW, Q, KG, PW, TK>(g, par, two, esize, false, cc, pl, true) && pl->smem <= 74 * 1024) return true;
+        return plan_tiles_opt<R, S, SW, DW, Q, KG, PW, TK>(g, par, two, esize, false, 2, pl, true);
+    }
     for (int cc = 8; cc >= 4; cc -= 2) {
         const size_t budget = (two_resident ? 112 : (cc == 4 ? 74 : 56)) * 1024;
         TiledPlan cand = *pl;

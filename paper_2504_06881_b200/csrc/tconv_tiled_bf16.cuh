@@ -65,16 +65,12 @@ __device__ __forceinline__ void load_words(const unsigned* base, unsigned* out) 
         }
     }
 }
-// The pixel pair whose first element sits E elements past the first loaded word:
-// elements (E, E + SW).
-template <int SW, int E>
-__device__ __forceinline__ unsigned pixel_pair(const unsigned* xw) {
-    if constexpr (SW == 1) {
-        if constexpr (E % 2 == 0) return xw[E / 2];
-        else return __byte_perm(xw[E / 2], xw[E / 2 + 1], 0x5432);
-    } else {
-        return __byte_perm(xw[E / 2], xw[E / 2 + 1], (E % 2) ? 0x7632 : 0x5410);
-    }
+// The pixel pair whose first element sits e elements past the first loaded word: elements (e, e + SW).
+// (e is a constant wherever the surrounding loops are unrolled.)
+template <int SW>
+__device__ __forceinline__ unsigned pixel_pair(const unsigned* xw, int e) {
+    if (SW == 1) return (e & 1) ? __byte_perm(xw[e / 2], xw[e / 2 + 1], 0x5432) : xw[e / 2];
+    return __byte_perm(xw[e / 2], xw[e / 2 + 1], (e & 1) ? 0x7632 : 0x5410);
 }
 
 // Weight repack for the bf16 kernels: every weight becomes the pair {w, w}.  (A template so
@@ -124,28 +120,37 @@ __device__ __forceinline__ unsigned short load_x(const unsigned short* x, size_t
     return __bfloat16_as_ushort(__float2bfloat16_rn(reinterpret_cast<const float*>(x)[i]));
 }
 
-// Extremum m of R rows of three tap sums (pixel pairs) and, per half, the lowest tap that attains it,
-// shifted left by SH.  NaN taps (neutral padding) never equal it.
-template <int R, int SH>
+// Extremum m of R rows of S tap sums (pixel pairs) and, per half, the lowest tap that attains it, shifted
+// left by SH.  NaN taps (neutral padding) never equal it.
+template <int R, int S, int SH>
 __device__ __forceinline__ unsigned win_taps(const unsigned* t, bool is_min, unsigned& m) {
     auto eq = [](unsigned a, unsigned b) { return __heq2_mask(as_bf162(a), as_bf162(b)); };
     auto pick = [](unsigned mask, unsigned a, unsigned b) { return (mask & a) | (~mask & b); };
     constexpr unsigned one = 0x00010001u << SH;
     unsigned row[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) row[r] = hext2u(hext2u(t[3 * r], t[3 * r + 1], is_min), t[3 * r + 2], is_min);
+    for (int r = 0; r < R; ++r) {
+        row[r] = t[S * r];
+#pragma unroll
+        for (int i = 1; i < S; ++i) row[r] = hext2u(row[r], t[S * r + i], is_min);
+    }
     m = row[0];
 #pragma unroll
     for (int r = 1; r < R; ++r) m = hext2u(m, row[r], is_min);
-    unsigned u = t[3 * (R - 1)], v = t[3 * (R - 1) + 1], first = 3 * (R - 1) * one;
+    unsigned u[S - 1], first = S * (R - 1) * one;       // the winning row's taps but the last
+#pragma unroll
+    for (int i = 0; i < S - 1; ++i) u[i] = t[S * (R - 1) + i];
 #pragma unroll
     for (int r = R - 2; r >= 0; --r) {
         const unsigned e = eq(row[r], m);
-        u = pick(e, t[3 * r], u);
-        v = pick(e, t[3 * r + 1], v);
-        first = pick(e, 3 * r * one, first);
+#pragma unroll
+        for (int i = 0; i < S - 1; ++i) u[i] = pick(e, t[S * r + i], u[i]);
+        first = pick(e, S * r * one, first);
     }
-    return first + pick(eq(u, m), 0u, pick(eq(v, m), one, 2 * one));
+    unsigned col = (S - 1) * one;
+#pragma unroll
+    for (int i = S - 2; i >= 0; --i) col = pick(eq(u[i], m), i * one, col);
+    return first + col;
 }
 
 // KPT words of packed weights of one tap (one or two 16-byte loads)
@@ -165,7 +170,6 @@ template <int MODE, int CHAN, bool WIN, bool XTMA, bool RAG, int R, int S, int S
           bool STATS = false>
 __global__ void __launch_bounds__(KG * PW * 32)
 fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParams p) {
-    static_assert(S == 3, "the pixel-pair selection below is written for 3 taps per row");
     static_assert(KPT == 8 || KPT == 4, "output channels per thread");
     constexpr int RS = R * S;
     constexpr int TILE_K = KG * KPT;
@@ -352,7 +356,7 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
     const size_t plane = (size_t)g.OH * g.OW;
     // Sum forms with winners: where this thread's codes of (its first output channel, the next input
     // channel) go, the distance between two output channels, and how many of its channels exist
-    const size_t cplane = (size_t)g.OH * g.OWP, kstep = (size_t)g.C * cplane;
+    const size_t cplane = (size_t)g.OH * g.OWP * (RS > 16 ? 2 : 1), kstep = (size_t)g.C * cplane;
     const int klim = g.K - (kt * TILE_K + kg * KPT);
     uint8_t* code_ptr[Q];
     bool code_ok[Q];
@@ -363,7 +367,7 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
         if constexpr (WIN && SUMF) {
             code_ok[q] = out_row[q] >= 0 && qcol[q] < g.OW;
             const int n = max(out_row[q], 0) / g.OH, oh = max(out_row[q], 0) - n * g.OH;
-            code_ptr[q] = reinterpret_cast<uint8_t*>(p.winners) + ((size_t)n * g.K + kt * TILE_K + kg * KPT) * kstep + (size_t)oh * g.OWP + qcol[q];
+            code_ptr[q] = reinterpret_cast<uint8_t*>(p.winners) + ((size_t)n * g.K + kt * TILE_K + kg * KPT) * kstep + ((size_t)oh * g.OWP + qcol[q]) * (RS > 16 ? 2 : 1);
         }
     }
     const int row_step = g.dh * pitch_w;
@@ -410,6 +414,7 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
                 // selects, and the first of its taps that equals the extremum (win_taps).  13 instructions
                 // per branch and pair; comparing every tap took 16 and tracking the tap while folding 26.
                 constexpr bool DO_MIN = TWO || TAP_MIN, DO_MAX = TWO || !TAP_MIN;
+                constexpr bool WIDE = RS > 16;      // 16-bit codes
                 float av[KPT], bv[KPT];
                 if constexpr (TWO) {
                     loadn<KPT>(as + cc * TILE_K, av);
@@ -419,10 +424,9 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
                 for (int q = 0; q < Q; ++q) {
                     unsigned xp[RS][2];
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        xp[r * 3][0] = pixel_pair<SW, EODD + 0 * SW + 0 * DW>(xw[q][r]); xp[r * 3][1] = pixel_pair<SW, EODD + 2 * SW + 0 * DW>(xw[q][r]);
-                        xp[r * 3 + 1][0] = pixel_pair<SW, EODD + 0 * SW + 1 * DW>(xw[q][r]); xp[r * 3 + 1][1] = pixel_pair<SW, EODD + 2 * SW + 1 * DW>(xw[q][r]);
-                        xp[r * 3 + 2][0] = pixel_pair<SW, EODD + 0 * SW + 2 * DW>(xw[q][r]); xp[r * 3 + 2][1] = pixel_pair<SW, EODD + 2 * SW + 2 * DW>(xw[q][r]);
+                    for (int tap = 0; tap < RS; ++tap) {
+                        xp[tap][0] = pixel_pair<SW>(xw[q][tap / S], EODD + (tap % S) * DW);
+                        xp[tap][1] = pixel_pair<SW>(xw[q][tap / S], EODD + 2 * SW + (tap % S) * DW);
                     }
                     uint8_t* dst = code_ptr[q];
 #pragma unroll
@@ -446,8 +450,8 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
                                     if constexpr (PAR) tb[tap] = hadd2u(xp[tap][pp], h == 0 ? wb[tap].x : wb[tap].y);
                                 }
                                 unsigned lo = 0u, hi = 0u, code = 0u;
-                                if constexpr (DO_MIN) code = win_taps<R, 0>(ta, true, lo);
-                                if constexpr (DO_MAX) code |= win_taps<R, 4>(PAR ? tb : ta, false, hi);
+                                if constexpr (DO_MIN) code = win_taps<R, S, 0>(ta, true, lo);
+                                if constexpr (DO_MAX) code |= win_taps<R, S, WIDE ? 8 : 4>(PAR ? tb : ta, false, hi);
                                 float* a2 = acc[k][q] + 2 * pp;
                                 if constexpr (TWO) {
                                     fma2(av[k], bf_lo(lo), bf_hi(lo), a2[0], a2[1]);
@@ -459,7 +463,10 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
                                 c2[pp] = code;
                             }
                             // the quad's 4 codes in one store (code rows are padded to whole quads)
-                            if (k < klim && code_ok[q]) *reinterpret_cast<unsigned*>(dst) = __byte_perm(c2[0], c2[1], 0x6420);
+                            if (k < klim && code_ok[q]) {
+                                if constexpr (WIDE) *reinterpret_cast<uint2*>(dst) = make_uint2(c2[0], c2[1]);
+                                else *reinterpret_cast<unsigned*>(dst) = __byte_perm(c2[0], c2[1], 0x6420);
+                            }
                             dst += kstep;
                         }
                     }
@@ -488,10 +495,7 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
                             for (int u = 0; u < 3; ++u)
                                 if (u < nt) {
                                     const int tap = t0 + u;
-                                    const int r = tap / S, sx = tap % S;
-                                    if (sx == 0) xp[u] = pp == 0 ? pixel_pair<SW, EODD + 0 * SW + 0 * DW>(xw[q][r]) : pixel_pair<SW, EODD + 2 * SW + 0 * DW>(xw[q][r]);
-                                    else if (sx == 1) xp[u] = pp == 0 ? pixel_pair<SW, EODD + 0 * SW + 1 * DW>(xw[q][r]) : pixel_pair<SW, EODD + 2 * SW + 1 * DW>(xw[q][r]);
-                                    else xp[u] = pp == 0 ? pixel_pair<SW, EODD + 0 * SW + 2 * DW>(xw[q][r]) : pixel_pair<SW, EODD + 2 * SW + 2 * DW>(xw[q][r]);
+                                    xp[u] = pixel_pair<SW>(xw[q][tap / S], EODD + 2 * pp * SW + (tap % S) * DW);
                                 }
 #pragma unroll
                             for (int k = 0; k < KPT; ++k) {
@@ -654,10 +658,10 @@ fwd_tiled_bf16_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParam
     }
 }
 
-// PLAIN_ONLY: instantiate only the kernel without TMA and without ragged tiles (what small maps
-// use); a plan that wants either is left to the caller's next choice.
+// PLAIN_ONLY: instantiate only the kernel without TMA and without ragged tiles (what small maps use); a plan
+// that wants either is left to the caller's next choice, or (PLAN_PLAIN) not made.
 template <int MODE, int CHAN, bool WIN, int R, int S, int SW, int DW, int Q, int KG, int PW, int KPT = 8,
-          bool PLAIN_ONLY = false>
+          bool PLAIN_ONLY = false, bool PLAN_PLAIN = false>
 int launch_tiled_variant_bf16(FwdArgs& a) {
     constexpr bool TWO = (MODE == TCONV_COMPOUND || MODE == TCONV_PARALLEL);
     constexpr bool PAR = (MODE == TCONV_PARALLEL);
@@ -665,7 +669,7 @@ int launch_tiled_variant_bf16(FwdArgs& a) {
     if (g.C > 65535) return TCONV_ERR_UNSUPPORTED;   // winner channel kept in 16 bits
     TiledPlan pl;
     pl.p.g = g;
-    if (!plan_tiles<R, S, SW, DW, Q, KG, PW, KPT>(g, PAR, TWO, 2, &pl)) return TCONV_ERR_UNSUPPORTED;
+    if (!plan_tiles<R, S, SW, DW, Q, KG, PW, KPT>(g, PAR, TWO, 2, &pl, PLAN_PLAIN)) return TCONV_ERR_UNSUPPORTED;
     if (PLAIN_ONLY && (pl.xtma || pl.p.ragged)) return TCONV_ERR_UNSUPPORTED;
     const size_t need = pl.ws_w * (PAR ? 2 : 1) + (TWO ? 2 * pl.ws_ab : 0);
     if (!a.ws || a.ws_bytes < need) return TCONV_ERR_WORKSPACE_TOO_SMALL;
@@ -703,7 +707,7 @@ int launch_tiled_variant_bf16(FwdArgs& a) {
     }
     if constexpr (PLAIN_ONLY) {
         TCONV_LAUNCH_BF16(false, false)
-        a.name = WIN ? "fwd_tiled_bf16_k4_win" : "fwd_tiled_bf16_k4";
+        a.name = PLAN_PLAIN ? (WIN ? "fwd_tiled_bf16_win" : "fwd_tiled_bf16") : (WIN ? "fwd_tiled_bf16_k4_win" : "fwd_tiled_bf16_k4");
     } else if (pl.xtma) {
         if (pl.p.ragged) TCONV_LAUNCH_BF16(true, true) else TCONV_LAUNCH_BF16(true, false)
         a.name = WIN ? "fwd_tiled_bf16_tma_win" : "fwd_tiled_bf16_tma";
@@ -746,12 +750,15 @@ int launch_tiled_geom_bf16(FwdArgs& a) {
     // 1 x 3: the 1-D layers as signals of unit height
     if (g.R == 1 && g.S == 3 && g.sw == 1 && g.dw == 1)
         return launch_tiled_variant_bf16<MODE, CHAN, WIN, 1, 3, 1, 1, Q, 4, 1>(a);
+    // 5 x 5 (LeNet); 4 channels per thread where winners and their 25 tap sums share the registers.  Against the
+    // any-shape kernel: N=19 C=217 K=164 31x38 compound training 23.2 -> 4.36 ms, N=3 C=16 K=300 10x19 107 -> 20 us.
+    if (g.R == 5 && g.S == 5 && g.sw == 1 && g.dw == 1)
+        return launch_tiled_variant_bf16<MODE, CHAN, WIN, 5, 5, 1, 1, Q, 4, 1, (WIN && CHAN == CH_SUM) ? 4 : 8, true, true>(a);
     return TCONV_ERR_UNSUPPORTED;
 }
 
 template <int MODE, int CHAN>
 int launch_fwd_tiled_bf16_inst(FwdArgs& a) {
-    if (a.g.wide) return TCONV_ERR_UNSUPPORTED;
     if ((double)a.g.N * a.g.C * a.g.H * a.g.W >= 2.0e9) return TCONV_ERR_UNSUPPORTED;
     if (a.winners) return launch_tiled_geom_bf16<MODE, CHAN, true>(a);
     return launch_tiled_geom_bf16<MODE, CHAN, false>(a);
