@@ -241,60 +241,14 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
     bool bias_done = false;
     if (g.chan != CH_SUM) {
         const int32_t* idx = (const int32_t*)winners;
-        int thi = 0;
-        size_t smem = 0;
         if (gx) {
-            if (tiled && plan_idx_gx(g, &thi, &smem)) {
-                const int tiles = (g.H + thi - 1) / thi;
-                const unsigned magic = g.RS == 1 ? 0u : (0xFFFFFFFFu / (unsigned)g.RS) + 1u;
-                if (g.RS <= 15) {
-                    // the phases of this form are latency-bound: aim at three resident CTAs per SM
-                    // (the tile shares the CTA's shared memory with the staging columns)
-                    const size_t stage = (size_t)kIdxGxKB * 256 * 2 * sizeof(float);
-                    const size_t row = (size_t)g.C * g.W * sizeof(float);
-                    const int halo = (g.R - 1) * g.dh;
-                    int thi2 = thi;
-                    while ((row * thi2 + stage > 73 * 1024 || row * thi2 + stage > kBwdSmemAttr) &&
-                           (thi2 + 1) / 2 >= 2 * halo && thi2 > 4)
-                        thi2 = (thi2 + 1) / 2;
-                    if (row * thi2 + stage > kBwdSmemAttr) thi2 = 0;
-                    // among the band heights down to that one's half: the fewest rounds of resident
-                    // CTAs times the rows a CTA scans (a band that leaves a few CTAs for a last round
-                    // costs a whole round)
-                    if (thi2 > 0) {
-                        long best_cost = -1;
-                        int best = thi2;
-                        for (int t = thi2; t >= 4 && t >= 2 * halo && 2 * t >= thi2; --t) {
-                            const size_t sm = row * t + stage;
-                            long per_sm = (long)((227 * 1024) / (sm + 1024));
-                            if (per_sm > 8) per_sm = 8;
-                            if (per_sm < 1) continue;
-                            const long ctas = (long)g.N * ((g.H + t - 1) / t);
-                            const long rounds = (ctas + 148 * per_sm - 1) / (148 * per_sm);
-                            const long cost = rounds * (t + halo);
-                            if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = t; }
-                        }
-                        thi2 = best;
-                    }
-                    auto kern = g.RS == 9 ? bwd_idx_gx2_kernel<T, 9> : bwd_idx_gx2_kernel<T, 0>;
-                    if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess)
-                        return cuda_fail(cudaGetLastError());
-                    if (thi2 > 0) {
-                        const int tiles2 = (g.H + thi2 - 1) / thi2;
-                        kern<<<(unsigned)(g.N * tiles2), 256, (size_t)g.C * g.W * sizeof(float) * thi2 + stage, st>>>(
-                            g, (const T*)gy, idx, (T*)gx, thi2, tiles2, magic);
-                    } else {
-                        auto kern1 = bwd_idx_gx_kernel<T>;
-                        if (allow_smem(kern1, kBwdSmemAttr) != cudaSuccess)
-                            return cuda_fail(cudaGetLastError());
-                        kern1<<<(unsigned)(g.N * tiles), 256, smem, st>>>(g, (const T*)gy, idx, (T*)gx, thi, tiles, magic);
-                    }
-                } else {
-                    auto kern = bwd_idx_gx_kernel<T>;
-                    if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess)
-                        return cuda_fail(cudaGetLastError());
-                    kern<<<(unsigned)(g.N * tiles), 256, smem, st>>>(g, (const T*)gy, idx, (T*)gx, thi, tiles, magic);
-                }
+            IdxGxPlan pl;
+            if (tiled && plan_idx_gx(g, &pl)) {
+                auto kern = bwd_idx_gx_kernel<T>;
+                if (allow_smem(kern, (int)kIdxSmemMost) != cudaSuccess) return cuda_fail(cudaGetLastError());
+                kern<<<pl.grid, pl.threads, pl.smem, st>>>(g, (const T*)gy, idx, (T*)gx, pl,
+                                                           g.RS == 1 ? 0u : (0xFFFFFFFFu / (unsigned)g.RS) + 1u,
+                                                           65536u / (unsigned)g.S + 1u);
                 name = "bwd_idx";
             } else {
                 const size_t total = (size_t)g.N * g.C * g.H * g.W;
@@ -303,27 +257,17 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
             }
             g_launches += 1;
         }
-        int chunks = 0;
-        if ((gw || gbias) && tiled && plan_idx_gw(g, &chunks, &smem) && ws && ws_bytes >= bwd_ws_bytes(g)) {
-            const size_t CRS = (size_t)g.C * g.RS;
-            float* pw = (float*)ws;
-            float* pb = pw + (size_t)chunks * g.K * CRS;
-            auto kern = bwd_idx_gw_kernel<T>;
-            if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess)
-                return cuda_fail(cudaGetLastError());
-            const int npc = (g.N + chunks - 1) / chunks;
-            kern<<<dim3((unsigned)g.K, (unsigned)chunks), 256, smem, st>>>(g, (const T*)gy, idx, pw, pb, npc);
-            g_launches += 1;
-            if (gw) {
-                const size_t len = (size_t)g.K * CRS;
-                bwd_reduce_partials_kernel<<<(unsigned)((len + 255) / 256), 256, 0, st>>>(pw, gw, len, chunks);
-                g_launches += 1;
-            }
-            if (gbias) {
-                bwd_reduce_partials_kernel<<<(unsigned)((g.K + 255) / 256), 256, 0, st>>>(pb, gbias, (size_t)g.K, chunks);
-                g_launches += 1;
-                bias_done = true;
-            }
+        IdxGwPlan pw;
+        if ((gw || gbias) && tiled && plan_idx_gw(g, (((uintptr_t)gy | (uintptr_t)idx) & 15) == 0, &pw) && ws && ws_bytes >= pw.part_floats * sizeof(float)) {
+            float* part = (float*)ws;
+            float* part_b = part + (size_t)pw.chunks * pw.nkg * g.C * g.RS * 32;
+            auto kern = pw.vec == 4 ? bwd_idx_gw_kernel<T, 4> : bwd_idx_gw_kernel<T, 1>;
+            if (allow_smem(kern, (int)kIdxSmemMost) != cudaSuccess) return cuda_fail(cudaGetLastError());
+            kern<<<dim3((unsigned)(pw.nkg * pw.nblk), (unsigned)pw.chunks), 32, pw.smem, st>>>(g, (const T*)gy, idx, part, part_b, pw);
+            bwd_idx_gw_finish_kernel<<<dim3((unsigned)(((size_t)g.C * g.RS + 3) / 4 + 1), (unsigned)pw.nkg), dim3(32, 4, 8), 0, st>>>(
+                g, pw, part, part_b, gw, gbias);
+            g_launches += 2;
+            bias_done = true;
             name = "bwd_idx";
         } else if (gw) {
             bwd_gw_generic_kernel<T><<<(unsigned)((size_t)g.K * g.C * g.RS), 256, 0, st>>>(
