@@ -300,8 +300,9 @@ int backward_sum_t(const Geo& g, const void* x, const void* w, const void* w2, c
         if (part_bytes && ws_bytes >= pad_bytes + part_bytes) {
             a.gy = gy;
             if (pad_bytes) {
-                const size_t total = (size_t)g.N * g.K * g.OH * g.OWP;
-                pad_grad_kernel<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(g, (const T*)gy, (T*)ws);
+                const size_t rows = (size_t)g.N * g.K * g.OH;
+                const unsigned rpb = g.OWP <= 1024 ? 1024u / (unsigned)g.OWP : 1u;
+                pad_grad_kernel<T><<<(unsigned)((rows + 4 * rpb - 1) / (4 * rpb)), 256, 0, st>>>(g, (const T*)gy, (T*)ws, rows, rpb);
                 g_launches += 1;
                 a.gy = ws;
             }

@@ -64,16 +64,36 @@ inline size_t bwd_ws_bytes(const Geo& g) {
     return part > bias ? part : bias;
 }
 
-// grad_y with rows padded by zeros to OWP elements: one thread per padded element.
+__device__ __forceinline__ void store_quad(float* o, const float* v) {
+    *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store_quad(__nv_bfloat16* o, const __nv_bfloat16* v) {
+    __nv_bfloat162* p = reinterpret_cast<__nv_bfloat162*>(o);
+    p[0] = __halves2bfloat162(v[0], v[1]);
+    p[1] = __halves2bfloat162(v[2], v[3]);
+}
+
+// grad_y with rows padded by zeros to OWP elements: one thread per four of them (one store).
+// N=80 K=152 71x142 fp32 (983 MB) took 492 us with one thread and two divisions per element.
 template <typename T>
 __global__ void __launch_bounds__(256)
-pad_grad_kernel(Geo g, const T* __restrict__ gy, T* __restrict__ out) {
-    const size_t total = (size_t)g.N * g.K * g.OH * g.OWP;
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    const int ow = (int)(i % g.OWP);
-    const size_t row = i / g.OWP;
-    out[i] = ow < g.OW ? gy[row * g.OW + ow] : zero_of<T>();
+pad_grad_kernel(Geo g, const T* __restrict__ gy, T* __restrict__ out, size_t rows, unsigned rpb) {
+    const unsigned QPR = (unsigned)g.OWP >> 2, r = threadIdx.x / QPR, q0 = threadIdx.x - r * QPR;
+    const unsigned step = QPR < 256 ? QPR : 256;
+    if (r >= rpb) return;
+    // a block takes rpb whole rows at once (long rows: one, in steps of 256 threads), four times
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const size_t row = ((size_t)blockIdx.x * 4 + u) * rpb + r;
+        if (row >= rows) return;
+        for (unsigned q = q0; q < QPR; q += step) {
+            const T* p = gy + row * g.OW + 4 * q;
+            T v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = (int)(4 * q) + j < g.OW ? __ldg(p + j) : zero_of<T>();
+            store_quad(out + (row * QPR + q) * 4, v);
+        }
+    }
 }
 
 constexpr int kBwdSmemAttr = 200 * 1024;       // opt-in ceiling set on the kernels

@@ -56,16 +56,20 @@ int launch_all(SumBwdArgs& a) {
     else if (a.gx) rc = br == 0 ? launch_gx_window<T, 0, true, false>(a, xp, part_ab, part_gx)
                         : br == 1 ? launch_gx_window<T, 1, true, false>(a, xp, part_ab, part_gx) : launch_gx_window<T, 2, true, false>(a, xp, part_ab, part_gx);
     if (rc == TCONV_OK && a.gx && xp.nrow * xp.ncol > 1) {
-        bwd_sum_edges_kernel<T><<<dim3((unsigned)(g.N * g.C), (unsigned)((g.H * g.W + 255) / 256)), 256, 0, a.st>>>(g, part_gx, (T*)a.gx, xp);
+        bwd_sum_edges_kernel<T><<<dim3((unsigned)(g.N * g.C), (unsigned)(((g.H + 3) / 4 * ((g.W + 31) / 32) + 7) / 8)), 256, 0, a.st>>>(g, part_gx, (T*)a.gx, xp);
         ++a.launches;
     }
     if (rc != TCONV_OK || !params) return rc;
     rc = br == 0 ? launch_gw_window<T, 0>(a, gp, part) : br == 1 ? launch_gw_window<T, 1>(a, gp, part) : launch_gw_window<T, 2>(a, gp, part);
     if (rc != TCONV_OK) return rc;
     const size_t pairs = (size_t)g.K * g.C;
-    const unsigned nb_w = a.gw || a.gw2 || a.gbias ? (unsigned)((pairs * g.RS + 255) / 256) : 0u, nb_ab = ab ? (unsigned)((pairs + 31) / 32) : 0u;
-    bwd_sum_finish_kernel<T><<<nb_w + nb_ab, 256, 0, a.st>>>(g, br, gp.splits, part, (int)xp.ctas, part_ab, (const T*)a.w,
-                                                            (const T*)a.w2, a.alpha, a.beta, a.gw, a.gw2, a.galpha, a.gbeta, a.gbias, nb_w);
+    // slices of the splits: a power of two, about eight splits each
+    int ws = 1;
+    while (ws < 32 && ws * 8 < gp.splits) ws *= 2;
+    const unsigned nb_w = a.gw || a.gw2 ? (unsigned)((pairs * g.RS * ws + 255) / 256) : 0u, nb_ab = ab ? (unsigned)((pairs + 15) / 16) : 0u;
+    const unsigned nb_bias = a.gbias ? (unsigned)((g.K + 7) / 8) : 0u;
+    bwd_sum_finish_kernel<T><<<nb_w + nb_ab + nb_bias, 256, 0, a.st>>>(g, br, gp.splits, part, (int)xp.ctas, part_ab, (const T*)a.w,
+                                                            (const T*)a.w2, a.alpha, a.beta, a.gw, a.gw2, a.galpha, a.gbeta, a.gbias, nb_w, nb_ab, ws);
     ++a.launches;
     return TCONV_OK;
 }

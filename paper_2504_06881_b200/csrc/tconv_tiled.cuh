@@ -240,12 +240,16 @@ template <int S, int DW, int ESIZE = 4> struct TmaShift {
 // the ALU / FMA pipes and want four or more warps per scheduler to hide their latencies.
 constexpr int kMinBlocksSingle = 4;   // single-branch kernels
 constexpr int kMinBlocksWinSum = 3;   // Sum forms that emit winners (168 registers)
+// Max / Min combine with winners: the running winners live beside the running extrema.  Three CTAs (168 registers,
+// no spills) against two without a bound: N=128 C=64 K=64 32x32 3x3 426 -> 384 us; four CTAs spill, and four
+// channels per thread with five CTAs read the input twice as often (388 us).
+constexpr int kMinBlocksWinExt = 3;
 constexpr int kQuadsCarried = 2;      // quads per thread of the carried max-plus / min-plus chain
 // STATS (winner-emitting kernels only): also leave the per-tile channel statistics.
 template <int MODE, int CHAN, bool WIN, bool XTMA, bool RAG, int R, int S, int SW, int DW, int Q, int KG, int PW, int TK, bool STATS = false>
 __global__ void __launch_bounds__(KG * PW * 32,
                                   (WIN && CHAN == CH_SUM) ? kMinBlocksWinSum
-                                  : WIN ? 1
+                                  : WIN ? kMinBlocksWinExt
                                   : (MODE == TCONV_COMPOUND || MODE == TCONV_PARALLEL) ? (TK == 4 ? 4 : 1)
                                   : kMinBlocksSingle)
 fwd_tiled_f32_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParams p) {
