@@ -17,6 +17,9 @@ ROOT = PKG.parent
 CSRC = PKG / "csrc"
 LIB = PKG / "libtconv.so"
 EXT = PKG / "_tconv_torch.so"
+# The compiler that nvcc takes for host code, whatever CXX says: one that links its C++ library statically puts a
+# second copy of it beside torch's, and formatting a number for an error message then crashed.
+HOST_CXX = "g++"
 OBJ = PKG / "build"
 
 # (exported launcher, tconv_mode_t, channel combine: 1 sum, 2 max, 3 min)
@@ -61,7 +64,7 @@ def _torch_flags():
 def _compile(job):
     src, obj, defs, verbose = job
     if src.suffix == ".cpp":
-        cmd = [os.environ.get("CXX", "g++")] + _torch_flags()[0] + ["-c", str(src), "-o", str(obj)]
+        cmd = [HOST_CXX] + _torch_flags()[0] + ["-c", str(src), "-o", str(obj)]
     else:
         cmd = _nvcc_base(verbose) + defs + ["-c", str(src), "-o", str(obj)]
     r = subprocess.run(cmd, capture_output=True, text=True)
@@ -96,7 +99,7 @@ def build(force: bool = False, verbose: bool = False) -> Path:
     subprocess.run(cmd, check=True)
     os.replace(tmp, LIB)
     tmp = EXT.with_suffix(f".{os.getpid()}.tmp.so")
-    subprocess.run([os.environ.get("CXX", "g++"), "-shared", str(ext_obj)] + _torch_flags()[1] + ["-o", str(tmp)], check=True)
+    subprocess.run([HOST_CXX, "-shared", str(ext_obj)] + _torch_flags()[1] + ["-o", str(tmp)], check=True)
     os.replace(tmp, EXT)
     return LIB
 
