@@ -343,7 +343,7 @@ __device__ __forceinline__ TapRange tap_range(int i, int pad, int dil, int strid
 constexpr int kGx3Slices = 8;
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kGx3Slices)
+__global__ void __launch_bounds__(32 * kGx3Slices, 6)
 bwd3d_gx_kernel(Geo3 g, const float* __restrict__ alpha, const float* __restrict__ beta,
                 const T* __restrict__ gy, const void* __restrict__ winners, T* __restrict__ gx) {
     __shared__ float part[32 * kGx3Slices];
@@ -380,30 +380,25 @@ bwd3d_gx_kernel(Geo3 g, const float* __restrict__ alpha, const float* __restrict
                     if (nw < 0 || ow * g.sw != nw || ow >= g.OW) continue;
                     const unsigned tap = (unsigned)((t * g.R + r) * g.S + s);
                     const int pos = (od * g.OH + oh) * g.OW + ow;
-                    for (int k0 = slice; k0 < g.K; k0 += 4 * slices) {
-                        bool hmin[4], hmax[4];
+                    const unsigned want = (unsigned)(c * g.taps) + tap;
+                    auto take = [&](int k, unsigned v) {        // v: the winner code(s) of output channel k
+                        const bool hmin = codes ? use_min && (v & 0xFFu) == tap : use_min && v == want;
+                        const bool hmax = codes ? use_max && (v >> 8) == tap : use_max && v == want;
+                        if (!(hmin || hmax)) return;
+                        const float gv = to_f32(__ldg(gbase + (k * g.vol + pos)));
+                        if (hmin) acc = __fmaf_rn(twob && alpha ? alpha[k * g.C + c] : 1.0f, gv, acc);
+                        if (hmax) acc = __fmaf_rn(twob && beta ? beta[k * g.C + c] : 1.0f, gv, acc);
+                    };
+                    auto code = [&](int k) { return codes ? (unsigned)__ldg(cbase + (k * cstep + pos)) : (unsigned)__ldg(ibase + (k * g.vol + pos)); };
+                    int k = slice;
+                    for (; k + 3 * slices < g.K; k += 4 * slices) {
+                        unsigned v[4];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int k = min(k0 + u * slices, g.K - 1);
-                            if (codes) {
-                                const unsigned v = __ldg(cbase + (k * cstep + pos));
-                                hmin[u] = use_min && (v & 0xFFu) == tap;
-                                hmax[u] = use_max && (v >> 8) == tap;
-                            } else {
-                                const bool hit = (unsigned)__ldg(ibase + (k * g.vol + pos)) == (unsigned)(c * g.taps) + tap;
-                                hmin[u] = hit && use_min;
-                                hmax[u] = hit && !use_min;
-                            }
-                        }
+                        for (int u = 0; u < 4; ++u) v[u] = code(k + u * slices);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int k = k0 + u * slices;
-                            if (k >= g.K || !(hmin[u] || hmax[u])) continue;
-                            const float gv = to_f32(__ldg(gbase + (k * g.vol + pos)));
-                            if (hmin[u]) acc = __fmaf_rn(twob && alpha ? alpha[k * g.C + c] : 1.0f, gv, acc);
-                            if (hmax[u]) acc = __fmaf_rn(twob && beta ? beta[k * g.C + c] : 1.0f, gv, acc);
-                        }
+                        for (int u = 0; u < 4; ++u) take(k + u * slices, v[u]);
                     }
+                    for (; k < g.K; k += slices) take(k, code(k));
                 }
             }
         }

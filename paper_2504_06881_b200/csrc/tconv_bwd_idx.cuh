@@ -98,7 +98,9 @@ inline bool plan_idx_gx(const Geo& g, IdxGxPlan* best) {
                 if (best_cost < 0.0 || cost < 0.97 * best_cost) {
                     best_cost = cost;
                     p.smem = row * p.TH + 256 * sizeof(float);
-                    p.threads = 32 * warps;
+                    // (a tile of many channels: more warps to clear and store it)
+                    const size_t fill = row * p.TH / 4096;
+                    p.threads = 32 * (fill > 8 ? 8 : (int)fill > warps ? (int)fill : warps);
                     p.grid = (unsigned)ctas;
                     *best = p;
                 }
@@ -127,6 +129,7 @@ inline bool plan_idx_gw(const Geo& g, bool aligned, IdxGwPlan* p) {
     p->lk = g.K > 16 ? 5 : g.K > 8 ? 4 : g.K > 4 ? 3 : g.K > 2 ? 2 : g.K > 1 ? 1 : 0;
     p->smem = per_c * p->CB + 32 * sizeof(float) + kGwStages * kGwStageBytes;
     const long plane = (long)g.OH * g.OW;
+    while (p->lk < 5 && plane <= (32L << (5 - p->lk)) / 2) ++p->lk;    // small planes: no slices without pixels
     p->vec = plane % 4 == 0 && aligned ? 4 : 1;
     const long tile = 32L << (5 - p->lk);
     p->timg = (int)((plane + tile - 1) / tile);

@@ -752,6 +752,9 @@ int launch_tiled_geom_bf16(FwdArgs& a) {
         return launch_tiled_variant_bf16<MODE, CHAN, WIN, 1, 3, 1, 1, Q, 4, 1>(a);
     // 5 x 5 (LeNet); 4 channels per thread where winners and their 25 tap sums share the registers.  Against the
     // any-shape kernel: N=19 C=217 K=164 31x38 compound training 23.2 -> 4.36 ms, N=3 C=16 K=300 10x19 107 -> 20 us.
+    // (Max / Min winners rescan 25 taps of the winning channel: with fewer than 5 channels that outweighs the tap
+    // loop; N=79 C=3 K=14 42x82 min-plus 549 us here, 347 us in the any-shape kernel)
+    if (WIN && CHAN != CH_SUM && g.R == 5 && g.S == 5 && g.C < 5) return TCONV_ERR_UNSUPPORTED;
     if (g.R == 5 && g.S == 5 && g.sw == 1 && g.dw == 1)
         return launch_tiled_variant_bf16<MODE, CHAN, WIN, 5, 5, 1, 1, Q, 4, 1, (WIN && CHAN == CH_SUM) ? 4 : 8, true, true>(a);
     return TCONV_ERR_UNSUPPORTED;
