@@ -373,7 +373,8 @@ int backward3_t(const Geo3& g, const void* x, const void* w, const void* w2, con
         int slices = 1;
         while (slices < kGx3Slices && (size_t)slices < want && 2 * slices <= g.K) slices *= 2;
         const unsigned per_block = 32u * kGx3Slices / slices;
-        bwd3d_gx_kernel<T><<<(unsigned)((total + per_block - 1) / per_block), dim3(per_block, (unsigned)slices), 0, st>>>(
+        auto kern = two ? bwd3d_gx_kernel<T, true, true> : g.chan == CH_SUM ? bwd3d_gx_kernel<T, true, false> : bwd3d_gx_kernel<T, false, false>;
+        kern<<<(unsigned)((total + per_block - 1) / per_block), dim3(per_block, (unsigned)slices), 0, st>>>(
             g, alpha, beta, (const T*)gy, winners, (T*)gx);
         g3_launches += 1;
     }

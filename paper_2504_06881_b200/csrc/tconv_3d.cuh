@@ -340,10 +340,12 @@ __device__ __forceinline__ TapRange tap_range(int i, int pad, int dil, int strid
 // element; the slices' partial sums are then added in slice order.  (Small 3-D layers have few input elements:
 // the slices keep enough warps in flight to hide the dependent loads.)  Four channels' winners are requested
 // together; a gradient is only read where one of them is the tap.
+// One instance per code form, five blocks per SM (48 registers): N=2 C=6 K=14 25^3 5^3 took 814 us with the form
+// decided in the loop at 64 registers, four blocks.
 constexpr int kGx3Slices = 8;
 
-template <typename T>
-__global__ void __launch_bounds__(32 * kGx3Slices, 6)
+template <typename T, bool CODES, bool TWO>
+__global__ void __launch_bounds__(32 * kGx3Slices, 5)
 bwd3d_gx_kernel(Geo3 g, const float* __restrict__ alpha, const float* __restrict__ beta,
                 const T* __restrict__ gy, const void* __restrict__ winners, T* __restrict__ gx) {
     __shared__ float part[32 * kGx3Slices];
@@ -351,8 +353,8 @@ bwd3d_gx_kernel(Geo3 g, const float* __restrict__ alpha, const float* __restrict
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int slice = threadIdx.y, slices = blockDim.y;
     const bool live = i < total;
-    const bool twob = two_branch(g.mode), codes = g.chan == CH_SUM;
-    const bool use_min = g.mode != TCONV_MAX_PLUS, use_max = g.mode != TCONV_MIN_PLUS;
+    // TWO: two branches; else the codes of a single branch or the winner index decide
+    const bool is_max = g.mode == TCONV_MAX_PLUS;
     float acc = 0.0f;
     if (live) {
         const unsigned ui = (unsigned)i;                    // (every tensor has fewer than 2^31 elements)
@@ -382,14 +384,18 @@ bwd3d_gx_kernel(Geo3 g, const float* __restrict__ alpha, const float* __restrict
                     const int pos = (od * g.OH + oh) * g.OW + ow;
                     const unsigned want = (unsigned)(c * g.taps) + tap;
                     auto take = [&](int k, unsigned v) {        // v: the winner code(s) of output channel k
-                        const bool hmin = codes ? use_min && (v & 0xFFu) == tap : use_min && v == want;
-                        const bool hmax = codes ? use_max && (v >> 8) == tap : use_max && v == want;
-                        if (!(hmin || hmax)) return;
-                        const float gv = to_f32(__ldg(gbase + (k * g.vol + pos)));
-                        if (hmin) acc = __fmaf_rn(twob && alpha ? alpha[k * g.C + c] : 1.0f, gv, acc);
-                        if (hmax) acc = __fmaf_rn(twob && beta ? beta[k * g.C + c] : 1.0f, gv, acc);
+                        if constexpr (TWO) {
+                            const bool hmin = (v & 0xFFu) == tap, hmax = (v >> 8) == tap;
+                            if (!(hmin || hmax)) return;
+                            const float gv = to_f32(__ldg(gbase + (k * g.vol + pos)));
+                            if (hmin) acc = __fmaf_rn(alpha ? alpha[k * g.C + c] : 1.0f, gv, acc);
+                            if (hmax) acc = __fmaf_rn(beta ? beta[k * g.C + c] : 1.0f, gv, acc);
+                        } else {
+                            const unsigned mine = !CODES ? v : is_max ? v >> 8 : v & 0xFFu;
+                            if (mine == (CODES ? tap : want)) acc += to_f32(__ldg(gbase + (k * g.vol + pos)));
+                        }
                     };
-                    auto code = [&](int k) { return codes ? (unsigned)__ldg(cbase + (k * cstep + pos)) : (unsigned)__ldg(ibase + (k * g.vol + pos)); };
+                    auto code = [&](int k) { return CODES ? (unsigned)__ldg(cbase + (k * cstep + pos)) : (unsigned)__ldg(ibase + (k * g.vol + pos)); };
                     int k = slice;
                     for (; k + 3 * slices < g.K; k += 4 * slices) {
                         unsigned v[4];

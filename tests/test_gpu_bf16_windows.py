@@ -24,5 +24,6 @@ def test_five_by_five(mode, chan):
         d = dict(d, mode=mode, chan=chan, dtype="bf16")
         t = inputs.draw(d, 2300 + i)
         parity.check_forward(d, t)
-        assert tconv.tconv_last_kernel().startswith("fwd_tiled_bf16"), d
+        tiled = chan == "sum" or d["C"] >= 5      # Max / Min winners of few channels: the any-shape kernel
+        assert tconv.tconv_last_kernel().startswith("fwd_tiled_bf16" if tiled else "fwd_generic"), d
         parity.check_layer(d, None, 2300 + i, recompute=False)
