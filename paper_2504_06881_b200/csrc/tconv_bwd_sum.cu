@@ -7,9 +7,9 @@ namespace {
 template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW>
 int launch_gx(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx) {
     auto kern = bwd_sum_gx_kernel<T, BR, GX, AB, WIDE, KW>;
-    if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
+    if (allow_smem(kern, kSgSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
     kern<<<pl.ctas * (unsigned)a.g.C, pl.threads, pl.smem, a.st>>>(
-        a.g, a.x, a.alpha, a.beta, (const T*)a.gy, a.codes, (T*)a.gx, part_ab, part_gx, pl);
+        a.g, a.x, (const T*)a.w, (const T*)a.w2, a.alpha, a.beta, (const T*)a.gy, a.codes, (T*)a.gx, part_ab, part_gx, pl);
     ++a.launches;
     return TCONV_OK;
 }
@@ -68,8 +68,8 @@ int launch_all(SumBwdArgs& a) {
     while (ws < 32 && ws * 8 < gp.splits) ws *= 2;
     const unsigned nb_w = a.gw || a.gw2 ? (unsigned)((pairs * g.RS * ws + 255) / 256) : 0u, nb_ab = ab ? (unsigned)((pairs + 15) / 16) : 0u;
     const unsigned nb_bias = a.gbias ? (unsigned)((g.K + 7) / 8) : 0u;
-    bwd_sum_finish_kernel<T><<<nb_w + nb_ab + nb_bias, 256, 0, a.st>>>(g, br, gp.splits, part, (int)xp.ctas, part_ab, (const T*)a.w,
-                                                            (const T*)a.w2, a.alpha, a.beta, a.gw, a.gw2, a.galpha, a.gbeta, a.gbias, nb_w, nb_ab, ws);
+    bwd_sum_finish_kernel<<<nb_w + nb_ab + nb_bias, 256, 0, a.st>>>(g, br, gp.splits, part, (int)xp.ctas, part_ab,
+                                                            a.alpha, a.beta, a.gw, a.gw2, a.galpha, a.gbeta, a.gbias, nb_w, nb_ab, ws);
     ++a.launches;
     return TCONV_OK;
 }

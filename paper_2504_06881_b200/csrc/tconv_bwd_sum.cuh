@@ -6,15 +6,15 @@
 //                       channels k.  It adds coef * g into its private per-tap accumulators, which a
 //                       gather over the taps turns into grad_x at the end.  For grad_alpha / grad_beta
 //                       the inputs of its windows sit beside the accumulators, so the input of a winner
-//                       is read through the address of its accumulator; g * x is summed over the warp
-//                       per k.
+//                       is read through the address of its accumulator; with the winning weight it gives
+//                       the branch value as the forward rounded it, and g * (x + w) is summed over the
+//                       warp per k.
 //   bwd_sum_edges_kernel  where an image is cut into tiles: adds the (overlapping) input regions the
 //                       tiles' outputs reach.
 //   bwd_sum_gw_kernel   a warp owns one (k, c) pair and a share of its (image, pixel) items; every
 //                       lane keeps a private histogram of g over the *pair* of winning taps, so that
 //                       an item costs one shared-memory read-modify-write for both branches.
-//   bwd_sum_finish_kernel  sums the partials in a fixed order, applies alpha / beta, and completes
-//                       grad_alpha = sum g * (x + w) at the winners with sum_tap w * histogram.
+//   bwd_sum_finish_kernel  sums the partials in a fixed order and applies alpha / beta.
 //
 // No atomics; every accumulator has one writer and a fixed order.
 #pragma once
@@ -26,8 +26,9 @@ namespace tconv {
 
 // ---------------------------------------------------------------------------------- plans
 constexpr int kSgThreads = 256;         // most threads of a grad_x CTA: one quad each
-constexpr int kSgKB = 32;               // output channels staged per round
+constexpr int kSgKB = 8;                // output channels per stage of coefficients and weights
 constexpr size_t kSgSmem = 112 * 1024;  // two CTAs per SM (other windows than 3 x 3)
+constexpr int kSgSmemAttr = 214 * 1024; // opt-in ceiling: accumulators of kBwdSmemAttr and their stages
 
 struct SumGxPlan {
     int threads;
@@ -49,6 +50,23 @@ struct SumGwPlan {
     size_t smem;
 };
 
+// Stage of eight output channels' operands: weights [channel][tap], {alpha, beta} behind them, then (parallel) the
+// weights of the max branch.  Both tables and the two stages start at multiples of 256 bytes, so that a winner's
+// weight is addressed by putting tap * 4 into the low byte.  (Single-branch layers: alpha and beta only.)
+struct SumStage {
+    int coef, w2, stride, bytes;       // offsets of {alpha, beta} and w2, distance of the two stages, bytes of both
+};
+__host__ __device__ inline SumStage sum_stage(int mode, int RS) {
+    SumStage t;
+    t.coef = two_branch(mode) ? kSgKB * RS * 4 : 0;
+    const int len = t.coef + kSgKB * 8;
+    t.w2 = mode == TCONV_PARALLEL ? (len + 255) / 256 * 256 : 0;
+    const int all = mode == TCONV_PARALLEL ? t.w2 + kSgKB * RS * 4 : len;
+    t.stride = (all + 255) / 256 * 256;
+    t.bytes = t.stride + all;
+    return t;
+}
+
 // Picks the tile of outputs with the least work: lanes (idle ones included) times output channels, and
 // the input region a tile leaves for the final sum.
 inline bool plan_sum_gx(const Geo& g, SumGxPlan* best) {
@@ -56,7 +74,8 @@ inline bool plan_sum_gx(const Geo& g, SumGxPlan* best) {
     const size_t group = (size_t)g.RS * 256 * (ab ? 8 : 4);     // accumulators (and window inputs) of 64 threads
     const int halo_h = (g.R - 1) * g.dh, halo_w = (g.S - 1) * g.dw, QPR = (g.OW + 3) / 4;
     int most = kSgThreads;
-    while (most > 64 && most / 64 * group > kSgSmem) most -= 64;
+    const size_t stages = sum_stage(g.mode, g.RS).bytes;
+    while (most > 64 && most / 64 * group + stages > kSgSmem) most -= 64;
     if (most / 64 * group > kBwdSmemAttr) return false;
     double best_cost = -1.0;
     for (int ncol = 1; ncol <= QPR; ++ncol) {
@@ -88,7 +107,7 @@ inline bool plan_sum_gx(const Geo& g, SumGxPlan* best) {
         const double ctas = (double)((g.N + p.imgs - 1) / p.imgs) * p.nrow * ncol;
         if (ctas * g.C > 2.0e9) continue;
         p.ctas = (unsigned)ctas;
-        p.smem = (k3 ? kSgThreads / 64 : (p.threads + 63) / 64) * group;
+        p.smem = (k3 ? kSgThreads / 64 : (p.threads + 63) / 64) * group + stages;
         const double per_sm = ctas * g.C / 148.0;
         const double cost = ctas * (4.0 * p.threads * g.K + (p.nrow * ncol > 1 ? 2.0 * p.ER * p.EC : 0.0)) * (per_sm < 1.0 ? 1.0 / per_sm : 1.0);
         if (best_cost < 0.0 || cost < best_cost) { best_cost = cost; *best = p; }
@@ -197,6 +216,16 @@ template <typename T> __device__ __forceinline__ void unpack_g4(const float* raw
         gv[2] = __uint_as_float(b << 16); gv[3] = __uint_as_float(b & 0xffff0000u);
     }
 }
+__device__ __forceinline__ float ahead_value(const float* p) {
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ahead_value(const __nv_bfloat16* p) {
+    unsigned short v;
+    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __bfloat162float(__ushort_as_bfloat16(v));
+}
 template <bool WIDE, bool KEEP>
 __device__ __forceinline__ Codes4<WIDE> ahead_codes4(const uint8_t* p) {
     Codes4<WIDE> r;
@@ -248,26 +277,61 @@ template <> struct QuadTaps<true, 8> {
     __device__ __forceinline__ unsigned tmin(int j) const { return __byte_perm(j < 2 ? c.lo : c.hi, 0u, 0x4404u + (unsigned)((2 * (j & 1)) << 4)); }
     __device__ __forceinline__ unsigned tmax(int j) const { return __byte_perm(j < 2 ? c.lo : c.hi, 0u, 0x4404u + (unsigned)((2 * (j & 1) + 1) << 4)); }
 };
+// Shared-memory address of the winning weight of pixel j: table (at a multiple of 256 bytes) + tap * 4.
+template <bool WIDE> struct QuadWeights;
+template <> struct QuadWeights<false> {
+    unsigned lo, hi;
+    __device__ __forceinline__ explicit QuadWeights(const Codes4<false>& c) : lo((c.lo << 2) & 0x3c3c3c3cu), hi((c.lo >> 2) & 0x3c3c3c3cu) {}
+    __device__ __forceinline__ unsigned tmin(unsigned table, int j) const { return __byte_perm(lo, table, 0x7650u + (unsigned)j); }
+    __device__ __forceinline__ unsigned tmax(unsigned table, int j) const { return __byte_perm(hi, table, 0x7650u + (unsigned)j); }
+};
+template <> struct QuadWeights<true> {
+    QuadTaps<true, 8> t;
+    __device__ __forceinline__ explicit QuadWeights(const Codes4<true>& c) : t(c) {}
+    __device__ __forceinline__ unsigned tmin(unsigned table, int j) const { return table + (t.tmin(j) >> 6); }
+    __device__ __forceinline__ unsigned tmax(unsigned table, int j) const { return table + (t.tmax(j) >> 6); }
+};
+__device__ __forceinline__ float load_shared(unsigned at) {
+    return *reinterpret_cast<const float*>(__cvta_shared_to_generic(at));
+}
+
+// Branch values z = x + w of a quad as the forward rounds them (one rounded add; bf16: the fp32 sum of two bf16
+// values keeps more than twice their bits, so rounding it equals the bf16 add).
+__device__ __forceinline__ void branch_values(const float* x, const float* w, float* z, float) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) z[j] = __fadd_rn(x[j], w[j]);
+}
+__device__ __forceinline__ void branch_values(const float* x, const float* w, float* z, __nv_bfloat16) {
+#pragma unroll
+    for (int j = 0; j < 4; j += 2) {
+        const __nv_bfloat162 v = __floats2bfloat162_rn(__fadd_rn(x[j], w[j]), __fadd_rn(x[j + 1], w[j + 1]));
+        z[j] = __low2float(v);
+        z[j + 1] = __high2float(v);
+    }
+}
 
 // BR: 0 both branches, 1 min branch only, 2 max branch only.  GX: grad_x.  AB: grad_alpha / grad_beta (BR 0).
 // KW: 3 or 5 for 3 x 3 (narrow codes) and 5 x 5 windows (wide codes), else 0 (any window).
 // Shared memory: accumulators [4][tap][TP] floats per TP threads, then (AB) the window inputs in the same
-// layout; TP is 256 for 3 x 3 windows (and the taps of a column lie 1024 bytes apart), 64 otherwise (256
+// layout, at the end two stages of eight output channels' coefficients and (AB) weights; TP is 256 for 3 x 3 windows (and the taps of a column lie 1024 bytes apart), 64 otherwise (256
 // bytes apart): one PRMT and one add address an accumulator, and the winner's input lies at a constant
 // distance from it.
+// Bound by the shared-memory accesses of a quad and output channel: per branch four loads and four stores of
+// accumulators, four inputs, four weights.  The weights cost the training pass of N=128 C=64 K=64 32x32 fp32
+// 2.27 -> 2.41 ms against sums of g * x completed by the weights times the histograms; but those are the gradient
+// of an unrounded x + w, lose what x + w cancels, and are NaN where an infinite weight never wins.
 template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW>
 __global__ void __launch_bounds__(kSgThreads, KW == 3 ? 3 : 2)
-bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const float* __restrict__ alpha, const float* __restrict__ beta,
-                  const T* __restrict__ gy, const uint8_t* __restrict__ codes, T* __restrict__ gx,
-                  float* __restrict__ part_ab, float* __restrict__ part_gx, SumGxPlan pl) {
+bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, const T* __restrict__ w2,
+                  const float* __restrict__ alpha, const float* __restrict__ beta, const T* __restrict__ gy,
+                  const uint8_t* __restrict__ codes, T* __restrict__ gx, float* __restrict__ part_ab, float* __restrict__ part_gx, SumGxPlan pl) {
     constexpr bool K3 = KW == 3;
     constexpr int TP = K3 ? kSgThreads : 64, TS = TP * 4;      // columns side by side, bytes between two taps
     const int RS = KW ? KW * KW : g.RS;
     const int WR = KW ? KW : g.R, WS = KW ? KW : g.S;
     const int gbytes = RS * TS * (AB ? 8 : 4);                 // bytes of TP threads
-    extern __shared__ __align__(16) char smem[];
-    __shared__ float coef[kSgKB * 2];                          // [KB] {alpha, beta}
-    __shared__ float part[kSgThreads / 32 * kSgKB * 2];        // [warps][KB][2]
+    extern __shared__ __align__(256) char smem[];
+    __shared__ float part[2][kSgThreads / 32][kSgKB * 2];      // g * branch value of a warp, by stage
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int c = blockIdx.x % g.C;
     const unsigned tile = blockIdx.x / g.C;
@@ -301,8 +365,14 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const float* __restrict__ a
         float raw[PF][sizeof(T)];      // (4 floats, or 4 bf16 in two registers)
         Codes4<WIDE> cq[PF];
         int more = g.K - 1;
+        if constexpr (AB) {            // a repeated quad has no gradient
+#pragma unroll
+            for (int u = 0; u < PF; ++u)
+#pragma unroll
+                for (int i = 0; i < (int)sizeof(T); ++i) raw[u][i] = 0.0f;
+        }
         auto request = [&](int u) {
-            ahead_g4<T, false>(gbase + goff, raw[u]);
+            if (!AB || live) ahead_g4<T, false>(gbase + goff, raw[u]);
             cq[u] = ahead_codes4<WIDE, false>(cbase + (size_t)coff * (4 * CW));
             if (more > 0) { goff += plane; coff += cstep; }
             --more;
@@ -340,64 +410,116 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const float* __restrict__ a
             }
         }
 
-        for (int kb0 = 0; kb0 < g.K; kb0 += kSgKB) {
-            const int kn = min(kSgKB, g.K - kb0);
-            __syncthreads();     // the previous round's staging is consumed
-            for (int e = tid; e < kSgKB; e += blockDim.x) {
-                const bool ok = e < kn;
-                const size_t i = (size_t)(kb0 + e) * g.C + c;
-                coef[2 * e] = ok ? (alpha ? alpha[i] : 1.0f) : 0.0f;      // (no alpha / beta in single-branch layers)
-                coef[2 * e + 1] = ok ? (beta ? beta[i] : 1.0f) : 0.0f;
+        // The operands of the next stage are requested before this stage's are used and stored behind them (one a
+        // thread; the rest of a large window's weights are copied then).
+        const SumStage lay = sum_stage(g.mode, RS);
+        char* stage = smem + pl.smem - lay.bytes;
+        const int nw = AB ? kSgKB * RS : 0, nstage = 2 * kSgKB + nw * (AB && g.mode == TCONV_PARALLEL ? 2 : 1);
+        struct Operand {
+            const void* from;      // of the first stage; null: all ones
+            int kk, to;            // output channel within the stage, place in it
+            bool coef;
+        };
+        auto operand = [&](int e) {
+            Operand o;
+            o.coef = e < 2 * kSgKB;
+            if (o.coef) {
+                const float* ab = (e & 1) ? beta : alpha;
+                o.kk = e >> 1;
+                o.to = lay.coef + 4 * e;
+                o.from = ab ? ab + (size_t)o.kk * g.C + c : nullptr;
+            } else {
+                e -= 2 * kSgKB;
+                const bool second = e >= nw;
+                if (second) e -= nw;
+                o.kk = e / RS;
+                o.to = (second ? lay.w2 : 0) + 4 * e;
+                o.from = (second ? w2 : w) + ((size_t)o.kk * g.C + c) * RS + e % RS;
             }
-            __syncthreads();
-            for (int k8 = 0; k8 < kn; k8 += 8) {
-                float s[AB ? 16 : 1];
+            return o;
+        };
+        auto fetch = [&](const Operand& o, int k0) {
+            if (k0 + o.kk >= g.K) return 0.0f;
+            if (o.coef) return o.from ? ahead_value(static_cast<const float*>(o.from) + (size_t)k0 * g.C) : 1.0f;
+            return ahead_value(static_cast<const T*>(o.from) + (size_t)k0 * g.C * RS);
+        };
+        auto copy = [&](int e0, int k0, char* to) {
+            for (int e = e0; e < nstage; e += blockDim.x) {
+                const Operand o = operand(e);
+                *reinterpret_cast<float*>(to + o.to) = fetch(o, k0);
+            }
+        };
+        copy(tid, 0, stage);
+        __syncthreads();
+        int buf = 0;
+        for (int k0 = 0; k0 < g.K; k0 += kSgKB, buf ^= 1) {
+            const bool more_k = k0 + kSgKB < g.K;
+            float ahead = 0.0f;
+            if (more_k && tid < nstage) ahead = fetch(operand(tid), k0 + kSgKB);
+            // (output channels past K repeat the last one with zero coefficients)
+            const char* st = stage + buf * lay.stride;
+            const unsigned table = (unsigned)__cvta_generic_to_shared(st);
+            float s[AB ? 16 : 1];
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
-                    const int u = kk % PF;
-                    if (kk % 2 == 0) {
-                        request((u + 2) % PF);
-                        request((u + 3) % PF);
+            for (int kk = 0; kk < kSgKB; ++kk) {
+                const int u = kk % PF;
+                if (kk % 2 == 0) {
+                    request((u + 2) % PF);
+                    request((u + 3) % PF);
+                }
+                float gv[4];
+                unpack_g4<T>(raw[u], gv);
+                const float2 cf = *reinterpret_cast<const float2*>(st + lay.coef + kk * 8);
+                const QuadTaps<WIDE, K3 ? 10 : 8> taps(cq[u]);
+                const QuadWeights<WIDE> wtaps(cq[u]);
+                // one branch: the four pixels' accumulators are distinct, so their loads go out together
+                auto branch = [&](bool is_min, float a) {
+                    char* p[4];
+                    float v[4], xv[4], wv[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) p[j] = Ab + (is_min ? taps.tmin(j) : taps.tmax(j));
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        if constexpr (GX) v[j] = *reinterpret_cast<const float*>(p[j] + j * RS * TS);
+                        if constexpr (AB) {
+                            xv[j] = *reinterpret_cast<const float*>(p[j] + (4 + j) * RS * TS);
+                            wv[j] = load_shared((is_min ? wtaps.tmin(table, j) : wtaps.tmax(table + lay.w2, j)) + kk * RS * 4);
+                        }
                     }
-                    float gv[4];
-                    unpack_g4<T>(raw[u], gv);
-                    const float2 cf = *reinterpret_cast<const float2*>(coef + 2 * (k8 + kk));
-                    const QuadTaps<WIDE, K3 ? 10 : 8> taps(cq[u]);
-                    // one branch: the four pixels' accumulators are distinct, so their loads go out together
-                    auto branch = [&](bool is_min, float a) {
-                        char* p[4];
-                        float v[4], xv[4];
+                    float sum = 0.0f;
+                    if constexpr (GX) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) p[j] = Ab + (is_min ? taps.tmin(j) : taps.tmax(j));
+                        for (int j = 0; j < 4; ++j) *reinterpret_cast<float*>(p[j] + j * RS * TS) = __fmaf_rn(a, gv[j], v[j]);
+                    }
+                    if constexpr (AB) {
+                        float z[4];
+                        branch_values(xv, wv, z, T());
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if constexpr (GX) v[j] = *reinterpret_cast<const float*>(p[j] + j * RS * TS);
-                            if constexpr (AB) xv[j] = *reinterpret_cast<const float*>(p[j] + (4 + j) * RS * TS);
-                        }
-                        float sum = 0.0f;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if constexpr (GX) *reinterpret_cast<float*>(p[j] + j * RS * TS) = __fmaf_rn(a, gv[j], v[j]);
-                            if constexpr (AB) sum = __fmaf_rn(gv[j], xv[j], sum);
-                        }
-                        return sum;
-                    };
-                    float sa = 0.0f, sb = 0.0f;
-                    if constexpr (BR != 2) sa = branch(true, cf.x);
-                    if constexpr (BR != 1) sb = branch(false, cf.y);
-                    if constexpr (AB) { s[2 * kk] = sa; s[2 * kk + 1] = sb; }
-                }
-                if constexpr (AB) {
-                    const float v = warp_sum16(s, lane);
-                    if (!(lane & 1)) part[(warp * kSgKB + k8) * 2 + (lane >> 1)] = v;
-                }
+                        for (int j = 0; j < 4; ++j) sum = __fmaf_rn(gv[j], z[j], sum);
+                    }
+                    return sum;
+                };
+                float sa = 0.0f, sb = 0.0f;
+                if constexpr (BR != 2) sa = branch(true, cf.x);
+                if constexpr (BR != 1) sb = branch(false, cf.y);
+                if constexpr (AB) { s[2 * kk] = sa; s[2 * kk + 1] = sb; }
             }
             if constexpr (AB) {
-                __syncthreads();
-                for (int e = tid; e < 2 * kn; e += blockDim.x) {
+                const float v = warp_sum16(s, lane);
+                if (!(lane & 1)) part[buf][warp][lane >> 1] = v;
+            }
+            if (more_k) {
+                char* to = stage + (buf ^ 1) * lay.stride;
+                if (tid < nstage) *reinterpret_cast<float*>(to + operand(tid).to) = ahead;
+                copy(tid + blockDim.x, k0 + kSgKB, to);
+            }
+            __syncthreads();     // this stage is used, the next one and its sums are stored
+            if constexpr (AB) {
+                if (tid < 2 * kSgKB && 2 * k0 + tid < 2 * g.K) {
                     float t = 0.0f;
-                    for (int i = 0; i < nwarps; ++i) t += part[i * kSgKB * 2 + e];
-                    part_ab[((size_t)tile * g.C + c) * g.K * 2 + 2 * kb0 + e] = t;
+#pragma unroll
+                    for (int i = 0; i < kSgThreads / 32; ++i) t += i < nwarps ? part[buf][i][tid] : 0.0f;
+                    part_ab[((size_t)tile * g.C + c) * g.K * 2 + 2 * k0 + tid] = t;
                 }
             }
         }
@@ -673,14 +795,12 @@ bwd_sum_gw_kernel(Geo g, const T* __restrict__ gy, const uint8_t* __restrict__ c
 // ---------------------------------------------------------------------------------- finish
 // Blocks [0, nb_w): grad_w / grad_w2, 256 / ws (k, c, tap) entries per block; ws slices share the splits and are
 // added in slice order.  The next nb_ab blocks: grad_alpha / grad_beta, 16 (c, k) entries per block; sixteen slices
-// share the partial rows and the splits, and are added in slice order.  The rest: grad_bias, a warp per output channel (the sum of a pair's histogram is the sum
+// share the partial rows and are added in slice order.  The rest: grad_bias, a warp per output channel (the sum of a pair's histogram is the sum
 // of grad_y), its lanes added in a fixed tree.  All sums are chains of loads from L2, kept eight deep in flight:
 // N=92 C=3 K=12 23x33 5x5 took 42 us where one thread per channel summed splits x taps values.
-template <typename T>
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 bwd_sum_finish_kernel(Geo g, int br, int splits, const float* __restrict__ part, int rows, const float* __restrict__ part_ab,
-                      const T* __restrict__ w, const T* __restrict__ w2, const float* __restrict__ alpha,
-                      const float* __restrict__ beta, float* __restrict__ gw, float* __restrict__ gw2,
+                      const float* __restrict__ alpha, const float* __restrict__ beta, float* __restrict__ gw, float* __restrict__ gw2,
                       float* __restrict__ galpha, float* __restrict__ gbeta, float* __restrict__ gbias, unsigned nb_w,
                       unsigned nb_ab, int ws) {
     const size_t pairs = (size_t)g.K * g.C, len = pairs * 2 * g.RS;
@@ -736,18 +856,6 @@ bwd_sum_finish_kernel(Geo g, int br, int splits, const float* __restrict__ part,
         for (int r = sl; r < rows; r += 16) {
             const float2 v = __ldg(reinterpret_cast<const float2*>(part_ab) + r * pairs + e);
             s.x += v.x; s.y += v.y;
-        }
-        const size_t pair = k * g.C + c;
-        const T* wk = w + pair * g.RS;
-        const T* wm = (g.mode == TCONV_PARALLEL ? w2 : w) + pair * g.RS;
-        const float* p = part + pair * 2 * g.RS;
-        for (int sp = sl; sp < splits; sp += 16) {
-            const float* q = p + sp * len;
-#pragma unroll 9
-            for (int t = 0; t < g.RS; ++t) {
-                s.x = __fmaf_rn(to_f32(wk[t]), __ldg(q + t), s.x);
-                s.y = __fmaf_rn(to_f32(wm[t]), __ldg(q + g.RS + t), s.y);
-            }
         }
     }
     red[threadIdx.x] = s;

@@ -1,0 +1,83 @@
+"""grad_alpha / grad_beta are sums of grad_y times the branch values as the forward rounded them.  Tolerance: the
+products of the bf16 layers are exact in fp32 and a value passes fewer than 100 fp32 additions, so that the result
+is within 100 * 2^-24 < 1e-5 of the sum of |contributions|; fp32 layers round each branch value and product as well.
+Also: what cancels inside a branch value does not reach the sums, and taps that never win add nothing, whatever
+their weight (infinite weights are how a caller masks a tap: +inf under min, -inf under max)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import tconv_oracle as ora
+from paper_2504_06881_b200 import inputs, tconv
+import parity
+
+pytestmark = pytest.mark.gpu
+
+L = inputs.layer
+RTOL = 1e-5
+PARAMS = ("grad_w", "grad_w2", "grad_alpha", "grad_beta", "grad_bias")
+LAYERS = [
+    L(2, 3, 32, 32, 33, pad=1),                     # one tile of 256 quads, output channels past a whole stage
+    L(1, 2, 37, 70, 9, pad=2, dil=2),               # several tiles, ragged rows
+    L(19, 3, 7, 7, 12, stride=2, pad=1),            # several images per tile
+    L(2, 2, 20, 23, 5, R=5, S=5, pad=2),            # 16-bit codes
+    L(1, 2, 24, 25, 3, R=4, S=4, pad=1),
+]
+
+
+def device_grads(d, t, winners=None):
+    g = parity.to_dev(t, d)
+    la = parity.layer_args(d, g)
+    if winners is None:
+        _, winners = tconv.forward(d, g["x"], g["w"], la["w2"], la["alpha"], la["beta"], g["bias"], want_winners=True)
+    return tconv.backward(d, g["x"], g["w"], g["g"], la["w2"], la["alpha"], la["beta"], winners)
+
+
+def oracle_grads(d, t):
+    la = parity.layer_args(d, t)
+    return ora.backward(d, t["x"], t["w"], t["g"], la["w2"], la["alpha"], la["beta"])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("mode", ["compound", "parallel"])
+def test_dense(mode, dtype):
+    for i, d in enumerate(LAYERS):
+        d = dict(d, mode=mode, dtype=dtype)
+        t = inputs.draw(d, 4100 + i)
+        got, ref = device_grads(d, t), oracle_grads(d, t)
+        assert tconv.tconv_last_kernel() == "bwd_sum"
+        parity.compare_grads(d, {k: got[k] for k in PARAMS if k in got}, ref, rtol=RTOL)
+
+
+@pytest.mark.parametrize("mode", ["compound", "parallel"])
+def test_dense_offset_inputs(mode):
+    """Inputs around 4096 under weights around -4096: |x| and |w| are thousands of times |x + w|."""
+    for i, d in enumerate(LAYERS[:3]):
+        d = dict(d, mode=mode, dtype="f32", pad_h=0, pad_w=0)
+        t = inputs.draw(d, 4200 + i, x=("normal", 4096.0, 1.0), w=("normal", -4096.0, 1.0))
+        parity.compare_grads(d, device_grads(d, t), oracle_grads(d, t), rtol=RTOL)
+
+
+def masked(t):
+    """Every other tap of the min branch and the others of the max branch masked (the middle one in neither)."""
+    taps = t["w"].reshape(t["w"].shape[:2] + (-1,)).shape[2]
+    keep = taps // 2
+    for name, start, v in (("w", 0, np.inf), ("w2", 1, -np.inf)):
+        flat = t[name].reshape(t[name].shape[:2] + (taps,))
+        flat[..., [i for i in range(start, taps, 2) if i != keep]] = v
+    return t
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_dense_masked_taps(dtype):
+    for i, d in enumerate(LAYERS[:3]):
+        d = dict(d, mode="parallel", dtype=dtype)
+        t = masked(inputs.draw(d, 4300 + i))
+        ref = ora.forward(d, t["x"], t["w"], t["w2"], t["alpha"], t["beta"], t["bias"])
+        # (the fp32 forward recovers winners from differences of tap sums, which infinite sums do not have: the
+        # oracle's winners are passed to the backward)
+        OH, OW = inputs.output_hw(d)
+        codes = np.zeros((d["N"], d["K"], d["C"], OH, (OW + 3) // 4 * 4), np.uint8)
+        codes[..., :OW] = ref["codes"]
+        got = device_grads(d, t, torch.from_numpy(codes).cuda().reshape(-1))
+        parity.compare_grads(d, {k: got[k] for k in PARAMS}, oracle_grads(d, t), rtol=RTOL)
