@@ -4,9 +4,9 @@
 namespace tconv {
 namespace {
 
-template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW>
+template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW, bool TAIL>
 int launch_gx(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx) {
-    auto kern = bwd_sum_gx_kernel<T, BR, GX, AB, WIDE, KW>;
+    auto kern = bwd_sum_gx_kernel<T, BR, GX, AB, WIDE, KW, TAIL>;
     if (allow_smem(kern, kSgSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
     kern<<<pl.ctas * (unsigned)a.g.C, pl.threads, pl.smem, a.st>>>(
         a.g, a.x, (const T*)a.w, (const T*)a.w2, a.alpha, a.beta, (const T*)a.gy, a.codes, (T*)a.gx, part_ab, part_gx, pl);
@@ -17,10 +17,11 @@ int launch_gx(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx
 template <typename T, int BR, bool GX, bool AB>
 int launch_gx_window(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx) {
     const Geo& g = a.g;
-    if (g.wide) return g.R == 5 && g.S == 5 ? launch_gx<T, BR, GX, AB, true, 5>(a, pl, part_ab, part_gx)
-                                            : launch_gx<T, BR, GX, AB, true, 0>(a, pl, part_ab, part_gx);
-    return g.R == 3 && g.S == 3 ? launch_gx<T, BR, GX, AB, false, 3>(a, pl, part_ab, part_gx)
-                                : launch_gx<T, BR, GX, AB, false, 0>(a, pl, part_ab, part_gx);
+    if (g.wide) return g.R == 5 && g.S == 5 ? launch_gx<T, BR, GX, AB, true, 5, true>(a, pl, part_ab, part_gx)
+                                            : launch_gx<T, BR, GX, AB, true, 0, true>(a, pl, part_ab, part_gx);
+    if (g.R != 3 || g.S != 3) return launch_gx<T, BR, GX, AB, false, 0, true>(a, pl, part_ab, part_gx);
+    return g.K % kSgKB ? launch_gx<T, BR, GX, AB, false, 3, true>(a, pl, part_ab, part_gx)
+                       : launch_gx<T, BR, GX, AB, false, 3, false>(a, pl, part_ab, part_gx);
 }
 
 template <typename T, int BR, bool PAIRS, bool WIDE>

@@ -320,7 +320,10 @@ __device__ __forceinline__ void branch_values(const float* x, const float* w, fl
 // accumulators, four inputs, four weights.  The weights cost the training pass of N=128 C=64 K=64 32x32 fp32
 // 2.27 -> 2.41 ms against sums of g * x completed by the weights times the histograms; but those are the gradient
 // of an unrounded x + w, lose what x + w cancels, and are NaN where an infinite weight never wins.
-template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW>
+// TAIL: the last stage may have output channels past K.  They repeat the last one, and their gradients are dropped
+// by selection (times a zero coefficient an infinite one would be NaN); selecting in every stage costs 3 x 3 layers
+// 3 %, so they have an instance for multiples of eight channels without it.
+template <typename T, int BR, bool GX, bool AB, bool WIDE, int KW, bool TAIL>
 __global__ void __launch_bounds__(kSgThreads, KW == 3 ? 3 : 2)
 bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, const T* __restrict__ w2,
                   const float* __restrict__ alpha, const float* __restrict__ beta, const T* __restrict__ gy,
@@ -456,7 +459,6 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
             const bool more_k = k0 + kSgKB < g.K;
             float ahead = 0.0f;
             if (more_k && tid < nstage) ahead = fetch(operand(tid), k0 + kSgKB);
-            // (output channels past K repeat the last one with zero coefficients)
             const char* st = stage + buf * lay.stride;
             const unsigned table = (unsigned)__cvta_generic_to_shared(st);
             float s[AB ? 16 : 1];
@@ -469,6 +471,10 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
                 }
                 float gv[4];
                 unpack_g4<T>(raw[u], gv);
+                if constexpr (TAIL) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) gv[j] = k0 + kk < g.K ? gv[j] : 0.0f;
+                }
                 const float2 cf = *reinterpret_cast<const float2*>(st + lay.coef + kk * 8);
                 const QuadTaps<WIDE, K3 ? 10 : 8> taps(cq[u]);
                 const QuadWeights<WIDE> wtaps(cq[u]);

@@ -81,3 +81,19 @@ def test_dense_masked_taps(dtype):
         codes[..., :OW] = ref["codes"]
         got = device_grads(d, t, torch.from_numpy(codes).cuda().reshape(-1))
         parity.compare_grads(d, {k: got[k] for k in PARAMS}, oracle_grads(d, t), rtol=RTOL)
+
+
+@pytest.mark.parametrize("mode,chan", [("compound", "sum"), ("parallel", "sum"), ("max_plus", "sum")])
+@pytest.mark.parametrize("K", [8, 9, 12])
+def test_dense_infinite_gradient(mode, chan, K):
+    """One infinite gradient in the last output channel reaches its winners' inputs as an infinity, nothing else."""
+    for i, shape in enumerate([dict(N=2, C=3, H=12, W=13), dict(N=1, C=2, H=40, W=72)]):
+        d = L(shape["N"], shape["C"], shape["H"], shape["W"], K, pad=1, mode=mode, chan=chan)
+        t = inputs.draw(d, 4400 + i)
+        t["alpha"] += 0.5
+        t["beta"] += 0.5
+        t["g"][0, K - 1, 5, 6] = np.inf
+        got = device_grads(d, t)["grad_x"].cpu().numpy()
+        ref = oracle_grads(d, t)["grad_x"][0]
+        assert not np.isnan(got).any()
+        assert np.array_equal(np.isinf(got), np.isinf(ref)) and np.isinf(got).any()
