@@ -170,7 +170,7 @@ struct PlanParams3 {
 PlanParams3 plan_params3(const Geo3& g) {
     PlanParams3 p;
     const int branches = two_branch(g.mode) ? 2 : 1;
-    auto bytes = [&](int tb) { return ((size_t)branches * (g.taps + 1) * tb + 2 * (size_t)g.taps + 3 * (size_t)(tb / 32)) * 4; };
+    auto bytes = [&](int tb) { return ((size_t)branches * (g.taps + 1) * tb + 4 * (size_t)g.taps + 3 * (size_t)(tb / 32)) * 4; };
     p.tb = 128;
     while (p.tb > 32 && bytes(p.tb) > 48 * 1024) p.tb /= 2;
     p.smem = bytes(p.tb);
@@ -387,8 +387,8 @@ int backward3_t(const Geo3& g, const void* x, const void* w, const void* w2, con
         float* pb = ab + (size_t)p.nsplit * kc * 2;
         if (allow_smem(bwd3d_params_kernel<T>, (int)kSmem1d) != cudaSuccess) return TCONV_ERR_CUDA;
         bwd3d_params_kernel<T><<<dim3((unsigned)kc, (unsigned)p.nsplit), p.tb, p.smem, st>>>(
-            g, p.nsplit, (const T*)x, (const T*)gy, winners, hist, ab, pb);
-        bwd3d_params_finish_kernel<T><<<(unsigned)kc, 128, 0, st>>>(g, p.nsplit, (const T*)w, (const T*)w2, alpha, beta, hist, ab,
+            g, p.nsplit, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, winners, hist, ab, pb);
+        bwd3d_params_finish_kernel<<<(unsigned)kc, 128, 0, st>>>(g, p.nsplit, alpha, beta, hist, ab,
                                                                   pb, gw, gw2, galpha, gbeta, gbias);
         g3_launches += 2;
         return check(cudaGetLastError());

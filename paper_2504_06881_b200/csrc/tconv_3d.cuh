@@ -421,13 +421,13 @@ bwd3d_gx_kernel(Geo3 g, const float* __restrict__ alpha, const float* __restrict
 // All parameter gradients but their last sum.  Block (k * C + c, split) walks its share of the (n, position)
 // range; every thread keeps private columns in shared memory, one per tap and branch (col[tap][tb], one more
 // for items that another channel won), so that an item costs one read-modify-write per branch; grad_alpha /
-// grad_beta: g * x at the winner (zero in the padding), the weights' share is added by the finishing kernel from
-// the same histograms.  part_hist [split][k*C+c][2][taps], part_ab [split][k*C+c][2], part_bias [split][k].
+// grad_beta: g times the branch value, rebuilt from the winner (x zero in the padding) as the forward rounded it.
+// part_hist [split][k*C+c][2][taps], part_ab [split][k*C+c][2], part_bias [split][k].
 template <typename T>
 __global__ void __launch_bounds__(128)
-bwd3d_params_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __restrict__ gy,
-                    const void* __restrict__ winners, float* __restrict__ part_hist, float* __restrict__ part_ab,
-                    float* __restrict__ part_bias) {
+bwd3d_params_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __restrict__ w, const T* __restrict__ w2,
+                    const T* __restrict__ gy, const void* __restrict__ winners, float* __restrict__ part_hist,
+                    float* __restrict__ part_ab, float* __restrict__ part_bias) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, tb = blockDim.x, taps = g.taps;
     const int kc = blockIdx.x, k = kc / g.C, c = kc - k * g.C, split = blockIdx.y;
@@ -438,12 +438,18 @@ bwd3d_params_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __rest
     float* cmax = cmin + (use_min ? (taps + 1) * tb : 0);
     int* tofs = reinterpret_cast<int*>(cmin + branches * (taps + 1) * tb);   // input offset of a tap from its window's corner
     int* tcrd = tofs + taps;                                                 // its (depth, row, column) distance, 10 bits each
-    float* red = reinterpret_cast<float*>(tcrd + taps);                      // [3][tb / 32]
+    T* wmin = reinterpret_cast<T*>(tcrd + taps);                             // weights of the pair, either branch
+    T* wmax = wmin + taps;
+    float* red = reinterpret_cast<float*>(tcrd + 3 * taps);                  // [3][tb / 32]
     for (int i = tid; i < branches * (taps + 1) * tb; i += tb) cmin[i] = 0.0f;
     for (int i = tid; i < taps; i += tb) {
         const int t = i / (g.R * g.S), r = (i / g.S) % g.R, s = i % g.S;
         tofs[i] = (t * g.dd * g.H + r * g.dh) * g.W + s * g.dw;
         tcrd[i] = (t << 20) | (r << 10) | s;
+        if (twob) {
+            wmin[i] = w[(size_t)kc * taps + i];
+            wmax[i] = (g.mode == TCONV_PARALLEL ? w2 : w)[(size_t)kc * taps + i];
+        }
     }
     __syncthreads();
     const int total = g.N * g.vol, per = (total + nsplit - 1) / nsplit;
@@ -477,7 +483,7 @@ bwd3d_params_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __rest
             }
         }
         if (twob) {
-            float xa[U], xb[U];
+            float za[U], zb[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const unsigned q = (unsigned)pos[u] / (unsigned)g.OW;
@@ -485,19 +491,20 @@ bwd3d_params_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __rest
                 const int d0 = od * g.sd - g.pd, h0 = oh * g.sh - g.ph, w0 = ow * g.sw - g.pw;
                 const T* xc = x + (size_t)(n[u] * g.C + c) * g.D * g.H * g.W;
                 const int corner = (d0 * g.H + h0) * g.W + w0;
-                auto at = [&](int tap) {
+                auto at = [&](int tap, const T* wt) {
                     const int p = tcrd[tap];
                     const int id = d0 + (p >> 20) * g.dd, ih = h0 + ((p >> 10) & 1023) * g.dh, iw = w0 + (p & 1023) * g.dw;
                     const bool ok = (unsigned)id < (unsigned)g.D && (unsigned)ih < (unsigned)g.H && (unsigned)iw < (unsigned)g.W;
-                    return ok ? to_f32(__ldg(xc + corner + tofs[tap])) : 0.0f;
+                    return tap_add(ok ? __ldg(xc + corner + tofs[tap]) : zero_of<T>(), wt[tap]);
                 };
-                xa[u] = at(amn[u]);
-                xb[u] = at(amx[u]);
+                za[u] = at(amn[u], wmin);
+                zb[u] = at(amx[u], wmax);
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                sa = __fmaf_rn(gv[u], xa[u], sa);
-                sb = __fmaf_rn(gv[u], xb[u], sb);
+                if (jb + u * tb >= j1) break;
+                sa = __fmaf_rn(gv[u], za[u], sa);
+                sb = __fmaf_rn(gv[u], zb[u], sb);
             }
         }
 #pragma unroll
@@ -533,21 +540,16 @@ bwd3d_params_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __rest
     }
 }
 
-// One block per (k, c): sums its partials over the splits in order, applies alpha / beta and completes
-// grad_alpha / grad_beta with sum_tap w * histogram.
-template <typename T>
-__global__ void __launch_bounds__(128)
-bwd3d_params_finish_kernel(Geo3 g, int nsplit, const T* __restrict__ w, const T* __restrict__ w2,
-                           const float* __restrict__ alpha, const float* __restrict__ beta,
+// One block per (k, c): sums its partials over the splits in order and applies alpha / beta.
+static __global__ void __launch_bounds__(128)
+bwd3d_params_finish_kernel(Geo3 g, int nsplit, const float* __restrict__ alpha, const float* __restrict__ beta,
                            const float* __restrict__ part_hist, const float* __restrict__ part_ab,
                            const float* __restrict__ part_bias, float* __restrict__ gw, float* __restrict__ gw2,
                            float* __restrict__ galpha, float* __restrict__ gbeta, float* __restrict__ gbias) {
-    __shared__ float red[2][4];
     const int kc = blockIdx.x, k = kc / g.C, c = kc - k * g.C, tid = threadIdx.x;
     const size_t pairs = (size_t)g.K * g.C;
     const bool twob = two_branch(g.mode), par = g.mode == TCONV_PARALLEL;
     const float a = twob && alpha ? alpha[kc] : 1.0f, b = twob && beta ? beta[kc] : 1.0f;
-    float sa = 0.0f, sb = 0.0f;
     for (int t = tid; t < g.taps; t += 128) {
         float tmin = 0.0f, tmax = 0.0f;
         for (int s = 0; s < nsplit; ++s) {
@@ -565,25 +567,13 @@ bwd3d_params_finish_kernel(Geo3 g, int nsplit, const T* __restrict__ w, const T*
             } else if (gw) {
                 gw[i] = __fmaf_rn(a, tmin, b * tmax);
             }
-            sa = __fmaf_rn(to_f32(w[i]), tmin, sa);
-            sb = __fmaf_rn(to_f32(par ? w2[i] : w[i]), tmax, sb);
         }
     }
-    if (twob && (galpha || gbeta)) {
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) {
-            sa += __shfl_xor_sync(0xffffffffu, sa, d);
-            sb += __shfl_xor_sync(0xffffffffu, sb, d);
-        }
-        if ((tid & 31) == 0) { red[0][tid >> 5] = sa; red[1][tid >> 5] = sb; }
-        __syncthreads();
-        if (tid < 2) {
-            float s = 0.0f;
-            for (int sp = 0; sp < nsplit; ++sp) s += part_ab[(sp * pairs + kc) * 2 + tid];
-            for (int q = 0; q < 4; ++q) s += red[tid][q];
-            float* to = tid == 0 ? galpha : gbeta;
-            if (to) to[kc] = s;
-        }
+    if (twob && tid < 2) {
+        float s = 0.0f;
+        for (int sp = 0; sp < nsplit; ++sp) s += part_ab[(sp * pairs + kc) * 2 + tid];
+        float* to = tid == 0 ? galpha : gbeta;
+        if (to) to[kc] = s;
     }
     if (gbias && c == 0 && tid == 2) {
         float s = 0.0f;

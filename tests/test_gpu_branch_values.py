@@ -7,8 +7,8 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import tconv_oracle as ora
-from paper_2504_06881_b200 import inputs, tconv
+from oracle import tconv3d_oracle as ora3, tconv_oracle as ora
+from paper_2504_06881_b200 import inputs, tconv, tconv3d
 import parity
 
 pytestmark = pytest.mark.gpu
@@ -97,3 +97,46 @@ def test_dense_infinite_gradient(mode, chan, K):
         ref = oracle_grads(d, t)["grad_x"][0]
         assert not np.isnan(got).any()
         assert np.array_equal(np.isinf(got), np.isinf(ref)) and np.isinf(got).any()
+
+
+VOLUMES = [
+    inputs.layer3d(4, 6, 6, 6, 6, 16, T=5, R=5, S=5),
+    inputs.layer3d(2, 3, 9, 11, 10, 8, T=3, R=3, S=3, stride=(2, 3, 2), pad=1, dil=(1, 2, 1)),
+    inputs.layer3d(3, 2, 1, 9, 40, 3, T=1, R=3, S=3, pad=(0, 1, 1)),
+]
+
+
+def volume_grads(d, t):
+    dt = tconv.TORCH_DTYPE[d["dtype"]]
+    dev = {k: torch.from_numpy(v).cuda().to(dt if k in ("x", "w", "w2", "g") else torch.float32) for k, v in t.items()}
+    w2 = dev["w2"] if d["mode"] == "parallel" else None
+    _, win = tconv3d.forward(d, dev["x"], dev["w"], w2, dev["alpha"], dev["beta"], dev["bias"], want_winners=True)
+    return tconv3d.backward(d, dev["x"], dev["w"], dev["g"], w2, dev["alpha"], dev["beta"], win)
+
+
+def check_volume(d, t):
+    got = volume_grads(d, t)
+    ref = ora3.backward(d, t["x"], t["w"], t["g"], t["w2"] if d["mode"] == "parallel" else None, t["alpha"], t["beta"])
+    parity.compare_grads(d, {k: got[k] for k in PARAMS if k in got}, ref, rtol=RTOL)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("mode", ["compound", "parallel"])
+def test_volume(mode, dtype):
+    for i, d in enumerate(VOLUMES):
+        d = dict(d, mode=mode, dtype=dtype)
+        check_volume(d, inputs.draw3d(d, 4500 + i))
+
+
+@pytest.mark.parametrize("mode", ["compound", "parallel"])
+def test_volume_offset_inputs(mode):
+    for i, d in enumerate(VOLUMES):
+        d = dict(d, mode=mode, pad=(0, 0, 0))
+        check_volume(d, inputs.draw3d(d, 4600 + i, x=("normal", 4096.0, 1.0), w=("normal", -4096.0, 1.0)))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_volume_masked_taps(dtype):
+    for i, d in enumerate(VOLUMES):
+        d = dict(d, mode="parallel", dtype=dtype)
+        check_volume(d, masked(inputs.draw3d(d, 4700 + i)))
