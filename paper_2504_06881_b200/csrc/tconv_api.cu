@@ -443,30 +443,7 @@ int dw_backward_t(const Geo& g, const void* x, const void* w, const void* w2, co
         if (rc != TCONV_OK) return rc;
         codes = (const uint8_t*)ws;
     }
-    const bool params = gw || gw2 || galpha || gbeta || gbias;
-    const bool s1 = g.R == 3 && g.S == 3 && g.dh == 1 && g.dw == 1 && g.sh == 1 && g.sw == 1;
-    if constexpr (sizeof(T) == 4) {
-        if (gx && params && twob && s1 && g.ph <= 2 && g.pw <= 2 && dw_chunks(g) <= g.N && g.OH * g.OW >= 100) {
-            // fp32, two branches: grad_x and the parameters together (tiny planes: too few strips per image; bf16
-            // and single branches: the separate kernels' packed or shorter loops are faster, 197 against 370 us for
-            // 15 x 483 x 60 x 60 bf16)
-            const DwBwdPlan pl = plan_dw_bwd3(g, dw_chunks(g));
-            const dim3 grid((unsigned)g.C, (unsigned)pl.nch);
-            const int need_ab = (galpha || gbeta) ? 1 : 0, QPRI = (g.W + 3) / 4;
-            const bool vec = g.pw == 1 && (g.OW & 3) == 0;
-            auto kern = par ? (vec ? dw_bwd3_kernel<true, true> : dw_bwd3_kernel<true, false>)
-                            : (vec ? dw_bwd3_kernel<false, true> : dw_bwd3_kernel<false, false>);
-            kern<<<grid, 256, 0, st>>>(g, (const float*)x, (const float*)w, (const float*)w2, alpha, beta, (const float*)gy,
-                                       codes, (float*)gx, partial, pl, need_ab, QPRI);
-            const int n = g.C * kDwAcc;
-            dw_bwd_finish_kernel<<<(n + 255) / 256, 256, 0, st>>>(g, partial, pl.nch, g.mode, alpha, beta, gw, gw2, galpha,
-                                                                 gbeta, gbias);
-            g_launches += 2;
-            snprintf(g_last_kernel, sizeof(g_last_kernel), "%s", "dw_bwd");
-            return check_launch();
-        }
-    }
-    if (gx && s1) {
+    if (gx && g.R == 3 && g.S == 3 && g.dh == 1 && g.dw == 1 && g.sh == 1 && g.sw == 1) {
         // 3x3, stride 1: strips of 4 input columns x 6 input rows over a register window
         const int QPRI = (g.W + 3) / 4, strips = (g.H + 5) / 6;
         const size_t total = (size_t)g.N * g.C * strips * QPRI;
@@ -499,7 +476,7 @@ int dw_backward_t(const Geo& g, const void* x, const void* w, const void* w2, co
 #undef TCONV_DW_GX
         g_launches += 1;
     }
-    if (params) {
+    if (gw || gw2 || galpha || gbeta || gbias) {
         const int nch = dw_chunks(g);
         const dim3 grid((unsigned)g.C, (unsigned)nch);
         const size_t smem = (size_t)kDwAcc * 256 * sizeof(float);

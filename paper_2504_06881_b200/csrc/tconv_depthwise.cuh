@@ -933,208 +933,6 @@ dw_bwd_params3_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, c
     }
 }
 
-// All gradients of fp32 two-branch layers with 3x3 windows, stride 1, dilation 1 in one pass over x, grad_y and the
-// codes, each read once (two kernels read grad_y and the codes twice and rebuild the branch values from x).  CTA
-// (c, chunk) walks strips of RT input rows x 4 columns of its images.  Every (output, tap) pair is met once, at the
-// input it reads (those in the padding belong to the strips and quads at the border), and adds grad_y to that
-// input's branch sum and to the tap's histogram, both predicated on one comparison;
-// grad_alpha = sum grad_y * (x + w) at the minima = sum over inputs of x * branch sum + sum over taps of
-// w * histogram.  Output rows come in one by one, the next in flight; an input row is finished by the third.
-// Padding up to 2.  N=128 C=144 56x56 compound (520 MB of reads, 231 MB of writes: 117 us): 355 us in two kernels,
-// 308 us in this one, bound by issue: 18 comparisons and 36 predicated adds per input at 16 warps per SM.
-struct DwBwdPlan {
-    int nch, RT, strips;
-};
-inline DwBwdPlan plan_dw_bwd3(const Geo& g, int most) {
-    const long slots = 2 * 148;
-    DwBwdPlan best{1, 1, 1};
-    double best_cost = -1.0;
-    if (most > g.N) most = g.N;
-    for (int nch = most; nch >= 1 && nch >= most / 2; --nch)
-        for (int s0 = 1; s0 <= g.H; s0 *= 2) {
-            const int RT = (g.H + s0 - 1) / s0, strips = (g.H + RT - 1) / RT;
-            if (RT > 32) continue;
-            const long items = (long)((g.N + nch - 1) / nch) * strips * ((g.W + 3) / 4);
-            // rounds of 256 strips, each with the equivalent of 2.5 rows of halo; the reduction takes about 3 rows
-            const double cost = (double)(((long)g.C * nch + slots - 1) / slots) * ((double)((items + 255) / 256) * (RT + 2.5) + 3.0);
-            if (best_cost < 0.0 || cost < best_cost) {
-                best_cost = cost;
-                best = DwBwdPlan{nch, RT, strips};
-            }
-            if (RT <= 4) break;
-        }
-    return best;
-}
-
-// Where tap is the wanted one, both sums take v.  Predicated: as branches the same kernel took 773 us for 331, and
-// v * (0 or 1) would spread infinities.
-__device__ __forceinline__ void dw_add_at(unsigned tap, int want, float v, float& s0, float& s1) {
-    asm("{.reg .pred p; setp.eq.u32 p, %2, %3; @p add.f32 %0, %0, %4; @p add.f32 %1, %1, %4;}"
-        : "+f"(s0), "+f"(s1) : "r"(tap), "r"(want), "f"(v));
-}
-__device__ __forceinline__ void dw_add_at(unsigned tap, int want, float v, float& s0) {
-    asm("{.reg .pred p; setp.eq.u32 p, %1, %2; @p add.f32 %0, %0, %3;}" : "+f"(s0) : "r"(tap), "r"(want), "f"(v));
-}
-
-template <bool PAR, bool VEC>
-__global__ void __launch_bounds__(256, 2)
-dw_bwd3_kernel(Geo g, const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ w2,
-               const float* __restrict__ alpha, const float* __restrict__ beta, const float* __restrict__ gy,
-               const uint8_t* __restrict__ codes, float* __restrict__ gx, float* __restrict__ partial, DwBwdPlan pl,
-               int need_ab, int QPR) {
-    constexpr int L = 6;
-    const int c = blockIdx.x, chunk = blockIdx.y, tid = threadIdx.x;
-    const float a = alpha ? alpha[c] : 1.0f, b = beta ? beta[c] : 1.0f;
-    const int per = (g.N + pl.nch - 1) / pl.nch;
-    const int n_lo = min(g.N, chunk * per), n_hi = min(g.N, n_lo + per);
-    const unsigned sq = (unsigned)pl.strips * QPR, nitems = (unsigned)(n_hi - n_lo) * sq;
-    const size_t plane = (size_t)g.OH * g.OW;
-    float hist[2][9], sab[2] = {0.0f, 0.0f};
-#pragma unroll
-    for (int i = 0; i < 9; ++i) hist[0][i] = hist[1][i] = 0.0f;
-    for (unsigned it = tid; it < nitems; it += 256) {
-        const unsigned nl = it / sq, rem = it - nl * sq;
-        const int st = (int)(rem / (unsigned)QPR), iw0 = (int)(rem - (unsigned)st * QPR) * 4;
-        const size_t nc = (size_t)(n_lo + nl) * g.C + c;
-        const int ih0 = st * pl.RT, rows = min(pl.RT, g.H - ih0);
-        const int ob = ih0 + g.ph - 2, c0 = iw0 + g.pw - 2;     // first output row / column that reaches the strip
-        const bool left = iw0 == 0 && g.pw, right = iw0 + 4 >= g.W && g.pw, far = g.pw == 2 || g.W % 4;
-        const unsigned cmask = dw_col_mask(c0, L, g.OW), xmask = dw_col_mask(iw0, 4, g.W);
-        const bool full = xmask == 15u && (g.W & 3) == 0;
-        const float* grp = gy + nc * plane + (ptrdiff_t)ob * g.OW + c0;
-        const uint8_t* crp = codes + nc * plane + (ptrdiff_t)ob * g.OW + c0;
-        const size_t xo = (nc * g.H + ih0) * (size_t)g.W + iw0;
-        float gr[2][L], xr[4];
-        unsigned cr[2][3];                                      // codes: first column, four columns, last column
-        auto request = [&](int k, int slot) {                   // output row k of the strip
-            const bool ok = k < rows + 2 && ob + k >= 0 && ob + k < g.OH;
-            const unsigned m = ok ? cmask : 0u;
-            dw_load_row<float, L, VEC>(grp + (ptrdiff_t)k * g.OW, ok, cmask, gr[slot]);
-            const uint8_t* cp = crp + (ptrdiff_t)k * g.OW;
-            cr[slot][0] = (m & 1u) ? __ldg(cp) : 0u;
-            if constexpr (VEC) {
-                cr[slot][1] = (m & 2u) ? __ldg(reinterpret_cast<const unsigned*>(cp + 1)) : 0u;
-            } else {
-                unsigned v = 0u;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) v |= ((m >> (i + 1)) & 1u) ? (unsigned)__ldg(cp + 1 + i) << (8 * i) : 0u;
-                cr[slot][1] = v;
-            }
-            cr[slot][2] = (m & 32u) ? __ldg(cp + 5) : 0u;
-        };
-        float acc[3][2][4];
-        request(0, 0);
-        // six rows per trip: the two slots of grad_y and the three of the sums are constants
-        for (int k0 = 0; k0 < rows + 2; k0 += 6) {
-#pragma unroll
-            for (int u = 0; u < 6; ++u) {
-                const int k = k0 + u;
-                if (k >= rows + 2) break;
-                request(k + 1, (u + 1) & 1);
-                if (full && need_ab && k >= 2) {                // input row k - 2
-                    load4(x + xo + (ptrdiff_t)(k - 2) * g.W, xr);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        xr[j] = need_ab && k >= 2 && ((xmask >> j) & 1u) ? __ldg(x + xo + (ptrdiff_t)(k - 2) * g.W + j) : 0.0f;
-                }
-#pragma unroll
-                for (int v = 0; v < 2; ++v)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[u % 3][v][j] = 0.0f;
-                auto tap_of = [&](int o, int v) {
-                    const unsigned* cd = cr[u & 1];
-                    return (o == 0 ? cd[0] >> (4 * v) : o == 5 ? cd[2] >> (4 * v) : cd[1] >> (8 * (o - 1) + 4 * v)) & 15u;
-                };
-#pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    const int i = k + r - 2;                    // input row: slot (k + r - 2) % 3
-                    if ((i < 0 && ih0 > 0) || (i >= rows && ih0 + rows < g.H)) continue;   // another strip's
-#pragma unroll
-                    for (int o = 0; o < L; ++o)
-#pragma unroll
-                        for (int v = 0; v < 2; ++v)
-#pragma unroll
-                            for (int sx = 0; sx < 3; ++sx) {
-                                const int j = o + sx - 2;
-                                if (j < 0 || j > 3) continue;
-                                dw_add_at(tap_of(o, v), r * 3 + sx, gr[u & 1][o], acc[(u + r + 1) % 3][v][j], hist[v][r * 3 + sx]);
-                            }
-                    // columns in the padding: histogram only
-                    auto beyond = [&](int o, int sx) {
-#pragma unroll
-                        for (int v = 0; v < 2; ++v) dw_add_at(tap_of(o, v), r * 3 + sx, gr[u & 1][o], hist[v][r * 3 + sx]);
-                    };
-                    if (left) {
-                        beyond(1, 0);
-                        if (g.pw == 2) { beyond(0, 0); beyond(0, 1); }
-                    }
-                    if (right) {
-                        beyond(4, 2);
-                        if (far) { beyond(5, 1); beyond(5, 2); }
-                    }
-                }
-                if (k >= 2) {                                   // input row k - 2 is complete
-                    float out[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float p0 = acc[(u + 1) % 3][0][j], p1 = acc[(u + 1) % 3][1][j];
-                        out[j] = __fmaf_rn(a, p0, b * p1);
-                        // (an infinite input that wins nowhere adds nothing)
-                        sab[0] = p0 != 0.0f ? __fmaf_rn(xr[j], p0, sab[0]) : sab[0];
-                        sab[1] = p1 != 0.0f ? __fmaf_rn(xr[j], p1, sab[1]) : sab[1];
-                    }
-                    float* op = gx + xo + (ptrdiff_t)(k - 2) * g.W;
-                    if (full) {
-                        *reinterpret_cast<float4*>(op) = make_float4(out[0], out[1], out[2], out[3]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if ((xmask >> j) & 1u) op[j] = out[j];
-                    }
-                }
-            }
-        }
-    }
-    // per accumulator: a fixed tree over each warp's lanes, then the warps in order
-    __shared__ float red[8][20];
-    const int warp = tid >> 5, lane = tid & 31;
-    auto reduce = [&](float v, int slot) {
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
-        if (lane == 0) red[warp][slot] = v;
-    };
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-#pragma unroll
-        for (int i = 0; i < 9; ++i) reduce(hist[v][i], v * 9 + i);
-        reduce(sab[v], 18 + v);
-    }
-    __syncthreads();
-    if (tid < 20) {
-        float v = 0.0f;
-        for (int e = 0; e < 8; ++e) v += red[e][tid];
-        red[0][tid] = v;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        const float* wmax = (PAR ? w2 : w) + (size_t)c * 9;
-        float* out = partial + ((size_t)chunk * g.C + c) * kDwAcc;
-        float A = red[0][18], B = red[0][19], total = 0.0f;
-        for (int i = 0; i < 9; ++i) {
-            const float h0 = red[0][i], h1 = red[0][9 + i];
-            out[i] = h0;
-            out[16 + i] = h1;
-            A = __fmaf_rn(__ldg(w + (size_t)c * 9 + i), h0, A);
-            B = __fmaf_rn(__ldg(wmax + i), h1, B);
-            total += h0;
-        }
-        out[32] = A;
-        out[33] = B;
-        out[34] = total;
-    }
-}
-
 // One thread per (c, accumulator): sums the chunk partials in order and writes the gradients.
 __global__ void dw_bwd_finish_kernel(Geo g, const float* __restrict__ partial, int nchunks, int mode,
                                      const float* __restrict__ alpha, const float* __restrict__ beta,

@@ -140,3 +140,52 @@ def test_volume_masked_taps(dtype):
     for i, d in enumerate(VOLUMES):
         d = dict(d, mode="parallel", dtype=dtype)
         check_volume(d, masked(inputs.draw3d(d, 4700 + i)))
+
+
+def depthwise(d, t):
+    """Gradients of a depthwise layer and the oracle's."""
+    dt, par = tconv.TORCH_DTYPE[d["dtype"]], d["mode"] == "parallel"
+    dev = {k: torch.from_numpy(v).cuda().to(dt if k in ("x", "w", "w2", "g") else torch.float32) for k, v in t.items()}
+    w2 = dev["w2"] if par else None
+    _, win = tconv.dw_forward(d, dev["x"], dev["w"], w2, dev["alpha"], dev["beta"], None, want_winners=True)
+    got = tconv.dw_backward(d, dev["x"], dev["w"], dev["g"], w2, dev["alpha"], dev["beta"], win)
+    return got, ora.depthwise_backward(d, t["x"], t["w"], t["g"], t["w2"] if par else None, t["alpha"], t["beta"])
+
+
+DEPTHWISE = [L(3, 4, 12, 12, 4, pad=1), L(2, 3, 37, 9, 3, pad=1), L(5, 2, 33, 46, 2, pad=(2, 1)), L(3, 2, 14, 13, 2, stride=2)]
+
+
+def draw_depthwise(d, seed, x=("normal", 0.0, 1.0), w=("normal", 0.0, 0.3)):
+    t = inputs.draw(dict(d, C=1, K=d["C"]), seed, x=x, w=w)          # weights [C][1][R][S], one alpha and beta per channel
+    t["x"], t["g"] = (inputs.draw(dict(d, K=d["C"]), seed, x=x)[k] for k in ("x", "g"))
+    t["w"], t["w2"] = (np.ascontiguousarray(t[k][:, 0]) for k in ("w", "w2"))
+    t["alpha"], t["beta"] = (np.ascontiguousarray(t[k][:, 0]) for k in ("alpha", "beta"))
+    return t
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("mode", ["compound", "parallel"])
+def test_depthwise(mode, dtype):
+    for i, d in enumerate(DEPTHWISE):
+        d = dict(d, mode=mode, dtype=dtype)
+        got, ref = depthwise(d, draw_depthwise(d, 4800 + i))
+        parity.compare_grads(d, {k: got[k] for k in PARAMS if k in got}, ref, rtol=RTOL)
+
+
+@pytest.mark.parametrize("mode", ["compound", "parallel"])
+def test_depthwise_offset_inputs(mode):
+    for i, d in enumerate(DEPTHWISE):
+        d = dict(d, mode=mode, pad_h=0, pad_w=0)
+        got, ref = depthwise(d, draw_depthwise(d, 4900 + i, x=("normal", 4096.0, 1.0), w=("normal", -4096.0, 1.0)))
+        parity.compare_grads(d, {k: got[k] for k in PARAMS if k in got}, ref, rtol=RTOL)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_depthwise_masked_taps(dtype):
+    for i, d in enumerate(DEPTHWISE):
+        d = dict(d, mode="parallel", dtype=dtype)
+        t = draw_depthwise(d, 5000 + i)
+        for name, v in (("w", np.inf), ("w2", -np.inf)):
+            t[name].reshape(-1, 9)[:, [0, 2, 6, 8] if name == "w" else [1, 3, 5, 7]] = v
+        got, ref = depthwise(d, t)
+        parity.compare_grads(d, {k: got[k] for k in PARAMS}, ref, rtol=RTOL)
