@@ -1,4 +1,6 @@
 // Launches of the Sum-form backward kernels (tconv_bwd_sum.cuh).
+#include <algorithm>
+
 #include "tconv_bwd_sum.cuh"
 
 namespace tconv {
@@ -57,7 +59,8 @@ int launch_all(SumBwdArgs& a) {
     else if (a.gx) rc = br == 0 ? launch_gx_window<T, 0, true, false>(a, xp, part_ab, part_gx)
                         : br == 1 ? launch_gx_window<T, 1, true, false>(a, xp, part_ab, part_gx) : launch_gx_window<T, 2, true, false>(a, xp, part_ab, part_gx);
     if (rc == TCONV_OK && a.gx && xp.nrow * xp.ncol > 1) {
-        bwd_sum_edges_kernel<T><<<dim3((unsigned)(g.N * g.C), (unsigned)(((g.H + 3) / 4 * ((g.W + 31) / 32) + 7) / 8)), 256, 0, a.st>>>(g, part_gx, (T*)a.gx, xp);
+        const unsigned tasks = (unsigned)((g.H + 3) / 4) * (unsigned)((g.W + 31) / 32);
+        bwd_sum_edges_kernel<T><<<dim3((unsigned)(g.N * g.C), std::min((tasks + 7) / 8, 65535u)), 256, 0, a.st>>>(g, part_gx, (T*)a.gx, xp);
         ++a.launches;
     }
     if (rc != TCONV_OK || !params) return rc;

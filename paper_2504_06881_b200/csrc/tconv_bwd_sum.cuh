@@ -586,7 +586,7 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
 }
 
 // grad_x of an image cut into tiles: every input element adds the regions that cover it, tile rows and
-// columns ascending.  grid (N * C, eight warps' tasks each).
+// columns ascending.  grid (N * C, eight warps' tasks each; tall maps have more than the 65535 blocks of that axis).
 // A warp takes four rows of 32 columns: the tiles that reach a column (two divisions) once for the four rows, the
 // sums' loads together.  N=19 C=75 118x93 bf16 (85 MB) took 122 us with one thread and four divisions per element.
 template <typename T>
@@ -594,43 +594,45 @@ __global__ void __launch_bounds__(256)
 bwd_sum_edges_kernel(Geo g, const float* __restrict__ part_gx, T* __restrict__ gx, SumGxPlan pl) {
     constexpr int RPT = 4;
     const unsigned chunks = ((unsigned)g.W + 31) / 32;
-    const unsigned task = blockIdx.y * 8 + (threadIdx.x >> 5), rg = task / chunks;
-    const unsigned xi = (task - rg * chunks) * 32 + (threadIdx.x & 31), y0 = rg * RPT;
-    if (y0 >= (unsigned)g.H || xi >= (unsigned)g.W) return;
     const unsigned n = blockIdx.x / (unsigned)g.C, c = blockIdx.x - n * (unsigned)g.C;
     const unsigned sr = pl.TR * g.sh, sc = pl.TQ * 4 * g.sw;     // input distance between two tiles
     const unsigned ER = pl.ER, EC = pl.EC, area = ER * EC;
-    const unsigned x = xi + g.pw;
-    const unsigned c1 = min((unsigned)pl.ncol - 1, x / sc);
-    unsigned c0 = c1;
-    while (c0 > 0 && x - (c0 - 1) * sc < EC) --c0;
-    const bool covered = x - c1 * sc < EC;
-    const float* base = part_gx + ((size_t)n * pl.nrow * pl.ncol * g.C + c) * area;
-    const size_t tile = (size_t)g.C * area;
-    T* out = gx + ((size_t)blockIdx.x * g.H + y0) * g.W + xi;
-    // the last tile that covers each element first, all rows together; then the others, ascending
-    unsigned r0[RPT], r1[RPT], at = min((unsigned)pl.nrow - 1, (y0 + g.ph) / sr);
-    float sum[RPT];
+    for (unsigned task = blockIdx.y * 8 + (threadIdx.x >> 5);; task += gridDim.y * 8) {
+        const unsigned rg = task / chunks, xi = (task - rg * chunks) * 32 + (threadIdx.x & 31), y0 = rg * RPT;
+        if (y0 >= (unsigned)g.H) break;
+        if (xi >= (unsigned)g.W) continue;
+        const unsigned x = xi + g.pw;
+        const unsigned c1 = min((unsigned)pl.ncol - 1, x / sc);
+        unsigned c0 = c1;
+        while (c0 > 0 && x - (c0 - 1) * sc < EC) --c0;
+        const bool covered = x - c1 * sc < EC;
+        const float* base = part_gx + ((size_t)n * pl.nrow * pl.ncol * g.C + c) * area;
+        const size_t tile = (size_t)g.C * area;
+        T* out = gx + ((size_t)blockIdx.x * g.H + y0) * g.W + xi;
+        // the last tile that covers each element first, all rows together; then the others, ascending
+        unsigned r0[RPT], r1[RPT], at = min((unsigned)pl.nrow - 1, (y0 + g.ph) / sr);
+        float sum[RPT];
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-        const unsigned y = y0 + i + g.ph;
-        while (at + 1 < (unsigned)pl.nrow && (at + 1) * sr <= y) ++at;
-        r1[i] = r0[i] = at;
-        while (r0[i] > 0 && y - (r0[i] - 1) * sr < ER) --r0[i];
-        sum[i] = y - at * sr < ER && covered ? __ldg(base + (r1[i] * pl.ncol + c1) * tile + (y - r1[i] * sr) * EC + (x - c1 * sc)) : 0.0f;
-    }
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-        const unsigned y = y0 + i + g.ph;
-        if (r0[i] == r1[i] && c0 == c1) {
-            if (y0 + i < (unsigned)g.H) out[(size_t)i * g.W] = from_f32<T>(sum[i]);
-            continue;
+        for (int i = 0; i < RPT; ++i) {
+            const unsigned y = y0 + i + g.ph;
+            while (at + 1 < (unsigned)pl.nrow && (at + 1) * sr <= y) ++at;
+            r1[i] = r0[i] = at;
+            while (r0[i] > 0 && y - (r0[i] - 1) * sr < ER) --r0[i];
+            sum[i] = y - at * sr < ER && covered ? __ldg(base + (r1[i] * pl.ncol + c1) * tile + (y - r1[i] * sr) * EC + (x - c1 * sc)) : 0.0f;
         }
-        for (unsigned r = r0[i]; r <= r1[i]; ++r)
-            for (unsigned q = c0; q <= c1; ++q)
-                if ((r != r1[i] || q != c1) && y - r * sr < ER && x - q * sc < EC)
-                    sum[i] += __ldg(base + (r * pl.ncol + q) * tile + (y - r * sr) * EC + (x - q * sc));
-        if (y0 + i < (unsigned)g.H) out[(size_t)i * g.W] = from_f32<T>(sum[i]);
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const unsigned y = y0 + i + g.ph;
+            if (r0[i] == r1[i] && c0 == c1) {
+                if (y0 + i < (unsigned)g.H) out[(size_t)i * g.W] = from_f32<T>(sum[i]);
+                continue;
+            }
+            for (unsigned r = r0[i]; r <= r1[i]; ++r)
+                for (unsigned q = c0; q <= c1; ++q)
+                    if ((r != r1[i] || q != c1) && y - r * sr < ER && x - q * sc < EC)
+                        sum[i] += __ldg(base + (r * pl.ncol + q) * tile + (y - r * sr) * EC + (x - q * sc));
+            if (y0 + i < (unsigned)g.H) out[(size_t)i * g.W] = from_f32<T>(sum[i]);
+        }
     }
 }
 

@@ -47,3 +47,9 @@ def test_single_gradients(need):
     assert set(part) == set(need)
     for k in need:
         assert (part[k] == full[k]).all(), k
+
+
+def test_more_rows_than_blocks_of_one_grid_axis():
+    d = L(1, 1, 2_100_000, 4, 1, pad=1, mode="compound")
+    parity.check_layer(d, None, 1760, recompute=False)
+    assert tconv.tconv_last_kernel() == "bwd_sum"
