@@ -19,9 +19,10 @@ int launch_gx(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx
 template <typename T, int BR, bool GX, bool AB>
 int launch_gx_window(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* part_gx) {
     const Geo& g = a.g;
-    if (g.wide) return g.R == 5 && g.S == 5 ? launch_gx<T, BR, GX, AB, true, 5, true>(a, pl, part_ab, part_gx)
-                                            : launch_gx<T, BR, GX, AB, true, 0, true>(a, pl, part_ab, part_gx);
-    if (g.R != 3 || g.S != 3) return launch_gx<T, BR, GX, AB, false, 0, true>(a, pl, part_ab, part_gx);
+    const bool far = sum_far(g);
+    if (g.wide) return g.R == 5 && g.S == 5 && !far ? launch_gx<T, BR, GX, AB, true, 5, true>(a, pl, part_ab, part_gx)
+                                                    : launch_gx<T, BR, GX, AB, true, 0, true>(a, pl, part_ab, part_gx);
+    if (g.R != 3 || g.S != 3 || far) return launch_gx<T, BR, GX, AB, false, 0, true>(a, pl, part_ab, part_gx);
     return g.K % kSgKB ? launch_gx<T, BR, GX, AB, false, 3, true>(a, pl, part_ab, part_gx)
                        : launch_gx<T, BR, GX, AB, false, 3, false>(a, pl, part_ab, part_gx);
 }

@@ -19,6 +19,7 @@
 // No atomics; every accumulator has one writer and a fixed order.
 #pragma once
 #include <cstring>
+#include <type_traits>
 
 #include "tconv_bwd.cuh"
 
@@ -167,9 +168,9 @@ inline const SumPlans& sum_plans(const Geo& g, int esize) {
     SumPlans& p = kept[next];
     p.g = g;
     p.esize = esize;
-    p.ok = (double)g.N * g.OH * g.OWP < 2.0e9 && (double)g.H * g.W < 1.6e7 && (double)g.N * g.C < 2.0e9 && (double)g.OH * g.OWP * g.K < 1.0e9 &&
-           (double)g.OH * g.OWP * g.K * g.C < 1.6e10 && plan_sum_gx(g, &p.gx) &&
-           plan_sum_gw(g, &p.gw);
+    // 31-bit counts: quads of all images (a share's last round may end past them), positions of a map, images x channels
+    p.ok = (double)g.N * g.OH * g.OWP < 8.0e9 && (double)g.OH * g.OWP < 2.1e9 && (double)g.H * g.W < 2.1e9 &&
+           (double)g.N * g.C < 2.0e9 && plan_sum_gx(g, &p.gx) && plan_sum_gw(g, &p.gw);
     next = (next + 1) % kKept;
     if (used < kKept) ++used;
     return p;
@@ -183,6 +184,10 @@ inline size_t sum_part_ab_bytes(const Geo& g, const SumGxPlan& p) {
 }
 inline size_t sum_part_gx_bytes(const Geo& g, const SumGxPlan& p) {
     return p.nrow * p.ncol > 1 ? ((size_t)p.ctas * g.C * p.ER * p.EC * sizeof(float) + 255) / 256 * 256 : 0;
+}
+// Images of 2^32 gradients or of 2^32 quads of winners and more.
+inline bool sum_far(const Geo& g) {
+    return (double)g.OH * g.OW * g.K > 4.2e9 || (double)g.OH * g.OW * g.K * g.C > 1.6e10;
 }
 // Bytes of all partial sums; 0 when the layer does not fit the kernels.  g: widened to whole quads.
 inline size_t sum_ws_bytes(const Geo& g, int esize) {
@@ -311,7 +316,8 @@ __device__ __forceinline__ void branch_values(const float* x, const float* w, fl
 }
 
 // BR: 0 both branches, 1 min branch only, 2 max branch only.  GX: grad_x.  AB: grad_alpha / grad_beta (BR 0).
-// KW: 3 or 5 for 3 x 3 (narrow codes) and 5 x 5 windows (wide codes), else 0 (any window).
+// KW: 3 or 5 for 3 x 3 (narrow codes) and 5 x 5 windows (wide codes), else 0 (any window, and images whose
+// gradients or winners exceed 32-bit counts: sum_far).
 // Shared memory: accumulators [4][tap][TP] floats per TP threads, then (AB) the window inputs in the same
 // layout, at the end two stages of eight output channels' coefficients and (AB) weights; TP is 256 for 3 x 3 windows (and the taps of a column lie 1024 bytes apart), 64 otherwise (256
 // bytes apart): one PRMT and one add address an accumulator, and the winner's input lies at a constant
@@ -344,12 +350,16 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
     const int oh0 = rt * pl.TR, oq0 = ct * pl.TQ;
     const int tr = min(pl.TR, g.OH - oh0), tq = min(pl.TQ, (g.OW >> 2) - oq0);   // output rows, quads per row
     const int NQ1 = tr * tq, NQ = NQ1 * nimg;
-    const unsigned plane = (unsigned)g.OH * (unsigned)g.OW;    // (below 2^30 with all K channels)
+    const unsigned plane = (unsigned)g.OH * (unsigned)g.OW;
     constexpr int CW = WIDE ? 2 : 1;                           // bytes per code
-    // addresses: a base of the CTA plus a 32-bit count of the thread, elements of grad_y and quads of codes
+    constexpr bool FAR = KW == 0;
+    // addresses: a base of the CTA plus a 32-bit count of the thread, elements of grad_y and quads of codes.  FAR: the
+    // output channels advance the base, the count is that of the image and pixel (several images only of maps of at
+    // most 256 quads); as 64-bit sums they cost 3 x 3 layers 3 %
     const T* gbase = gy + (size_t)n_first * g.K * plane;
     const uint8_t* cbase = codes + ((size_t)n_first * g.K * g.C + c) * plane * CW;
-    const unsigned cstep = (unsigned)g.C * (plane >> 2);       // quads of codes between two output channels
+    using Count = std::conditional_t<FAR, size_t, unsigned>;
+    const Count cstep = (Count)g.C * (plane >> 2);             // quads of codes between two output channels
     {
         // a thread without a quad repeats the last one into columns nobody reads
         const bool live = tid < NQ;
@@ -358,7 +368,7 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
         const int oh = oh0 + orow, ow0 = (oq0 + q1 - orow * tq) * 4;
         const unsigned pix = (unsigned)(oh * g.OW + ow0);
         unsigned goff = (unsigned)(il * g.K) * plane + pix;
-        unsigned coff = (unsigned)(il * g.K) * cstep + (pix >> 2);
+        unsigned coff = (unsigned)(il * g.K) * (unsigned)cstep + (pix >> 2);
         char* Ab = smem + (size_t)(tid / TP) * gbytes + (tid % TP) * 4;
 
         // gradients and codes of a pair of output channels are requested together, one pair ahead: the loads
@@ -377,7 +387,10 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
         auto request = [&](int u) {
             if (!AB || live) ahead_g4<T, false>(gbase + goff, raw[u]);
             cq[u] = ahead_codes4<WIDE, false>(cbase + (size_t)coff * (4 * CW));
-            if (more > 0) { goff += plane; coff += cstep; }
+            if (more > 0) {
+                if constexpr (FAR) { gbase += plane; cbase += cstep * (4 * CW); }
+                else { goff += plane; coff += cstep; }
+            }
             --more;
         };
         request(0);
