@@ -12,8 +12,8 @@
 //   bwd_idx_gw_finish_kernel  sums the ranges' histograms in a fixed order.
 //
 // Measured at N=128 C=64 K=64 32x32 3x3 fp32 (67 MB of winners and gradients, 10 us at the copy rate):
-// grad_x 133 -> 84 us, bound by the latency of its chain (classes x K / 4 steps of some 250 cycles of dependent
-// shared-memory accesses) at the six warps per SM that the tile leaves; grad_w 93 -> 23 us, memory traffic.
+// grad_x 133 -> 80 us, bound by the latency of its chain (row classes x K / 4 steps of some 800 cycles: addresses,
+// then three column classes of dependent shared-memory accesses) at the few warps per SM that the tile leaves; grad_w 93 -> 23 us, memory traffic.
 // One row of 10303 samples, 53 channels: 825 -> 22 us (column tiles instead of one warp along the row).
 #pragma once
 #include "tconv_common.cuh"
@@ -52,10 +52,14 @@ __host__ __device__ inline int idx_class_count(int n, int gd, int m, int cls) {
     return n / period * gd + (rest < 0 ? 0 : rest < gd ? rest : gd);
 }
 
-// Tile (rows, columns, channel block) with the shortest estimated time.  A CTA's rows of one class run on a warp
-// each, its classes and the columns of a row one after another, about 100 cycles of dependent shared-memory
-// accesses per (channel class step, 4 output channels) of which 45 are issue slots: a tile costs classes x column
-// chunks, resident warps beyond about two per scheduler queue up.
+// Tile (rows, columns, channel block) and threads with the shortest estimated time, in cycles.  A CTA's rows of one
+// class run on a warp each, its classes and the columns of a row one after another; a step of four output channels
+// takes 460 cycles + 115 per column class, or, with more warps on an SM than that hides, their 14 + 31 issue slots
+// each.  Clearing and storing the tile: 244 cycles per element of a thread, more where 16 warps share an SM.  Fitted
+// to 3600 launches of 21 layers (the choice is 8 % off the best on average, 39 % at worst).  Residency counts the
+// registers as well: without them N=64 C=512 K=512 12x12 fp32 ran in three rounds of two CTAs per SM instead of one
+// of two (549 against 187 us).
+constexpr int kIdxGxRegs = 112;          // per thread, as allocated (107 used)
 inline bool plan_idx_gx(const Geo& g, IdxGxPlan* best) {
     if ((double)g.K * g.OH * g.OW > 2.0e9 || (double)g.N * g.H > 2.0e9) return false;
     int gdh, mr, gdw, mc;
@@ -63,47 +67,50 @@ inline bool plan_idx_gx(const Geo& g, IdxGxPlan* best) {
     idx_classes(g.S, g.dw, g.sw, &gdw, &mc);
     double best_cost = -1.0;
     const int halo_h = (g.R - 1) * g.dh, halo_w = (g.S - 1) * g.dw;
-    for (int nblk = 1; nblk <= 64 && nblk <= g.C; ++nblk) {
+    const double step = 460.0 + 115.0 * mc, slots = 14.0 + 31.0 * mc, k4 = (g.K + 3) / 4;
+    for (const int nblk : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64}) {
+        if (nblk > g.C) break;
         IdxGxPlan p;
         p.gdh = gdh; p.mr = mr; p.gdw = gdw; p.mc = mc;
         p.CB = (g.C + nblk - 1) / nblk;
         p.nblk = (g.C + p.CB - 1) / p.CB;
-        if (p.nblk != nblk) continue;
         for (int tw0 = g.W; ; tw0 = (tw0 + 1) / 2) {
             p.ncol = (g.W + tw0 - 1) / tw0;
             p.TW = (g.W + p.ncol - 1) / p.ncol;
             const size_t row = (size_t)p.CB * p.TW * sizeof(float);
             int cols = (p.TW + halo_w - 1) / g.sw + 1;               // outputs that reach a tile's columns
             if (cols > g.OW) cols = g.OW;
-            for (int per_sm = 12; per_sm >= 1; per_sm = per_sm > 6 ? 6 : per_sm - 1) {
-                size_t budget = (size_t)(220 * 1024) / per_sm - 2560;
-                if (budget > kIdxSmemMost - 2048) budget = kIdxSmemMost - 2048;
-                int th = (int)(budget / row);
-                if (th < 1) continue;
-                if (th > g.H) th = g.H;
-                const int bands = (g.H + th - 1) / th;
-                p.TH = (g.H + bands - 1) / bands;
+            for (int b = 1; ; b = b < 4 ? b + 1 : b + b / 2) {
+                if (b > g.H) b = g.H;
+                p.TH = (g.H + b - 1) / b;
                 p.bands = (g.H + p.TH - 1) / p.TH;
+                p.smem = row * p.TH + 256 * sizeof(float);
                 const double ctas = (double)g.N * p.bands * p.ncol * p.nblk;
-                if (ctas > 2.0e9) continue;
-                int rows = (p.TH + halo_h - 1) / g.sh + 1;
-                if (rows > g.OH) rows = g.OH;
-                int tasks = idx_class_count(rows, gdh, mr, 0);
-                if (cols <= 32) tasks = (tasks + 32 / cols - 1) / (32 / cols);
-                const int warps = tasks < 1 ? 1 : tasks > 8 ? 8 : tasks;
-                const double resident = ctas < 148.0 * per_sm ? ctas / 148.0 : per_sm;
-                const double load = 0.45 * resident * warps / 4.0;
-                const double rounds = (double)(long)((ctas + 148.0 * per_sm - 1) / (148.0 * per_sm));
-                const double cost = rounds * ((tasks + warps - 1) / warps) * ((cols + 31) / 32) * (load > 1.0 ? load : 1.0);
-                if (best_cost < 0.0 || cost < 0.97 * best_cost) {
-                    best_cost = cost;
-                    p.smem = row * p.TH + 256 * sizeof(float);
-                    // (a tile of many channels: more warps to clear and store it)
-                    const size_t fill = row * p.TH / 4096;
-                    p.threads = 32 * (fill > 8 ? 8 : (int)fill > warps ? (int)fill : warps);
-                    p.grid = (unsigned)ctas;
-                    *best = p;
+                if (p.smem <= kIdxSmemMost && ctas <= 2.0e9) {
+                    int rows = (p.TH + halo_h - 1) / g.sh + 1;
+                    if (rows > g.OH) rows = g.OH;
+                    int tasks = idx_class_count(rows, gdh, mr, 0);
+                    if (cols <= 32) tasks = (tasks + 32 / cols - 1) / (32 / cols);
+                    const int warps = tasks < 1 ? 1 : tasks > 8 ? 8 : tasks;
+                    for (const int nw : {warps, 8}) {                // (eight: to clear and store the tile)
+                        long per_sm = (long)(228 * 1024 / (p.smem + 1024));
+                        if (per_sm > 65536 / (kIdxGxRegs * 32 * nw)) per_sm = 65536 / (kIdxGxRegs * 32 * nw);
+                        const double rounds = (double)(long)((ctas + 148.0 * per_sm - 1) / (148.0 * per_sm));
+                        double resident = (double)(long)((ctas + 147.0) / 148.0);
+                        if (resident > per_sm) resident = per_sm;
+                        const double issue = resident * warps * slots, crowd = resident * nw / 16.0;
+                        const double chain = (double)mr * ((tasks + warps - 1) / warps) * ((cols + 31) / 32) * k4;
+                        const double cost = rounds * (chain * (issue > step ? issue : step) +
+                                                      244.0 * row / 4 * p.TH / (32 * nw) * (crowd > 1.0 ? crowd : 1.0));
+                        if (best_cost < 0.0 || cost < best_cost) {
+                            best_cost = cost;
+                            p.threads = 32 * nw;
+                            p.grid = (unsigned)ctas;
+                            *best = p;
+                        }
+                    }
                 }
+                if (b == g.H) break;
             }
             if (tw0 <= 32) break;
         }
@@ -195,8 +202,7 @@ bwd_idx_gx_kernel(Geo g, const T* __restrict__ gy, const int32_t* __restrict__ i
                 const int cbase = ow * g.sw - g.pw - iw0;
                 const int ccls = live ? (ow / pl.gdw) % pl.mc : -1;
                 unsigned off = live ? (unsigned)(oh * g.OW + ow) : 0u;
-                // winners and gradients of four output channels at a time, the next twelve in flight (a step takes
-                // some 300 cycles, a load two to three times that)
+                // winners and gradients of four output channels at a time, the next twelve in flight
                 constexpr int U = 4, B = 4;
                 int32_t id[B][U];
                 float gv[B][U];
