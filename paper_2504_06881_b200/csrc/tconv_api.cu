@@ -264,7 +264,8 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
             auto kern = pw.vec == 4 ? bwd_idx_gw_kernel<T, 4> : bwd_idx_gw_kernel<T, 1>;
             if (allow_smem(kern, (int)kIdxSmemMost) != cudaSuccess) return cuda_fail(cudaGetLastError());
             kern<<<dim3((unsigned)(pw.nkg * pw.nblk), (unsigned)pw.chunks), 32, pw.smem, st>>>(g, (const T*)gy, idx, part, part_b, pw);
-            bwd_idx_gw_finish_kernel<<<dim3((unsigned)(((size_t)g.C * g.RS + 3) / 4 + 1), (unsigned)pw.nkg), dim3(32, 4, 8), 0, st>>>(
+            const unsigned slices = pw.chunks >= 8 ? 8 : pw.chunks >= 4 ? 4 : pw.chunks >= 2 ? 2 : 1;
+            bwd_idx_gw_finish_kernel<<<dim3((unsigned)(((size_t)g.C * g.RS + 3) / 4 + 1), (unsigned)pw.nkg), dim3(32, 4, slices), 0, st>>>(
                 g, pw, part, part_b, gw, gbias);
             g_launches += 2;
             bias_done = true;
