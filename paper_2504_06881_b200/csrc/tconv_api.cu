@@ -242,8 +242,9 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
     if (g.chan != CH_SUM) {
         const int32_t* idx = (const int32_t*)winners;
         if (gx) {
-            IdxGxPlan pl;
-            if (tiled && plan_idx_gx(g, &pl)) {
+            const IdxGxPlan* kept = tiled ? idx_gx_plan(g) : nullptr;
+            if (kept) {
+                const IdxGxPlan& pl = *kept;
                 auto kern = bwd_idx_gx_kernel<T>;
                 if (allow_smem(kern, (int)kIdxSmemMost) != cudaSuccess) return cuda_fail(cudaGetLastError());
                 kern<<<pl.grid, pl.threads, pl.smem, st>>>(g, (const T*)gy, idx, (T*)gx, pl,

@@ -16,6 +16,8 @@
 // then three column classes of dependent shared-memory accesses) at the few warps per SM that the tile leaves; grad_w 93 -> 23 us, memory traffic.
 // One row of 10303 samples, 53 channels: 825 -> 22 us (column tiles instead of one warp along the row).
 #pragma once
+#include <cstring>
+
 #include "tconv_common.cuh"
 
 namespace tconv {
@@ -116,6 +118,23 @@ inline bool plan_idx_gx(const Geo& g, IdxGxPlan* best) {
         }
     }
     return best_cost >= 0.0;
+}
+
+// The plan of a layer, or null.  The search is some microseconds of host work, so the last few are kept per host
+// thread (they depend on nothing but the geometry).
+inline const IdxGxPlan* idx_gx_plan(const Geo& g) {
+    constexpr int kKept = 16;
+    struct Entry { Geo g; IdxGxPlan plan; bool ok; };
+    static thread_local Entry kept[kKept];
+    static thread_local int used = 0, next = 0;
+    for (int i = 0; i < used; ++i)
+        if (memcmp(&kept[i].g, &g, sizeof(Geo)) == 0) return kept[i].ok ? &kept[i].plan : nullptr;
+    Entry& e = kept[next];
+    e.g = g;
+    e.ok = plan_idx_gx(g, &e.plan);
+    next = (next + 1) % kKept;
+    if (used < kKept) ++used;
+    return e.ok ? &e.plan : nullptr;
 }
 
 // One stage of the pixel ring: 32 lanes' winners and gradients of 32 pixels, rows padded against bank conflicts.
