@@ -452,19 +452,20 @@ bwd3d_params_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __rest
         }
     }
     __syncthreads();
-    const int total = g.N * g.vol, per = (total + nsplit - 1) / nsplit;
-    const int j0 = min(total, split * per), j1 = min(total, j0 + per);
+    // (unsigned: up to 2^31 - 1 items, and a round may end past them)
+    const unsigned total = (unsigned)(g.N * g.vol), per = (total + nsplit - 1) / nsplit;
+    const unsigned j0 = min(total, split * per), j1 = min(total, j0 + per);
     float sa = 0.0f, sb = 0.0f, sg = 0.0f;
     constexpr int U = 4;          // items whose loads go out together
-    for (int jb = j0 + tid; jb < j1; jb += U * tb) {
+    for (unsigned jb = j0 + tid; jb < j1; jb += U * tb) {
         unsigned raw[U];
         float gv[U];
         int n[U], pos[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int j = jb + u * tb, jj = j < j1 ? j : jb;
-            n[u] = (int)((unsigned)jj / (unsigned)g.vol);
-            pos[u] = jj - n[u] * g.vol;
+            const unsigned j = jb + u * tb, jj = j < j1 ? j : jb;
+            n[u] = (int)(jj / (unsigned)g.vol);
+            pos[u] = (int)(jj - (unsigned)n[u] * (unsigned)g.vol);
             const int row = n[u] * g.K + k;
             raw[u] = codes ? (unsigned)__ldg((const uint16_t*)winners + ((row * g.C + c) * g.vol + pos[u]))
                            : (unsigned)__ldg((const int32_t*)winners + (row * g.vol + pos[u]));
