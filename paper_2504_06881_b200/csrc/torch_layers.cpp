@@ -10,6 +10,7 @@
 #include <array>
 #include <optional>
 #include <string>
+#include <vector>
 
 #include "tconv.h"
 #include "tconv3d.h"
@@ -88,6 +89,13 @@ void check(const Tensor& t, at::IntArrayRef shape, const char* name) {
     TORCH_CHECK_VALUE(t.is_cuda() && t.sizes() == shape, name, ": need a contiguous CUDA tensor of shape ", shape, ", got ",
                       t.sizes(), " on ", t.device());
 }
+// A tensor of the backward: saved-tensor hooks may hand back another one than the forward kept.
+void check_saved(const Tensor& t, const at::Device& dev, at::ScalarType type, at::IntArrayRef shape, const char* name) {
+    if (!t.defined()) return;
+    TORCH_CHECK_VALUE(t.is_cuda() && t.device() == dev && t.scalar_type() == type && t.is_contiguous() && t.sizes() == shape, name,
+                      ": need the contiguous ", type, " tensor of shape ", shape, " on ", dev, " that the forward saved, got ",
+                      t.scalar_type(), " ", t.sizes(), " on ", t.device());
+}
 void* ptr(const Tensor& t) { return t.defined() ? t.data_ptr() : nullptr; }
 float* fptr(const Tensor& t) { return t.defined() ? t.data_ptr<float>() : nullptr; }
 void* stream() { return (void*)at::cuda::getCurrentCUDAStream().stream(); }
@@ -150,19 +158,39 @@ struct Grads {
 };
 
 Grads run_backward(const Geom& g, const Saved& s, const Tensor& gy_in, bool need_x) {
-    c10::cuda::CUDAGuard guard(s.x.device());
+    const at::Device dev = s.x.device();
+    const auto dt = type_of(g);
+    const int wd = g.kind == kVolume ? 5 : g.kind == kDense ? 4 : 3;
+    TORCH_CHECK_VALUE(dev.is_cuda(), "x: need the CUDA tensor that the forward saved, got one on ", dev);
+    TORCH_CHECK_VALUE(s.w.dim() == wd, "w: need the tensor of ", wd, " dimensions that the forward saved, got ", s.w.dim());
+    c10::cuda::CUDAGuard guard(dev);
     const Desc d = make_desc(g, s.x, s.w);
-    const Tensor gy = as(gy_in, type_of(g));
-    check(gy, d.out(), "grad_y");
+    const Tensor gy = as(gy_in, dt);
+    check_saved(gy, dev, dt, d.out(), "grad_y");
     const bool two = g.mode == TCONV_COMPOUND || g.mode == TCONV_PARALLEL, par = g.mode == TCONV_PARALLEL;
     const auto opt = s.x.options(), f32 = opt.dtype(at::kFloat);
     const int64_t K = d.y[1], C = s.x.size(1);
+    const int64_t kc[2] = {K, C};
+    const at::IntArrayRef scalars = g.kind == kDepthwise ? at::IntArrayRef(kc, 1) : at::IntArrayRef(kc, 2);
+    {
+        std::vector<int64_t> ws = s.w.sizes().vec();
+        ws[0] = K;
+        if (g.kind != kDepthwise) ws[1] = C;
+        const int64_t wb[1] = {(int64_t)(g.kind == kVolume      ? tconv3d_winner_bytes(&d.d3)
+                                         : g.kind == kDepthwise ? tconv_dw_winner_bytes(&d.d2)
+                                                                : tconv_winner_bytes(&d.d2))};
+        check_saved(s.x, dev, dt, s.x.sizes(), "x");
+        check_saved(s.w, dev, dt, ws, "w");
+        check_saved(s.w2, dev, dt, ws, "w2");
+        check_saved(s.alpha, dev, at::kFloat, scalars, "alpha");
+        check_saved(s.beta, dev, at::kFloat, scalars, "beta");
+        TORCH_CHECK_VALUE(s.winners.defined(), "winners: need the tensor that the forward saved");
+        check_saved(s.winners, dev, at::kByte, wb, "winners");
+    }
     Grads r;
     if (need_x || g.kind == kDepthwise) r.x = at::empty(s.x.sizes(), opt);
     r.w = at::empty(s.w.sizes(), f32);
     if (par) r.w2 = at::empty(s.w.sizes(), f32);
-    const int64_t kc[2] = {K, C};
-    const at::IntArrayRef scalars = g.kind == kDepthwise ? at::IntArrayRef(kc, 1) : at::IntArrayRef(kc, 2);
     if (two) {
         r.alpha = at::empty(scalars, f32);
         r.beta = at::empty(scalars, f32);
