@@ -261,6 +261,9 @@ public:
 Tensor layer(const Geom& g, const Tensor& x, const Tensor& w, const std::optional<Tensor>& w2_, const std::optional<Tensor>& alpha_,
              const std::optional<Tensor>& beta_, const std::optional<Tensor>& bias_) {
     const Tensor w2 = given(w2_), alpha = given(alpha_), beta = given(beta_), bias = given(bias_);
+    // (a tangent would be dropped without a word where nothing is recorded)
+    for (const Tensor* t : {&x, &w, &w2, &alpha, &beta, &bias})
+        TORCH_CHECK_NOT_IMPLEMENTED(!t->defined() || !t->_fw_grad(0).defined(), "tropical layers have no forward-mode derivative");
     bool record = false;
     if (at::GradMode::is_enabled())
         for (const Tensor* t : {&x, &w, &w2, &alpha, &beta, &bias}) record = record || (t->defined() && t->requires_grad());

@@ -57,3 +57,11 @@ def test_other_saved_tensors_are_refused(kind, pack):
         y = m(x)
     with pytest.raises(ValueError):
         y.sum().backward()
+
+
+@pytest.mark.parametrize("kind", ["dense", "depthwise", "volume"])
+@pytest.mark.parametrize("record", [True, False])
+def test_forward_mode_is_refused(kind, record):
+    m, x = make(kind, "cpu")
+    with torch.set_grad_enabled(record), fwad.dual_level(), pytest.raises(NotImplementedError):
+        m(fwad.make_dual(x, torch.ones_like(x)))
