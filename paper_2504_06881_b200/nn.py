@@ -58,7 +58,7 @@ _geoms = tconv.KeptPlans(lambda kind, mode, chan, dtype, stride, pad, dil: _nati
 
 def _layer(kind, mode, chan, dtype, stride, pad, dil, x, w, w2, alpha, beta, bias):
     """One layer through the native autograd path (csrc/torch_layers.cpp)."""
-    geom = (kind, mode, chan, dtype, stride, pad, dil)
+    geom = (kind, mode, chan, dtype, tuple(stride), tuple(pad), tuple(dil))
     return _native.layer(_geoms.get(geom, *geom), x, w, w2, alpha, beta, bias)
 
 

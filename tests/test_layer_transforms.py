@@ -65,3 +65,12 @@ def test_forward_mode_is_refused(kind, record):
     m, x = make(kind, "cpu")
     with torch.set_grad_enabled(record), fwad.dual_level(), pytest.raises(NotImplementedError):
         m(fwad.make_dual(x, torch.ones_like(x)))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["dense", "depthwise", "volume"])
+def test_geometry_as_lists(kind):
+    m, x = make(kind)
+    ref = m(x)
+    m.stride, m.padding, m.dilation = list(m.stride), list(m.padding), list(m.dilation)
+    assert torch.equal(m(x), ref)
