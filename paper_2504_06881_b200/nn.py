@@ -14,7 +14,7 @@ import math
 import torch
 import torch.nn as nn
 
-from . import tconv
+from . import tconv, tconv3d
 try:
     from . import _tconv_torch as _native
 except ImportError as err:
@@ -40,31 +40,26 @@ def _as(t, dtype):
     return t if t.is_contiguous() else t.contiguous()
 
 
-def _make_desc2d(xs, ws, geom, x_f32):
-    (N, C, H, W), (K, _, R, S), (mode, chan, dtype, stride, pad, dil, _rec) = xs, ws, geom
-    d = tconv.PlannedDesc(N=N, C=C, H=H, W=W, K=K, R=R, S=S, stride_h=stride[0], stride_w=stride[1], pad_h=pad[0],
-                          pad_w=pad[1], dil_h=dil[0], dil_w=dil[1], mode=mode, chan=chan, dtype=dtype)
-    if x_f32:
-        d["x_dtype"] = "f32"
-    return d
-
-
-_descs2d = tconv.KeptPlans(_make_desc2d)
-
 _KINDS = {"dense": 0, "depthwise": 1, "volume": 2}
 _geoms = tconv.KeptPlans(lambda kind, mode, chan, dtype, stride, pad, dil: _native.Geom(
     _KINDS[kind], tconv.MODES[mode], tconv.CHANS[chan], tconv.DTYPES[dtype], stride, pad, dil))
 
 
 def _layer(kind, mode, chan, dtype, stride, pad, dil, x, w, w2, alpha, beta, bias):
-    """One layer through the native autograd path (csrc/torch_layers.cpp)."""
-    geom = (kind, mode, chan, dtype, tuple(stride), tuple(pad), tuple(dil))
-    return _native.layer(_geoms.get(geom, *geom), x, w, w2, alpha, beta, bias)
+    """One layer through the native autograd path (csrc/torch_layers.cpp).  Under ``torch.jit.trace`` through the
+    Python Function, which a trace records as one operation: of the native path it would record the allocations."""
+    geom = (mode, chan, dtype, tuple(stride), tuple(pad), tuple(dil))
+    if torch.jit.is_tracing():
+        fn = {"dense": TropicalConvFn, "depthwise": TropicalDepthwiseFn, "volume": TropicalConv3dFn}[kind]
+        return fn.apply(x, w, w2, alpha, beta, bias, geom if kind != "depthwise" else (mode,) + geom[2:])
+    return _native.layer(_geoms.get((kind,) + geom, kind, *geom), x, w, w2, alpha, beta, bias)
 
 
 class TropicalConvFn(torch.autograd.Function):
     """y = tconv_forward(x, w, w2, alpha, beta, bias); backward = tconv_backward with the stored winners.
-    The layers take the native path (csrc/torch_layers.cpp) unless one of the two settings below is on.
+    The layers take the native path (csrc/torch_layers.cpp) unless one of the two settings below is on or a trace is
+    recorded.  geom: mode, channel combine, type, stride, padding, dilation and optionally whether gradients are
+    recorded where the layer was called (inside a Function's forward the grad mode is always off).
 
     Master parameters may be fp32 while the layer computes in bf16: the cast happens here and the
     parameter gradients come back in fp32.  When ``TropicalConvFn.events`` is a list, every library
@@ -78,13 +73,18 @@ class TropicalConvFn(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, w, w2, alpha, beta, bias, geom):
-        dtype, recording = geom[2], geom[6]
+        mode, chan, dtype, stride, pad, dil = geom[:6]
+        recording = geom[6] if len(geom) > 6 else True
         dt = tconv.TORCH_DTYPE[dtype]
+        N, C, H, W = x.shape
+        K, _, R, S = w.shape
+        d = dict(N=N, C=C, H=H, W=W, K=K, R=R, S=S, stride_h=stride[0], stride_w=stride[1],
+                 pad_h=pad[0], pad_w=pad[1], dil_h=dil[0], dil_w=dil[1], mode=mode, chan=chan, dtype=dtype)
         # a float x for a bf16 layer is rounded by the kernel while it stages x (no cast kernel, no
         # bf16 copy); layers the tiled kernels do not serve fall back to the explicit cast
         fused_cast = TropicalConvFn.fuse_cast and dtype == "bf16" and x.dtype == torch.float32
-        desc_of = lambda f32x: _descs2d.get((x.shape, w.shape, geom, f32x), x.shape, w.shape, geom, f32x)
-        d = desc_of(fused_cast)
+        if fused_cast:
+            d["x_dtype"] = "f32"
         xc = _as(x, x.dtype if fused_cast else dt)
         wc, w2c = _as(w, dt), _as(w2, dt)
         al, be, bi = _as(alpha, torch.float32), _as(beta, torch.float32), _as(bias, torch.float32)
@@ -98,7 +98,7 @@ class TropicalConvFn(torch.autograd.Function):
         except tconv.TconvError as err:
             if not fused_cast or err.status != -2:
                 raise
-            d = desc_of(False)
+            del d["x_dtype"]
             xc = _as(x, dt)
             y, winners = tconv.forward(d, xc, wc, w2c, al, be, bi, want_winners=need_grad)
         if ev is not None:
@@ -377,6 +377,36 @@ class HybridResNet18(nn.Module):
         return [m for m in self.modules() if isinstance(m, TropicalConv2d)]
 
 
+class TropicalDepthwiseFn(torch.autograd.Function):
+    """Depthwise (groups = C) form over tconv_dw_forward / tconv_dw_backward; see TropicalConvFn."""
+
+    @staticmethod
+    def forward(ctx, x, w, w2, alpha, beta, bias, geom):
+        mode, dtype, stride, pad, dil = geom
+        dt = tconv.TORCH_DTYPE[dtype]
+        N, C, H, W = x.shape
+        _, R, S = w.shape
+        d = dict(N=N, C=C, H=H, W=W, K=C, R=R, S=S, stride_h=stride[0], stride_w=stride[1],
+                 pad_h=pad[0], pad_w=pad[1], dil_h=dil[0], dil_w=dil[1], mode=mode, chan="sum", dtype=dtype)
+        xc, wc, w2c = _as(x, dt), _as(w, dt), _as(w2, dt)
+        al, be, bi = _as(alpha, torch.float32), _as(beta, torch.float32), _as(bias, torch.float32)
+        y, winners = tconv.dw_forward(d, xc, wc, w2c, al, be, bi,
+                                      want_winners=_emit_winners(True, x, w, w2, alpha, beta, bias))
+        ctx.d, ctx.in_dtype = d, x.dtype
+        ctx.save_for_backward(xc, wc, w2c, al, be, winners)
+        ctx.has = (w2 is not None, alpha is not None, beta is not None, bias is not None)
+        return y.to(x.dtype) if x.dtype != dt else y
+
+    @staticmethod
+    def backward(ctx, gy):
+        xc, wc, w2c, al, be, winners = ctx.saved_tensors
+        grads = tconv.dw_backward(ctx.d, xc, wc, _as(gy, tconv.TORCH_DTYPE[ctx.d["dtype"]]), w2c, al, be, winners)
+        has_w2, has_a, has_b, has_bias = ctx.has
+        return (grads["grad_x"].to(ctx.in_dtype), grads["grad_w"], grads.get("grad_w2") if has_w2 else None,
+                grads.get("grad_alpha") if has_a else None, grads.get("grad_beta") if has_b else None,
+                grads["grad_bias"] if has_bias else None, None)
+
+
 class TropicalDepthwiseConv2d(nn.Module):
     """Depthwise tropical convolution (``nn.Conv2d(channels, channels, k, groups=channels)``'s place in
     a MobileNetV2 block): per channel one window of weights, one alpha and one beta.
@@ -426,6 +456,38 @@ class TropicalDepthwiseConv2d(nn.Module):
                 alpha, beta = self.alpha_fixed, self.beta_fixed
         return _layer("depthwise", self.mode, "sum", self.dtype, self.stride, self.padding, self.dilation, x, self.weight,
                       self.weight2, alpha, beta, self.bias)
+
+
+class TropicalConv3dFn(torch.autograd.Function):
+    """y = tconv3d_forward(...); backward = tconv3d_backward with the stored winners; see TropicalConvFn."""
+
+    @staticmethod
+    def forward(ctx, x, w, w2, alpha, beta, bias, geom):
+        mode, chan, dtype, stride, pad, dil = geom
+        dt = tconv.TORCH_DTYPE[dtype]
+        N, C, D, H, W = x.shape
+        K, _, T, R, S = w.shape
+        d = dict(N=N, C=C, D=D, H=H, W=W, K=K, T=T, R=R, S=S, stride=tuple(stride), pad=tuple(pad),
+                 dil=tuple(dil), mode=mode, chan=chan, dtype=dtype)
+        xc, wc, w2c = _as(x, dt), _as(w, dt), _as(w2, dt)
+        al, be, bi = _as(alpha, torch.float32), _as(beta, torch.float32), _as(bias, torch.float32)
+        y, winners = tconv3d.forward(d, xc, wc, w2c, al, be, bi,
+                                     want_winners=_emit_winners(True, x, w, w2, alpha, beta, bias))
+        ctx.d, ctx.in_dtype = d, x.dtype
+        ctx.save_for_backward(xc, wc, w2c, al, be, winners)
+        ctx.has = (w2 is not None, alpha is not None, beta is not None, bias is not None)
+        return y.to(x.dtype) if x.dtype != dt else y
+
+    @staticmethod
+    def backward(ctx, gy):
+        xc, wc, w2c, al, be, winners = ctx.saved_tensors
+        grads = tconv3d.backward(ctx.d, xc, wc, _as(gy, tconv.TORCH_DTYPE[ctx.d["dtype"]]), w2c, al, be, winners,
+                                 need_grad_x=ctx.needs_input_grad[0])
+        has_w2, has_a, has_b, has_bias = ctx.has
+        gx = grads["grad_x"].to(ctx.in_dtype) if "grad_x" in grads else None
+        return (gx, grads["grad_w"], grads.get("grad_w2") if has_w2 else None,
+                grads.get("grad_alpha") if has_a else None, grads.get("grad_beta") if has_b else None,
+                grads["grad_bias"] if has_bias else None, None)
 
 
 class TropicalConv3d(TropicalConv2d):

@@ -256,16 +256,6 @@ class Plan:
         self.bwd_ws_stored = max(0, self.bwd_ws - (self.winner_bytes + 255) // 256 * 256)
 
 
-class PlannedDesc(dict):
-    """A descriptor dict that carries its plan (made on first use; the dict must not change after that)."""
-
-    __slots__ = ("plan",)
-
-    def __init__(self, *args, **kw):
-        super().__init__(*args, **kw)
-        self.plan = None
-
-
 class KeptPlans:
     """A bounded table of plans by key; when it is full the oldest half goes."""
 
@@ -309,18 +299,10 @@ _dw_plans = KeptPlans(DwPlan)
 
 
 def dw_plan_of(d: dict) -> DwPlan:
-    if type(d) is PlannedDesc:
-        if d.plan is None:
-            d.plan = DwPlan(d)
-        return d.plan
     return _dw_plans.get(tuple(map(d.get, _FIELDS)), d)
 
 
 def plan_of(d: dict) -> Plan:
-    if type(d) is PlannedDesc:
-        if d.plan is None:
-            d.plan = Plan(d)
-        return d.plan
     return _plans.get(tuple(map(d.get, _FIELDS)), d)
 
 

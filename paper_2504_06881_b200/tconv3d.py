@@ -10,8 +10,8 @@ import ctypes
 
 import torch
 
-from .tconv import (CHANS, DTYPES, MODES, TORCH_DTYPE, KeptPlans, PlannedDesc, TconvError, _check, _lib, _on_stream,
-                    _p, _ptr, _raw_stream, _stream)
+from .tconv import (CHANS, DTYPES, MODES, TORCH_DTYPE, KeptPlans, TconvError, _check, _lib, _on_stream, _p,
+                    _ptr, _raw_stream, _stream)
 
 # every symbol include/tconv3d.h declares
 SYMBOLS = ("tconv3d_output_shape", "tconv3d_winner_bytes", "tconv3d_workspace_bytes", "tconv3d_forward",
@@ -118,10 +118,6 @@ _FIELDS = ("N", "C", "D", "H", "W", "K", "T", "R", "S", "stride", "pad", "dil", 
 
 
 def plan_of(d: dict) -> Plan3:
-    if type(d) is PlannedDesc:
-        if d.plan is None:
-            d.plan = Plan3(d)
-        return d.plan
     return _plans.get(tuple(tuple(v) if isinstance(v, list) else v for v in map(d.get, _FIELDS)), d)
 
 

@@ -74,3 +74,37 @@ def test_geometry_as_lists(kind):
     ref = m(x)
     m.stride, m.padding, m.dilation = list(m.stride), list(m.padding), list(m.dilation)
     assert torch.equal(m(x), ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("record", [True, False])
+def test_traced_layers_compute(kind, record):
+    m, x = make(kind)
+    for p in m.parameters():
+        p.requires_grad_(record)
+    traced = torch.jit.trace(m, x, check_trace=False)
+    other = torch.randn_like(x)
+    assert torch.equal(traced(other), m(other))
+    if record:
+        assert all(torch.equal(a, b) for a, b in zip(gradients(m, other), gradients(m, other, traced)))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", KINDS)
+def test_transforms_are_refused(kind):
+    m, x = make(kind)
+    with pytest.raises(RuntimeError):
+        torch.func.vmap(m)(torch.stack([x, x]))
+    with pytest.raises(RuntimeError), torch.no_grad():
+        torch.func.vmap(m)(torch.stack([x, x]))
+    with pytest.raises(RuntimeError):
+        torch.func.grad(lambda v: m(v).sum())(x)
+
+
+@pytest.mark.gpu
+def test_functions_take_the_geometry_alone():
+    m, x = make("dense")
+    geom = (m.mode, m.chan, m.dtype, m.stride, m.padding, m.dilation)
+    y = tnn.TropicalConvFn.apply(x, m.weight, m.weight2, m.alpha, m.beta, m.bias, geom)
+    assert torch.equal(y, m(x)) and y.requires_grad
