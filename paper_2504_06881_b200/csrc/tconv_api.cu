@@ -259,10 +259,10 @@ int backward_t(const Geo& g, const void* x, const void* w, const void* w2, const
             g_launches += 1;
         }
         IdxGwPlan pw;
-        if ((gw || gbias) && tiled && plan_idx_gw(g, (((uintptr_t)gy | (uintptr_t)idx) & 15) == 0, &pw) && ws && ws_bytes >= pw.part_floats * sizeof(float)) {
+        if ((gw || gbias) && tiled && plan_idx_gw(g, &pw) && ws && ws_bytes >= pw.part_floats * sizeof(float)) {
             float* part = (float*)ws;
             float* part_b = part + (size_t)pw.chunks * pw.nkg * g.C * g.RS * 32;
-            auto kern = pw.vec == 4 ? bwd_idx_gw_kernel<T, 4> : bwd_idx_gw_kernel<T, 1>;
+            auto kern = pw.shift ? bwd_idx_gw_kernel<T, true> : bwd_idx_gw_kernel<T, false>;
             if (allow_smem(kern, (int)kIdxSmemMost) != cudaSuccess) return cuda_fail(cudaGetLastError());
             kern<<<dim3((unsigned)(pw.nkg * pw.nblk), (unsigned)pw.chunks), 32, pw.smem, st>>>(g, (const T*)gy, idx, part, part_b, pw);
             const unsigned slices = pw.chunks >= 8 ? 8 : pw.chunks >= 4 ? 4 : pw.chunks >= 2 ? 2 : 1;

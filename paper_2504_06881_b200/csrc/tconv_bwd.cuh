@@ -59,7 +59,7 @@ inline size_t bwd_ws_bytes(const Geo& g) {
     // grad_bias partials of the any-shape path; Max / Min combine: the histograms of bwd_idx_gw_kernel
     const size_t bias = (size_t)16 * g.K * sizeof(float) + 256;
     IdxGwPlan p;
-    if (g.chan == CH_SUM || !plan_idx_gw(g, false, &p)) return bias;
+    if (g.chan == CH_SUM || !plan_idx_gw(g, &p)) return bias;
     const size_t part = p.part_floats * sizeof(float) + 256;
     return part > bias ? part : bias;
 }

@@ -37,7 +37,7 @@ struct IdxGwPlan {
     int CB, nblk;           // channels per table, channel blocks
     int nkg;                // groups of 32 output channels
     int lk;                 // log2 of the lanes that take different output channels (the others: more pixels)
-    int vec;                // pixels per load (4 or 1)
+    int shift;              // 1: planes that are not a multiple of four, rows start inside a piece of four
     int timg;               // tiles of 32 pixels per lane slice, per image
     int chunks, per;        // ranges of the flattened (image, tile) space, tiles per range
     size_t smem, part_floats;
@@ -142,7 +142,7 @@ constexpr int kGwPitch = 36;                        // words per lane row (16-by
 constexpr int kGwStages = 4;
 constexpr size_t kGwStageBytes = 2 * 32 * kGwPitch * 4;
 
-inline bool plan_idx_gw(const Geo& g, bool aligned, IdxGwPlan* p) {
+inline bool plan_idx_gw(const Geo& g, IdxGwPlan* p) {
     const size_t per_c = (size_t)g.RS * 32 * sizeof(float);
     if (per_c > 150 * 1024 || (double)g.N * g.K * g.OH * g.OW > 6.0e10 || (double)g.N * g.OH * g.OW > 2.0e9) return false;
     p->CB = (int)(73 * 1024 / per_c);
@@ -156,7 +156,7 @@ inline bool plan_idx_gw(const Geo& g, bool aligned, IdxGwPlan* p) {
     p->smem = per_c * p->CB + 32 * sizeof(float) + kGwStages * kGwStageBytes;
     const long plane = (long)g.OH * g.OW;
     while (p->lk < 5 && plane <= (32L << (5 - p->lk)) / 2) ++p->lk;    // small planes: no slices without pixels
-    p->vec = plane % 4 == 0 && aligned ? 4 : 1;
+    p->shift = plane % 4 != 0;
     const long tile = 32L << (5 - p->lk);
     p->timg = (int)((plane + tile - 1) / tile);
     const long tiles = (long)g.N * p->timg;
@@ -290,17 +290,25 @@ bwd_idx_gx_kernel(Geo g, const T* __restrict__ gy, const int32_t* __restrict__ i
 }
 
 // ---------------------------------------------------------------------------------- grad_w, grad_bias
-__device__ __forceinline__ void gw_copy16(unsigned dst, const void* src, bool on) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
+// bytes of a piece of 16 (8), then zeros
+__device__ __forceinline__ void gw_copy16(unsigned dst, const void* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void gw_copy8(unsigned dst, const void* src, bool on) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(on ? 8 : 0) : "memory");
+__device__ __forceinline__ void gw_copy8(unsigned dst, const void* src, int bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
-__device__ __forceinline__ void gw_copy4(unsigned dst, const void* src, bool on) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(on ? 4 : 0) : "memory");
+// Elements s .. s + 3 of eight.
+__device__ __forceinline__ uint4 gw_shift(const uint4& a, const uint4& b, int s) {
+    const bool one = s & 1, two = s & 2;
+    const unsigned t0 = one ? a.y : a.x, t1 = one ? a.z : a.y, t2 = one ? a.w : a.z, t3 = one ? b.x : a.w, t4 = one ? b.y : b.x,
+                   t5 = one ? b.z : b.y;
+    return make_uint4(two ? t2 : t0, two ? t3 : t1, two ? t4 : t2, two ? t5 : t3);
 }
 
-template <typename T, int V>
+// SHIFT: planes that are not a multiple of four.  A row of 32 pixels may start inside a piece of four; its nine pieces
+// are copied whole and four pixels selected out of two pieces when they are read.  Copied pixel by pixel such planes
+// took four times the copies (N=64 C=512 K=512 15x15 bf16: 818 us).
+template <typename T, bool SHIFT>
 __global__ void __launch_bounds__(32)
 bwd_idx_gw_kernel(Geo g, const T* __restrict__ gy, const int32_t* __restrict__ idx, float* __restrict__ part,
                   float* __restrict__ part_b, IdxGwPlan pl) {
@@ -315,34 +323,28 @@ bwd_idx_gw_kernel(Geo g, const T* __restrict__ gy, const int32_t* __restrict__ i
     const int i0 = chunk * pl.per, i1 = min(total, i0 + pl.per);
     const int tile_px = 32 << (5 - pl.lk), kmask = (1 << pl.lk) - 1;
     constexpr bool HALF = sizeof(T) == 2;
-    int n = i0 / pl.timg, t = i0 - n * pl.timg, next = i0;
+    const int n0 = i0 / pl.timg, t0 = i0 - n0 * pl.timg;
+    int n = n0, t = t0, next = i0;
     // Pixels past the plane's end and output channels past K arrive as zeros: nothing added.
     auto request = [&](int stage) {
         if (next < i1) {
             float* st = smem_gw + stage * (kGwStageBytes / 4);
             const unsigned si = (unsigned)__cvta_generic_to_shared(st), sg = si + 32 * kGwPitch * 4;
-            if constexpr (V == 4) {
+            // piece j (four pixels) of a row: `left` pixels of the row and those before it in its first piece remain
+            auto copy = [&](int row, int j) {
+                const int k = kg * 32 + (row & kmask), p0 = t * tile_px + (row >> pl.lk) * 32, cnt = min(32, plane - p0);
+                const bool on = k < g.K && cnt > 0;
+                size_t at = on ? ((size_t)n * g.K + k) * plane + p0 : 0;
+                const int before = SHIFT ? (int)(at & 3) : 0;
+                const int left = on ? min(4, max(0, cnt + before - 4 * j)) : 0;
+                at = left ? at - before + 4 * j : 0;
+                gw_copy16(si + (row * kGwPitch + 4 * j) * 4, idx + at, left * 4);
+                if constexpr (HALF) gw_copy8(sg + row * (kGwPitch * 2) + j * 8, gy + at, left * 2);
+                else gw_copy16(sg + (row * kGwPitch + 4 * j) * 4, gy + at, left * 4);
+            };
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {                     // eight lanes copy 32 pixels of one row
-                    const int row = u * 4 + (lane >> 3), j = (lane & 7) * 4;
-                    const int k = kg * 32 + (row & kmask), p = t * tile_px + (row >> pl.lk) * 32 + j;
-                    const bool on = k < g.K && p < plane;
-                    const size_t at = on ? ((size_t)n * g.K + k) * plane + p : 0;
-                    gw_copy16(si + (row * kGwPitch + j) * 4, idx + at, on);
-                    if constexpr (HALF) gw_copy8(sg + row * (kGwPitch * 2) + j * 2, gy + at, on);
-                    else gw_copy16(sg + (row * kGwPitch + j) * 4, gy + at, on);
-                }
-            } else {
-#pragma unroll 8
-                for (int row = 0; row < 32; ++row) {
-                    const int k = kg * 32 + (row & kmask), p = t * tile_px + (row >> pl.lk) * 32 + lane;
-                    const bool on = k < g.K && p < plane;
-                    const size_t at = on ? ((size_t)n * g.K + k) * plane + p : 0;
-                    gw_copy4(si + (row * kGwPitch + lane) * 4, idx + at, on);
-                    if constexpr (HALF) st[32 * kGwPitch + row * kGwPitch + lane] = on ? to_f32(__ldg(gy + at)) : 0.0f;
-                    else gw_copy4(sg + (row * kGwPitch + lane) * 4, gy + at, on);
-                }
-            }
+            for (int u = 0; u < 8; ++u) copy(u * 4 + (lane >> 3), lane & 7);       // eight lanes, 32 pixels of one row
+            if constexpr (SHIFT) copy(lane, 8);
             if (++t == pl.timg) { t = 0; ++n; }
         }
         ++next;
@@ -375,28 +377,45 @@ bwd_idx_gw_kernel(Geo g, const T* __restrict__ gy, const int32_t* __restrict__ i
 #pragma unroll 4
     for (int e = lane; e < (pl.CB * g.RS + 1) * 8; e += 32) tab4[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     int stage = 0;
+    const unsigned kmine = kg * 32 + (lane & kmask);
+    unsigned nu = n0;                                             // image of the tile in use
+    int tu = t0;
     for (int i = i0; i < i1; ++i) {
         asm volatile("cp.async.wait_group %0;" ::"n"(kGwStages - 2) : "memory");
         __syncwarp();
         request((stage + kGwStages - 1) % kGwStages);
         const float* st = smem_gw + stage * (kGwStageBytes / 4);
-        const int4* ri = reinterpret_cast<const int4*>(st + lane * kGwPitch);
-        auto grad = [&](int j) {
-            if constexpr (HALF && V == 4) {
+        const int before = SHIFT ? (int)(((nu * g.K + kmine) * (unsigned)plane) & 3u) : 0;
+        if (++tu == pl.timg) { tu = 0; ++nu; }
+        const uint4* ri = reinterpret_cast<const uint4*>(st + lane * kGwPitch);
+        auto grads = [&](int j) {                                 // (bf16: four in two words)
+            if constexpr (HALF) {
                 const uint2 f = reinterpret_cast<const uint2*>(st + 32 * kGwPitch + lane * (kGwPitch / 2))[j];
-                return make_float4(__uint_as_float(f.x << 16), __uint_as_float(f.x & 0xffff0000u),
-                                   __uint_as_float(f.y << 16), __uint_as_float(f.y & 0xffff0000u));
+                return make_uint4(f.x, f.y, 0u, 0u);
             } else {
-                return reinterpret_cast<const float4*>(st + 32 * kGwPitch + lane * kGwPitch)[j];
+                return reinterpret_cast<const uint4*>(st + 32 * kGwPitch + lane * kGwPitch)[j];
             }
         };
-        int4 q = ri[0];
-        float4 f = grad(0);
+        uint4 q = ri[0], f = grads(0);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int4 q1 = ri[(j + 1) & 7];
-            const float4 f1 = grad((j + 1) & 7);
-            add(q, f);
+            const int j1 = SHIFT ? j + 1 : (j + 1) & 7;
+            const uint4 q1 = ri[j1], f1 = grads(j1);
+            uint4 w = q, v = f;
+            if constexpr (SHIFT) {
+                w = gw_shift(q, q1, before);
+                if constexpr (HALF) {
+                    const bool two = before & 2;
+                    const unsigned h = (before & 1) * 16, a = two ? f.y : f.x, b = two ? f1.x : f.y, c = two ? f1.y : f1.x;
+                    v.x = __funnelshift_r(a, b, h);
+                    v.y = __funnelshift_r(b, c, h);
+                } else {
+                    v = gw_shift(f, f1, before);
+                }
+            }
+            if constexpr (HALF) v = make_uint4(v.x << 16, v.x & 0xffff0000u, v.y << 16, v.y & 0xffff0000u);
+            add(make_int4(w.x, w.y, w.z, w.w),
+                make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w)));
             q = q1;
             f = f1;
         }

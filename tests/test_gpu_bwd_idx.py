@@ -32,3 +32,18 @@ LAYERS = [
 def test_classes_and_tiles(mode, chan, dtype):
     for i, d in enumerate(LAYERS):
         parity.check_layer(dict(d, mode=mode, chan=chan, dtype=dtype), None, 2400 + i, recompute=False)
+
+
+ODD = [
+    L(3, 2, 9, 7, 33, pad=1),                            # rows that start at odd elements, the last at the tensor's end
+    L(1, 1, 5, 5, 1, pad=1),
+    L(5, 70, 15, 15, 40, pad=1),                         # several tiles of a plane, channel blocks
+    L(2, 3, 11, 13, 3, pad=1),                           # lanes of one channel on several pixel slices
+    L(3, 2, 7, 10, 5, pad=1),                            # an even plane that is not a multiple of four
+]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_odd_planes(dtype):
+    for i, d in enumerate(ODD):
+        parity.check_layer(dict(d, mode="max_plus", dtype=dtype), None, 2500 + i, recompute=False)
