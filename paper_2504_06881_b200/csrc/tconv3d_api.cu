@@ -62,30 +62,7 @@ size_t winner_bytes3(const Geo3& g) {
     return (size_t)g.N * g.K * g.vol * sizeof(int32_t);
 }
 
-// Splits of the (n, position) range for the grad_w partial sums: enough blocks to fill the SMs
-// when K*C is small, each split at least four stages long.
-int gw_splits(const Geo3& g) {
-    const long long total = (long long)g.N * g.vol;
-    long long want = (2 * 148 + (long long)g.K * g.C - 1) / ((long long)g.K * g.C);
-    const long long most = (total + 4 * kGw3Stage - 1) / (4 * kGw3Stage);
-    if (want > most) want = most;
-    if (want < 1) want = 1;
-    if (want > 64) want = 64;
-    return (int)want;
-}
-
-// Splits of the same range for the grad_bias partial sums (K blocks otherwise).
-int bias_splits(const Geo3& g) {
-    const long long total = (long long)g.N * g.vol;
-    long long want = (2 * 148 + g.K - 1) / g.K;
-    const long long most = (total + 4095) / 4096;
-    if (want > most) want = most;
-    if (want < 1) want = 1;
-    if (want > 64) want = 64;
-    return (int)want;
-}
-
-// TCONV_FORCE_GENERIC=1 keeps every call on the any-shape kernels (read once per process).
+// TCONV_FORCE_GENERIC=1 keeps 1-D layers on the kernels of the other layers (read once per process).
 bool force_generic3() {
     static const int v = [] {
         const char* e = getenv("TCONV_FORCE_GENERIC");
@@ -189,10 +166,7 @@ PlanParams3 plan_params3(const Geo3& g) {
 
 size_t backward_scratch_floats(const Geo3& g) {
     const Plan1 p = plan_1d(g);
-    if (p.ok) return p.scratch_floats;
-    if (!force_generic3()) return plan_params3(g).scratch_floats;
-    const size_t ns = (size_t)gw_splits(g);
-    return 2 * ns * g.K * g.C * g.taps + 2 * ns * g.K * g.C + (size_t)bias_splits(g) * g.K;
+    return p.ok ? p.scratch_floats : plan_params3(g).scratch_floats;
 }
 
 int check(cudaError_t e) { return e == cudaSuccess ? TCONV_OK : TCONV_ERR_CUDA; }
@@ -378,48 +352,18 @@ int backward3_t(const Geo3& g, const void* x, const void* w, const void* w2, con
             g, alpha, beta, (const T*)gy, winners, (T*)gx);
         g3_launches += 1;
     }
-    if (!force_generic3()) {
-        if (!(gw || gw2 || gbias || (two && (galpha || gbeta)))) return check(cudaGetLastError());
-        const PlanParams3 p = plan_params3(g);
-        const size_t kc = (size_t)g.K * g.C;
-        float* hist = (float*)ws;
-        float* ab = hist + (size_t)p.nsplit * kc * 2 * g.taps;
-        float* pb = ab + (size_t)p.nsplit * kc * 2;
-        if (allow_smem(bwd3d_params_kernel<T>, (int)kSmem1d) != cudaSuccess) return TCONV_ERR_CUDA;
-        bwd3d_params_kernel<T><<<dim3((unsigned)kc, (unsigned)p.nsplit), p.tb, p.smem, st>>>(
-            g, p.nsplit, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, winners, hist, ab, pb);
-        bwd3d_params_finish_kernel<<<(unsigned)kc, 128, 0, st>>>(g, p.nsplit, alpha, beta, hist, ab,
-                                                                  pb, gw, gw2, galpha, gbeta, gbias);
-        g3_launches += 2;
-        return check(cudaGetLastError());
-    }
-    const int nsplit = gw_splits(g);
-    const size_t count = (size_t)g.K * g.C * g.taps;
-    float* pmin = (float*)ws;
-    float* pmax = pmin + (size_t)nsplit * count;
-    float* pab = pmax + (size_t)nsplit * count;          // [nsplit][K*C][2]
-    float* pbias = pab + (size_t)nsplit * g.K * g.C * 2;  // [bias splits][K]
-    if (gw || gw2) {
-        bwd3d_gw_kernel<T><<<dim3((unsigned)(g.K * g.C), (unsigned)nsplit), 256, 0, st>>>(
-            g, nsplit, (const T*)gy, winners, pmin, pmax);
-        bwd3d_gw_finish_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(g, nsplit, alpha, beta, pmin,
-                                                                               pmax, gw, gw2);
-        g3_launches += 2;
-    }
-    if (two && (galpha || gbeta)) {
-        bwd3d_gab_kernel<T><<<dim3((unsigned)(g.K * g.C), (unsigned)nsplit), 256, 0, st>>>(
-            g, nsplit, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, winners, pab);
-        const int kc = g.K * g.C;
-        if (galpha) bwd3d_sum_splits_kernel<<<(kc + 255) / 256, 256, 0, st>>>(kc, nsplit, 2, 0, pab, galpha);
-        if (gbeta) bwd3d_sum_splits_kernel<<<(kc + 255) / 256, 256, 0, st>>>(kc, nsplit, 2, 1, pab, gbeta);
-        g3_launches += 1 + (galpha ? 1 : 0) + (gbeta ? 1 : 0);
-    }
-    if (gbias) {
-        const int bs = bias_splits(g);
-        bwd3d_bias_kernel<T><<<dim3((unsigned)g.K, (unsigned)bs), 256, 0, st>>>(g, bs, (const T*)gy, pbias);
-        bwd3d_sum_splits_kernel<<<(g.K + 255) / 256, 256, 0, st>>>(g.K, bs, 1, 0, pbias, gbias);
-        g3_launches += 2;
-    }
+    if (!(gw || gw2 || gbias || (two && (galpha || gbeta)))) return check(cudaGetLastError());
+    const PlanParams3 p = plan_params3(g);
+    const size_t kc = (size_t)g.K * g.C;
+    float* hist = (float*)ws;
+    float* ab = hist + (size_t)p.nsplit * kc * 2 * g.taps;
+    float* pb = ab + (size_t)p.nsplit * kc * 2;
+    if (allow_smem(bwd3d_params_kernel<T>, (int)kSmem1d) != cudaSuccess) return TCONV_ERR_CUDA;
+    bwd3d_params_kernel<T><<<dim3((unsigned)kc, (unsigned)p.nsplit), p.tb, p.smem, st>>>(
+        g, p.nsplit, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, winners, hist, ab, pb);
+    bwd3d_params_finish_kernel<<<(unsigned)kc, 128, 0, st>>>(g, p.nsplit, alpha, beta, hist, ab, pb, gw, gw2, galpha, gbeta,
+                                                             gbias);
+    g3_launches += 2;
     return check(cudaGetLastError());
 }
 

@@ -303,22 +303,6 @@ fwd3d_split_kernel(Geo3 g, int PX, int ts, int cg, const T* __restrict__ x, cons
     if (WIN && g.chan != CH_SUM) ((int32_t*)winners)[o] = win;
 }
 
-// The winning taps of (n, k, c, position) as two ints; -1 where the layer has no such branch or
-// (Max / Min channel combine) another channel won.
-__device__ __forceinline__ void winners3(const Geo3& g, const void* winners, int n, int k, int c, int pos,
-                                         int& amn, int& amx) {
-    if (g.chan == CH_SUM) {
-        const unsigned v = ((const uint16_t*)winners)[(((size_t)n * g.K + k) * g.C + c) * g.vol + pos];
-        amn = (g.mode == TCONV_MAX_PLUS) ? -1 : (int)(v & 0xFFu);
-        amx = (g.mode == TCONV_MIN_PLUS) ? -1 : (int)(v >> 8);
-    } else {
-        const int v = ((const int32_t*)winners)[((size_t)n * g.K + k) * g.vol + pos] - c * g.taps;
-        const int tap = (v >= 0 && v < g.taps) ? v : -1;
-        amn = (g.mode == TCONV_MIN_PLUS) ? tap : -1;
-        amx = (g.mode == TCONV_MIN_PLUS) ? -1 : tap;
-    }
-}
-
 // Taps t of one axis through which an output reads input index i: i + pad - t * dil = stride * o with
 // 0 <= o < out.  The walk visits exactly those when dil is 1 (step = stride), else it tests every tap.
 struct TapRange {
@@ -583,52 +567,6 @@ bwd3d_params_finish_kernel(Geo3 g, int nsplit, const float* __restrict__ alpha, 
     }
 }
 
-constexpr int kGw3Stage = 1024;  // (winner, gradient) pairs staged per pass
-
-// grad_w partial sums: block (k*C + c, split) stages the winners and gradients of its share of
-// the (n, position) range in shared memory; thread `tap` then walks the staged pairs in order and
-// adds the gradients whose winner it is (the pairs are broadcast reads).  part[split][k*C+c][tap]
-// receives the min-branch and max-branch sums.
-template <typename T>
-__global__ void __launch_bounds__(256)
-bwd3d_gw_kernel(Geo3 g, int nsplit, const T* __restrict__ gy, const void* __restrict__ winners,
-                float* __restrict__ part_min, float* __restrict__ part_max) {
-    __shared__ unsigned code_s[kGw3Stage];
-    __shared__ float g_s[kGw3Stage];
-    const int kc = blockIdx.x, k = kc / g.C, c = kc % g.C, split = blockIdx.y;
-    const long long total = (long long)g.N * g.vol;
-    const long long per = (total + nsplit - 1) / nsplit;
-    const long long j0 = split * per, j1 = min(total, j0 + per);
-    const int tap = threadIdx.x;
-    float smin = 0.0f, smax = 0.0f;
-    for (long long base = j0; base < j1; base += kGw3Stage) {
-        const int cnt = (int)min((long long)kGw3Stage, j1 - base);
-        __syncthreads();
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-            const long long j = base + i;
-            const int n = (int)(j / g.vol), pos = (int)(j % g.vol);
-            int amn, amx;
-            winners3(g, winners, n, k, c, pos, amn, amx);
-            code_s[i] = ((unsigned)amn & 0xFFFFu) | ((unsigned)amx << 16);   // -1 stays 0xFFFF: matches no tap
-            g_s[i] = to_f32(gy[((size_t)n * g.K + k) * g.vol + pos]);
-        }
-        __syncthreads();
-        if (tap < g.taps) {
-            for (int i = 0; i < cnt; ++i) {
-                const unsigned code = code_s[i];
-                const float gv = g_s[i];
-                if ((code & 0xFFFFu) == (unsigned)tap) smin += gv;
-                if ((code >> 16) == (unsigned)tap) smax += gv;
-            }
-        }
-    }
-    if (tap < g.taps) {
-        const size_t o = ((size_t)split * g.K * g.C + kc) * g.taps + tap;
-        part_min[o] = smin;
-        part_max[o] = smax;
-    }
-}
-
 // Sums the partials over the splits in order and applies alpha / beta: one thread per (k, c, tap).
 __global__ void __launch_bounds__(256)
 bwd3d_gw_finish_kernel(Geo3 g, int nsplit, const float* __restrict__ alpha, const float* __restrict__ beta,
@@ -654,66 +592,6 @@ bwd3d_gw_finish_kernel(Geo3 g, int nsplit, const float* __restrict__ alpha, cons
         if (gw) gw[i] = a * tmin;
         if (gw2) gw2[i] = b * tmax;
     }
-}
-
-// grad_alpha / grad_beta partial sums: block (k*C + c, split) sums grad_y * MinPlus3d resp.
-// grad_y * MaxPlus3d over its share of the (n, position) range, the branch values rebuilt from the
-// winning taps.  part[split][k*C + c][2].
-template <typename T>
-__global__ void __launch_bounds__(256)
-bwd3d_gab_kernel(Geo3 g, int nsplit, const T* __restrict__ x, const T* __restrict__ w, const T* __restrict__ w2,
-                 const T* __restrict__ gy, const void* __restrict__ winners, float* __restrict__ part) {
-    __shared__ float red[256];
-    const int c = blockIdx.x % g.C, k = blockIdx.x / g.C, split = blockIdx.y;
-    const long long total = (long long)g.N * g.vol;
-    const long long per = (total + nsplit - 1) / nsplit;
-    const long long j0 = split * per, j1 = min(total, j0 + per);
-    const T* wmin = w + ((size_t)k * g.C + c) * g.taps;
-    const T* wmax = (g.mode == TCONV_PARALLEL ? w2 : w) + ((size_t)k * g.C + c) * g.taps;
-    float sa = 0.0f, sb = 0.0f;
-    for (long long j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-        const int n = (int)(j / g.vol), pos = (int)(j % g.vol);
-        const int ow = pos % g.OW, oh = (pos / g.OW) % g.OH, od = pos / (g.OW * g.OH);
-        int am[2];
-        winners3(g, winners, n, k, c, pos, am[0], am[1]);
-        const float gv = to_f32(gy[((size_t)n * g.K + k) * g.vol + pos]);
-        const T* xc = x + ((size_t)n * g.C + c) * g.D * g.H * g.W;
-#pragma unroll
-        for (int br = 0; br < 2; ++br) {
-            const int tap = am[br];
-            const int t = tap / (g.R * g.S), r = (tap / g.S) % g.R, s = tap % g.S;
-            const int id = od * g.sd - g.pd + t * g.dd, ih = oh * g.sh - g.ph + r * g.dh,
-                      iw = ow * g.sw - g.pw + s * g.dw;
-            T xv = zero_of<T>();
-            if (id >= 0 && id < g.D && ih >= 0 && ih < g.H && iw >= 0 && iw < g.W)
-                xv = xc[((size_t)id * g.H + ih) * g.W + iw];
-            const float v = tap_add(xv, br == 0 ? wmin[tap] : wmax[tap]);
-            if (br == 0) sa = __fmaf_rn(gv, v, sa); else sb = __fmaf_rn(gv, v, sb);
-        }
-    }
-    const float ta = block_sum(sa, red);
-    const float tb = block_sum(sb, red);
-    if (threadIdx.x == 0) {
-        float* o = part + ((size_t)split * g.K * g.C + blockIdx.x) * 2;
-        o[0] = ta;
-        o[1] = tb;
-    }
-}
-
-// grad_bias partial sums: block (k, split); part[split][k].
-template <typename T>
-__global__ void __launch_bounds__(256)
-bwd3d_bias_kernel(Geo3 g, int nsplit, const T* __restrict__ gy, float* __restrict__ part) {
-    __shared__ float red[256];
-    const int k = blockIdx.x, split = blockIdx.y;
-    const long long total = (long long)g.N * g.vol;
-    const long long per = (total + nsplit - 1) / nsplit;
-    const long long j0 = split * per, j1 = min(total, j0 + per);
-    float s = 0.0f;
-    for (long long j = j0 + threadIdx.x; j < j1; j += blockDim.x)
-        s += to_f32(gy[((size_t)(j / g.vol) * g.K + k) * g.vol + (j % g.vol)]);
-    const float t = block_sum(s, red);
-    if (threadIdx.x == 0) part[(size_t)split * g.K + k] = t;
 }
 
 // Sums partials over the splits in order: out[i] = sum_split part[(split * count + i) * stride + off].
