@@ -53,7 +53,7 @@ struct SumGwPlan {
 
 // Stage of eight output channels' operands: weights [channel][tap], {alpha, beta} behind them, then (parallel) the
 // weights of the max branch.  Both tables and the two stages start at multiples of 256 bytes, so that a winner's
-// weight is addressed by putting tap * 4 into the low byte.  (Single-branch layers: alpha and beta only.)
+// weight is addressed by putting tap * 4 into the low byte.  (Single-branch layers have none of them.)
 struct SumStage {
     int coef, w2, stride, bytes;       // offsets of {alpha, beta} and w2, distance of the two stages, bytes of both
 };
@@ -64,7 +64,7 @@ __host__ __device__ inline SumStage sum_stage(int mode, int RS) {
     t.w2 = mode == TCONV_PARALLEL ? (len + 255) / 256 * 256 : 0;
     const int all = mode == TCONV_PARALLEL ? t.w2 + kSgKB * RS * 4 : len;
     t.stride = (all + 255) / 256 * 256;
-    t.bytes = t.stride + all;
+    t.bytes = two_branch(mode) ? t.stride + all : 0;
     return t;
 }
 
@@ -430,7 +430,7 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
         // thread; the rest of a large window's weights are copied then).
         const SumStage lay = sum_stage(g.mode, RS);
         char* stage = smem + pl.smem - lay.bytes;
-        const int nw = AB ? kSgKB * RS : 0, nstage = 2 * kSgKB + nw * (AB && g.mode == TCONV_PARALLEL ? 2 : 1);
+        const int nw = AB ? kSgKB * RS : 0, nstage = BR != 0 ? 0 : 2 * kSgKB + nw * (AB && g.mode == TCONV_PARALLEL ? 2 : 1);
         struct Operand {
             const void* from;      // of the first stage; null: all ones
             int kk, to;            // output channel within the stage, place in it
@@ -465,13 +465,15 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
                 *reinterpret_cast<float*>(to + o.to) = fetch(o, k0);
             }
         };
-        copy(tid, 0, stage);
-        __syncthreads();
+        if constexpr (BR == 0) {
+            copy(tid, 0, stage);
+            __syncthreads();
+        }
         int buf = 0;
         for (int k0 = 0; k0 < g.K; k0 += kSgKB, buf ^= 1) {
             const bool more_k = k0 + kSgKB < g.K;
             float ahead = 0.0f;
-            if (more_k && tid < nstage) ahead = fetch(operand(tid), k0 + kSgKB);
+            if (BR == 0 && more_k && tid < nstage) ahead = fetch(operand(tid), k0 + kSgKB);
             const char* st = stage + buf * lay.stride;
             const unsigned table = (unsigned)__cvta_generic_to_shared(st);
             float s[AB ? 16 : 1];
@@ -488,7 +490,7 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
 #pragma unroll
                     for (int j = 0; j < 4; ++j) gv[j] = k0 + kk < g.K ? gv[j] : 0.0f;
                 }
-                const float2 cf = *reinterpret_cast<const float2*>(st + lay.coef + kk * 8);
+                const float2 cf = BR == 0 ? *reinterpret_cast<const float2*>(st + lay.coef + kk * 8) : make_float2(1.0f, 1.0f);
                 const QuadTaps<WIDE, K3 ? 10 : 8> taps(cq[u]);
                 const QuadWeights<WIDE> wtaps(cq[u]);
                 // one branch: the four pixels' accumulators are distinct, so their loads go out together
@@ -527,12 +529,12 @@ bwd_sum_gx_kernel(Geo g, const void* __restrict__ x, const T* __restrict__ w, co
                 const float v = warp_sum16(s, lane);
                 if (!(lane & 1)) part[buf][warp][lane >> 1] = v;
             }
-            if (more_k) {
+            if (BR == 0 && more_k) {
                 char* to = stage + (buf ^ 1) * lay.stride;
                 if (tid < nstage) *reinterpret_cast<float*>(to + operand(tid).to) = ahead;
                 copy(tid + blockDim.x, k0 + kSgKB, to);
             }
-            __syncthreads();     // this stage is used, the next one and its sums are stored
+            if constexpr (BR == 0) __syncthreads();     // this stage is used, the next one and its sums are stored
             if constexpr (AB) {
                 if (tid < 2 * kSgKB && 2 * k0 + tid < 2 * g.K) {
                     float t = 0.0f;
