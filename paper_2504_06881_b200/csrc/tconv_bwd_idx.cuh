@@ -181,7 +181,7 @@ template <typename T>
 __global__ void __launch_bounds__(256, 2)
 bwd_idx_gx_kernel(Geo g, const T* __restrict__ gy, const int32_t* __restrict__ idx, T* __restrict__ gx, IdxGxPlan pl,
                   unsigned magic_rs, unsigned magic_s) {
-    extern __shared__ float tile[];          // [CB][TH][W], then a dummy word per thread
+    extern __shared__ float tile[];          // [CB][TH][TW], then a dummy word per thread
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int cblk = blockIdx.x % pl.nblk;
     int bt = blockIdx.x / pl.nblk;

@@ -1,6 +1,6 @@
-"""All gradients of 3x3 stride-1 depthwise layers at the sizes where the one-pass backward changes: one strip and
+"""All gradients of 3x3 stride-1 depthwise layers at the sizes where the strips of the backward change: one strip and
 several, a short last strip, widths that are not whole quads, no padding and padding 2 (winners in the padding),
-one image per chunk and several."""
+one image per chunk of the parameter sums and several."""
 import pytest
 
 from paper_2504_06881_b200 import inputs
