@@ -48,11 +48,18 @@ _geoms = tconv.KeptPlans(lambda kind, mode, chan, dtype, stride, pad, dil: _nati
 def _layer(kind, mode, chan, dtype, stride, pad, dil, x, w, w2, alpha, beta, bias):
     """One layer through the native autograd path (csrc/torch_layers.cpp).  Under ``torch.jit.trace`` through the
     Python Function, which a trace records as one operation: of the native path it would record the allocations."""
-    geom = (mode, chan, dtype, tuple(stride), tuple(pad), tuple(dil))
-    if torch.jit.is_tracing():
-        fn = {"dense": TropicalConvFn, "depthwise": TropicalDepthwiseFn, "volume": TropicalConv3dFn}[kind]
-        return fn.apply(x, w, w2, alpha, beta, bias, geom if kind != "depthwise" else (mode,) + geom[2:])
-    return _native.layer(_geoms.get((kind,) + geom, kind, *geom), x, w, w2, alpha, beta, bias)
+    geom = (kind, mode, chan, dtype, stride, pad, dil)
+    try:
+        g = _geoms.get(geom, *geom)
+    except TypeError:            # (geometry set as lists)
+        stride, pad, dil = tuple(stride), tuple(pad), tuple(dil)
+        geom = (kind, mode, chan, dtype, stride, pad, dil)
+        g = _geoms.get(geom, *geom)
+    y = _native.layer(g, x, w, w2, alpha, beta, bias)
+    if y is not None:
+        return y
+    fn = {"dense": TropicalConvFn, "depthwise": TropicalDepthwiseFn, "volume": TropicalConv3dFn}[kind]
+    return fn.apply(x, w, w2, alpha, beta, bias, (mode, dtype, stride, pad, dil) if kind == "depthwise" else geom[1:])
 
 
 class TropicalConvFn(torch.autograd.Function):
