@@ -50,7 +50,7 @@ PROBES_BF16 = {"max_plus": ("bf16x2_add_max", "bf16x2_fma_max", "bf16x2_mix_max"
                "min_plus": ("bf16x2_add_max", "bf16x2_fma_max", "bf16x2_mix_max"),
                "compound": ("bf16x2_add_minmax", "bf16x2_fma_minmax", "bf16x2_mix_minmax"),
                "parallel": ("bf16x2_2add_minmax", "bf16x2_2fma_minmax", "bf16x2_2mix_minmax")}
-# register-only probes of the winner-emitting Sum-form inner loop (sums, extrema, FMA keys, key fold)
+# register-only probes of the winner-emitting Sum-form inner loop (sums, extrema by rows, first equal row and tap)
 WIN_PROBES = {"compound": "f32_win_compound", "parallel": "f32_win_parallel"}
 
 

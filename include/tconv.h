@@ -35,10 +35,9 @@
  *
  * Every function that returns int returns TCONV_OK (0) or a negative
  * tconv_status_t; nothing throws, aborts or prints.  Non-finite inputs are
- * outside the contract.  Winner codes of the fp32 Sum forms (incl. compound and
- * parallel) are recovered from scaled differences of tap sums: they are exact for
- * |x + w| < 2^95 (windows of up to 16 taps) and |x + w| < 2^86 (larger windows);
- * beyond that the outputs y are still exact but winners may be wrong.  There is no
+ * outside the contract.  Winner codes of the depthwise fp32 entry points are recovered
+ * from scaled differences of tap sums: they are exact for |x + w| < 2^95; beyond that the outputs
+ * y are still exact but winners may be wrong.  There is no
  * CPU implementation behind this interface.
  */
 #ifndef TCONV_H

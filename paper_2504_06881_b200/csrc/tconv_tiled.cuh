@@ -15,52 +15,15 @@
 
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "tconv_common.cuh"
+#include "tconv_winners.cuh"
 
 namespace tconv {
 
 // ----------------------------------------------------------------------------------
 // small device helpers
-__device__ __forceinline__ float ext3(float a, float b, float c, bool is_min) {
-    float d;
-    if (is_min) asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    else asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ float ext2(float a, float b, bool is_min) {
-    return is_min ? fminf(a, b) : fmaxf(a, b);
-}
-// {lo, hi} = {x + wlo, x + whi}: one packed fp32 add for two output channels.
-__device__ __forceinline__ void add2(float x, float wlo, float whi, float& lo, float& hi) {
-    unsigned long long xx, ww, tt;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(xx) : "f"(x));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(ww) : "f"(wlo), "f"(whi));
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(tt) : "l"(xx), "l"(ww));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(tt));
-}
-// Extremum of v[0..RS)[h] with 3-input min / max: a fresh chain opens with three values,
-// every later step folds two more.
-template <int RS>
-__device__ __forceinline__ float fold_taps(const float (*v)[2], int h, bool is_min) {
-    float m;
-    if constexpr (RS >= 3) m = ext3(v[0][h], v[1][h], v[2][h], is_min);
-    else if constexpr (RS == 2) m = ext2(v[0][h], v[1][h], is_min);
-    else m = v[0][h];
-#pragma unroll
-    for (int i = 3; i + 1 < RS; i += 2) m = ext3(m, v[i][h], v[i + 1][h], is_min);
-    if constexpr (RS > 3 && ((RS - 3) & 1)) m = ext2(m, v[RS - 1][h], is_min);
-    return m;
-}
-// {c0, c1} = a * {v0, v1} + {c0, c1}: one packed fused multiply-add (scalar a splat)
-__device__ __forceinline__ void fma2s(float a, float v0, float v1, float& c0, float& c1) {
-    unsigned long long aa, vv, cc;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(a));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(vv) : "f"(v0), "f"(v1));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(cc) : "f"(c0), "f"(c1));
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(cc) : "l"(aa), "l"(vv));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(c0), "=f"(c1) : "l"(cc));
-}
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
@@ -240,6 +203,9 @@ template <int S, int DW, int ESIZE = 4> struct TmaShift {
 // the ALU / FMA pipes and want four or more warps per scheduler to hide their latencies.
 constexpr int kMinBlocksSingle = 4;   // single-branch kernels
 constexpr int kMinBlocksWinSum = 3;   // Sum forms that emit winners (168 registers)
+// The same with 5 x 5 windows: three CTAs spill.  N=16 C=64 K=64 32x32, compound 391 -> 370 us, parallel 490 -> 415 us
+// (reading the weights for every pixel anew; with all of them in registers three CTAs take 412 and 1239 us).
+constexpr int kMinBlocksWinWide = 2;
 // Max / Min combine with winners: the running winners live beside the running extrema.  Three CTAs (168 registers,
 // no spills) against two without a bound: N=128 C=64 K=64 32x32 3x3 426 -> 384 us; four CTAs spill, and four
 // channels per thread with five CTAs read the input twice as often (388 us).
@@ -248,7 +214,7 @@ constexpr int kQuadsCarried = 2;      // quads per thread of the carried max-plu
 // STATS (winner-emitting kernels only): also leave the per-tile channel statistics.
 template <int MODE, int CHAN, bool WIN, bool XTMA, bool RAG, int R, int S, int SW, int DW, int Q, int KG, int PW, int TK, bool STATS = false>
 __global__ void __launch_bounds__(KG * PW * 32,
-                                  (WIN && CHAN == CH_SUM) ? kMinBlocksWinSum
+                                  (WIN && CHAN == CH_SUM) ? (R * S > 16 ? kMinBlocksWinWide : kMinBlocksWinSum)
                                   : WIN ? kMinBlocksWinExt
                                   : (MODE == TCONV_COMPOUND || MODE == TCONV_PARALLEL) ? (TK == 4 ? 4 : 1)
                                   : kMinBlocksSingle)
@@ -471,26 +437,19 @@ fwd_tiled_f32_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParams
             const float* wc2 = ws2 + cc * (RS * TILE_K);
 
             if constexpr (WIN && CHAN == CH_SUM) {
-                // Sum forms that emit winners.  Per pair of output channels and per pixel the RS tap
-                // sums stay in registers, feed the extrema, and then give the winning taps on the
-                // FMA pipe: with m the exact extremum, d = (t - m) * 2^32 is computed with one
-                // rounding and is zero exactly for the taps that attain m;
-                // key = |d| * (-2^125) + (2^23 + rank(tap)) equals 2^23 + rank for those taps and is
-                // below 2^23 for every other tap, so the largest key belongs to the lowest winning
-                // tap when rank decreases with the tap, and the low mantissa bits of that key are
-                // rank itself: 15 - tap for the min branch (low nibble of the code), 16 * (15 - tap)
-                // for the max branch (high nibble), both read back with one complement-and-mask.
-                // (a non-zero |d| * 2^125 is at least 256 > 240, the largest rank; |x + w| < 2^95 is assumed.)
-                // Windows above 16 taps use 16-bit codes: rank = 255 - tap (low byte) and
-                // 256 * (255 - tap) (high byte); the scale grows to 2^41 so that a non-zero
-                // |d| * 2^125 (at least 2^17) still exceeds every rank, |x + w| < 2^86 assumed.
+                // Sum forms that emit winners.  Per pair of output channels and per pixel the RS tap sums stay in
+                // registers, give the extrema row by row and then the winning taps (add_winner), which are counted
+                // into floats from 2^23 on: byte (RS > 16: 16 bits) j of the mantissas holds argmin + 16 argmax
+                // (256 argmax) of pixel j.
+                // Bound by the half-rate pipe (71 % of its slots: 16 three-input min / max, 8 compares, 8 selects per
+                // (output, input channel) with two branches) and its dependences: N=128 C=64 K=64 32x32 fp32,
+                // compound 1285 -> 947 us, parallel 1377 -> 1040 us against keys formed from every tap by two packed
+                // FMAs (exact only for |x + w| < 2^95).  Four CTAs per SM, eight or two channels per thread, and
+                // selects as predicated FMAs measured the same or slower.
                 constexpr bool WIDE = RS > 16;
                 constexpr int CW = WIDE ? 2 : 1;             // bytes per code
-                constexpr int RTOP = WIDE ? 255 : 15, RMUL = WIDE ? 256 : 16;
-                constexpr float kS = WIDE ? 2199023255552.0f : 4294967296.0f;   // 2^41 : 2^32
-                constexpr float kH = 4.253529586511731e37f;  // 2^125
-                constexpr float kB = 8388608.0f;             // 2^23
-                constexpr bool DO_MIN = TWO || TAP_MIN, DO_MAX = TWO || !TAP_MIN;
+                constexpr float kUnitMax = WIDE ? 256.0f : 16.0f;
+                constexpr int PPW = WIDE ? 1 : 2;            // pixels counted in one float (16 bits of its mantissa)
                 const int c = ch * p.CC + cc;
                 float av[TK], bv[TK];
                 if constexpr (TWO) {
@@ -499,81 +458,55 @@ fwd_tiled_f32_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParams
                 }
 #pragma unroll
                 for (int kp = 0; kp < TK / 2; ++kp) {
-                    float wa[RS][2], wb[PAR ? RS : 1][2];
-#pragma unroll
-                    for (int tap = 0; tap < RS; ++tap) {
-                        loadn<2>(wc + tap * TILE_K + 2 * kp, wa[tap]);
-                        if constexpr (PAR) loadn<2>(wc2 + tap * TILE_K + 2 * kp, wb[tap]);
-                    }
 #pragma unroll
                     for (int q = 0; q < Q; ++q) {
-                        unsigned packed[2] = {0u, 0u}, packed_hi[2] = {0u, 0u};   // 4 codes per channel (wide: two words)
+                        float cnt[2][4 / PPW];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            float ta[RS][2], tb[PAR ? RS : 1][2];
+                        for (int h = 0; h < 2; ++h)
 #pragma unroll
-                            for (int tap = 0; tap < RS; ++tap) {
-                                const float xv = xr[q][tap / S][j * SW + (tap % S) * DW];
-                                add2(xv, wa[tap][0], wa[tap][1], ta[tap][0], ta[tap][1]);
-                                if constexpr (PAR) add2(xv, wb[tap][0], wb[tap][1], tb[tap][0], tb[tap][1]);
-                            }
-                            const float (*tm)[2] = PAR ? tb : ta;   // sums of the max branch
-                            unsigned bits_min[2] = {0u, 0u}, bits_max[2] = {0u, 0u};
-                            float lo[2] = {0.0f, 0.0f}, hi[2] = {0.0f, 0.0f};
-                            if constexpr (DO_MIN) {
-                                lo[0] = fold_taps<RS>(ta, 0, true);
-                                lo[1] = fold_taps<RS>(ta, 1, true);
-                            }
-                            if constexpr (DO_MAX) {
-                                hi[0] = fold_taps<RS>(tm, 0, false);
-                                hi[1] = fold_taps<RS>(tm, 1, false);
-                            }
+                            for (int i = 0; i < 4 / PPW; ++i) cnt[h][i] = 8388608.0f;
+                        // parallel layers make one pass per branch, so that one set of weights and sums is live
+                        auto pass = [&](auto min_branch, auto max_branch, const float* wsrc) {
+                            constexpr bool DO_MIN = decltype(min_branch)::value, DO_MAX = decltype(max_branch)::value;
+                            float wa[RS][2];
 #pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                float& a = acc[2 * kp + h][q][j];
-                                if constexpr (TWO) {
-                                    a = __fmaf_rn(av[2 * kp + h], lo[h], a);
-                                    a = __fmaf_rn(bv[2 * kp + h], hi[h], a);
-                                } else {
-                                    a = __fadd_rn(a, TAP_MIN ? lo[h] : hi[h]);
+                            for (int tap = 0; tap < RS; ++tap) loadn<2>(wsrc + tap * TILE_K + 2 * kp, wa[tap]);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                float t[RS][2], lo[2] = {0.0f, 0.0f}, hi[2] = {0.0f, 0.0f}, rmin[2][R], rmax[2][R];
+#pragma unroll
+                                for (int tap = 0; tap < RS; ++tap)
+                                    add2(xr[q][tap / S][j * SW + (tap % S) * DW], wa[tap][0], wa[tap][1], t[tap][0], t[tap][1]);
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) {
+                                    const auto th = [&](int tap) { return t[tap][h]; };
+                                    if constexpr (DO_MIN) lo[h] = fold_rows<R, S>(th, true, rmin[h]);
+                                    if constexpr (DO_MAX) hi[h] = fold_rows<R, S>(th, false, rmax[h]);
+                                }
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) {
+                                    float& a = acc[2 * kp + h][q][j];
+                                    if constexpr (TWO) {
+                                        if constexpr (DO_MIN) a = __fmaf_rn(av[2 * kp + h], lo[h], a);
+                                        if constexpr (DO_MAX) a = __fmaf_rn(bv[2 * kp + h], hi[h], a);
+                                    } else {
+                                        a = __fadd_rn(a, TAP_MIN ? lo[h] : hi[h]);
+                                    }
+                                }
+                                const float unit = j % PPW ? 256.0f : 1.0f;
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) {
+                                    const auto th = [&](int tap) { return t[tap][h]; };
+                                    if constexpr (DO_MIN) add_winner<R, S>(th, rmin[h], lo[h], unit, cnt[h][j / PPW]);
+                                    if constexpr (DO_MAX) add_winner<R, S>(th, rmax[h], hi[h], kUnitMax * unit, cnt[h][j / PPW]);
                                 }
                             }
-                            if constexpr (DO_MIN) {
-                                const float e0 = -lo[0] * kS, e1 = -lo[1] * kS;
-                                float key[RS][2];
-#pragma unroll
-                                for (int tap = 0; tap < RS; ++tap) {
-                                    float d0 = e0, d1 = e1;
-                                    fma2s(kS, ta[tap][0], ta[tap][1], d0, d1);             // >= 0
-                                    key[tap][0] = key[tap][1] = kB + (float)(RTOP - tap);
-                                    fma2s(-kH, d0, d1, key[tap][0], key[tap][1]);
-                                }
-                                bits_min[0] = __float_as_uint(fold_taps<RS>(key, 0, false));
-                                bits_min[1] = __float_as_uint(fold_taps<RS>(key, 1, false));
-                            }
-                            if constexpr (DO_MAX) {
-                                const float e0 = -hi[0] * kS, e1 = -hi[1] * kS;
-                                float key[RS][2];
-#pragma unroll
-                                for (int tap = 0; tap < RS; ++tap) {
-                                    float d0 = e0, d1 = e1;
-                                    fma2s(kS, tm[tap][0], tm[tap][1], d0, d1);             // <= 0
-                                    key[tap][0] = key[tap][1] = kB + (float)(RMUL * (RTOP - tap));
-                                    fma2s(kH, d0, d1, key[tap][0], key[tap][1]);
-                                }
-                                bits_max[0] = __float_as_uint(fold_taps<RS>(key, 0, false));
-                                bits_max[1] = __float_as_uint(fold_taps<RS>(key, 1, false));
-                            }
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                unsigned code;
-                                constexpr unsigned MLO = WIDE ? 0x00ffu : 0x0fu, MHI = WIDE ? 0xff00u : 0xf0u;
-                                if constexpr (TWO) code = (~bits_min[h] & MLO) | (~bits_max[h] & MHI);
-                                else code = TAP_MIN ? (~bits_min[h] & MLO) : (~bits_max[h] & MHI);
-                                if constexpr (!WIDE) packed[h] |= code << (8 * j);
-                                else if (j < 2) packed[h] |= code << (16 * j);
-                                else packed_hi[h] |= code << (16 * (j - 2));
-                            }
+                        };
+                        if constexpr (PAR) {
+                            pass(std::true_type(), std::false_type(), wc);
+                            pass(std::false_type(), std::true_type(), wc2);
+                        } else {
+                            pass(std::bool_constant<TWO || TAP_MIN>(), std::bool_constant<TWO || !TAP_MIN>(), wc);
                         }
                         // one byte per (n, k, c, oh, ow): low nibble argmin tap, high nibble argmax tap
                         if (out_row[q] >= 0) {
@@ -583,8 +516,10 @@ fwd_tiled_f32_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParams
                                 if (kt * TILE_K + kl >= g.K) continue;
                                 uint8_t* dst = code_base[q] + ((size_t)kl * g.C + c) * cplane * CW;
                                 if (qcol[q] < g.OW) {   // the quad's 4 codes in one store (rows are padded)
-                                    if constexpr (WIDE) *reinterpret_cast<uint2*>(dst) = make_uint2(packed[h], packed_hi[h]);
-                                    else *reinterpret_cast<unsigned*>(dst) = packed[h];
+                                    const float* w16 = cnt[h];   // 16 bits each
+                                    auto pair = [&](int i) { return __byte_perm(__float_as_uint(w16[i]), __float_as_uint(w16[i + 1]), 0x5410); };
+                                    if constexpr (WIDE) *reinterpret_cast<uint2*>(dst) = make_uint2(pair(0), pair(2));
+                                    else *reinterpret_cast<unsigned*>(dst) = pair(0);
                                 }
                             }
                         }
