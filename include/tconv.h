@@ -35,10 +35,8 @@
  *
  * Every function that returns int returns TCONV_OK (0) or a negative
  * tconv_status_t; nothing throws, aborts or prints.  Non-finite inputs are
- * outside the contract.  Winner codes of the depthwise fp32 entry points are recovered
- * from scaled differences of tap sums: they are exact for |x + w| < 2^95; beyond that the outputs
- * y are still exact but winners may be wrong.  There is no
- * CPU implementation behind this interface.
+ * outside the contract.  There is no CPU
+ * implementation behind this interface.
  */
 #ifndef TCONV_H
 #define TCONV_H
