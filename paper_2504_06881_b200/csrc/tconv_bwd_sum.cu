@@ -29,7 +29,8 @@ int launch_gx_window(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* 
 
 template <typename T, int BR, bool PAIRS, bool WIDE>
 int launch_gw(SumBwdArgs& a, const SumGwPlan& pl, float* part) {
-    auto kern = pl.flat ? bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, true> : bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false>;
+    auto kern = pl.flat ? bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, true, false>
+                : pl.blocks ? bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false, true> : bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false, false>;
     if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
     kern<<<pl.grid, 128, pl.smem, a.st>>>(a.g, (const T*)a.gy, a.codes, part, pl);
     ++a.launches;

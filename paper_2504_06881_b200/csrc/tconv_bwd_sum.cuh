@@ -43,6 +43,7 @@ struct SumGxPlan {
 
 struct SumGwPlan {
     int flat;                      // items run over the flattened (image, quad) space
+    int blocks;                    // an image is whole blocks of 128 quads, and so are the shares
     int splits;                    // shares of a pair's items
     int per;                       // quads (flat) or rounds of 32 quads per share
     int pairs;                     // 1: one table over the pair of winners, 0: one table per branch
@@ -145,6 +146,8 @@ inline bool plan_sum_gw(const Geo& g, SumGwPlan* p) {
         if (best > 0.92) break;
     }
     p->per = (int)((items + s - 1) / s);
+    p->blocks = !p->flat && rpi % 4 == 0;
+    if (p->blocks) p->per = (p->per + 3) / 4 * 4;
     p->splits = (int)((items + p->per - 1) / p->per);
     p->grid = (unsigned)((pairs * p->splits + 3) / 4);
     return true;
@@ -299,6 +302,22 @@ template <> struct QuadWeights<true> {
 __device__ __forceinline__ float load_shared(unsigned at) {
     return *reinterpret_cast<const float*>(__cvta_shared_to_generic(at));
 }
+__device__ __forceinline__ float& at_shared(unsigned at) { return *reinterpret_cast<float*>(__cvta_shared_to_generic(at)); }
+// Address base + tap * 256 of a pixel's bin.  Narrow codes: the nibbles in the high halves of the bytes, and one dot
+// product of bytes picks, scales and adds one of them (7 x 7 x 512 bf16 compound: 724 -> 707 us against a byte
+// permutation and an add; the table over pairs of winners has more bits than a byte's half and keeps those).
+template <bool WIDE> struct BinAddress {
+    QuadTaps<WIDE, 8> t;
+    __device__ __forceinline__ explicit BinAddress(const Codes4<WIDE>& c) : t(c) {}
+    __device__ __forceinline__ unsigned tmin(unsigned base, int j) const { return base + t.tmin(j); }
+    __device__ __forceinline__ unsigned tmax(unsigned base, int j) const { return base + t.tmax(j); }
+};
+template <> struct BinAddress<false> {
+    unsigned lo, hi;
+    __device__ __forceinline__ explicit BinAddress(const Codes4<false>& c) : lo((c.lo << 4) & 0xf0f0f0f0u), hi(c.lo & 0xf0f0f0f0u) {}
+    __device__ __forceinline__ unsigned tmin(unsigned base, int j) const { return __dp4a(lo, 16u << (8 * j), base); }
+    __device__ __forceinline__ unsigned tmax(unsigned base, int j) const { return __dp4a(hi, 16u << (8 * j), base); }
+};
 
 // Branch values z = x + w of a quad as the forward rounds them (one rounded add; bf16: the fp32 sum of two bf16
 // values keeps more than twice their bits, so rounding it equals the bf16 add).
@@ -658,7 +677,13 @@ bwd_sum_edges_kernel(Geo g, const float* __restrict__ part_gx, T* __restrict__ g
 // read-modify-write serves both; the finishing sums over rows / columns of the table give the two
 // histograms.  Else one table per branch.
 // FLAT: the share is a range of the flattened (image, quad) space; else an image is whole rounds of 32 quads.
-template <typename T, int BR, bool PAIRS, bool WIDE, bool FLAT>
+// BLOCKS (not FLAT): an image is a multiple of four rounds, whose operands lie at constant distances.
+// Bound by the shared-memory path (two accesses of the table per item beside the streamed operands) and the issue
+// slots, so what is left out is address arithmetic.  Against one address per round with a test for the end of the
+// image, and (FLAT) a test for the end of the share in every round: N=128 C=64 K=64 32x32 fp32 compound 320 -> 268 us,
+// 8 x 256 x 256 channels 128x256 bf16 7704 -> 6977 us; FLAT: 28 x 28 x 128 bf16 parallel 487 -> 430 us, 7 x 7 x 512
+// bf16 compound 831 -> 707 us, 56 -> 28 fp32 parallel 271 -> 255 us.
+template <typename T, int BR, bool PAIRS, bool WIDE, bool FLAT, bool BLOCKS>
 __global__ void __launch_bounds__(128)
 bwd_sum_gw_kernel(Geo g, const T* __restrict__ gy, const uint8_t* __restrict__ codes, float* __restrict__ part, SumGwPlan pl) {
     extern __shared__ float tabs[];
@@ -669,39 +694,38 @@ bwd_sum_gw_kernel(Geo g, const T* __restrict__ gy, const uint8_t* __restrict__ c
     const int split = (int)(wid / pairs), pair = (int)(wid - (long)split * pairs);
     const int k = pair / g.C, c = pair - k * g.C;
     float* tab = tabs + (size_t)(warp >> 1) * pl.nbins * 64 + (warp & 1) * 32;
-    char* mine = reinterpret_cast<char*>(tab + lane);
-    char* mine_max = mine + (BR == 0 ? g.RS * 256 : 0);      // (one table per branch)
+    // (32-bit shared-memory addresses: 449 -> 430 us on 28 x 28 bf16 parallel against generic pointers)
+    const unsigned mine = (unsigned)__cvta_generic_to_shared(tab + lane);
+    const unsigned mine_max = mine + (BR == 0 ? g.RS * 256 : 0);      // (one table per branch)
     for (int b = 0; b < pl.nbins; ++b) tab[b * 64 + lane] = 0.0f;
     constexpr int CW = WIDE ? 2 : 1;
     const int NQ = g.OH * (g.OW >> 2);
     const size_t plane = (size_t)g.OH * g.OW, gstep = (size_t)g.K * plane, cstep = gstep * g.C * CW;
     const unsigned skip = 16u - (unsigned)g.RS;
-    auto add_two = [&](char* base, unsigned o0, unsigned o1, float g0, float g1) {
-        float* p0 = reinterpret_cast<float*>(base + o0);
-        float* p1 = reinterpret_cast<float*>(base + o1);
+    auto add_two = [&](unsigned p0, unsigned p1, float g0, float g1) {
         // both loads first; where the two bins are one, the second store holds both gradients
-        const float v0 = *p0, v1 = *p1;
+        const float v0 = at_shared(p0), v1 = at_shared(p1);
         const float t0 = v0 + g0;
-        const float t1 = (o0 == o1 ? t0 : v1) + g1;
-        *p0 = t0;
-        *p1 = t1;
+        const float t1 = (p0 == p1 ? t0 : v1) + g1;
+        at_shared(p0) = t0;
+        at_shared(p1) = t1;
     };
     auto add_quad = [&](const float* gv, const Codes4<WIDE>& code) {
         if constexpr (PAIRS) {
             // four bins, one per byte (no borrow crosses a byte: each is at least skip * high nibble)
             const unsigned top = (code.lo >> 4) & 0x0f0f0f0fu, bins = code.lo - skip * top;
-            auto at = [&](int j) { return __byte_perm(bins, 0u, 0x4404u + (unsigned)(j << 4)); };
-            add_two(mine, at(0), at(1), gv[0], gv[1]);
-            add_two(mine, at(2), at(3), gv[2], gv[3]);
+            auto at = [&](int j) { return mine + __byte_perm(bins, 0u, 0x4404u + (unsigned)(j << 4)); };
+            add_two(at(0), at(1), gv[0], gv[1]);
+            add_two(at(2), at(3), gv[2], gv[3]);
         } else {
-            const QuadTaps<WIDE, 8> t(code);
+            const BinAddress<WIDE> bin(code);
             if constexpr (BR != 2) {
-                add_two(mine, t.tmin(0), t.tmin(1), gv[0], gv[1]);
-                add_two(mine, t.tmin(2), t.tmin(3), gv[2], gv[3]);
+                add_two(bin.tmin(mine, 0), bin.tmin(mine, 1), gv[0], gv[1]);
+                add_two(bin.tmin(mine, 2), bin.tmin(mine, 3), gv[2], gv[3]);
             }
             if constexpr (BR != 1) {
-                add_two(mine_max, t.tmax(0), t.tmax(1), gv[0], gv[1]);
-                add_two(mine_max, t.tmax(2), t.tmax(3), gv[2], gv[3]);
+                add_two(bin.tmax(mine_max, 0), bin.tmax(mine_max, 1), gv[0], gv[1]);
+                add_two(bin.tmax(mine_max, 2), bin.tmax(mine_max, 3), gv[2], gv[3]);
             }
         }
     };
@@ -722,26 +746,43 @@ bwd_sum_gw_kernel(Geo g, const T* __restrict__ gy, const uint8_t* __restrict__ c
         const int dn = 32 / NQ, dq = 32 - dn * NQ;
         const size_t gadv = dn * gstep + 4 * dq, cadv = dn * cstep + 4 * dq * CW;
         const size_t gwrap = gstep - plane, cwrap = cstep - plane * CW;
-        auto request = [&](int u) {
+        auto request = [&](int u, bool advance) {
             ahead_g4<T, true>(gp, raw[u]);
             cq[u] = ahead_codes4<WIDE, true>(cp);
-            it += 32;
-            if (it < hi) {
+            if (advance) {
                 q += dq;
                 gp += gadv;
                 cp += cadv;
                 if (q >= NQ) { q -= NQ; gp += gwrap; cp += cwrap; }
             }
         };
+        auto request_to_end = [&](int u) {
+            it += 32;
+            request(u, it < hi);
+        };
 #pragma unroll
-        for (int u = 0; u < HB; ++u) request(u);
-        const int rounds = (hi - lo + 31) / 32;
-        for (int r0 = 0; r0 < rounds; r0 += PF) {
+        for (int u = 0; u < HB; ++u) request_to_end(u);
+        const int rounds = (hi - lo + 31) / 32, full = (hi - lo) / 32;
+        int r0 = 0;
+        // while all that is requested and the round behind it are whole rounds
+        for (; r0 + PF + HB < full; r0 += PF, it += 32 * PF) {
 #pragma unroll
             for (int u = 0; u < PF; ++u) {
                 if (u % HB == 0) {
 #pragma unroll
-                    for (int v = 0; v < HB; ++v) request((u + HB + v) % PF);
+                    for (int v = 0; v < HB; ++v) request((u + HB + v) % PF, true);
+                }
+                float gv[4];
+                unpack_g4<T>(raw[u], gv);
+                add_quad(gv, cq[u]);
+            }
+        }
+        for (; r0 < rounds; r0 += PF) {
+#pragma unroll
+            for (int u = 0; u < PF; ++u) {
+                if (u % HB == 0) {
+#pragma unroll
+                    for (int v = 0; v < HB; ++v) request_to_end((u + HB + v) % PF);
                 }
                 float gv[4];
                 unpack_g4<T>(raw[u], gv);
@@ -751,6 +792,45 @@ bwd_sum_gw_kernel(Geo g, const T* __restrict__ gy, const uint8_t* __restrict__ c
                     for (int j = 0; j < 4; ++j) gv[j] = in ? gv[j] : 0.0f;
                 }
                 add_quad(gv, cq[u]);
+            }
+        }
+    } else if constexpr (BLOCKS) {
+        const int bpi = NQ / 128;                        // blocks of an image; shares are whole blocks
+        const int lo = split * (pl.per / 4), hi = min(g.N * bpi, lo + pl.per / 4);
+        const int n0 = lo / bpi;
+        int left = bpi - (lo - n0 * bpi), more = hi - lo;      // blocks left in the image, in the share
+        const size_t off = (size_t)((lo - n0 * bpi) * 128 + lane) * 4;
+        const T* gp = gy + ((size_t)n0 * g.K + k) * plane + off;
+        const uint8_t* cp = codes + ((((size_t)n0 * g.K + k) * g.C + c) * plane + off) * CW;
+        const size_t gwrap = gstep - plane, cwrap = cstep - plane * CW;
+        auto request = [&](int u0) {                     // (past the share its last block is read again)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                ahead_g4<T, true>(gp + v * 128, raw[u0 + v]);
+                cq[u0 + v] = ahead_codes4<WIDE, true>(cp + v * 128 * CW);
+            }
+            if (--more > 0) {
+                gp += 512;
+                cp += 512 * CW;
+                if (--left == 0) {
+                    left = bpi;
+                    gp += gwrap;
+                    cp += cwrap;
+                }
+            }
+        };
+        request(0);
+        for (int i = lo; i < hi; i += 2) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                if (half && i + 1 >= hi) break;
+                request(half ? 0 : 4);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    float gv[4];
+                    unpack_g4<T>(raw[4 * half + v], gv);
+                    add_quad(gv, cq[4 * half + v]);
+                }
             }
         }
     } else {

@@ -1,0 +1,32 @@
+"""Parameter gradients of the Sum forms where the loops over a share's items change: images of one and of several whole
+blocks of 128 quads, rounds that are not whole blocks, flattened ranges around the eight rounds of a step and their last
+partial round, shares of one block, one or two branches and wide codes."""
+import pytest
+
+from paper_2504_06881_b200 import inputs, tconv
+import parity
+
+pytestmark = pytest.mark.gpu
+
+L = inputs.layer
+LAYERS = [
+    L(1, 1, 16, 32, 1, pad=1),                           # one block
+    L(3, 2, 16, 32, 3, pad=1),                           # three images of one block, an odd number of blocks
+    L(9, 3, 32, 32, 4, pad=1),                           # two blocks an image, several shares
+    L(5, 2, 16, 24, 3, pad=1),                           # three rounds an image: whole rounds, no blocks
+    L(2, 2, 32, 48, 3, pad=1),                           # three blocks an image
+    L(1, 2, 11, 23, 3, pad=1),                           # flattened: 66 quads
+    L(4, 3, 24, 16, 5, pad=0),                           # flattened: 88 quads an image, 11 rounds
+    L(7, 2, 13, 61, 4, pad=1),                           # flattened: shares that start inside an image
+    L(32, 1, 20, 20, 2, pad=1),                          # flattened: 100 rounds, a last one of 4 lanes
+    L(3, 2, 16, 32, 3, R=5, S=5, pad=2),                 # wide codes, one block
+    L(3, 2, 9, 21, 3, R=5, S=5, pad=2),                  # wide codes, flattened
+]
+
+
+@pytest.mark.parametrize("mode", ["compound", "parallel", "max_plus"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_shares(mode, dtype):
+    for i, d in enumerate(LAYERS):
+        parity.check_layer(dict(d, mode=mode, chan="sum", dtype=dtype), None, 2700 + i, recompute=False)
+        assert tconv.tconv_last_kernel() == "bwd_sum", d
