@@ -14,6 +14,7 @@
 #include <type_traits>
 
 #include "tconv_3d.cuh"
+#include "tconv_winners.cuh"
 
 namespace tconv {
 
@@ -70,6 +71,12 @@ __host__ __device__ constexpr bool has_max(int br) { return br != 0; }
 // Output channels per thread: eight while one extremum per output is live, else four.
 __host__ __device__ constexpr int f1_kt(int br, bool win) { return (br >= 2 || win) ? 4 : 8; }
 
+// Resident blocks per SM that the fp32 kernels with winners are compiled for.  Two branches: stride 4 has up to 212
+// registers without a bound (audio opening layer, compound: 318 us; three blocks 279, four 279, parallel 356 / 302 /
+// 335), strides 1 and 2 gain from four in spite of some spills (16 -> 64 channels, k=9: 204 -> 179, k=21 s=2: 162 ->
+// 150 us).  One branch: four at stride 4 (193 -> 175 us), none at 1 and 2 (a bound of three costs them 20 %).
+__host__ __device__ constexpr int f1_blocks(int st, int br) { return br >= 2 ? (st == 4 ? 3 : 4) : (st == 4 ? 4 : 1); }
+
 // Row pitch of the staged signal segment: the window of the last lane ends at 4 * 31 + q4 + 3.
 __host__ __device__ constexpr int f1_xw(int q4) { return (kF1Pos + q4 + 4 + 7) & ~7; }
 
@@ -81,7 +88,7 @@ __host__ __device__ constexpr int f1_xw(int q4) { return (kF1Pos + q4 + 4 + 7) &
 // rounded up to a multiple of four.  WIN: a second copy of the weights by output channel follows,
 // wst[4 * KT][q4 * ST] in the layer's type (twice in parallel mode).
 template <typename T, int ST, int BR, bool WIN>
-__global__ void __launch_bounds__(kF1Threads)
+__global__ void __launch_bounds__(kF1Threads, WIN && sizeof(T) == 4 ? f1_blocks(ST, BR) : 1)
 fwd1d_kernel(Geo3 g, int q4, const T* __restrict__ x, const T* __restrict__ w, const T* __restrict__ w2,
              const float* __restrict__ alpha, const float* __restrict__ beta,
              const float* __restrict__ bias, T* __restrict__ y, void* __restrict__ winners) {
@@ -245,12 +252,15 @@ fwd1d_kernel(Geo3 g, int q4, const T* __restrict__ x, const T* __restrict__ w, c
                 }
             }
         } else {
-            // Winners in two steps.  First the windows are walked in blocks of BQ q (BQ * ST = 4 or
-            // 8 consecutive taps, blocks ascending): a block's extremum replaces the running one only
-            // when it is strictly better, and the block is remembered.  Then, per output and branch,
-            // the taps of the remembered block are formed again, highest first, and the lowest one
-            // that equals the extremum is the winner.
-            constexpr int BQ = ST == 4 ? 2 : 4;
+            // Winners in two steps.  First the windows are walked in blocks of BQ q (fp32: BQ * ST = 4
+            // consecutive taps, bf16: 4 or 8; blocks ascending): a block's extremum replaces the running
+            // one only when it is strictly better, and the block is remembered.  Then, per output and
+            // branch, the taps of the remembered block are formed again and the lowest one that equals the
+            // extremum is the winner.  The second step's loads (each lane its own block: some four passes
+            // of the shared-memory path each) cost fp32 more than remembering twice as many blocks: with
+            // blocks of eight taps, scalar adds and fresh extrema per block the audio opening layer (N=32,
+            // 128 channels, k=80, s=4, compound) took 310 us, now 279 us.
+            constexpr int BQ = PK ? (ST == 4 ? 2 : 4) : 4 / ST;
             const T* xl = xs + 4 * lane;
             int bmn[KT][4], bmx[KT][4];
 #pragma unroll
@@ -356,51 +366,54 @@ fwd1d_kernel(Geo3 g, int q4, const T* __restrict__ x, const T* __restrict__ w, c
                     *reinterpret_cast<Vec<T, 4>*>(r[p] + 4) =
                         *reinterpret_cast<const Vec<T, 4>*>(xl + p * xw + q0 + 4);
                 }
+                // a block's extremum continues the running one, so that one compare says whether it is better
                 float cmn[KT][4], cmx[KT][4];
 #pragma unroll
-                for (int dq = 0; dq < 4; dq += 2) {
-                    if (dq % BQ == 0) {
+                for (int i = 0; i < 4 * ST; i += 2) {            // taps q0 * ST + i and the next
+                    if (i % 4 == 0) {
 #pragma unroll
                         for (int kk = 0; kk < KT; ++kk)
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) { cmn[kk][j] = INFINITY; cmx[kk][j] = -INFINITY; }
+                            for (int j = 0; j < 4; ++j) { cmn[kk][j] = mn[kk][j]; cmx[kk][j] = mx[kk][j]; }
+                    }
+                    const int s0 = q0 * ST + i;
+                    const float* x0 = r[i % ST] + i / ST;
+                    const float* x1 = r[(i + 1) % ST] + (i + 1) / ST;
+                    const Vec<T, KT> wa0 = *reinterpret_cast<const Vec<T, KT>*>(ws + s0 * KB + wv * KT);
+                    const Vec<T, KT> wa1 = *reinterpret_cast<const Vec<T, KT>*>(ws + (s0 + 1) * KB + wv * KT);
+                    Vec<T, KT> wb0 = wa0, wb1 = wa1;
+                    if constexpr (BR == 3) {
+                        wb0 = *reinterpret_cast<const Vec<T, KT>*>(ws2 + s0 * KB + wv * KT);
+                        wb1 = *reinterpret_cast<const Vec<T, KT>*>(ws2 + (s0 + 1) * KB + wv * KT);
                     }
 #pragma unroll
-                    for (int p = 0; p < ST; ++p) {
-                        const int s0 = (q0 + dq) * ST + p, s1 = s0 + ST;
-                        const Vec<T, KT> wa0 = *reinterpret_cast<const Vec<T, KT>*>(ws + s0 * KB + wv * KT);
-                        const Vec<T, KT> wa1 = *reinterpret_cast<const Vec<T, KT>*>(ws + s1 * KB + wv * KT);
-                        Vec<T, KT> wb0 = wa0, wb1 = wa1;
-                        if constexpr (BR == 3) {
-                            wb0 = *reinterpret_cast<const Vec<T, KT>*>(ws2 + s0 * KB + wv * KT);
-                            wb1 = *reinterpret_cast<const Vec<T, KT>*>(ws2 + s1 * KB + wv * KT);
-                        }
+                    for (int kk = 0; kk < KT; kk += 2)
 #pragma unroll
-                        for (int kk = 0; kk < KT; ++kk)
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const float t0 = tap_add(r[p][dq + j], wa0.v[kk]);
-                                const float t1 = tap_add(r[p][dq + 1 + j], wa1.v[kk]);
-                                if constexpr (MIN) cmn[kk][j] = fmin3(cmn[kk][j], t0, t1);
-                                if constexpr (BR == 3) {
-                                    const float u0 = tap_add(r[p][dq + j], wb0.v[kk]);
-                                    const float u1 = tap_add(r[p][dq + 1 + j], wb1.v[kk]);
-                                    cmx[kk][j] = fmax3(cmx[kk][j], u0, u1);
-                                } else if constexpr (MAX) {
-                                    cmx[kk][j] = fmax3(cmx[kk][j], t0, t1);
-                                }
+                        for (int j = 0; j < 4; ++j) {
+                            float t0[2], t1[2];
+                            add2(x0[j], wa0.v[kk], wa0.v[kk + 1], t0[0], t0[1]);
+                            add2(x1[j], wa1.v[kk], wa1.v[kk + 1], t1[0], t1[1]);
+                            if constexpr (MIN) {
+                                cmn[kk][j] = fmin3(cmn[kk][j], t0[0], t1[0]);
+                                cmn[kk + 1][j] = fmin3(cmn[kk + 1][j], t0[1], t1[1]);
                             }
-                    }
-                    if ((dq + 2) % BQ == 0) {   // the block that starts at q0 + dq + 2 - BQ is complete
-                        const int qb = q0 + dq + 2 - BQ;
+                            if constexpr (BR == 3) {
+                                add2(x0[j], wb0.v[kk], wb0.v[kk + 1], t0[0], t0[1]);
+                                add2(x1[j], wb1.v[kk], wb1.v[kk + 1], t1[0], t1[1]);
+                            }
+                            if constexpr (MAX) {
+                                cmx[kk][j] = fmax3(cmx[kk][j], t0[0], t1[0]);
+                                cmx[kk + 1][j] = fmax3(cmx[kk + 1][j], t0[1], t1[1]);
+                            }
+                        }
+                    if (i % 4 == 2) {
+                        const int qb = q0 + (i - 2) / ST;
 #pragma unroll
                         for (int kk = 0; kk < KT; ++kk)
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
-                                if constexpr (MIN)
-                                    if (cmn[kk][j] < mn[kk][j]) { mn[kk][j] = cmn[kk][j]; bmn[kk][j] = qb; }
-                                if constexpr (MAX)
-                                    if (cmx[kk][j] > mx[kk][j]) { mx[kk][j] = cmx[kk][j]; bmx[kk][j] = qb; }
+                                if constexpr (MIN) { bmn[kk][j] = cmn[kk][j] < mn[kk][j] ? qb : bmn[kk][j]; mn[kk][j] = cmn[kk][j]; }
+                                if constexpr (MAX) { bmx[kk][j] = cmx[kk][j] > mx[kk][j] ? qb : bmx[kk][j]; mx[kk][j] = cmx[kk][j]; }
                             }
                     }
                 }
@@ -408,38 +421,26 @@ fwd1d_kernel(Geo3 g, int q4, const T* __restrict__ x, const T* __restrict__ w, c
             const int span = q4 * ST;
             const T* wt = wst + wv * KT * span;
             const T* wt2 = (BR == 3 ? wst2 : wst) + wv * KT * span;
+            auto lowest = [&](const T* wk, int j, int qb, float m) {
+                const T* wq = wk + qb * ST;
+                const T* xq = xl + j + qb;
+                constexpr int NB = BQ * ST;
+                [[maybe_unused]] T wv4[NB];
+                if constexpr (!PK) *reinterpret_cast<Vec<T, 4>*>(wv4) = *reinterpret_cast<const Vec<T, 4>*>(wq);
+                int first = NB - 1;
+#pragma unroll
+                for (int i = NB - 2; i >= 0; --i) {
+                    const float t = tap_add(xq[(i % ST) * xw + i / ST], PK ? wq[i] : wv4[i]);
+                    first = t == m ? i : first;
+                }
+                return qb * ST + first;
+            };
 #pragma unroll
             for (int kk = 0; kk < KT; ++kk)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    if constexpr (MIN) {
-                        const int qb = bmn[kk][j];
-                        const float m = mn[kk][j];
-                        int am = 0;
-#pragma unroll
-                        const T* wq = wt + kk * span + qb * ST;
-                        const T* xq = xl + j + qb;
-#pragma unroll
-                        for (int i = BQ * ST - 1; i >= 0; --i) {
-                            const float t = tap_add(xq[(i % ST) * xw + i / ST], wq[i]);
-                            if (t == m) am = qb * ST + i;
-                        }
-                        amn[kk][j] = am;
-                    }
-                    if constexpr (MAX) {
-                        const int qb = bmx[kk][j];
-                        const float m = mx[kk][j];
-                        int am = 0;
-#pragma unroll
-                        const T* wq = wt2 + kk * span + qb * ST;
-                        const T* xq = xl + j + qb;
-#pragma unroll
-                        for (int i = BQ * ST - 1; i >= 0; --i) {
-                            const float t = tap_add(xq[(i % ST) * xw + i / ST], wq[i]);
-                            if (t == m) am = qb * ST + i;
-                        }
-                        amx[kk][j] = am;
-                    }
+                    if constexpr (MIN) amn[kk][j] = lowest(wt + kk * span, j, bmn[kk][j], mn[kk][j]);
+                    if constexpr (MAX) amx[kk][j] = lowest(wt2 + kk * span, j, bmx[kk][j], mx[kk][j]);
                 }
         }
         // channel combine, channels ascending
