@@ -897,7 +897,7 @@ bwd_sum_gw_kernel(Geo g, const T* __restrict__ gy, const uint8_t* __restrict__ c
 
 // ---------------------------------------------------------------------------------- finish
 // Blocks [0, nb_w): grad_w / grad_w2, 256 / ws (k, c, tap) entries per block; ws slices share the splits and are
-// added in slice order.  The next nb_ab blocks: grad_alpha / grad_beta, 16 (c, k) entries per block; sixteen slices
+// added in slice order.  The next nb_ab blocks: grad_alpha / grad_beta, 256 / as (c, k) entries per block; as slices
 // share the partial rows and are added in slice order.  The rest: grad_bias, a warp per output channel (the sum of a pair's histogram is the sum
 // of grad_y), its lanes added in a fixed tree.  All sums are chains of loads from L2, kept eight deep in flight:
 // N=92 C=3 K=12 23x33 5x5 took 42 us where one thread per channel summed splits x taps values.
@@ -905,7 +905,7 @@ static __global__ void __launch_bounds__(256)
 bwd_sum_finish_kernel(Geo g, int br, int splits, const float* __restrict__ part, int rows, const float* __restrict__ part_ab,
                       const float* __restrict__ alpha, const float* __restrict__ beta, float* __restrict__ gw, float* __restrict__ gw2,
                       float* __restrict__ galpha, float* __restrict__ gbeta, float* __restrict__ gbias, unsigned nb_w,
-                      unsigned nb_ab, int ws) {
+                      unsigned nb_ab, int ws, int as) {
     const size_t pairs = (size_t)g.K * g.C, len = pairs * 2 * g.RS;
     __shared__ float2 red[256];
     if (blockIdx.x < nb_w) {
@@ -950,13 +950,13 @@ bwd_sum_finish_kernel(Geo g, int br, int splits, const float* __restrict__ part,
         if (lane == 0) gbias[k] = s;
         return;
     }
-    const int el = threadIdx.x & 15, sl = threadIdx.x >> 4;
-    const size_t e = (size_t)(blockIdx.x - nb_w) * 16 + el;      // c * K + k
+    const int epb = 256 / as, el = threadIdx.x % epb, sl = threadIdx.x / epb;
+    const size_t e = (size_t)(blockIdx.x - nb_w) * epb + el;      // c * K + k
     const size_t c = e / g.K, k = e - c * g.K;
     float2 s = make_float2(0.0f, 0.0f);
     if (e < pairs) {
 #pragma unroll 8
-        for (int r = sl; r < rows; r += 16) {
+        for (int r = sl; r < rows; r += as) {
             const float2 v = __ldg(reinterpret_cast<const float2*>(part_ab) + r * pairs + e);
             s.x += v.x; s.y += v.y;
         }
@@ -964,7 +964,7 @@ bwd_sum_finish_kernel(Geo g, int br, int splits, const float* __restrict__ part,
     red[threadIdx.x] = s;
     __syncthreads();
     if (sl == 0 && e < pairs) {
-        for (int i = 1; i < 16; ++i) { s.x += red[i * 16 + el].x; s.y += red[i * 16 + el].y; }
+        for (int i = 1; i < as; ++i) { s.x += red[i * epb + el].x; s.y += red[i * epb + el].y; }
         if (galpha) galpha[k * g.C + c] = s.x;
         if (gbeta) gbeta[k * g.C + c] = s.y;
     }
