@@ -238,11 +238,11 @@ dw_fwd3_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, const T*
             const auto tmax = [&](int tap) { return tm[tap]; };
             const float unit = j % 2 ? 256.0f : 1.0f;
             if constexpr (DO_MIN) {
-                mn[j] = fold_rows<3, 3>(tmin, true, rows);
+                mn[j] = WIN ? fold_rows<3, 3>(tmin, true, rows) : dw_fold9(ta, true);
                 if constexpr (WIN) add_winner<3, 3>(tmin, rows, mn[j], unit, cnt[j / 2]);
             }
             if constexpr (DO_MAX) {
-                mx[j] = fold_rows<3, 3>(tmax, false, rows);
+                mx[j] = WIN ? fold_rows<3, 3>(tmax, false, rows) : dw_fold9(tm, false);
                 if constexpr (WIN) add_winner<3, 3>(tmax, rows, mx[j], 16.0f * unit, cnt[j / 2]);
             }
         }
