@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256) alu_probe_kernel(int iters, float seed, f
         // and pixel, nine packed tap sums, their extrema by rows, the channel combine, the winning
         // taps (add_winner) and the code bytes.
         constexpr bool TWOB = (V != PROBE_F32_WIN_SINGLE), PARB = (V == PROBE_F32_WIN_PARALLEL);
-        float x[12], wa[2][9][2], wb[PARB ? 2 : 1][9][2], acc[4][4], al[4], be[4];
+        float x[12], wa[2][9][2], acc[4][4], al[4], be[4];
         unsigned codes = 0u;
         const float dx = seed * 1.0e-3f;
         for (int j = 0; j < 12; ++j) x[j] = seed * (float)(j + threadIdx.x);
@@ -172,7 +172,6 @@ __global__ void __launch_bounds__(256) alu_probe_kernel(int iters, float seed, f
             for (int t = 0; t < 9; ++t)
                 for (int h = 0; h < 2; ++h) {
                     wa[kp][t][h] = seed * (float)(kp * 18 + t * 2 + h + 3);
-                    if (PARB) wb[kp][t][h] = seed * (float)(kp * 18 + t * 2 + h + 5);
                 }
         for (int k = 0; k < 4; ++k) {
             al[k] = seed * (float)(k + 1); be[k] = seed * (float)(k + 2);
@@ -186,7 +185,6 @@ __global__ void __launch_bounds__(256) alu_probe_kernel(int iters, float seed, f
 #pragma unroll
                 for (int t = 0; t < 9; ++t) {
                     TCONV_OPAQUE_F(wa[kp][t][0]); TCONV_OPAQUE_F(wa[kp][t][1]);
-                    if constexpr (PARB) { TCONV_OPAQUE_F(wb[kp][t][0]); TCONV_OPAQUE_F(wb[kp][t][1]); }
                 }
 #pragma unroll
             for (int kp = 0; kp < 2; ++kp) {
@@ -197,7 +195,7 @@ __global__ void __launch_bounds__(256) alu_probe_kernel(int iters, float seed, f
 #pragma unroll
                     for (int t = 0; t < 9; ++t) {
                         add2f(x[j + t], wa[kp][t][0], wa[kp][t][1], ta[t][0], ta[t][1]);
-                        if constexpr (PARB) add2f(x[j + t], wb[kp][t][0], wb[kp][t][1], tb[t][0], tb[t][1]);
+                        if constexpr (PARB) add2f(x[j + t], wa[kp][8 - t][0], wa[kp][8 - t][1], tb[t][0], tb[t][1]);   // (the same registers in another order)
                     }
                     const float (*tm)[2] = PARB ? tb : ta;
                     float lo[2] = {0.0f, 0.0f}, hi[2], rmin[2][3], rmax[2][3];
