@@ -77,8 +77,9 @@ int launch_all(SumBwdArgs& a) {
     const int as = xp.ctas <= 16 && pairs >= 148 * 256 ? 1 : 16;
     const unsigned nb_w = a.gw || a.gw2 ? (unsigned)((pairs * g.RS * ws + 255) / 256) : 0u, nb_ab = ab ? (unsigned)((pairs * as + 255) / 256) : 0u;
     const unsigned nb_bias = a.gbias ? (unsigned)((g.K + 7) / 8) : 0u;
-    bwd_sum_finish_kernel<<<nb_w + nb_ab + nb_bias, 256, 0, a.st>>>(g, br, gp.splits, part, (int)xp.ctas, part_ab,
-                                                            a.alpha, a.beta, a.gw, a.gw2, a.galpha, a.gbeta, a.gbias, nb_w, nb_ab, ws, as);
+    auto finish = as == 1 ? bwd_sum_finish_kernel<1> : bwd_sum_finish_kernel<16>;
+    finish<<<nb_w + nb_ab + nb_bias, 256, 0, a.st>>>(g, br, gp.splits, part, (int)xp.ctas, part_ab, a.alpha, a.beta, a.gw, a.gw2,
+                                                     a.galpha, a.gbeta, a.gbias, nb_w, nb_ab, ws);
     ++a.launches;
     return TCONV_OK;
 }

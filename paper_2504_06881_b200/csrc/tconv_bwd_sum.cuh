@@ -897,15 +897,19 @@ bwd_sum_gw_kernel(Geo g, const T* __restrict__ gy, const uint8_t* __restrict__ c
 
 // ---------------------------------------------------------------------------------- finish
 // Blocks [0, nb_w): grad_w / grad_w2, 256 / ws (k, c, tap) entries per block; ws slices share the splits and are
-// added in slice order.  The next nb_ab blocks: grad_alpha / grad_beta, 256 / as (c, k) entries per block; as slices
-// share the partial rows and are added in slice order.  The rest: grad_bias, a warp per output channel (the sum of a pair's histogram is the sum
-// of grad_y), its lanes added in a fixed tree.  All sums are chains of loads from L2, kept eight deep in flight:
-// N=92 C=3 K=12 23x33 5x5 took 42 us where one thread per channel summed splits x taps values.
-static __global__ void __launch_bounds__(256)
+// added in slice order.  The next nb_ab blocks: grad_alpha / grad_beta, 256 / AS (c, k) entries per block; AS slices
+// share the partial rows and are added in slice order.  The rest: grad_bias, a warp per output channel (the sum of a
+// pair's histogram is the sum of grad_y), its lanes added in a fixed tree.  All sums are chains of loads from L2, kept eight
+// deep in flight: N=92 C=3 K=12 23x33 5x5 took 42 us where one thread per channel summed splits x taps values.  Short
+// blocks, so eight on an SM: 46 registers leave five.  3 -> 36 channels 1 x 15623 N=64 (7872 rows), 400 -> 197 64x45 5x5 N=3
+// (24), 512 x 512 7x7 N=64 (4 rows, one slice): five blocks, an unrolled loop and what eights leave one by one 42, 32 and 55
+// us; a variable number of slices and 32 registers 81, 25 and 24; constant slices, the rest in twos, 32 registers 30, 23, 24.
+template <int AS>
+__global__ void __launch_bounds__(256, 8)
 bwd_sum_finish_kernel(Geo g, int br, int splits, const float* __restrict__ part, int rows, const float* __restrict__ part_ab,
                       const float* __restrict__ alpha, const float* __restrict__ beta, float* __restrict__ gw, float* __restrict__ gw2,
                       float* __restrict__ galpha, float* __restrict__ gbeta, float* __restrict__ gbias, unsigned nb_w,
-                      unsigned nb_ab, int ws, int as) {
+                      unsigned nb_ab, int ws) {
     const size_t pairs = (size_t)g.K * g.C, len = pairs * 2 * g.RS;
     __shared__ float2 red[256];
     if (blockIdx.x < nb_w) {
@@ -950,21 +954,19 @@ bwd_sum_finish_kernel(Geo g, int br, int splits, const float* __restrict__ part,
         if (lane == 0) gbias[k] = s;
         return;
     }
-    const int epb = 256 / as, el = threadIdx.x % epb, sl = threadIdx.x / epb;
-    const size_t e = (size_t)(blockIdx.x - nb_w) * epb + el;      // c * K + k
+    constexpr int EPB = 256 / AS;
+    const int el = threadIdx.x % EPB, sl = threadIdx.x / EPB;
+    const size_t e = (size_t)(blockIdx.x - nb_w) * EPB + el;      // c * K + k
     const size_t c = e / g.K, k = e - c * g.K;
     float2 s = make_float2(0.0f, 0.0f);
     if (e < pairs) {
-#pragma unroll 8
-        for (int r = sl; r < rows; r += as) {
-            const float2 v = __ldg(reinterpret_cast<const float2*>(part_ab) + r * pairs + e);
-            s.x += v.x; s.y += v.y;
-        }
+        const float2* at = reinterpret_cast<const float2*>(part_ab) + sl * pairs + e;
+        s = sum_in_order<8, float2>((rows - sl + AS - 1) / AS, [&](int i) { return __ldg(at + (size_t)i * AS * pairs); });
     }
     red[threadIdx.x] = s;
     __syncthreads();
     if (sl == 0 && e < pairs) {
-        for (int i = 1; i < as; ++i) { s.x += red[i * epb + el].x; s.y += red[i * epb + el].y; }
+        for (int i = 1; i < AS; ++i) { s.x += red[i * EPB + el].x; s.y += red[i * EPB + el].y; }
         if (galpha) galpha[k * g.C + c] = s.x;
         if (gbeta) gbeta[k * g.C + c] = s.y;
     }

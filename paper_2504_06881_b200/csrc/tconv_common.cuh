@@ -82,6 +82,30 @@ inline cudaError_t allow_smem_ptr(const void* kern, int bytes) {
 }
 template <typename F> inline cudaError_t allow_smem(F* kern, int bytes) { return allow_smem_ptr((const void*)kern, bytes); }
 
+// load(0) + ... + load(n - 1) in that order, U loads in flight, the rest in twos.
+__device__ __forceinline__ void accumulate(float& s, float v) { s += v; }
+__device__ __forceinline__ void accumulate(float2& s, float2 v) { s.x += v.x; s.y += v.y; }
+template <int U, typename V, typename Load>
+__device__ __forceinline__ V sum_in_order(int n, Load load) {
+    V s = {};
+    int i = 0;
+    for (; i + U <= n; i += U) {
+        V v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = load(i + u);
+#pragma unroll
+        for (int u = 0; u < U; ++u) accumulate(s, v[u]);
+    }
+#pragma unroll 1
+    for (; i < n; i += 2) {
+        const bool two = i + 1 < n;
+        const V v = load(i), w = load(two ? i + 1 : i);
+        accumulate(s, v);
+        if (two) accumulate(s, w);
+    }
+    return s;
+}
+
 // Deterministic block-wide sum (fixed tree): every thread passes its partial,
 // thread 0 receives the total.  `red` holds blockDim.x floats.
 __device__ __forceinline__ float block_sum(float v, float* red) {

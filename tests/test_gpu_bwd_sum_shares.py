@@ -1,6 +1,6 @@
-"""Parameter gradients of the Sum forms where the loops over a share's items change: images of one and of several whole
-blocks of 128 quads, rounds that are not whole blocks, flattened ranges around the eight rounds of a step and their last
-partial round, shares of one block, one or two branches and wide codes."""
+"""Parameter gradients of the Sum forms where the loops over a share's items and over the partial rows change: images of one
+and of several whole blocks of 128 quads, rounds that are not whole blocks, flattened ranges around the eight rounds of a step
+and their last partial round, shares of one block, one or two branches and wide codes; slices of no row to seventeen."""
 import pytest
 
 from paper_2504_06881_b200 import inputs, tconv
@@ -30,3 +30,10 @@ def test_shares(mode, dtype):
     for i, d in enumerate(LAYERS):
         parity.check_layer(dict(d, mode=mode, chan="sum", dtype=dtype), None, 2700 + i, recompute=False)
         assert tconv.tconv_last_kernel() == "bwd_sum", d
+
+
+@pytest.mark.parametrize("N", [1, 4, 5, 30, 32, 33, 129, 144, 161, 272])
+def test_partial_rows(N):
+    """4, 16, 20, 120, 128, 132 rows of grad_alpha / grad_beta (four tiles an image), then one an image, in sixteen slices."""
+    parity.check_layer(dict(L(N, 2, 16, 64, 5, pad=1), mode="compound", chan="sum", dtype="f32"), None, 2800 + N, recompute=False)
+    assert tconv.tconv_last_kernel() == "bwd_sum"
