@@ -71,11 +71,15 @@ __host__ __device__ constexpr bool has_max(int br) { return br != 0; }
 // Output channels per thread: eight while one extremum per output is live, else four.
 __host__ __device__ constexpr int f1_kt(int br, bool win) { return (br >= 2 || win) ? 4 : 8; }
 
-// Resident blocks per SM that the fp32 kernels with winners are compiled for.  Two branches: stride 4 has up to 212
-// registers without a bound (audio opening layer, compound: 318 us; three blocks 279, four 279, parallel 356 / 302 /
-// 335), strides 1 and 2 gain from four in spite of some spills (16 -> 64 channels, k=9: 204 -> 179, k=21 s=2: 162 ->
-// 150 us).  One branch: four at stride 4 (193 -> 175 us), none at 1 and 2 (a bound of three costs them 20 %).
-__host__ __device__ constexpr int f1_blocks(int st, int br) { return br >= 2 ? (st == 4 ? 3 : 4) : (st == 4 ? 4 : 1); }
+// Resident blocks per SM that the kernels with winners are compiled for, 0: as the compiler sees fit (about four; a bound
+// of one lets it request the second step's loads far ahead, with 136 to 212 registers and half the blocks).  fp32 gains
+// from a bound where the second step is long: audio opening layer (k=80, stride 4), without one, three, four blocks
+// compound 312 / 271 / 267 us, parallel 349 / 296 / 329, max-plus 177 / 177 / 162.  16 -> 64 channels, N=16, k=9 / k=21
+// stride 2, bound of one, none, four: fp32 max-plus 135, 118, 119 / 111, 86, 89, compound 226, 194, 175 / 162, 159, 147;
+// bf16 max-plus 115, 97, 98 / 107, 86, 86, compound 159, 148, 154 / 161, 136, 136, parallel 170, 153, 160 / 173, 148, 152.
+__host__ __device__ constexpr int f1_blocks(int esize, int st, int br) {
+    return esize == 2 || (br < 2 && st < 4) ? 0 : br >= 2 && st == 4 ? 3 : 4;
+}
 
 // Row pitch of the staged signal segment: the window of the last lane ends at 4 * 31 + q4 + 3.
 __host__ __device__ constexpr int f1_xw(int q4) { return (kF1Pos + q4 + 4 + 7) & ~7; }
@@ -88,7 +92,7 @@ __host__ __device__ constexpr int f1_xw(int q4) { return (kF1Pos + q4 + 4 + 7) &
 // rounded up to a multiple of four.  WIN: a second copy of the weights by output channel follows,
 // wst[4 * KT][q4 * ST] in the layer's type (twice in parallel mode).
 template <typename T, int ST, int BR, bool WIN>
-__global__ void __launch_bounds__(kF1Threads, WIN && sizeof(T) == 4 ? f1_blocks(ST, BR) : 1)
+__global__ void __launch_bounds__(kF1Threads, WIN ? f1_blocks(sizeof(T), ST, BR) : 1)
 fwd1d_kernel(Geo3 g, int q4, const T* __restrict__ x, const T* __restrict__ w, const T* __restrict__ w2,
              const float* __restrict__ alpha, const float* __restrict__ beta,
              const float* __restrict__ bias, T* __restrict__ y, void* __restrict__ winners) {

@@ -1,8 +1,19 @@
 """Kernel instances whose speed hangs on how many blocks an SM holds stay within the registers that allows, without
 spilling to get there."""
+import pytest
+
 from nvcc_probe import resources
 
 FILE = 65536     # registers of an SM
+
+
+@pytest.mark.parametrize("dtype", ["float", "__nv_bfloat16"])
+def test_1d_forward_with_winners(dtype):
+    """Four blocks of 128 threads; three at stride 4 with two branches."""
+    most = {f"fwd1d_kernel<{dtype}, {st}, {br}, true>": FILE // 128 // (3 if st == 4 and br == 3 else 4)
+            for st in (1, 2, 4) for br in (1, 3)}
+    got = resources("tconv_1d.cuh", list(most))
+    assert all(got[k][0] <= most[k] // 8 * 8 for k in most), got
 
 
 def test_finishing_sum():
