@@ -773,27 +773,31 @@ dw_bwd_params_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, co
     }
 }
 
-// Resident blocks per SM the kernel below is compiled for.  The fp32 parallel kernel at stride 1 holds two sets of weights
-// and four input rows: with three blocks it spills (164 us against 124 at N=64 C=144 56x56); all others gain from the third
-// (bf16 compound 176 -> 108 us).
-__host__ __device__ constexpr int dw_params_blocks(int esize, bool par, int sw) { return esize == 4 && par && sw == 1 ? 2 : 3; }
+// Resident blocks per SM the kernel below is compiled for: three, two where both sets of weights and the wide rows of
+// stride 2 would spill with three (bf16 rows in whole vectors spill 24 bytes and still gain).  N=64 C=144, the fewest
+// chunks that fill one round, three against two blocks: 56x56 fp32 compound 93 / 116 us, parallel 104 / 121, stride 2
+// compound 40 / 46, bf16 parallel 113 / 142, stride 2 48 / 53; but fp32 parallel stride 2 51 / 46, 57x57 72 / 58, bf16
+// 57x57 66 / 59.
+__host__ __device__ constexpr int dw_params_blocks(int esize, bool par, int sw, bool vec) {
+    return par && sw == 2 && !(esize == 2 && vec) ? 2 : 3;
+}
 
 // Parameter gradients for 3x3 windows, dilation 1, stride SW: the same strips and register window
 // as the forward.  The branch values of grad_alpha / grad_beta are the extrema recomputed from the
 // window (no gathers); the per-tap sums take the winners from the codes.  CTA (c, chunk) walks the
 // strips of its images; accumulators and reduction as in dw_bwd_params_kernel.
-// Bound by latency: every output adds to two dependent table entries.  The entries of two outputs and both branches are
-// read together, the gradients and codes of the next row requested ahead (fp32 at stride 1: its input row too).
-// N=64 C=144 56x56, with the chunk count of dw_chunks: fp32 compound 110 -> 89 us, parallel 148 -> 124, max-plus
-// 81 -> 60; stride 2 compound 58 -> 46; bf16 compound 128 -> 108, parallel 188 -> 122.
+// Bound by latency: every output adds to two dependent table entries, and what hides it is resident warps.  One branch
+// has the registers to request the gradients and codes of the next row ahead: N=64 C=144 56x56 max-plus fp32 66 -> 58
+// us, bf16 50 -> 48.  Two branches lose by it (fp32 compound 93 -> 107, bf16 parallel 113 -> 136), as by reading the
+// entries of two outputs together (93 -> 99) and by a row of inputs ahead (57x57: 114 -> 134).
 template <typename T, int BR, bool PAR, int SW, bool VEC>
-__global__ void __launch_bounds__(256, dw_params_blocks(sizeof(T), PAR, SW))
+__global__ void __launch_bounds__(256, dw_params_blocks(sizeof(T), PAR, SW, VEC))
 dw_bwd_params3_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, const T* __restrict__ w2,
                       const T* __restrict__ gy, const uint8_t* __restrict__ codes,
                       float* __restrict__ partial, int nchunks, int need_ab, int QPR, int strips) {
     constexpr int RT = kDwRT;
     constexpr int L = 3 * SW + 3;
-    constexpr bool PACKED = sizeof(T) == 2 && SW == 1, AHEAD = sizeof(T) == 4 && SW == 1;
+    constexpr bool PACKED = sizeof(T) == 2 && SW == 1, AHEAD = BR != 0;
     extern __shared__ float col[];   // [kDwAcc][256]
     const int c = blockIdx.x, chunk = blockIdx.y, tid = threadIdx.x;
     for (int e = tid; e < kDwAcc * 256; e += 256) col[e] = 0.0f;
@@ -821,14 +825,12 @@ dw_bwd_params3_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, c
         const uint8_t* cp = codes + nc * plane + ow0;
         const bool full = (ow0 + 3 < g.OW) && ((g.OW & 3) == 0);
         const int ih0 = oh0 * SW - g.ph, c0 = ow0 * SW - g.pw;
-        // the gradients and codes of output row k + 1 and (AHEAD) its input rows are requested before row k is computed
-        constexpr int WR = AHEAD ? 4 : 3;
-        T win[WR][L];
+        T win[3][L];
         const unsigned cmask = need_ab ? dw_col_mask(c0, L, g.W) : 0u;
         const T* rp0 = x + nc * (size_t)g.H * g.W + (ptrdiff_t)ih0 * g.W + c0;
         auto load = [&](int rho) {
             const int ih = ih0 + rho;
-            dw_load_row<T, L, VEC>(rp0 + rho * g.W, need_ab && ih >= 0 && ih < g.H, cmask, win[rho % WR]);
+            dw_load_row<T, L, VEC>(rp0 + rho * g.W, need_ab && ih >= 0 && ih < g.H, cmask, win[rho % 3]);
         };
         float gnext[4];
         unsigned cnext;
@@ -851,24 +853,19 @@ dw_bwd_params3_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, c
         };
         load(0);
         load(1);
-        if constexpr (AHEAD) load(2);
-        load_out(oh0);
+        if constexpr (AHEAD) load_out(oh0);
 #pragma unroll
         for (int k = 0; k < RT; ++k) {
             const int oh = oh0 + k;
             if (oh >= g.OH) break;
-            if constexpr (!AHEAD) {
 #pragma unroll
-                for (int rho = (k == 0 ? 2 : (k - 1) * SW + 3); rho <= k * SW + 2; ++rho) load(rho);
-            }
+            for (int rho = (k == 0 ? 2 : (k - 1) * SW + 3); rho <= k * SW + 2; ++rho) load(rho);
+            if constexpr (!AHEAD) load_out(oh);
             float gq[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) gq[j] = gnext[j];
             const unsigned cq = cnext;
-            if (k + 1 < RT && oh + 1 < g.OH) {
-                if constexpr (AHEAD) load(k + 3);
-                load_out(oh + 1);
-            }
+            if (AHEAD && k + 1 < RT && oh + 1 < g.OH) load_out(oh + 1);
             // bf16 at stride 1: the branch values of the four outputs on packed pairs, as in the forward
             float bmn[4] = {0.0f, 0.0f, 0.0f, 0.0f}, bmx[4] = {0.0f, 0.0f, 0.0f, 0.0f};
             if constexpr (PACKED) {
@@ -878,7 +875,7 @@ dw_bwd_params3_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, c
                         unsigned ta[9], tb[PAR ? 9 : 1];
 #pragma unroll
                         for (int tap = 0; tap < 9; ++tap) {
-                            const T* row = win[(k + tap / 3) % WR];
+                            const T* row = win[(k + tap / 3) % 3];
                             const int i = 2 * pr + tap % 3;
                             const unsigned xv = (unsigned)__bfloat16_as_ushort(row[i]) |
                                                 ((unsigned)__bfloat16_as_ushort(row[i + 1]) << 16);
@@ -899,29 +896,14 @@ dw_bwd_params3_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, c
                     }
                 }
             }
-            // the tables' accesses of two outputs and both branches together (a column past the row adds zero)
-#pragma unroll
-            for (int j = 0; j < 4; j += 2) {
-                const unsigned c0q = cq >> (8 * j), c1q = c0q >> 8;
-                float* p0 = mine + (c0q & 15u) * 256;
-                float* p1 = mine + (c1q & 15u) * 256;
-                float* q0 = mine + (16 + ((c0q >> 4) & 15u)) * 256;
-                float* q1 = mine + (16 + ((c1q >> 4) & 15u)) * 256;
-                float v0 = 0.0f, v1 = 0.0f, u0 = 0.0f, u1 = 0.0f;
-                if (BR == 0 || BR == 1) { v0 = *p0; v1 = *p1; }
-                if (BR == 0 || BR == 2) { u0 = *q0; u1 = *q1; }
-                v0 += gq[j];
-                u0 += gq[j];
-                v1 = (p0 == p1 ? v0 : v1) + gq[j + 1];
-                u1 = (q0 == q1 ? u0 : u1) + gq[j + 1];
-                if (BR == 0 || BR == 1) { *p0 = v0; *p1 = v1; }
-                if (BR == 0 || BR == 2) { *q0 = u0; *q1 = u1; }
-                ss += gq[j] + gq[j + 1];
-            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 if (!full && ow0 + j >= g.OW) continue;
                 const float gv = gq[j];
+                const unsigned code = (cq >> (8 * j)) & 0xffu;
+                ss += gv;
+                if (BR == 0 || BR == 1) mine[(code & 15u) * 256] += gv;
+                if (BR == 0 || BR == 2) mine[(16 + (code >> 4)) * 256] += gv;
                 if (need_ab) {
                     if constexpr (PACKED) {
                         if (BR == 0 || BR == 1) sa = __fmaf_rn(gv, bmn[j], sa);
@@ -930,7 +912,7 @@ dw_bwd_params3_kernel(Geo g, const T* __restrict__ x, const T* __restrict__ w, c
                         float ta[9], tb[PAR ? 9 : 1];
 #pragma unroll
                         for (int tap = 0; tap < 9; ++tap) {
-                            const T xv = win[(k * SW + tap / 3) % WR][j * SW + tap % 3];
+                            const T xv = win[(k * SW + tap / 3) % 3][j * SW + tap % 3];
                             ta[tap] = tap_add(xv, wa[tap]);
                             if constexpr (PAR) tb[tap] = tap_add(xv, wb[tap]);
                         }

@@ -16,6 +16,16 @@ def test_1d_forward_with_winners(dtype):
     assert all(got[k][0] <= most[k] // 8 * 8 for k in most), got
 
 
+@pytest.mark.parametrize("dtype", ["float", "__nv_bfloat16"])
+def test_depthwise_parameter_gradients(dtype):
+    """Three blocks of 256 threads where they do not spill, two elsewhere: at most 32 bytes."""
+    names = [f"dw_bwd_params3_kernel<{dtype}, {br}, {par}, {sw}, {vec}>" for br, par in ((0, "false"), (0, "true"), (2, "false"))
+             for sw in (1, 2) for vec in ("true", "false")]
+    got = resources("tconv_depthwise.cuh", names)
+    assert all(regs <= FILE // 256 // 2 and spilled <= 32 for regs, spilled in got.values()), got
+    assert all(got[k][0] <= 80 for k in names if "true, 2" not in k), got
+
+
 def test_finishing_sum():
     """Eight blocks of 256 threads."""
     got = resources("tconv_bwd_sum.cuh", ["bwd_sum_finish_kernel<1>", "bwd_sum_finish_kernel<16>"])
