@@ -1,6 +1,5 @@
 // Host side of the C ABI declared in tconv.h: descriptor validation, workspace
 // accounting, kernel selection and launch.  No device memory is allocated here.
-#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -363,24 +362,6 @@ int make_dw_geo(const tconv_desc_t* d, Geo* g) {
     return TCONV_OK;
 }
 
-// Chunks of the per-channel reduction: enough CTAs to fill the GPU, at least 1024 items each; among up to four times
-// as many (no more than images) the count whose rounds of three resident CTAs per SM take the fewest steps of 256
-// strips of 4 columns x 6 rows (N=64 C=144 56x56: 3 instead of 5 chunks, one round instead of two).
-int dw_chunks(const Geo& g) {
-    const long items = (long)g.N * g.OH * g.OW;
-    long n = (592 + g.C - 1) / g.C;
-    const long most = (items + 1023) / 1024;
-    if (n > most) n = most;
-    if (n < 1) n = 1;
-    const long last = std::min(std::min(4 * n, most), (long)g.N);
-    long best = n;
-    const long sq = (long)((g.OW + 3) / 4) * ((g.OH + kDwRT - 1) / kDwRT);
-    auto cost = [&](long c) { return ((long)g.C * c + 443) / 444 * (((g.N + c - 1) / c * sq + 255) / 256); };
-    for (long c = n / 2 > 0 ? n / 2 : 1; c <= last; ++c)
-        if (cost(c) < cost(best)) best = c;
-    return (int)best;
-}
-
 template <typename T>
 int dw_forward_t(const Geo& g, const void* x, const void* w, const void* w2, const float* alpha,
                  const float* beta, const float* bias, void* y, void* winners, cudaStream_t st) {
@@ -488,7 +469,8 @@ int dw_backward_t(const Geo& g, const void* x, const void* w, const void* w2, co
         g_launches += 1;
     }
     if (gw || gw2 || galpha || gbeta || gbias) {
-        const int nch = dw_chunks(g);
+        const DwParamsPlan plan = plan_dw_params(g, (int)sizeof(T));
+        const int nch = plan.chunks;
         const dim3 grid((unsigned)g.C, (unsigned)nch);
         const size_t smem = (size_t)kDwAcc * 256 * sizeof(float);
         const int need_ab = (twob && (galpha || gbeta)) ? 1 : 0;
@@ -499,12 +481,9 @@ int dw_backward_t(const Geo& g, const void* x, const void* w, const void* w2, co
             return cuda_fail(cudaGetLastError());                                                    \
         kern<<<grid, 256, smem, st>>>(g, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, codes, partial, nch, need_ab); \
     }
-        const bool k3 = g.R == 3 && g.S == 3 && g.dh == 1 && g.dw == 1 && g.sh == g.sw && (g.sw == 1 || g.sw == 2) &&
-                        nch <= g.N && g.OH * g.OW >= 100;   // tiny planes: too few strips per image
-        if (k3) {
+        if (plan.strips) {
             // 3x3 windows: strips over a register window, the chunks are ranges of images
             const int QPR3 = (g.OW + 3) / 4, strips3 = (g.OH + kDwRT - 1) / kDwRT;
-            const bool vec3 = (g.pw == 1 && (g.W & 3) == 0);
 #define TCONV_DW_P3(BR, PARV, SWV, VECV)                                                              \
     {                                                                                                \
         auto kern = dw_bwd_params3_kernel<T, BR, PARV, SWV, VECV>;                                   \
@@ -513,7 +492,7 @@ int dw_backward_t(const Geo& g, const void* x, const void* w, const void* w2, co
         kern<<<grid, 256, smem, st>>>(g, (const T*)x, (const T*)w, (const T*)w2, (const T*)gy, codes, partial, nch, \
                                       need_ab, QPR3, strips3);                                       \
     }
-#define TCONV_DW_P3V(BR, PARV, SWV) { if (vec3) TCONV_DW_P3(BR, PARV, SWV, true) else TCONV_DW_P3(BR, PARV, SWV, false) }
+#define TCONV_DW_P3V(BR, PARV, SWV) { if (plan.vec) TCONV_DW_P3(BR, PARV, SWV, true) else TCONV_DW_P3(BR, PARV, SWV, false) }
 #define TCONV_DW_P3S(BR, PARV) { if (g.sw == 1) TCONV_DW_P3V(BR, PARV, 1) else TCONV_DW_P3V(BR, PARV, 2) }
             if (br == 0) { if (par) TCONV_DW_P3S(0, true) else TCONV_DW_P3S(0, false) }
             else if (br == 1) TCONV_DW_P3S(1, false)
@@ -684,7 +663,7 @@ size_t tconv_dw_winner_bytes(const tconv_desc_t* desc) {
 size_t tconv_dw_workspace_bytes(const tconv_desc_t* desc, int backward) {
     Geo g;
     if (make_dw_geo(desc, &g) != TCONV_OK || !backward) return 0;
-    return align_up((size_t)g.N * g.C * g.OH * g.OW, 256) + (size_t)dw_chunks(g) * g.C * kDwAcc * sizeof(float) + 256;
+    return align_up((size_t)g.N * g.C * g.OH * g.OW, 256) + (size_t)plan_dw_params(g, desc->dtype == TCONV_F32 ? 4 : 2).chunks * g.C * kDwAcc * sizeof(float) + 256;
 }
 
 int tconv_dw_forward(const tconv_desc_t* desc, const void* x, const void* w, const void* w2,

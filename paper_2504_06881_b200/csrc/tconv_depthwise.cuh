@@ -782,6 +782,58 @@ __host__ __device__ constexpr int dw_params_blocks(int esize, bool par, int sw, 
     return par && sw == 2 && !(esize == 2 && vec) ? 2 : 3;
 }
 
+// Which kernel sums the parameter gradients of a layer, and the chunks (blocks per channel) of its range.
+struct DwParamsPlan {
+    int strips;      // 1: dw_bwd_params3_kernel, chunks of images; 0: dw_bwd_params_kernel, chunks of outputs
+    int vec;         // strips: rows are read in whole vectors
+    int chunks;
+};
+// Chunks of a channel's range: among the fewest that fill one, two, ... rounds of the places of resident blocks those with
+// the least rounds x half-steps, where a block's start and end (clearing and summing the tables) weigh `ends`.  A chunk
+// is whole units of `each` items, a step takes `step` items.  The steps of a count are also those of fewer chunks; these
+// are taken, but no SM goes without a block that a step of items is there for.
+inline int dw_chunks(long channels, long places, long units, long each, long step, long ends) {
+    long best = 0, chunks = 1;
+    for (long r = (channels + places - 1) / places, i = 0; i < 8; ++r, ++i) {
+        long c = places * r / channels;
+        if (c > units) c = units;
+        const long steps = ((units + c - 1) / c * each + step - 1) / step, per = steps * step / each;
+        long least = 148 / channels;
+        if (least > units * each / step) least = units * each / step;
+        if (least > c) least = c;
+        c = (units + per - 1) / per;
+        if (c < least) c = least;
+        const long cost = (channels * c + places - 1) / places * (2 * steps + ends);
+        if (best == 0 || cost < best) {
+            best = cost;
+            chunks = c;
+        }
+        if (steps == 1 || c == units) break;
+    }
+    return (int)chunks;
+}
+// The strips kernel takes 3x3 windows of planes that give its threads work (100 outputs) where there are images for half as
+// many chunks as the any-window kernel would have.  Its work is counted in the strips of a warp, its ends weigh as one
+// strip of every thread (N=64 fp32 compound: C=144 56x56 3 chunks 93 us, 5 in two rounds 110; C=296 14x14 1 chunk 24, 3 in
+// two rounds 29; N=6 C=64 56x56: 6 chunks 7.5, any-window kernel 12.8).  The any-window kernel has four blocks resident and takes 1024 outputs a step,
+// its ends are some two steps (7x7, N=128 C=84 fp32 compound: 7 chunks 7.2 us, 3 chunks 8.0; N=64 C=160 max-plus: 2
+// chunks 5.1, 4 in two rounds 6.7; 28x28 dilation 2 N=64 C=296 max-plus: 2 chunks 31, 3 in two rounds 40).
+inline DwParamsPlan plan_dw_params(const Geo& g, int esize) {
+    DwParamsPlan p;
+    const long items = (long)g.N * g.OH * g.OW, full = (592 + g.C - 1) / g.C, most = (items + 1023) / 1024;
+    const bool images = 2 * (long)g.N >= (full < most ? full : most);
+    p.vec = g.pw == 1 && (g.W & 3) == 0;
+    p.strips = g.R == 3 && g.S == 3 && g.dh == 1 && g.dw == 1 && g.sh == g.sw && (g.sw == 1 || g.sw == 2) && images &&
+               g.OH * g.OW >= 100;
+    if (p.strips) {
+        const long places = 148L * dw_params_blocks(esize, g.mode == TCONV_PARALLEL, g.sw, p.vec);
+        p.chunks = dw_chunks(g.C, places, g.N, (long)((g.OW + 3) / 4) * ((g.OH + kDwRT - 1) / kDwRT), 32, 16);
+    } else {
+        p.chunks = dw_chunks(g.C, 592, items, 1, 1024, 4);
+    }
+    return p;
+}
+
 // Parameter gradients for 3x3 windows, dilation 1, stride SW: the same strips and register window
 // as the forward.  The branch values of grad_alpha / grad_beta are the extrema recomputed from the
 // window (no gathers); the per-tap sums take the winners from the codes.  CTA (c, chunk) walks the
@@ -948,8 +1000,10 @@ __global__ void dw_bwd_finish_kernel(Geo g, const float* __restrict__ partial, i
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.C * kDwAcc) return;
     const int c = i / kDwAcc, a = i - c * kDwAcc;
-    float s = 0.0f;
-    for (int ch = 0; ch < nchunks; ++ch) s += partial[((size_t)ch * g.C + c) * kDwAcc + a];
+    auto total = [&](int row) {
+        return sum_in_order<4, float>(nchunks, [&](int ch) { return __ldg(partial + ((size_t)ch * g.C + c) * kDwAcc + row); });
+    };
+    const float s = total(a);
     const bool two = two_branch(mode);
     const float al = (two && alpha) ? alpha[c] : 1.0f, be = (two && beta) ? beta[c] : 1.0f;
     if (a == 2 * 16 + 2) { if (gbias) gbias[c] = s; return; }
@@ -963,8 +1017,7 @@ __global__ void dw_bwd_finish_kernel(Geo g, const float* __restrict__ partial, i
         if (!gw) return;
         float v = (mode == TCONV_MAX_PLUS) ? 0.0f : al * s;
         if (mode == TCONV_MAX_PLUS || mode == TCONV_COMPOUND) {
-            float smax = 0.0f;
-            for (int ch = 0; ch < nchunks; ++ch) smax += partial[((size_t)ch * g.C + c) * kDwAcc + 16 + tap];
+            const float smax = total(16 + tap);
             v = (mode == TCONV_MAX_PLUS) ? smax : __fmaf_rn(be, smax, v);
         }
         gw[(size_t)c * g.RS + tap] = v;
