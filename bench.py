@@ -50,7 +50,8 @@ PROBES_BF16 = {"max_plus": ("bf16x2_add_max", "bf16x2_fma_max", "bf16x2_mix_max"
                "min_plus": ("bf16x2_add_max", "bf16x2_fma_max", "bf16x2_mix_max"),
                "compound": ("bf16x2_add_minmax", "bf16x2_fma_minmax", "bf16x2_mix_minmax"),
                "parallel": ("bf16x2_2add_minmax", "bf16x2_2fma_minmax", "bf16x2_2mix_minmax")}
-# register-only probes of the winner-emitting Sum-form inner loop (sums, extrema by rows, first equal row and tap)
+# replays of the winner-emitting Sum-form inner loop without its loads of x (sums, extrema by rows, first equal row and
+# tap); compound in two forms (both branches in one pass; "_fb": a pass each), the better counts
 WIN_PROBES = {"compound": "f32_win_compound", "parallel": "f32_win_parallel"}
 
 
@@ -458,8 +459,9 @@ def run_gpu(args):
                                 "and the backward do other work per tap than that mix and are held to the same "
                                 "denominator")}
     if dom_what == "fwd_winners" and dom_mode in WIN_PROBES:
-        # secondary: against a register-only replay of the kernel's own winner-emitting loop
-        roofline["frac_of_own_mix"] = achieved / (probe_rates[WIN_PROBES[dom_mode]] / 1e12)
+        # secondary: against a replay of the kernel's own winner-emitting loop
+        own = WIN_PROBES[dom_mode]
+        roofline["frac_of_own_mix"] = achieved / (max(probe_rates[own], probe_rates[own + "_fb"]) / 1e12)
     fwd_frac = {m: {"ms": per[m]["fwd"], "Ttap_s": L2.taps / (per[m]["fwd"] * 1e-3) / 1e12,
                     "frac_of_alu_peak": L2.taps / (per[m]["fwd"] * 1e-3) / peaks[m],
                     "kernel": per[m]["fwd_kernel"]}
@@ -488,9 +490,10 @@ def run_gpu(args):
             "alu_peak_Ttap_s": {"f32": {m: v / 1e12 for m, v in peaks.items()},
                                 "bf16": {m: v / 1e12 for m, v in peaks16.items()}},
             "alu_probe_Ttap_s": {k: v / 1e12 for k, v in probe_rates.items()},
-            "alu_probe_note": ("register-only loops; plain names advance their operands with extra adds (5 per 64 "
-                               "taps, uncorrected), _fb names feed tap sums back (no extra instruction); a mode's "
-                               "peak is the best of all its mixes in both forms")}
+            "alu_probe_note": ("register-only loops (f32_win_*: weights from shared memory); plain names advance their "
+                               "operands with extra adds (5 per 64 taps, uncorrected), _fb names feed tap sums back (no "
+                               "extra instruction; f32_win_compound_fb: a pass per branch); a mode's peak is the best of "
+                               "all its mixes in both forms")}
     print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()

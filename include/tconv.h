@@ -261,9 +261,9 @@ double tconv_paper_ops(const tconv_desc_t *desc);
 /*
  * Register-only throughput probe of the plain ALUs: every thread of a full-GPU
  * grid runs `iters` rounds of independent add + max/min chains in the
- * instruction mix `variant` (see tconv_alu_probe_name), with no memory traffic,
- * and one result is written to `sink` (device, >= 4 bytes) so the work cannot be
- * elided.  *taps_per_launch (host) receives the number of tropical taps
+ * instruction mix `variant` (see tconv_alu_probe_name), with no memory traffic
+ * (the f32_win mixes read their weights from shared memory), and one result is
+ * written to `sink` (device, >= 4 bytes) so the work cannot be elided.  *taps_per_launch (host) receives the number of tropical taps
  * (one x + w term folded into its running min and/or max) one launch performs.
  * Used to measure the add+max/min roofline the kernels are compared against.
  */

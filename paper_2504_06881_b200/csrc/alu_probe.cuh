@@ -10,29 +10,12 @@
 // iteration forms anyway become the next iteration's x operands, so that every
 // instruction of the loop body is a tap sum or a min / max.
 #pragma once
+#include <type_traits>
+
 #include "tconv_common.cuh"
 #include "tconv_winners.cuh"
 
 namespace tconv {
-
-__device__ __forceinline__ float max3f(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-__device__ __forceinline__ float min3f(float a, float b, float c) {
-    float d;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-// Packed fp32 add: {lo, hi} = {x + wlo, x + whi}, one instruction for two taps.
-__device__ __forceinline__ void add2f(float x, float wlo, float whi, float& lo, float& hi) {
-    unsigned long long xx, ww, tt;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(xx) : "f"(x));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(ww) : "f"(wlo), "f"(whi));
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(tt) : "l"(xx), "l"(ww));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(tt));
-}
 
 #define TCONV_OPAQUE_F(v) asm volatile("" : "+f"(v))
 #define TCONV_OPAQUE_R(v) asm volatile("" : "+r"(v))
@@ -160,67 +143,79 @@ __global__ void __launch_bounds__(256) alu_probe_kernel(int iters, float seed, f
             for (int j = 0; j < PX; ++j) r = __hadd2(r, __hadd2(mx[i][j], mn[i][j]));
         if (__low2float(r) == 12345.678f) sink[0] = __high2float(r);
     } else if constexpr (V == PROBE_F32_WIN_SINGLE || V == PROBE_F32_WIN_COMPOUND || V == PROBE_F32_WIN_PARALLEL) {
-        // The winner-emitting Sum-form inner loop on registers only: per pair of output channels
-        // and pixel, nine packed tap sums, their extrema by rows, the channel combine, the winning
-        // taps (add_winner) and the code bytes.
+        // The winner-emitting Sum-form inner loop: per pair of output channels and pixel, nine packed tap sums, their
+        // extrema by rows, the channel combine, the winning taps (add_winner) and the code bytes; the inputs in
+        // registers, a pass's weights from shared memory as the kernel reads them (another set every other iteration).
+        // Parallel: a pass per branch, as the kernel does.  Compound: one pass with both branches, as the kernel does,
+        // or (FEED) a pass per branch too, the sums formed anew from a second copy of the weights: the better of the two
+        // is what the mix can do (measured 5.68 and 6.04 Ttap/s, parallel 6.04).
         constexpr bool TWOB = (V != PROBE_F32_WIN_SINGLE), PARB = (V == PROBE_F32_WIN_PARALLEL);
-        float x[12], wa[2][9][2], acc[4][4], al[4], be[4];
+        __shared__ __align__(16) float ws[2][2][2][9][2];            // iteration, branch, channel pair, tap, channel
+        for (int e = threadIdx.x; e < 2 * 2 * 2 * 9 * 2; e += blockDim.x) {
+            const int id = V == PROBE_F32_WIN_COMPOUND ? e / 72 * 36 + e % 36 : e;       // (compound: both branches alike)
+            (&ws[0][0][0][0][0])[e] = seed * (float)(id * 37 % 101 + 3);
+        }
+        __syncthreads();
+        float x[12], acc[4][4], al[4], be[4];
         unsigned codes = 0u;
         const float dx = seed * 1.0e-3f;
         for (int j = 0; j < 12; ++j) x[j] = seed * (float)(j + threadIdx.x);
-        for (int kp = 0; kp < 2; ++kp)
-            for (int t = 0; t < 9; ++t)
-                for (int h = 0; h < 2; ++h) {
-                    wa[kp][t][h] = seed * (float)(kp * 18 + t * 2 + h + 3);
-                }
         for (int k = 0; k < 4; ++k) {
             al[k] = seed * (float)(k + 1); be[k] = seed * (float)(k + 2);
             for (int j = 0; j < 4; ++j) acc[k][j] = 0.0f;
         }
+#pragma unroll 1
         for (int it = 0; it < iters; ++it) {
 #pragma unroll
             for (int j = 0; j < 12; ++j) x[j] = __fadd_rn(x[j], dx);     // operands change every iteration
 #pragma unroll
-            for (int kp = 0; kp < 2; ++kp)
-#pragma unroll
-                for (int t = 0; t < 9; ++t) {
-                    TCONV_OPAQUE_F(wa[kp][t][0]); TCONV_OPAQUE_F(wa[kp][t][1]);
-                }
-#pragma unroll
             for (int kp = 0; kp < 2; ++kp) {
-                float cnt[2][2];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float ta[9][2], tb[PARB ? 9 : 1][2];
+                float cnt[2][2] = {{8388608.0f, 8388608.0f}, {8388608.0f, 8388608.0f}};
+                auto pass = [&](auto min_branch, auto max_branch, int branch) {
+                    constexpr bool DO_MIN = decltype(min_branch)::value, DO_MAX = decltype(max_branch)::value;
+                    float wa[9][2];
 #pragma unroll
                     for (int t = 0; t < 9; ++t) {
-                        add2f(x[j + t], wa[kp][t][0], wa[kp][t][1], ta[t][0], ta[t][1]);
-                        if constexpr (PARB) add2f(x[j + t], wa[kp][8 - t][0], wa[kp][8 - t][1], tb[t][0], tb[t][1]);   // (the same registers in another order)
-                    }
-                    const float (*tm)[2] = PARB ? tb : ta;
-                    float lo[2] = {0.0f, 0.0f}, hi[2], rmin[2][3], rmax[2][3];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        hi[h] = fold_rows<3, 3>([&](int t) { return tm[t][h]; }, false, rmax[h]);
-                        if constexpr (TWOB) lo[h] = fold_rows<3, 3>([&](int t) { return ta[t][h]; }, true, rmin[h]);
+                        const float2 v = *reinterpret_cast<const float2*>(ws[it & 1][branch][kp][t]);
+                        wa[t][0] = v.x; wa[t][1] = v.y;
                     }
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        if constexpr (TWOB) {
-                            acc[2 * kp + h][j] = __fmaf_rn(al[2 * kp + h], lo[h], acc[2 * kp + h][j]);
-                            acc[2 * kp + h][j] = __fmaf_rn(be[2 * kp + h], hi[h], acc[2 * kp + h][j]);
-                        } else {
-                            acc[2 * kp + h][j] = __fadd_rn(acc[2 * kp + h][j], hi[h]);
+                    for (int j = 0; j < 4; ++j) {
+                        float t[9][2], lo[2] = {0.0f, 0.0f}, hi[2] = {0.0f, 0.0f}, rmin[2][3], rmax[2][3];
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) add2(x[j + i], wa[i][0], wa[i][1], t[i][0], t[i][1]);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const auto th = [&](int i) { return t[i][h]; };
+                            if constexpr (DO_MIN) lo[h] = fold_rows<3, 3>(th, true, rmin[h]);
+                            if constexpr (DO_MAX) hi[h] = fold_rows<3, 3>(th, false, rmax[h]);
+                        }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            float& a = acc[2 * kp + h][j];
+                            if constexpr (TWOB) {
+                                if constexpr (DO_MIN) a = __fmaf_rn(al[2 * kp + h], lo[h], a);
+                                if constexpr (DO_MAX) a = __fmaf_rn(be[2 * kp + h], hi[h], a);
+                            } else {
+                                a = __fadd_rn(a, hi[h]);
+                            }
+                        }
+                        const float unit = j % 2 ? 256.0f : 1.0f;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const auto th = [&](int i) { return t[i][h]; };
+                            if constexpr (DO_MIN) add_winner<3, 3>(th, rmin[h], lo[h], unit, cnt[h][j / 2]);
+                            if constexpr (DO_MAX) add_winner<3, 3>(th, rmax[h], hi[h], 16.0f * unit, cnt[h][j / 2]);
                         }
                     }
-                    const float unit = j % 2 ? 256.0f : 1.0f;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float& code = cnt[h][j / 2];
-                        if (j % 2 == 0) code = 8388608.0f;
-                        if constexpr (TWOB) add_winner<3, 3>([&](int t) { return ta[t][h]; }, rmin[h], lo[h], unit, code);
-                        add_winner<3, 3>([&](int t) { return tm[t][h]; }, rmax[h], hi[h], 16.0f * unit, code);
-                    }
+                };
+                if constexpr (!TWOB) {
+                    pass(std::false_type(), std::true_type(), 0);
+                } else if constexpr (PARB || FEED) {
+                    pass(std::true_type(), std::false_type(), 0);
+                    pass(std::false_type(), std::true_type(), 1);
+                } else {
+                    pass(std::true_type(), std::true_type(), 0);
                 }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) codes ^= __byte_perm(__float_as_uint(cnt[h][0]), __float_as_uint(cnt[h][1]), 0x5410);
@@ -268,16 +263,16 @@ __global__ void __launch_bounds__(256) alu_probe_kernel(int iters, float seed, f
                     if constexpr (V == PROBE_F32_MAX2_ONLY || V == PROBE_F32_MAX3_ONLY) {
                         ta0 = x[j]; tb0 = w0[i]; ta1 = x[j + 1]; tb1 = w1[i + 1];
                     } else if constexpr (packed) {
-                        add2f(x[j], w0[i], w0[i + 1], ta0, tb0);
-                        add2f(x[j + 1], w1[i], w1[i + 1], ta1, tb1);
+                        add2(x[j], w0[i], w0[i + 1], ta0, tb0);
+                        add2(x[j + 1], w1[i], w1[i + 1], ta1, tb1);
                     } else {
                         ta0 = __fadd_rn(x[j], w0[i]); tb0 = __fadd_rn(x[j], w0[i + 1]);
                         ta1 = __fadd_rn(x[j + 1], w1[i]); tb1 = __fadd_rn(x[j + 1], w1[i + 1]);
                     }
                     if constexpr (par) {
                         if constexpr (packed) {
-                            add2f(x[j], v0[i], v0[i + 1], ua0, ub0);
-                            add2f(x[j + 1], v1[i], v1[i + 1], ua1, ub1);
+                            add2(x[j], v0[i], v0[i + 1], ua0, ub0);
+                            add2(x[j + 1], v1[i], v1[i + 1], ua1, ub1);
                         } else {
                             ua0 = __fadd_rn(x[j], v0[i]); ub0 = __fadd_rn(x[j], v0[i + 1]);
                             ua1 = __fadd_rn(x[j + 1], v1[i]); ub1 = __fadd_rn(x[j + 1], v1[i + 1]);
@@ -296,18 +291,18 @@ __global__ void __launch_bounds__(256) alu_probe_kernel(int iters, float seed, f
                         mx[i + 1][j] = fmaxf(fmaxf(mx[i + 1][j], tb0), tb1);
                     } else if constexpr (V == PROBE_F32_ADD_MAX3 || V == PROBE_F32_ADD2_MAX3 ||
                                          V == PROBE_F32_MAX3_ONLY) {
-                        mx[i][j] = max3f(mx[i][j], ta0, ta1);
-                        mx[i + 1][j] = max3f(mx[i + 1][j], tb0, tb1);
+                        mx[i][j] = ext3(mx[i][j], ta0, ta1, false);
+                        mx[i + 1][j] = ext3(mx[i + 1][j], tb0, tb1, false);
                     } else if constexpr (V == PROBE_F32_ADD_MINMAX2 || V == PROBE_F32_2ADD_MINMAX2) {
                         mx[i][j] = fmaxf(fmaxf(mx[i][j], ua0), ua1);
                         mx[i + 1][j] = fmaxf(fmaxf(mx[i + 1][j], ub0), ub1);
                         mn[i][j] = fminf(fminf(mn[i][j], ta0), ta1);
                         mn[i + 1][j] = fminf(fminf(mn[i + 1][j], tb0), tb1);
                     } else {
-                        mx[i][j] = max3f(mx[i][j], ua0, ua1);
-                        mx[i + 1][j] = max3f(mx[i + 1][j], ub0, ub1);
-                        mn[i][j] = min3f(mn[i][j], ta0, ta1);
-                        mn[i + 1][j] = min3f(mn[i + 1][j], tb0, tb1);
+                        mx[i][j] = ext3(mx[i][j], ua0, ua1, false);
+                        mx[i + 1][j] = ext3(mx[i + 1][j], ub0, ub1, false);
+                        mn[i][j] = ext3(mn[i][j], ta0, ta1, true);
+                        mn[i + 1][j] = ext3(mn[i + 1][j], tb0, tb1, true);
                     }
                 }
 #pragma unroll
