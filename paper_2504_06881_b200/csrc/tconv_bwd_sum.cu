@@ -29,8 +29,14 @@ int launch_gx_window(SumBwdArgs& a, const SumGxPlan& pl, float* part_ab, float* 
 
 template <typename T, int BR, bool PAIRS, bool WIDE>
 int launch_gw(SumBwdArgs& a, const SumGwPlan& pl, float* part) {
+    // fp32, one branch, wide codes: the loop over whole blocks takes 72 registers, seven CTAs an SM where the plan counts on
+    // eight, the loop over whole rounds 60.  Where that second round of CTAs is the price and shares are long, whole rounds:
+    // 24 -> 6 channels 5x5 128x256 N=25 (1116 CTAs of 208 rounds) 81 against 64 us, 64 -> 72 32x32 N=64 (1152 of 512) 186
+    // against 149, 24 -> 24 32x64 N=32 (1152 of 64) 27.7 against 25.5; else blocks: 13 -> 29 16x96 N=50 (1131 of 52) 19.3
+    // against 21.4, 64 -> 64 64x64 N=4 (8192 of 16) 50 against 52.  Blocks within 64 registers spill: 72, 169 and 27.5 us.
+    const bool second = sizeof(T) == 4 && WIDE && BR != 0 && pl.grid > 148 * 7 && pl.grid <= 148 * 8 && pl.per >= 64;
     auto kern = pl.flat ? bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, true, false>
-                : pl.blocks ? bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false, true> : bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false, false>;
+                : pl.blocks && !second ? bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false, true> : bwd_sum_gw_kernel<T, BR, PAIRS, WIDE, false, false>;
     if (allow_smem(kern, kBwdSmemAttr) != cudaSuccess) return TCONV_ERR_CUDA;
     kern<<<pl.grid, 128, pl.smem, a.st>>>(a.g, (const T*)a.gy, a.codes, part, pl);
     ++a.launches;

@@ -3,6 +3,7 @@ and of several whole blocks of 128 quads, rounds that are not whole blocks, flat
 and their last partial round, shares of one block, one or two branches and wide codes; slices of no row to seventeen."""
 import pytest
 
+from nvcc_probe import sum_gw_plans
 from paper_2504_06881_b200 import inputs, tconv
 import parity
 
@@ -37,3 +38,15 @@ def test_partial_rows(N):
     """4, 16, 20, 120, 128, 132 rows of grad_alpha / grad_beta (four tiles an image), then one an image, in sixteen slices."""
     parity.check_layer(dict(L(N, 2, 16, 64, 5, pad=1), mode="compound", chan="sum", dtype="f32"), None, 2800 + N, recompute=False)
     assert tconv.tconv_last_kernel() == "bwd_sum"
+
+
+@pytest.mark.parametrize("mode", ["max_plus", "min_plus"])
+def test_one_round_of_eight(mode):
+    """fp32, one branch, wide codes: more CTAs than seven per SM, with shares of 52 rounds (whole blocks) and of 64 (whole rounds)."""
+    layers = [L(50, 13, 16, 96, 29, R=5, S=5, pad=2), L(32, 24, 32, 64, 24, R=5, S=5, pad=2)]
+    for i, (d, per) in enumerate(zip(layers, (52, 64))):
+        d = dict(d, mode=mode, chan="sum", dtype="f32")
+        plan, = sum_gw_plans([d])
+        assert plan["blocks"] and plan["per"] == per and 148 * 28 < d["C"] * d["K"] * plan["splits"] <= 148 * 32
+        parity.check_layer(d, None, 2900 + i, recompute=False)
+        assert tconv.tconv_last_kernel() == "bwd_sum"
