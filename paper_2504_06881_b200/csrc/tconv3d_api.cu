@@ -183,19 +183,21 @@ int forward1d_t(const Geo3& g, const void* x, const void* w, const void* w2, con
     const size_t wcopy = (size_t)q4 * g.sw * kb * (br == 3 ? 2 : 1);
     const size_t smem = (size_t)g.sw * f1_xw(q4) * sizeof(T) + wcopy * 4 + (winners ? wcopy * sizeof(T) : 0);
     const dim3 grid((unsigned)((g.OW + kF1Pos - 1) / kF1Pos), (unsigned)((g.K + kb - 1) / kb), (unsigned)g.N);
+    const bool few = (double)grid.x * grid.y * grid.z <= 148.0 * 4;
     // (long windows with winners in parallel mode stage up to 67 KB: above the default limit)
-#define TCONV1_LAUNCH(STV, BRV, WINV)                                                     \
+#define TCONV1_LAUNCH(...)                                                                \
     {                                                                                     \
         if (smem > 48 * 1024 &&                                                           \
-            allow_smem(fwd1d_kernel<T, STV, BRV, WINV>, (int)kSmem1d) != cudaSuccess)     \
+            allow_smem(fwd1d_kernel<T, __VA_ARGS__>, (int)kSmem1d) != cudaSuccess)        \
             return TCONV_ERR_CUDA;                                                        \
-        fwd1d_kernel<T, STV, BRV, WINV><<<grid, kF1Threads, smem, st>>>(                   \
+        fwd1d_kernel<T, __VA_ARGS__><<<grid, kF1Threads, smem, st>>>(                      \
             g, q4, (const T*)x, (const T*)w, (const T*)w2, alpha, beta, bias, (T*)y, winners); \
     }
-#define TCONV1_BY_WIN(STV, BRV)                                  \
-    {                                                            \
-        if (winners) TCONV1_LAUNCH(STV, BRV, true)               \
-        else TCONV1_LAUNCH(STV, BRV, false)                      \
+#define TCONV1_BY_WIN(STV, BRV)                                                        \
+    {                                                                                  \
+        if (winners) TCONV1_LAUNCH(STV, BRV, true)                                     \
+        else if (few) TCONV1_LAUNCH(STV, BRV, false, f1_split(sizeof(T), STV, BRV))    \
+        else TCONV1_LAUNCH(STV, BRV, false)                                            \
     }
 #define TCONV1_BY_BR(STV)                                        \
     {                                                            \

@@ -81,6 +81,22 @@ __host__ __device__ constexpr int f1_blocks(int esize, int st, int br) {
     return esize == 2 || (br < 2 && st < 4) ? 0 : br >= 2 && st == 4 ? 3 : 4;
 }
 
+// The same for the kernels without winners.  With a bound of one all of these took 95 to 146 registers, which cost the
+// layers of many blocks up to two thirds; without one the compiler takes 64 to 119, which costs the layers of few blocks
+// up to a quarter.  So where four blocks per SM hold the whole grid (FEW) the kernel has a bound of four, else none; fp32
+// with one branch and at stride 4 has one bound that is good for both.  None / one / as chosen, us: fp32 max-plus 64 -> 64
+// channels k=5 stride 2 N=32 L=2000 152 / 253 / 153, k=9 stride 4 L=4000 260 / 354 / 257; compound 64 -> 128 k=3 N=16
+// L=4000 576 / 679 / 576, 40 -> 40 k=9 stride 2 N=1 103 / 91 / 91, 16 -> 64 k=33 stride 4 N=1 L=9000 78 / 64 / 64; parallel
+// k=33 94 / 74 / 74; bf16 compound 64 -> 64 k=11 N=32 209 / 266 / 209, parallel 64 -> 128 k=3 N=16 538 / 696 / 538,
+// max-plus 32 -> 64 k=8 stride 4 N=16 86 / 76 / 78, 64 -> 128 k=3 273 / 303 / 273.
+__host__ __device__ constexpr int f1_blocks_plain(int esize, int st, int br, bool few) {
+    if (esize == 4 && br == 2 && st == 4) return 1;
+    return (esize == 4 && (br < 2 || st == 4)) || few ? 4 : 0;
+}
+__host__ __device__ constexpr bool f1_split(int esize, int st, int br) {
+    return f1_blocks_plain(esize, st, br, true) != f1_blocks_plain(esize, st, br, false);
+}
+
 // Row pitch of the staged signal segment: the window of the last lane ends at 4 * 31 + q4 + 3.
 __host__ __device__ constexpr int f1_xw(int q4) { return (kF1Pos + q4 + 4 + 7) & ~7; }
 
@@ -91,8 +107,8 @@ __host__ __device__ constexpr int f1_xw(int q4) { return (kF1Pos + q4 + 4 + 7) &
 // s >= S; bf16 layers keep them as 4-byte {w, w} pairs), twice in parallel mode.  q4 = ceil(S / ST)
 // rounded up to a multiple of four.  WIN: a second copy of the weights by output channel follows,
 // wst[4 * KT][q4 * ST] in the layer's type (twice in parallel mode).
-template <typename T, int ST, int BR, bool WIN>
-__global__ void __launch_bounds__(kF1Threads, WIN ? f1_blocks(sizeof(T), ST, BR) : 1)
+template <typename T, int ST, int BR, bool WIN, bool FEW = false>
+__global__ void __launch_bounds__(kF1Threads, WIN ? f1_blocks(sizeof(T), ST, BR) : f1_blocks_plain(sizeof(T), ST, BR, FEW))
 fwd1d_kernel(Geo3 g, int q4, const T* __restrict__ x, const T* __restrict__ w, const T* __restrict__ w2,
              const float* __restrict__ alpha, const float* __restrict__ beta,
              const float* __restrict__ bias, T* __restrict__ y, void* __restrict__ winners) {

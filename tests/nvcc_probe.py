@@ -45,7 +45,7 @@ def sum_gw_plans(layers):
 
 
 def resources(header, kernels):
-    """{instance: (registers, bytes of spill stores)} of kernel instances like "fwd1d_kernel<float, 1, 1, true>"."""
+    """{instance: (registers, bytes of spill stores)} of kernel instances like "bwd_sum_finish_kernel<16>"."""
     with tempfile.TemporaryDirectory() as tmp:
         src = Path(tmp) / "probe.cu"
         src.write_text(f'#include "{header}"\nusing namespace tconv;\nvoid* const table[] = {{' +

@@ -93,3 +93,16 @@ def test_audio_opening_layer_at_the_benchmark_size(mode, dtype, N):
     window 80, stride 4), in full against the oracle: forward, winners and every gradient (the bf16
     oracle is slower: four signals)."""
     check(layer1d(N, 1, 16000, 128, 80, stride=4, mode=mode, dtype=dtype), 1300)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("mode,chan", [("max_plus", "default"), ("compound", "default"), ("parallel", "default")])
+@pytest.mark.parametrize("stride", [1, 2, 4])
+def test_grids_around_four_blocks_per_sm(mode, chan, dtype, stride):
+    """Without winners 592 blocks and 593 run different instances (single branches: 32 output channels per block)."""
+    kb = 32 if mode in ("max_plus", "min_plus") else 16
+    for blocks in (592, 593):
+        positions = 128 * (blocks // (16 if blocks == 592 else 1)) - 127
+        d = layer1d(16 if blocks == 592 else 1, 1, positions * stride + 4, kb - 3, 5, stride=stride, mode=mode, chan=chan, dtype=dtype)
+        assert -(-inputs.output_dhw(d)[2] // 128) * d["N"] == blocks
+        check(d, 1400 + blocks)

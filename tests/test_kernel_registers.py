@@ -10,10 +10,19 @@ FILE = 65536     # registers of an SM
 @pytest.mark.parametrize("dtype", ["float", "__nv_bfloat16"])
 def test_1d_forward_with_winners(dtype):
     """Four blocks of 128 threads; three at stride 4 with two branches."""
-    most = {f"fwd1d_kernel<{dtype}, {st}, {br}, true>": FILE // 128 // (3 if st == 4 and br == 3 else 4)
+    most = {f"fwd1d_kernel<{dtype}, {st}, {br}, true, false>": FILE // 128 // (3 if st == 4 and br == 3 else 4)
             for st in (1, 2, 4) for br in (1, 3)}
     got = resources("tconv_1d.cuh", list(most))
     assert all(got[k][0] <= most[k] // 8 * 8 for k in most), got
+
+
+@pytest.mark.parametrize("dtype", ["float", "__nv_bfloat16"])
+def test_1d_forward_without_winners(dtype):
+    """Four blocks of 128 threads; five with two branches and more blocks than four per SM hold."""
+    most = {f"fwd1d_kernel<{dtype}, {st}, {br}, false, {few}>": FILE // 128 // (5 if br >= 2 and few == "false" else 4)
+            for st in (1, 2, 4) for br in (1, 2, 3) for few in ("false", "true") if not (dtype == "float" and st == 4)}
+    got = resources("tconv_1d.cuh", list(most))
+    assert all(got[k][0] <= most[k] // 8 * 8 and got[k][1] <= 32 for k in most), got
 
 
 @pytest.mark.parametrize("dtype", ["float", "__nv_bfloat16"])
