@@ -18,7 +18,7 @@ LAYERS = [
     L(2, 2, 32, 48, 3, pad=1),                           # three blocks an image
     L(1, 2, 11, 23, 3, pad=1),                           # flattened: 66 quads
     L(4, 3, 24, 16, 5, pad=0),                           # flattened: 88 quads an image, 11 rounds
-    L(7, 2, 13, 61, 4, pad=1),                           # flattened: shares that start inside an image
+    L(7, 2, 13, 61, 4, pad=1),                           # flattened: 208 quads an image, 45 rounds and a last one of 16 lanes
     L(32, 1, 20, 20, 2, pad=1),                          # flattened: 100 rounds, a last one of 4 lanes
     L(3, 2, 16, 32, 3, R=5, S=5, pad=2),                 # wide codes, one block
     L(3, 2, 9, 21, 3, R=5, S=5, pad=2),                  # wide codes, flattened
@@ -50,3 +50,18 @@ def test_one_round_of_eight(mode):
         assert plan["blocks"] and plan["per"] == per and 148 * 28 < d["C"] * d["K"] * plan["splits"] <= 148 * 32
         parity.check_layer(d, None, 2900 + i, recompute=False)
         assert tconv.tconv_last_kernel() == "bwd_sum"
+
+
+@pytest.mark.parametrize("mode,layer", [("compound", L(40, 3, 11, 23, 4, pad=1)), ("parallel", L(9, 3, 31, 37, 4, pad=1)),
+                                        ("max_plus", L(17, 3, 13, 61, 4, pad=1)), ("compound", L(17, 3, 13, 61, 4, R=5, S=5, pad=2)),
+                                        ("min_plus", L(64, 3, 11, 23, 4, R=5, S=5, pad=2))])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_flattened_shares(mode, layer, dtype):
+    """Several shares of more than twelve rounds that start and end inside an image; the last one shorter in three layers."""
+    d = dict(layer, mode=mode, chan="sum", dtype=dtype)
+    OH, OW = inputs.output_hw(d)
+    quads = OH * ((OW + 3) // 4)
+    plan, = sum_gw_plans([d])
+    assert plan["flat"] and plan["splits"] >= 6 and plan["per"] > 12 * 32 and plan["per"] % quads and plan["per"] % 32
+    parity.check_layer(d, None, 2950, recompute=False)
+    assert tconv.tconv_last_kernel() == "bwd_sum"
