@@ -441,8 +441,8 @@ fwd_tiled_f32_kernel(const __grid_constant__ CUtensorMap xmap, const TiledParams
                 // registers, give the extrema row by row and then the winning taps (add_winner), which are counted
                 // into floats from 2^23 on: byte (RS > 16: 16 bits) j of the mantissas holds argmin + 16 argmax
                 // (256 argmax) of pixel j.
-                // Bound by the half-rate pipe (71 % of its slots: 16 three-input min / max, 8 compares, 8 selects per
-                // (output, input channel) with two branches) and its dependences: N=128 C=64 K=64 32x32 fp32,
+                // Bound by the half-rate pipe (71 % of its slots: 8 three-input min / max, 8 compares, 6.5 selects per
+                // (output, input channel) with two branches, 4.5 selects in parallel) and its dependences: N=128 C=64 K=64 32x32 fp32,
                 // compound 1285 -> 947 us, parallel 1377 -> 1040 us against keys formed from every tap by two packed
                 // FMAs (exact only for |x + w| < 2^95).  Four CTAs per SM, eight or two channels per thread, and
                 // selects as predicated FMAs measured the same or slower.

@@ -20,16 +20,13 @@ __device__ __forceinline__ void add2(float x, float wlo, float whi, float& lo, f
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(tt) : "l"(xx), "l"(ww));
     asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(tt));
 }
-// Extremum of N values with 3-input min / max: a fresh chain opens with three values, every later step folds two more.
+// Extremum of N values (N odd) with 3-input min / max: a fresh chain opens with three values, every later step folds two more.
 template <int N>
 __device__ __forceinline__ float fold_values(const float* v, bool is_min) {
-    float m;
-    if constexpr (N >= 3) m = ext3(v[0], v[1], v[2], is_min);
-    else if constexpr (N == 2) m = ext2(v[0], v[1], is_min);
-    else m = v[0];
+    static_assert(N % 2 == 1, "windows of 1, 3 or 5");
+    float m = v[0];
 #pragma unroll
-    for (int i = 3; i + 1 < N; i += 2) m = ext3(m, v[i], v[i + 1], is_min);
-    if constexpr (N > 3 && ((N - 3) & 1)) m = ext2(m, v[N - 1], is_min);
+    for (int i = 1; i < N; i += 2) m = ext3(m, v[i], v[i + 1], is_min);
     return m;
 }
 // Extremum of the R x S tap sums t(.), row by row; row[r] keeps the rows' own.
